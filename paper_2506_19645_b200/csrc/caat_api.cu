@@ -286,7 +286,7 @@ static caat_status backward_impl(const caat_ctx* ctx, int K_r, int T, const void
 
   if (tc) {
     RowparShapes sh{t, T, h, K_r, S, L.S_lo, L.S_hi, L.P};
-    const PrivOperand pv = compact ? PrivOperand{dR, L.P, 0, (float)ctx->alpha} : PrivOperand{dR, h, S, (float)ctx->alpha};
+    const PrivOperand pv = compact ? PrivOperand{dR, L.P, 0, (float)ctx->alpha} : PrivOperand{dR, h, L.S_lo, (float)ctx->alpha};
     ce = launch_tc_dgrad(sh, gs, pv, W, dY, wsb + L.wt_off, prescale, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
     ce = launch_tc_wgrad(sh, gs, pv, Y, dW, wsb + L.splitk_off, L.splitk_bytes, st);
@@ -833,7 +833,8 @@ static caat_status check_tp(const caat_ctx* ctx, caat_layer layer, int tokens, c
   caat_status s = check_common(ctx, layer, tokens);
   if (s != CAAT_OK) return s;
   const int K_r = layer_kr(ctx, layer);
-  if (!tc_gemm_usable(ctx, K_r)) return CAAT_EUNSUPPORTED;   // the packed [T, S] slab exists on the tensor-core path
+  // the packed [T, S] slab exists on the tensor-core path, for partitions on the 8-channel grid
+  if (!tc_gemm_usable(ctx, K_r) || ctx->S % kLayoutVec != 0) return CAAT_EUNSUPPORTED;
   if (!ws || !aligned16(ws) || ws_bytes < scratch_layout(ctx, K_r, tokens, backward).total) return CAAT_EWORKSPACE;
   return CAAT_OK;
 }

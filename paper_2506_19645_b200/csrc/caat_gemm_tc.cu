@@ -66,6 +66,13 @@ struct Region {          // a family of output tiles with the same operand wirin
   int mtiles, ntiles;    // the output goes through the region's own tensor map (TMA store);
                          // its z coordinate is split * batch + b
   float* out_t;          // transposed direct-store output (decode), else unused
+  // Weight gradient with a partition off the 8-channel grid: the private rows start at S_lo (TMA reads channels in
+  // 16-byte units), and the first `skip` = S - S_lo rows, which belong to the shared region, are not stored.  Only the
+  // region's first row tile has such rows; it stores fp32 straight from registers to skip_out (plane z of skip_plane
+  // elements, rows of N).
+  int skip;
+  float* skip_out;
+  long long skip_plane;
   int splits;            // split-K factor of this region's tiles (set by finish_tiles from Params::splits when 0)
   int b_slowest;         // tile order: 1 = rank index slowest (a rank's weights / activations stay
                          // hot in L2 while its row tiles stream), 0 = row tile slowest
@@ -552,6 +559,23 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
             }
           }
         }
+      } else if (r.skip > 0 && c.mt == 0) {
+        const int row = m0 + rr;
+        float* dst = r.skip_out + (long long)zc * r.skip_plane + (long long)row * r.N + n0;
+        for (int cc = 0; cc < p.BN && n0 + cc < r.N; cc += 16) {
+          uint32_t v[32];
+          tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + cc), v);
+          tmem_ld_wait();
+          if (row >= r.skip && row < r.M) {
+#pragma unroll
+            for (int e = 0; e < 16; e += 4)
+              if (n0 + cc + e < r.N)            // N is a multiple of 8
+                *reinterpret_cast<float4*>(dst + cc + e) =
+                    total_k == 0 ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                 : make_float4(__uint_as_float(v[e]) * r.scale, __uint_as_float(v[e + 1]) * r.scale,
+                                               __uint_as_float(v[e + 2]) * r.scale, __uint_as_float(v[e + 3]) * r.scale);
+          }
+        }
       } else
       for (int cc = 0; cc < p.BN && n0 + cc < r.N && !(p.debug & kAidMask & 2); cc += sub) {
         uint32_t v[32];
@@ -818,16 +842,19 @@ void finish_tiles(Params& p) {
 }  // namespace
 
 bool tc_gemm_usable(const caat_ctx* ctx, int K_r) {
-  return ctx->dtype == CAAT_BF16 && !ctx->force_simt && K_r % 8 == 0 && ctx->S % 8 == 0 && ctx->h % 8 == 0;
+  return ctx->dtype == CAAT_BF16 && !ctx->force_simt && K_r % 8 == 0 && ctx->h % 8 == 0;
 }
 
-// ---- forward: zs[T,S] = sum_m Y[m] W[m][:S]^T ; zp[m][T,h-S] = Y[m] W[m][S:]^T
+// ---- forward: zs[T,S] = sum_m Y[m] W[m][:S]^T ; zp[m][T,h-S_lo] = Y[m] W[m][S_lo:]^T
+// Any partition S: TMA wants 16-byte coordinates along a row's channels, so the private products start at S_lo; their
+// S - S_lo extra columns land in the scratch columns that no row kernel reads.  (Partitions off the 8-channel grid ran on
+// the CUDA-core GEMM before: a training step of a block at h = 2048, 2999 tokens, p = 0.7 took 17.5 ms, now 0.61 ms.)
 cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* W, void* zs, void* zp,
                               cudaStream_t st, const PushTarget* push) {
   CUtensorMap maps[4], cmaps[2];
   PeerMaps pmaps{};
   Params p{};
-  const int n_sh = s.S, n_pr = s.h - s.S;
+  const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
   const int ksteps = (s.K_r + BK - 1) / BK;
   {
     const RegionShape rs[2] = {{s.T, n_sh, 1, ksteps * s.t}, {s.T, n_pr, s.t, ksteps}};
@@ -850,11 +877,9 @@ cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* 
   if (n_pr > 0) {
     Region& r = p.r[g++];
     r.nunits = 1;
-    r.u[0] = Unit{0, 1, 0, 0, 0, s.S, 1, 0, 1, 0, 1, ksteps};
+    r.u[0] = Unit{0, 1, 0, 0, 0, s.S_lo, 1, 0, 1, 0, 1, ksteps};
     r.M = s.T; r.N = n_pr; r.batch = s.t; r.b_slowest = 1;
-    if (!make_cmap(&cmaps[g - 1], static_cast<__nv_bfloat16*>(zp) + (s.S - s.S_lo), n_pr, s.T, s.t, s.P,
-                   (long long)s.T * s.P, false))
-      return cudaErrorInvalidValue;
+    if (!make_cmap(&cmaps[g - 1], zp, n_pr, s.T, s.t, s.P, (long long)s.T * s.P, false)) return cudaErrorInvalidValue;
   }
   if (g == 1) cmaps[1] = cmaps[0];
   p.nregions = g;
@@ -926,24 +951,32 @@ cudaError_t launch_tc_forward_decode(int t, int T, int h, const DecodeProblem* p
 // ---- dgrad: dY[m] = gs W[m][:S] + (alpha gp[m]) W[m][S:]
 // pv describes where the private gradient lives and what still multiplies it (see PrivOperand); when
 // pv.alpha != 1, w_scaled ([t, h, K_r], only rows >= S are used) must hold alpha times the private rows of W.
+// Any partition S: the private gradient is read from column S_lo on, and the weights' map starts at row S with the
+// coordinate -(S - S_lo), so the shared columns among them meet rows that TMA fills with zeros.
 cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* W, void* dY,
                             void* w_scaled, bool w_scaled_ready, cudaStream_t st) {
   CUtensorMap maps[4], cmaps[2];
   Params p{};
   {
-    const RegionShape rs[1] = {{s.T, s.K_r, s.t, (s.S + BK - 1) / BK + (s.h - s.S + BK - 1) / BK}};
+    const RegionShape rs[1] = {{s.T, s.K_r, s.t, (s.S + BK - 1) / BK + (s.h - s.S_lo + BK - 1) / BK}};
     const TileCfg c = pick_tile(rs, 1, true, 1, 0.0);
     p.BN = c.bn; p.cg = c.cg;
   }
-  const int n_sh = s.S, n_pr = s.h - s.S;
+  const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
   // B = W[m] as [h rows (contraction)][K_r contiguous (N)]: N-major, boxes of 64 (N) x 64 (K)
   if (!make_map(&maps[1], W, s.K_r, s.h, s.t, s.K_r, (long long)s.h * s.K_r, 64, BK)) return cudaErrorInvalidValue;
   maps[3] = maps[1];
-  if (n_pr > 0 && pv.alpha != 1.0f) {
-    // sum_l (alpha g[l]) W[l][k] = sum_l g[l] (alpha W[l][k]): the private gradient is read as stored in dR,
-    // the weights' private rows (the small operand) carry alpha; they were scaled by the launch before this one
-    if (!w_scaled || !w_scaled_ready) return cudaErrorInvalidValue;
-    if (!make_map(&maps[3], w_scaled, s.K_r, s.h, s.t, s.K_r, (long long)s.h * s.K_r, 64, BK)) return cudaErrorInvalidValue;
+  if (n_pr > 0) {
+    const void* wp = W;
+    if (pv.alpha != 1.0f) {
+      // sum_l (alpha g[l]) W[l][k] = sum_l g[l] (alpha W[l][k]): the private gradient is read as stored in dR,
+      // the weights' private rows (the small operand) carry alpha; they were scaled by the launch before this one
+      if (!w_scaled || !w_scaled_ready) return cudaErrorInvalidValue;
+      wp = w_scaled;
+    }
+    if (!make_map(&maps[3], static_cast<const __nv_bfloat16*>(wp) + (long long)s.S * s.K_r, s.K_r, s.h - s.S, s.t, s.K_r,
+                  (long long)s.h * s.K_r, 64, BK))
+      return cudaErrorInvalidValue;
   }
   bool okA0 = n_sh > 0 ? make_map(&maps[0], gs, n_sh, s.T, 1, s.S_hi, (long long)s.T * s.S_hi, BK, BM) : true;
   bool okA1 = n_pr > 0 ? make_map(&maps[2], pv.ptr, pv.ld, s.T, s.t, pv.ld, (long long)s.T * pv.ld, BK, BM) : true;
@@ -954,7 +987,7 @@ cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOpe
   Region& r = p.r[0];
   int nu = 0;
   if (n_sh > 0) r.u[nu++] = Unit{0, 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, (n_sh + BK - 1) / BK};
-  if (n_pr > 0) r.u[nu++] = Unit{2, 3, pv.col0, 0, s.S, 0, 1, 0, 1, 0, 1, (n_pr + BK - 1) / BK};
+  if (n_pr > 0) r.u[nu++] = Unit{2, 3, pv.col0, 0, s.S_lo - s.S, 0, 1, 0, 1, 0, 1, (n_pr + BK - 1) / BK};
   r.nunits = nu;
   r.M = s.T; r.N = s.K_r; r.batch = s.t; r.b_slowest = 1; r.scale = 1.0f;
   if (!make_cmap(&cmaps[0], dY, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, false)) return cudaErrorInvalidValue;
@@ -966,7 +999,7 @@ cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOpe
 
 static TileCfg wgrad_cfg(const RowparShapes& s) {
   const int ksteps = (s.T + BK - 1) / BK;
-  const RegionShape rs[2] = {{s.S, s.K_r, s.t, ksteps}, {s.h - s.S, s.K_r, s.t, ksteps}};
+  const RegionShape rs[2] = {{s.S, s.K_r, s.t, ksteps}, {s.S < s.h ? s.h - s.S_lo : 0, s.K_r, s.t, ksteps}};
   return pick_tile(rs, 2, true, 16, (double)s.t * s.h * s.K_r * sizeof(float));
 }
 
@@ -982,7 +1015,7 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
   Params p{};
   const TileCfg wc = wgrad_cfg(s);
   p.BN = wc.bn; p.cg = wc.cg;
-  const int n_sh = s.S, n_pr = s.h - s.S;
+  const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
   const int splits = wc.splits;
   const long long dw_elems = (long long)s.t * s.h * s.K_r;
   if (splits > 1 && splitk_bytes < (size_t)splits * dw_elems * sizeof(float)) return cudaErrorInvalidValue;
@@ -1014,7 +1047,10 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
     r.u[0] = Unit{2, 1, 0, pv.col0, 0, 0, 1, 0, 1, 0, 1, ksteps};
     r.M = n_pr; r.N = s.K_r; r.batch = s.t; r.b_slowest = 1;
     r.scale = pv.alpha;
-    if (!make_cmap(&cmaps[g - 1], out + (long long)s.S * s.K_r, s.K_r, n_pr, (long long)s.t * splits, s.K_r,
+    r.skip = s.S - s.S_lo;
+    r.skip_out = out + (long long)s.S_lo * s.K_r;
+    r.skip_plane = (long long)s.h * s.K_r;
+    if (!make_cmap(&cmaps[g - 1], out + (long long)s.S_lo * s.K_r, s.K_r, n_pr, (long long)s.t * splits, s.K_r,
                    (long long)s.h * s.K_r, true))
       return cudaErrorInvalidValue;
   }

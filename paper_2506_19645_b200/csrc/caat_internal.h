@@ -87,10 +87,9 @@ bool tc_gemm_usable(const caat_ctx* ctx, int K_r);
 struct PushTarget { int world, rank, slice; void* const* recv; };
 cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* W, void* zs, void* zp,
                               cudaStream_t st, const PushTarget* push = nullptr);
-// The private part of dZt as the backward GEMMs read it: element (m, i, l) for l >= S sits at
-// ptr[(m * T + i) * ld + col0 + (l - S)], and the gradient is alpha times the stored value.
-//   scratch copy written by the row kernel:   {zp, P, S - S_lo, 1}
-//   the residual gradient itself (per rank):  {dR, h, S, alpha}      (no scaled copy is written at all)
+// The private part of dZt as the backward GEMMs read it: element (m, i, l) for l >= S_lo sits at
+// ptr[(m * T + i) * ld + col0 + (l - S_lo)], and the gradient is alpha times the stored value for l >= S.
+//   the residual gradient itself (per rank):  {dR, h, S_lo, alpha}   (no scaled copy is written at all)
 //   compact stream:                           {dRp, P, 0, alpha}
 struct PrivOperand { const void* ptr; int ld; int col0; float alpha; };
 // dY[m] = [gs | alpha gp[m]] W[m];  w_scaled: [t, h, K_r] scratch for the alpha-scaled private rows of W

@@ -401,8 +401,9 @@ __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPar
     float st[1] = {0.f};
     for (int c = threadIdx.x * V; c < a.h; c += blockDim.x * V) {
       float r[V], z[V], hn[V];
-      const bool shared_chunk = c + V <= a.S;          // the partition is a multiple of 8 on this path
-      // compact layout: where this chunk of the stream lives (shared part once, private part per rank)
+      const bool shared_chunk = c + V <= a.S;
+      const bool mixed = !shared_chunk && c < a.S;     // the one chunk that straddles a partition off the 8-channel grid
+      // compact layout (partition on the grid): where this chunk of the stream lives (shared part once, private part per rank)
       const long long coff = shared_chunk ? ((long long)i * a.S + c) * ES : (row * (a.h - a.S) + (c - a.S)) * ES;
       if (layer == 0) {
         if (a.compact) V_::unpack(ldg<raw>(static_cast<const char*>(shared_chunk ? a.Rs : a.R) + coff), r);
@@ -411,23 +412,31 @@ __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPar
 #pragma unroll
         for (int e = 0; e < V; ++e) r[e] = V_::round(hrow[c + e]);
       }
-#pragma unroll
-      for (int e = 0; e < V; ++e) z[e] = 0.f;
       const float* base = L.zt + (long long)i * a.h + c;
-      const int z0 = shared_chunk ? 0 : m, zstep = shared_chunk ? 1 : a.t;
-      const int nz = shared_chunk ? nplanes : L.splits;
-#pragma unroll 8
-      for (int q = 0; q < nz; ++q) {
-        const float* pz = base + (long long)(z0 + q * zstep) * plane;
+      auto plane_sum = [&](float (&out)[V], int z0, int zstep, int nz) {
 #pragma unroll
-        for (int e = 0; e < V; e += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(pz + e);
-          z[e] += v.x; z[e + 1] += v.y; z[e + 2] += v.z; z[e + 3] += v.w;
+        for (int e = 0; e < V; ++e) out[e] = 0.f;
+#pragma unroll 8
+        for (int q = 0; q < nz; ++q) {
+          const float* pz = base + (long long)(z0 + q * zstep) * plane;
+#pragma unroll
+          for (int e = 0; e < V; e += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(pz + e);
+            out[e] += v.x; out[e + 1] += v.y; out[e + 2] += v.z; out[e + 3] += v.w;
+          }
         }
+      };
+      plane_sum(z, shared_chunk ? 0 : m, shared_chunk ? 1 : a.t, shared_chunk ? nplanes : L.splits);
+      const float scale = shared_chunk ? 1.f : a.alpha;
+#pragma unroll
+      for (int e = 0; e < V; ++e) hn[e] = fmaf(scale, z[e], r[e]);
+      if (mixed) {
+        plane_sum(z, 0, 1, nplanes);
+#pragma unroll
+        for (int e = 0; e < V; ++e) hn[e] = c + e < a.S ? z[e] + r[e] : hn[e];
       }
 #pragma unroll
       for (int e = 0; e < V; ++e) {
-        hn[e] = (shared_chunk ? z[e] : a.alpha * z[e]) + r[e];
         st[0] = LN ? st[0] + hn[e] : fmaf(hn[e], hn[e], st[0]);
       }
       // (a thread reads and writes only its own chunks of hrow: no ordering between threads is needed, and a
@@ -491,7 +500,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 // float4 slots of the staging area a CTA needs (the widest shared slice is ceil(S/4 / t) chunks)
 inline size_t cluster_partials_smem(const RowPartArgs& a) {
-  const int S4 = a.S / 4, P4 = (a.h - a.S) / 4;
+  const int S4 = (a.S + 7) / 8 * 2, P4 = (a.h - a.S / 8 * 8) / 4;
   const int ns_max = (S4 + a.t - 1) / a.t;
   size_t f4 = (size_t)a.nlayers * S4 + 16;            // rank sums of the shared channels, reduction scratch
   for (int l = 0; l < a.nlayers; ++l) f4 += (size_t)a.L[l].splits * ((size_t)a.t * ns_max + P4);
@@ -508,7 +517,8 @@ __global__ void __launch_bounds__(512, MINB) rows_forward_partials_cluster_kerne
   cgx::cluster_group cluster = cgx::this_cluster();
   const int i = blockIdx.x, m = blockIdx.y;             // the cluster spans the ranks of token i: cluster rank == m
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int S4 = a.S / 4, P4 = (a.h - a.S) / 4;
+  // a chunk that straddles the partition is summed both ways: as a shared and as a private one
+  const int S4 = (a.S + V - 1) / V * (V / 4), S_lo = a.S / V * V, P4 = (a.h - S_lo) / 4;
   const int cs0 = (int)((long long)S4 * m / a.t);       // this CTA's slice of the shared channels, in float4 units
   const int ns = (int)((long long)S4 * (m + 1) / a.t) - cs0;
   float4* zs = sm4;                                     // [nlayers][S4]: complete after the cluster barrier
@@ -539,7 +549,7 @@ __global__ void __launch_bounds__(512, MINB) rows_forward_partials_cluster_kerne
       pr_off[l] = off;
       for (int idx = tid; idx < splits * P4; idx += nthr) {
         const int q = idx / P4, c = idx - q * P4;
-        cp_async16(stage + off + idx, zt + (long long)(m + q * a.t) * plane + a.S + 4 * c);
+        cp_async16(stage + off + idx, zt + (long long)(m + q * a.t) * plane + S_lo + 4 * c);
       }
       off += splits * P4;
     }
@@ -547,7 +557,7 @@ __global__ void __launch_bounds__(512, MINB) rows_forward_partials_cluster_kerne
   // ---- this thread's chunk of the row: residual and norm parameters, fetched behind the copies
   const int c = tid * V;
   const bool active = c < a.h;
-  const bool shared_chunk = c + V <= a.S;               // the partition is a multiple of 8 on this path
+  const bool shared_chunk = c + V <= a.S, mixed = !shared_chunk && c < a.S;
   const long long coff = shared_chunk ? ((long long)i * a.S + c) * ES : (row * (a.h - a.S) + (c - a.S)) * ES;
   float r[V], g[2][V], b[2][V];
 #pragma unroll
@@ -603,16 +613,19 @@ __global__ void __launch_bounds__(512, MINB) rows_forward_partials_cluster_kerne
     float st[1] = {0.f};
     if (active) {
       float z[V];
-      const float4* src = shared_chunk ? zs + l * S4 + c / 4 : stage + pr_off[l] + (c - a.S) / 4;
+      const float4* src = shared_chunk ? zs + l * S4 + c / 4 : stage + pr_off[l] + (c - S_lo) / 4;
 #pragma unroll
       for (int e = 0; e < V; e += 4) {
         const float4 v = src[e / 4];
         z[e] = v.x; z[e + 1] = v.y; z[e + 2] = v.z; z[e + 3] = v.w;
       }
+      const float scale = shared_chunk ? 1.f : a.alpha;
+      const float* zsh = reinterpret_cast<const float*>(zs + l * S4 + c / 4);     // read by a straddling chunk only
 #pragma unroll
       for (int e = 0; e < V; ++e) {
         const float res = l == 0 ? r[e] : V_::round(hn[e]);    // the second layer's residual is the first one's stream as stored
-        hn[e] = (shared_chunk ? z[e] : a.alpha * z[e]) + res;
+        hn[e] = fmaf(scale, z[e], res);
+        if (mixed && c + e < a.S) hn[e] = zsh[e] + res;
         st[0] = LN ? st[0] + hn[e] : fmaf(hn[e], hn[e], st[0]);
       }
       if (a.compact) {      // every rank's CTA forms the same shared values; rank 0's writes them
@@ -789,8 +802,7 @@ cudaError_t launch_rows_forward_partials(const RowPartArgs& a, caat_dtype dtype,
 #else
   constexpr int cluster_mode = 1;
 #endif
-  if (cluster_mode && dtype == CAAT_BF16 && a.t >= 2 && a.t <= 8 && a.h % V == 0 && a.h / V <= 512 && a.S % 4 == 0 &&
-      (a.h - a.S) % 4 == 0) {
+  if (cluster_mode && dtype == CAAT_BF16 && a.t >= 2 && a.t <= 8 && a.h % V == 0 && a.h / V <= 512) {
     const size_t csm = cluster_partials_smem(a);
     bool launched = false;
     cudaError_t e = cudaSuccess;

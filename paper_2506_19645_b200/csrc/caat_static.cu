@@ -44,7 +44,14 @@ extern "C" caat_status caat_rowpar_forward_noalloc(const caat_ctx* ctx, caat_lay
                                                    const void* beta, void* Hn, void* X, float* rstd, float* mean,
                                                    void* cuda_stream) {
   if (!ctx) return CAAT_EINVAL;
-  const size_t need = caat_workspace_bytes(ctx, layer, tokens, 0);
+  caat_ctx plain = *ctx;
+  size_t need = caat_workspace_bytes(ctx, layer, tokens, 0);
+  if (need > (size_t)CAAT_NOALLOC_SCRATCH_BYTES) {
+    // a few tokens of a wide layer: the decode path's fp32 planes do not fit, the large-batch path's scratch may
+    plain.no_decode = 1;
+    ctx = &plain;
+    need = caat_workspace_bytes(ctx, layer, tokens, 0);
+  }
   if (need == 0) {
     // let the regular entry point name the argument error (it fails before any launch)
     return caat_rowpar_forward(ctx, layer, tokens, Y, W, R, gamma, beta, Hn, X, rstd, mean, nullptr, 0, cuda_stream);
