@@ -194,24 +194,23 @@ static caat_status forward_impl(const caat_ctx* ctx, int K_r, int T, const void*
     ce = launch_tc_forward(sh, Y, W, zs, zp, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
   } else {
-    if (S > 0) {  // shared columns: one product over the whole contraction axis (all ranks)
-      GemmProblem g{};
+    GemmProblem pr[2] = {};
+    {  // shared columns: one product over the whole contraction axis (all ranks)
+      GemmProblem& g = pr[0];
       g.nseg = 1;
       g.seg[0] = GemmSeg{Y, W, 0, (long long)T * K_r, K_r, 1, 0, (long long)h * K_r, 1, K_r, t, K_r};
       g.C = zs; g.sCb = 0; g.sCi = L.S_hi; g.M = T; g.N = S; g.batch = 1; g.c_f32 = 0;
-      ce = launch_gemm_simt(g, ctx->dtype, st);
-      if (ce != cudaSuccess) return cuda_fail(ce);
     }
-    if (S < h) {  // private columns: one product per rank
-      GemmProblem g{};
+    {  // private columns: one product per rank
+      GemmProblem& g = pr[1];
       g.nseg = 1;
       g.seg[0] = GemmSeg{Y, static_cast<const char*>(W) + (size_t)S * K_r * e,
                          (long long)T * K_r, 0, K_r, 1, (long long)h * K_r, 0, 1, K_r, 1, K_r};
       g.C = static_cast<char*>(zp) + (size_t)(S - L.S_lo) * e;
       g.sCb = (long long)T * L.P; g.sCi = L.P; g.M = T; g.N = h - S; g.batch = t; g.c_f32 = 0;
-      ce = launch_gemm_simt(g, ctx->dtype, st);
-      if (ce != cudaSuccess) return cuda_fail(ce);
     }
+    ce = launch_gemm_simt(pr, 2, ctx->dtype, st);
+    if (ce != cudaSuccess) return cuda_fail(ce);
   }
   if (phase == 1) return CAAT_OK;
   RowFwdArgs a{zs, zp, R, gamma, beta, Hn, X, rstd, mean, t, T, h, S, L.S_lo, L.S_hi, L.P,
@@ -301,26 +300,25 @@ static caat_status backward_impl(const caat_ctx* ctx, int K_r, int T, const void
     g.seg[1] = GemmSeg{zp_priv, static_cast<const char*>(W) + (size_t)S * K_r * e,
                        (long long)T * L.P, 0, L.P, 1, (long long)h * K_r, 0, K_r, 1, 1, h - S};
     g.C = dY; g.sCb = (long long)T * K_r; g.sCi = K_r; g.M = T; g.N = K_r; g.batch = t; g.c_f32 = 0;
-    ce = launch_gemm_simt(g, ctx->dtype, st);
+    ce = launch_gemm_simt(&g, 1, ctx->dtype, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
   }
-  if (S > 0) {  // dW[m][:S] = gs^T Y[m]
-    GemmProblem g{};
+  GemmProblem pw[2] = {};
+  {  // dW[m][:S] = gs^T Y[m]
+    GemmProblem& g = pw[0];
     g.nseg = 1;
     g.seg[0] = GemmSeg{gs, Y, 0, 0, 1, L.S_hi, (long long)T * K_r, 0, K_r, 1, 1, T};
     g.C = dW; g.sCb = (long long)h * K_r; g.sCi = K_r; g.M = S; g.N = K_r; g.batch = t; g.c_f32 = 1;
-    ce = launch_gemm_simt(g, ctx->dtype, st);
-    if (ce != cudaSuccess) return cuda_fail(ce);
   }
-  if (S < h) {  // dW[m][S:] = zp[m]^T Y[m]
-    GemmProblem g{};
+  {  // dW[m][S:] = zp[m]^T Y[m]
+    GemmProblem& g = pw[1];
     g.nseg = 1;
     g.seg[0] = GemmSeg{zp_priv, Y, (long long)T * L.P, 0, 1, L.P, (long long)T * K_r, 0, K_r, 1, 1, T};
     g.C = dW + (size_t)S * K_r; g.sCb = (long long)h * K_r; g.sCi = K_r; g.M = h - S; g.N = K_r; g.batch = t;
     g.c_f32 = 1;
-    ce = launch_gemm_simt(g, ctx->dtype, st);
-    if (ce != cudaSuccess) return cuda_fail(ce);
   }
+  ce = launch_gemm_simt(pw, 2, ctx->dtype, st);
+  if (ce != cudaSuccess) return cuda_fail(ce);
   return CAAT_OK;
 }
 
@@ -766,7 +764,7 @@ caat_status caat_colpar_forward(const caat_ctx* ctx, caat_activation act, int n_
     g.nseg = 1;
     g.seg[0] = GemmSeg{X, A, (long long)T * h, 0, h, 1, (long long)n_out * h, 0, 1, h, 1, h};
     g.C = pre; g.sCb = (long long)T * n_out; g.sCi = n_out; g.M = T; g.N = n_out; g.batch = t; g.c_f32 = 0;
-    ce = launch_gemm_simt(g, ctx->dtype, st);
+    ce = launch_gemm_simt(&g, 1, ctx->dtype, st);
   }
   if (ce != cudaSuccess) return cuda_fail(ce);
   if (act != CAAT_ACT_NONE) {
@@ -813,7 +811,7 @@ caat_status caat_colpar_backward(const caat_ctx* ctx, caat_activation act, int n
     g.nseg = 1;
     g.seg[0] = GemmSeg{dpre, A, (long long)T * n_out, 0, n_out, 1, (long long)n_out * h, 0, h, 1, 1, n_out};
     g.C = dX; g.sCb = (long long)T * h; g.sCi = h; g.M = T; g.N = h; g.batch = t; g.c_f32 = 0;
-    ce = launch_gemm_simt(g, ctx->dtype, st);
+    ce = launch_gemm_simt(&g, 1, ctx->dtype, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
   }
   {  // dA[m] = dpre[m]^T X[m]
@@ -821,7 +819,7 @@ caat_status caat_colpar_backward(const caat_ctx* ctx, caat_activation act, int n
     g.nseg = 1;
     g.seg[0] = GemmSeg{dpre, X, (long long)T * n_out, 0, 1, n_out, (long long)T * h, 0, h, 1, 1, T};
     g.C = dA; g.sCb = (long long)n_out * h; g.sCi = h; g.M = n_out; g.N = h; g.batch = t; g.c_f32 = 1;
-    ce = launch_gemm_simt(g, ctx->dtype, st);
+    ce = launch_gemm_simt(&g, 1, ctx->dtype, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
   }
   return CAAT_OK;

@@ -56,8 +56,9 @@ inline size_t elem_size(caat_dtype d) { return d == CAAT_BF16 ? 2 : 4; }
 
 // ---- generic strided batched GEMM on CUDA cores (fp32 accumulate) -------------
 //   C[b][i][j] = sum_{seg} sum_{q < Q} sum_{k < Kd} A(b,q,i,k) * B(b,q,k,j)
-// with element strides for every index; A and B have the run's dtype, C has the
-// run's dtype or fp32.
+// with element strides for every index, the stride along k or along the row / column
+// being 1; A and B have the run's dtype, C has the run's dtype or fp32.  Every problem has a
+// segment 0 with Q, Kd >= 0; an empty segment contributes nothing.
 struct GemmSeg {
   const void* A;
   const void* B;
@@ -73,7 +74,8 @@ struct GemmProblem {
   int M, N, batch;
   int c_f32;           // 1: C is fp32 regardless of dtype
 };
-cudaError_t launch_gemm_simt(const GemmProblem& g, caat_dtype dtype, cudaStream_t st);
+// n <= 2 products that do not depend on each other, of one operand layout (forward, data or weight gradient), in one launch
+cudaError_t launch_gemm_simt(const GemmProblem* problems, int n, caat_dtype dtype, cudaStream_t st);
 
 // ---- tensor-core GEMMs (bf16, tcgen05 + TMA) -----------------------------------
 struct RowparShapes {
