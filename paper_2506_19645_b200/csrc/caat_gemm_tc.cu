@@ -38,7 +38,9 @@ constexpr int kAccCols = 256;     // column stride between the two accumulators
 constexpr int kTmemCols = 512;
 constexpr uint32_t kSpinCap = 1u << 22;
 constexpr int kMaxStages = 8;
-constexpr int kCBuf = 128 * 64;   // one output staging buffer: 128 rows x 64 bytes (32 bf16 / 16 fp32 columns)
+constexpr int kSlabBytes = 128;   // an epilogue warp drains slabs of 32 rows x 128 bytes (64 bf16 / 32 fp32 columns)
+constexpr int kCBuf = 32 * kSlabBytes;            // one output staging buffer of one epilogue warp
+constexpr int kCStage = 4 * 2 * kCBuf;            // four warps, two buffers each
 // Measurement aids that make results wrong (phase ablation: skipped loads, stores, barriers) and the
 // tile-shape overrides exist only in builds compiled with -DCAAT_MEASUREMENT_AIDS; the library as
 // built by build.py honours none of them.  Bit 1024 (a stage wait made to run out, for the time-out
@@ -98,7 +100,7 @@ struct Params {
   uint32_t spin_cap;     // polls of one mbarrier wait before the role gives up (kSpinCap; CAAT_TC_SPINCAP for the timeout test)
   int debug;             // measurement aid (env CAAT_TC_DEBUG, masked by kAidMask; results are then wrong): 1 = no operand loads,
                          // 2 = no epilogue work at all, 4 = no A loads, 8 = no B loads; epilogue stops after the
-                         // tensor-memory load (32) / after the staging stores (16); 64 = no slab barrier,
+                         // tensor-memory load (32) / after the staging stores (16);
                          // 128 = no TMA store; 512 = producer lanes take no second k-step; 1024 = the A boxes are
                          // announced to the stage barrier but never issued, so the consumers' waits run out
                          // (the timeout test: the kernel must flag it, drain and return)
@@ -197,7 +199,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, int x, int 
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
@@ -302,7 +303,8 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {   // arrives on
 // (tcgen05 cta_group::2): each CTA stages its own 128 rows of A and HALF of the B tile, the
 // leader (cluster rank 0) issues the MMAs for both and the tensor cores read B from both CTAs'
 // shared memory, so the operand bytes a CTA pulls from L2 per flop drop by a third.
-template <int CG>
+// SWAP: the operands are swapped (few tokens: weights on the 128-row side), fp32 planes stored straight from registers.
+template <int CG, bool SWAP>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
                const __grid_constant__ CUtensorMap map2, const __grid_constant__ CUtensorMap map3,
@@ -319,8 +321,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   const uint32_t stage_bytes = a_bytes + b_bytes;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t tiles_sa = smem_u32(base);
-  uint8_t* cstage = base + (size_t)p.nstages * stage_bytes;   // 3 output staging buffers of kCBuf bytes
-  uint64_t* bars = reinterpret_cast<uint64_t*>(cstage + 3 * kCBuf);
+  uint8_t* cstage = base + (size_t)p.nstages * stage_bytes;   // output staging, kCStage bytes
+  uint64_t* bars = reinterpret_cast<uint64_t*>(cstage + kCStage);
   // bars: full[nstages], empty[nstages], tfull[2], tempty[2]
   const uint32_t full0 = smem_u32(bars);
   const uint32_t empty0 = full0 + 8u * p.nstages;
@@ -372,7 +374,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     // measured: pays for multi-box operands (dgrad / wgrad -5...-8 %) and the weight stream of the decode
     // path (-5 %); a K-major operand of the large GEMMs gains nothing (its tiles wait for L2, not for the
     // issue) and a ring shorter than six stages loses more to pairwise refills than it gains
-    const int nki = ((multi || p.out_transposed) && p.nstages >= 6 && !(p.debug & kAidMask & 512)) ? kKI : 1;
+    const int nki = ((multi || SWAP) && p.nstages >= 6 && !(p.debug & kAidMask & 512)) ? kKI : 1;
     const int jk = lane / nbmax, box = lane - jk * nbmax;                         // this lane's k-step slot and box
     if (jk < nki) {
       int stage = 0; uint32_t phase = 0;
@@ -523,9 +525,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       }
       if (!mbar_wait(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) { ok = false; break; }
       tc_fence_after();
-      // Drain 64-byte-wide column slabs (32 bf16 / 16 fp32 columns): TMEM -> registers ->
-      // swizzled staging buffer -> TMA store (coalesced; rows and columns outside the region's
-      // extents are clipped by the tensor map).  Three buffers, one 128-thread barrier per slab.
+      // Every warp drains its 32 rows by itself in slabs of 128 bytes: TMEM -> registers -> swizzled staging buffer ->
+      // TMA store (whole 128-byte lines; rows and columns outside the region's extents are clipped by the tensor map).
+      // Two buffers per warp, no barrier across warps.  Short contractions are bound by this drain: the forward GEMM at
+      // t = 8, K_r = 256, h = 2048, 8192 tokens took 79.3 us with slabs of 64 bytes x 128 rows and a barrier per slab
+      // (54.5 without any epilogue), 71.5 like this; at p = 0.25 89.7 -> 78.8.
       const int n0 = c.nt * p.BN;
       const int m0 = c.mt * BMT + (int)rank * BM;
       const int zc = c.split * r.batch + c.b;
@@ -538,10 +542,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         omap = &pm.m[owner];
         om0 = m0 - owner * p.push_slice;
       }
-      const int sub = p.out_f32 ? 16 : 32;
       const int rr = quarter * 32 + lane;                 // row of the tile this thread holds
-      const uint32_t sw = (uint32_t)((rr >> 1) & 3);      // 64-byte swizzle: chunk ^= (row / 2) % 4
-      if (p.out_transposed) {
+      const uint32_t sw = (uint32_t)(lane & 7);           // 128-byte swizzle: 16-byte chunk ^= row % 8
+      // this warp's part of the accumulator is drained: tell the MMA issuer
+      auto release = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if (CG == 2) mbar_arrive_cluster(mapa_rank(tempty0 + 8u * acc, 0)); else mbar_arrive(tempty0 + 8u * acc);
+        }
+      };
+      if constexpr (SWAP) {
         // swap-AB (decode): TMEM lane = output channel, column = token.  For a fixed token the 32
         // lanes of a warp hold 32 consecutive channels: plain 128-byte coalesced stores.
         const long long chan = (long long)m0 + rr;
@@ -559,6 +570,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
             }
           }
         }
+        release();
       } else if (r.skip > 0 && c.mt == 0) {
         const int row = m0 + rr;
         float* dst = r.skip_out + (long long)zc * r.skip_plane + (long long)row * r.N + n0;
@@ -576,58 +588,65 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
                                                __uint_as_float(v[e + 2]) * r.scale, __uint_as_float(v[e + 3]) * r.scale);
           }
         }
-      } else
-      for (int cc = 0; cc < p.BN && n0 + cc < r.N && !(p.debug & kAidMask & 2); cc += sub) {
-        uint32_t v[32];
-        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + cc);
-        if (p.out_f32) tmem_ld16(taddr, v); else tmem_ld32(taddr, v);
-        tmem_ld_wait();
-        if (total_k == 0) {
+        release();
+      } else {
+        const int sub = p.out_f32 ? 32 : 64;
+        const int cols = (p.debug & kAidMask & 2) ? 0 : (r.N - n0 < p.BN ? r.N - n0 : p.BN);
+        const bool scaled = p.out_f32 && r.scale != 0.f && r.scale != 1.f;
+        if (cols <= 0) release();
+        for (int cc = 0; cc < cols; cc += sub) {
+          uint32_t v[32], w[32];
+          const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + cc);
+          tmem_ld32(taddr, v);
+          if (!p.out_f32) tmem_ld32(taddr + 32, w);
+          tmem_ld_wait();
+          if (cc + sub >= cols) release();
+          if (total_k == 0) {
 #pragma unroll
-          for (int e = 0; e < 32; ++e) v[e] = 0u;
-        }
-        if (p.out_f32 && r.scale != 0.f && r.scale != 1.f) {
-#pragma unroll
-          for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * r.scale);
-        }
-        const uint32_t buf = smem_u32(cstage + (size_t)(slab % 3) * kCBuf);
-        const uint32_t rowaddr = buf + (uint32_t)rr * 64u;
-        if (p.debug & kAidMask & 32) { ++slab; continue; }
-        if (p.out_f32) {
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4)
-            sts128(rowaddr + (((uint32_t)q4 ^ sw) << 4), v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
-        } else {
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            uint32_t w[4];
-#pragma unroll
-            for (int q2 = 0; q2 < 4; ++q2) {
-              __nv_bfloat162 bb = __floats2bfloat162_rn(__uint_as_float(v[8 * q4 + 2 * q2]), __uint_as_float(v[8 * q4 + 2 * q2 + 1]));
-              w[q2] = *reinterpret_cast<uint32_t*>(&bb);
-            }
-            sts128(rowaddr + (((uint32_t)q4 ^ sw) << 4), w[0], w[1], w[2], w[3]);
+            for (int e = 0; e < 32; ++e) v[e] = w[e] = 0u;
           }
+          if (p.debug & kAidMask & 32) { ++slab; continue; }
+          // the store that last used this buffer (two slabs ago) has finished reading it
+          if (lane == 0) bulk_wait_read1();
+          __syncwarp();
+          const uint32_t buf = smem_u32(cstage + (size_t)((quarter * 2 + (slab & 1)) * kCBuf));
+          const uint32_t rowaddr = buf + (uint32_t)lane * kSlabBytes;
+          if (p.out_f32) {
+            if (scaled) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * r.scale);
+            }
+#pragma unroll
+            for (int q4 = 0; q4 < 8; ++q4)
+              sts128(rowaddr + (((uint32_t)q4 ^ sw) << 4), v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
+          } else {
+            auto pack = [](uint32_t lo, uint32_t hi) {
+              __nv_bfloat162 bb = __floats2bfloat162_rn(__uint_as_float(lo), __uint_as_float(hi));
+              return *reinterpret_cast<uint32_t*>(&bb);
+            };
+#pragma unroll
+            for (int q4 = 0; q4 < 4; ++q4)
+              sts128(rowaddr + (((uint32_t)q4 ^ sw) << 4), pack(v[8 * q4], v[8 * q4 + 1]), pack(v[8 * q4 + 2], v[8 * q4 + 3]),
+                     pack(v[8 * q4 + 4], v[8 * q4 + 5]), pack(v[8 * q4 + 6], v[8 * q4 + 7]));
+#pragma unroll
+            for (int q4 = 0; q4 < 4; ++q4)
+              sts128(rowaddr + (((uint32_t)(q4 + 4) ^ sw) << 4), pack(w[8 * q4], w[8 * q4 + 1]), pack(w[8 * q4 + 2], w[8 * q4 + 3]),
+                     pack(w[8 * q4 + 4], w[8 * q4 + 5]), pack(w[8 * q4 + 6], w[8 * q4 + 7]));
+          }
+          if (p.debug & kAidMask & 16) { ++slab; continue; }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0 && !(p.debug & kAidMask & 128)) {
+            tma_store_3d(omap, n0 + cc, om0 + quarter * 32, zc, buf);
+            bulk_commit();
+          }
+          ++slab;
         }
-        if (p.debug & kAidMask & 16) { ++slab; continue; }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (!(p.debug & kAidMask & 64)) epi_barrier();
-        if (warp == 2 && lane == 0 && !(p.debug & kAidMask & 128)) {
-          tma_store_3d(omap, n0 + cc, om0, zc, buf);
-          bulk_commit();
-          bulk_wait_read1();     // the store before this one has finished reading its buffer
-        }
-        ++slab;
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {           // this CTA's part of the accumulator is drained: tell the MMA issuer
-        if (CG == 2) mbar_arrive_cluster(mapa_rank(tempty0 + 8u * acc, 0)); else mbar_arrive(tempty0 + 8u * acc);
       }
       acc ^= 1;
       if (acc == 0) acc_phase ^= 1u;
     }
-    if (warp == 2 && lane == 0) bulk_wait_all();   // all output stores of this CTA are complete
+    if (lane == 0) bulk_wait_all();   // all output stores of this warp are complete
     if (!ok && lane == 0) { *abort_flag = 1; atomicExch(p.status, 3u); }
   }
 
@@ -693,10 +712,10 @@ bool make_map(CUtensorMap* m, const void* base, long long d0, long long d1, long
   return r == CUDA_SUCCESS;
 }
 
-// Output map: slabs of 64 bytes x 128 rows, 64-byte swizzle (matches the epilogue's staging layout).
+// Output map: slabs of 128 bytes x 32 rows, 128-byte swizzle (matches the epilogue's staging layout).
 bool make_cmap(CUtensorMap* m, const void* base, long long d0, long long d1, long long d2, long long ld1,
                long long ld2, bool f32) {
-  return make_map(m, base, d0, d1, d2, ld1, ld2, f32 ? 16 : 32, BM, f32, CU_TENSOR_MAP_SWIZZLE_64B);
+  return make_map(m, base, d0, d1, d2, ld1, ld2, kSlabBytes / (f32 ? 4 : 2), 32, f32);
 }
 
 // ---- tile configuration ------------------------------------------------------------------
@@ -760,7 +779,7 @@ TileCfg pick_tile(const RegionShape* r, int nr, bool b_n_major, int max_splits, 
     }
     if (!ok) continue;
     if (force_cg && cg != force_cg && !(force_cg == 2 && cg == 1 && max_cg == 2)) continue;
-    const int step = b_n_major ? 64 * cg : 32 * cg;    // N-major B: whole 64-column chunks per CTA
+    const int step = b_n_major ? 64 * cg : 64;    // whole output slabs; N-major B: whole 64-column chunks per CTA
     for (int bn = 256; bn >= 64 * cg; bn -= step) {
       if (force_bn && bn != force_bn && force_bn % step == 0 && force_bn >= 64 * cg) continue;
       for (int splits = 1; splits <= max_splits; ++splits) {
@@ -778,17 +797,18 @@ cudaError_t launch(const CUtensorMap maps[4], const CUtensorMap cmaps[2], Params
   const LaunchLimits lim = effective_limits();
   const int stage_bytes = BM * BK * 2 + (p.BN / p.cg) * BK * 2;
   const int budget = lim.gemm_smem > 0 && lim.gemm_smem < 227 * 1024 ? lim.gemm_smem : 227 * 1024;
-  int nst = (budget - 2048 - 3 * kCBuf) / stage_bytes;
+  int nst = (budget - 2048 - kCStage) / stage_bytes;
   if (nst > kMaxStages) nst = kMaxStages;
   if (nst < 2) return cudaErrorInvalidConfiguration;
   p.nstages = nst;
-  const size_t smem = (size_t)nst * stage_bytes + 3 * kCBuf + 1024 /*alignment slack*/ + (2 * nst + 4) * 8 + 16;
+  const size_t smem = (size_t)nst * stage_bytes + kCStage + 1024 /*alignment slack*/ + (2 * nst + 4) * 8 + 16;
   static bool attr_set[64] = {};      // the attribute belongs to the device's copy of the kernel: once per device
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (std::lock_guard<std::mutex> lock(host_cache_mutex()); !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_gemm_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_gemm_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
@@ -823,9 +843,11 @@ cudaError_t launch(const CUtensorMap maps[4], const CUtensorMap cmaps[2], Params
   LaunchScope scope(kind, st);
   static const PeerMaps no_peers{};
   const PeerMaps& pm = peer_maps ? *peer_maps : no_peers;
+  if (p.out_transposed)
+    return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, true>, maps[0], maps[1], maps[2], maps[3], cmaps[0], cmaps[1], pm, p);
   if (p.cg == 2)
-    return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2>, maps[0], maps[1], maps[2], maps[3], cmaps[0], cmaps[1], pm, p);
-  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1>, maps[0], maps[1], maps[2], maps[3], cmaps[0], cmaps[1], pm, p);
+    return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, false>, maps[0], maps[1], maps[2], maps[3], cmaps[0], cmaps[1], pm, p);
+  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, false>, maps[0], maps[1], maps[2], maps[3], cmaps[0], cmaps[1], pm, p);
 }
 
 void finish_tiles(Params& p) {
