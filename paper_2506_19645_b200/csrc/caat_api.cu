@@ -115,8 +115,17 @@ Scratch scratch_layout(const caat_ctx* ctx, int K_r, int tokens, int backward) {
   if (!(backward && tc_gemm_usable(ctx, K_r)))   // the tensor-core backward reads the private gradient from dR
     off = align_up(off + (size_t)ctx->t * tokens * s.P * e, 256);
   s.zt_off = off;
-  if (!backward && tokens <= kDecodeMaxTokens && !ctx->no_decode && tc_gemm_usable(ctx, K_r))   // two layers' planes
+  const bool few = tokens <= kDecodeMaxTokens && !ctx->no_decode;
+  if (!backward && few && tc_gemm_usable(ctx, K_r))   // two layers' planes
     off = align_up(off + 2 * decode_planes_bytes(ctx, tokens), 256);
+  s.gp_off = off;
+  if (!backward && !few && !ctx->lean_scratch && ctx->S > 0 && tc_gemm_usable(ctx, K_r)) {
+    const size_t plane = (size_t)tokens * s.S_hi * sizeof(float), fit = kGroupPlanesBytes / plane;
+    if (fit >= 2) {
+      s.gp_groups = fit < (size_t)ctx->t ? (int)fit : ctx->t;
+      off = align_up(off + s.gp_groups * plane, 256);
+    }
+  }
   if (backward) {
     const size_t rows = (size_t)rows_backward_partial_rows(ctx->h, tokens, ctx->dtype);
     s.dgpart_off = off;
@@ -159,9 +168,10 @@ static caat_status check_common(const caat_ctx* ctx, caat_layer layer, int token
 static caat_status forward_impl(const caat_ctx* ctx, int K_r, int T, const void* Y, const void* W, const void* R,
                                 const void* gamma, const void* beta, void* Hn, void* X, float* rstd, float* mean,
                                 void* ws, cudaStream_t st, int compact = 0, const void* Rs = nullptr,
-                                void* Hns = nullptr, int phase = 0, int rows_mode = -1) {
+                                void* Hns = nullptr, int phase = 0, int rows_mode = -1, bool slab = false) {
   // phase: 0 = the whole layer; 1 = the GEMM only (leaves the partial sums in the scratch); 2 = the row
-  // kernel only (on what the scratch holds).  1 and 2 are the halves around a caller's all-reduce.
+  // kernel only (on what the scratch holds).  1 and 2 are the halves around a caller's all-reduce (slab: the shared
+  // part has to be in zs between them) or the block forward's side-by-side schedule.
   // compact: R / Hn are the private parts [t, T, h - S], Rs / Hns the shared part [T, S] stored once
   const Scratch L = scratch_layout(ctx, K_r, T, 0);
   char* wsb = static_cast<char*>(ws);
@@ -170,6 +180,7 @@ static caat_status forward_impl(const caat_ctx* ctx, int K_r, int T, const void*
   const int t = ctx->t, h = ctx->h, S = ctx->S;
   const size_t e = elem_size(ctx->dtype);
   cudaError_t ce;
+  int zgroups = 1;
 
   if (phase == 0 && T <= kDecodeMaxTokens && !ctx->no_decode && tc_gemm_usable(ctx, K_r)) {
     // few tokens (decode): the weights dominate the traffic; stream them with swapped operands and
@@ -188,10 +199,13 @@ static caat_status forward_impl(const caat_ctx* ctx, int K_r, int T, const void*
     return CAAT_OK;
   }
   if (phase == 2) {
-    // nothing to multiply
+    if (!slab && tc_gemm_usable(ctx, K_r))     // as the first half chose
+      zgroups = L.gp_groups ? tc_forward_groups(RowparShapes{t, T, h, K_r, S, L.S_lo, L.S_hi, L.P}, L.gp_groups) : 1;
   } else if (tc_gemm_usable(ctx, K_r)) {
     RowparShapes sh{t, T, h, K_r, S, L.S_lo, L.S_hi, L.P};
-    ce = launch_tc_forward(sh, Y, W, zs, zp, st);
+    // the row kernel sums the planes of a split itself; only a caller that exchanges the slab needs it in one piece
+    ce = launch_tc_forward(sh, Y, W, zs, zp, st, nullptr, L.gp_groups ? wsb + L.gp_off : nullptr, L.gp_groups,
+                           phase == 1 && slab ? nullptr : &zgroups);
     if (ce != cudaSuccess) return cuda_fail(ce);
   } else {
     GemmProblem pr[2] = {};
@@ -216,6 +230,7 @@ static caat_status forward_impl(const caat_ctx* ctx, int K_r, int T, const void*
   RowFwdArgs a{zs, zp, R, gamma, beta, Hn, X, rstd, mean, t, T, h, S, L.S_lo, L.S_hi, L.P,
                (float)ctx->alpha, (float)ctx->eps, ctx->norm};
   a.compact = compact; a.Rs = Rs; a.Hns = Hns;
+  a.zplanes = reinterpret_cast<const float*>(wsb + L.gp_off); a.zgroups = zgroups;
   ce = launch_rows_forward(a, ctx->dtype, rows_mode >= 0 ? rows_mode : ctx->direct_rows, st);
   if (ce != cudaSuccess) return cuda_fail(ce);
   return CAAT_OK;
@@ -393,6 +408,7 @@ caat_status caat_create(int h, int ffn, int t, double p, caat_dtype dtype, caat_
   c->alpha = std::sqrt((double)t);         // Section 4: private channels times sqrt(r)
   c->norm = 0; c->eps = 1e-5; c->force_simt = 0; c->direct_rows = 0; c->no_decode = 0; c->bwd_reduce = 0;
   c->groups = 1;
+  c->lean_scratch = 0;
   c->block_overlap = 2;
   *out = c;
   return CAAT_OK;
@@ -858,7 +874,7 @@ caat_status caat_tp_forward_local(const caat_ctx* ctx, caat_layer layer, int tok
   if (!Y || !W) return CAAT_EINVAL;
   if (!aligned16(Y) || !aligned16(W)) return CAAT_EALIGN;
   return forward_impl(ctx, layer_kr(ctx, layer), tokens, Y, W, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                      nullptr, workspace, static_cast<cudaStream_t>(cuda_stream), 0, nullptr, nullptr, 1);
+                      nullptr, workspace, static_cast<cudaStream_t>(cuda_stream), 0, nullptr, nullptr, 1, -1, true);
 }
 
 caat_status caat_tp_forward_finish(const caat_ctx* ctx, caat_layer layer, int tokens, const void* R, const void* gamma,
@@ -872,7 +888,7 @@ caat_status caat_tp_forward_finish(const caat_ctx* ctx, caat_layer layer, int to
   for (const void* p : ptrs)
     if (p && !aligned16(p)) return CAAT_EALIGN;
   return forward_impl(ctx, layer_kr(ctx, layer), tokens, nullptr, nullptr, R, gamma, beta, Hn, X, rstd, mean, workspace,
-                      static_cast<cudaStream_t>(cuda_stream), 0, nullptr, nullptr, 2);
+                      static_cast<cudaStream_t>(cuda_stream), 0, nullptr, nullptr, 2, -1, true);
 }
 
 caat_status caat_tp_backward_local(const caat_ctx* ctx, caat_layer layer, int tokens, const void* dX, const void* dHn,

@@ -76,6 +76,8 @@ struct Region {          // a family of output tiles with the same operand wirin
   float* skip_out;
   long long skip_plane;
   int splits;            // split-K factor of this region's tiles (set by finish_tiles from Params::splits when 0)
+  int qper;              // > 0: the splits divide the rank loop, qper ranks each, instead of the k-steps
+  int out_f32;
   int b_slowest;         // tile order: 1 = rank index slowest (a rank's weights / activations stay
                          // hot in L2 while its row tiles stream), 0 = row tile slowest
   float scale;           // fp32 outputs are multiplied by it in the epilogue (0 means 1)
@@ -87,7 +89,6 @@ struct Params {
   int BN;                // tile width (UMMA N): multiple of 16 (of 64 when B is N-major)
   int nstages;
   int a_mn, b_mn;        // 1: operand is MN-major in global memory
-  int out_f32;
   int out_transposed;    // 1: D is [channels x tokens]; store fp32 straight to the region's out_t[z][token][channel]
   long long out_t_ld;    // channels per token row of out_t
   int cg;                // CTAs per tile: 1, or 2 (tcgen05 cta_group::2, clusters of two)
@@ -252,10 +253,17 @@ __device__ __forceinline__ int tile_cols(const Params& p, const Region& r, int n
   return (left + q - 1) / q * q;
 }
 
-// k-step range of a unit for a split
-__device__ __forceinline__ void split_range(int splits, const Unit& u, int split, int& k_begin, int& k_end) {
-  if (splits == 1) { k_begin = 0; k_end = u.ksteps; return; }
-  const int per = (u.ksteps + splits - 1) / splits;
+// rank and k-step range of a unit for a split
+__device__ __forceinline__ void split_range(const Region& r, const Unit& u, int split, int& q_begin, int& q_end, int& k_begin,
+                                            int& k_end) {
+  q_begin = 0; q_end = u.Q; k_begin = 0; k_end = u.ksteps;
+  if (r.splits == 1) return;
+  if (r.qper > 0) {
+    q_begin = split * r.qper;
+    q_end = q_begin + r.qper < u.Q ? q_begin + r.qper : u.Q;
+    return;
+  }
+  const int per = (u.ksteps + r.splits - 1) / r.splits;
   k_begin = split * per;
   k_end = k_begin + per < u.ksteps ? k_begin + per : u.ksteps;
   if (k_begin > k_end) k_begin = k_end;
@@ -392,9 +400,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         for (int ui = 0; ui < r.nunits && ok; ++ui) {
           const Unit& u = r.u[ui];
           const CUtensorMap* map = maps[isA ? u.mapA : u.mapB];
-          int kb, ke;
-          split_range(r.splits, u, c.split, kb, ke);
-          for (int q = 0; q < u.Q && ok; ++q) {
+          int q0, q1, kb, ke;
+          split_range(r, u, c.split, q0, q1, kb, ke);
+          for (int q = q0; q < q1 && ok; ++q) {
             const int z = isA ? c.b * u.a_zb + q * u.a_zq : c.b * u.b_zb + q * u.b_zq;
             for (int k0 = kb; k0 < ke; k0 += nki) {
               const int ngrp = ke - k0 < nki ? ke - k0 : nki;      // k-steps of this group
@@ -473,9 +481,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         uint32_t accumulate = 0;
         for (int ui = 0; ui < r.nunits && ok; ++ui) {
           const Unit& u = r.u[ui];
-          int kb, ke;
-          split_range(r.splits, u, c.split, kb, ke);
-          for (int q = 0; q < u.Q && ok; ++q) {
+          int q0, q1, kb, ke;
+          split_range(r, u, c.split, q0, q1, kb, ke);
+          for (int q = q0; q < q1 && ok; ++q) {
             for (int kk = kb; kk < ke; ++kk) {
               if (!mbar_wait_warp(full_bar, phase, abort_flag, p.spin_cap)) { ok = false; break; }
               tc_fence_after();
@@ -519,9 +527,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       // a tile whose contraction range is empty leaves the accumulator undefined: its value is 0
       int total_k = 0;
       for (int ui = 0; ui < r.nunits; ++ui) {
-        int kb, ke;
-        split_range(r.splits, r.u[ui], c.split, kb, ke);
-        total_k += (ke - kb) * r.u[ui].Q;
+        int q0, q1, kb, ke;
+        split_range(r, r.u[ui], c.split, q0, q1, kb, ke);
+        total_k += (ke - kb) * (q1 - q0);
       }
       if (!mbar_wait(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) { ok = false; break; }
       tc_fence_after();
@@ -590,15 +598,16 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         }
         release();
       } else {
-        const int sub = p.out_f32 ? 32 : 64;
+        const bool out_f32 = r.out_f32 != 0;
+        const int sub = out_f32 ? 32 : 64;
         const int cols = (p.debug & kAidMask & 2) ? 0 : (r.N - n0 < p.BN ? r.N - n0 : p.BN);
-        const bool scaled = p.out_f32 && r.scale != 0.f && r.scale != 1.f;
+        const bool scaled = out_f32 && r.scale != 0.f && r.scale != 1.f;
         if (cols <= 0) release();
         for (int cc = 0; cc < cols; cc += sub) {
           uint32_t v[32], w[32];
           const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + cc);
           tmem_ld32(taddr, v);
-          if (!p.out_f32) tmem_ld32(taddr + 32, w);
+          if (!out_f32) tmem_ld32(taddr + 32, w);
           tmem_ld_wait();
           if (cc + sub >= cols) release();
           if (total_k == 0) {
@@ -611,7 +620,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           __syncwarp();
           const uint32_t buf = smem_u32(cstage + (size_t)((quarter * 2 + (slab & 1)) * kCBuf));
           const uint32_t rowaddr = buf + (uint32_t)lane * kSlabBytes;
-          if (p.out_f32) {
+          if (out_f32) {
             if (scaled) {
 #pragma unroll
               for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * r.scale);
@@ -676,6 +685,32 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float4* __rest
   }
 }
 
+// zs[i] = round(sum_g planes[g][i]), g ascending: the rank groups of a split shared region, 8 elements per thread.  With
+// slice > 0 row i of the sum goes to slot `rank` of GPU i / slice instead (the exchange over peer memory).
+struct SlotTarget { uint4* recv[CAAT_MAX_PEERS]; int slice, rank; };
+
+__global__ void __launch_bounds__(256) sum_groups_kernel(const float4* __restrict__ planes, uint4* __restrict__ zs, int T, int row8,
+                                                         int groups, const __grid_constant__ SlotTarget slots) {
+  pdl_wait();
+  const long long n8 = (long long)T * row8;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += (long long)gridDim.x * blockDim.x) {
+    float4 a = planes[2 * i], b = planes[2 * i + 1];
+    for (int g = 1; g < groups; ++g) {
+      const float4 x = planes[2 * (g * n8 + i)], y = planes[2 * (g * n8 + i) + 1];
+      a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+      b.x += y.x; b.y += y.y; b.z += y.z; b.w += y.w;
+    }
+    __nv_bfloat162 o[4] = {__floats2bfloat162_rn(a.x, a.y), __floats2bfloat162_rn(a.z, a.w), __floats2bfloat162_rn(b.x, b.y),
+                           __floats2bfloat162_rn(b.z, b.w)};
+    uint4* dst = zs + i;
+    if (slots.slice > 0) {
+      const int row = (int)(i / row8), q = row / slots.slice;
+      dst = slots.recv[q] + ((long long)slots.rank * slots.slice + (row - q * slots.slice)) * row8 + (i - (long long)row * row8);
+    }
+    *dst = *reinterpret_cast<uint4*>(o);
+  }
+}
+
 // ---------------------------------------------------------------- host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -728,30 +763,45 @@ bool make_cmap(CUtensorMap* m, const void* base, long long d0, long long d1, lon
 //    tile costs max(main loop, epilogue) plus a fixed hand-off (larger across a CTA pair);
 //  * tiles are dealt round-robin to 148 / cg workers: few tiles cost whole waves;
 //  * split-K partials are written and read back once (fp32).
+// Regions are dealt one after the other (the first one's tiles are the longest); a worker's load is the sum of its tiles.
 struct RegionShape { int M, N, batch, ksteps; };
 struct TileCfg { int bn, cg, splits; double cost; };
+
+// The busiest worker's load when n1 tiles of length a and then n2 of length b are dealt round-robin to W workers.
+double makespan(long long n1, double a, long long n2, double b, long long W) {
+  const long long r1 = n1 % W, rt = (n1 + n2) % W, edge[3] = {0, r1, rt};
+  double worst = 0;
+  for (long long w : edge) {
+    const long long c1 = n1 / W + (w < r1), ct = (n1 + n2) / W + (w < rt);
+    worst = fmax(worst, c1 * a + (ct - c1) * b);
+  }
+  return worst;
+}
 
 double estimate_cost(const RegionShape* r, int nr, int bn, int cg, int splits, double out_bytes, bool b_n_major) {
   const double workers = 148.0 / cg;
   const double step = (bn / 256.0) * fmax(1.0, 0.92 * (128.0 + (double)bn / cg) / bn);
   const double epi = 10.0 * bn / 256.0;
   const double handoff = cg == 2 ? 3.5 : 2.0;
-  double total = 0, ntiles = 0;
+  double total = 0, len[2] = {0, 0};
+  long long n[2] = {0, 0};
   for (int i = 0; i < nr; ++i) {
     if (r[i].M <= 0 || r[i].N <= 0) continue;
-    const double rows = (double)((r[i].M + 128 * cg - 1) / (128 * cg)) * r[i].batch * splits;
+    const long long rows = (long long)((r[i].M + 128 * cg - 1) / (128 * cg)) * r[i].batch * splits;
     const double ks = (double)((r[i].ksteps + splits - 1) / splits);
     const int full = r[i].N / bn, rest = r[i].N % bn;
-    total += rows * full * (fmax(ks * step, epi) + handoff);
-    ntiles += rows * full;
+    double region = rows * full * (fmax(ks * step, epi) + handoff);
+    n[i] = rows * full;
     if (rest) {   // the last, ragged tile: an N-major B operand is narrowed to whole 64-column chunks
       const double w = b_n_major ? (double)((rest + 64 * cg - 1) / (64 * cg) * (64 * cg)) / bn : 1.0;
-      total += rows * (fmax(ks * step * w, epi * w) + handoff);
-      ntiles += rows;
+      region += rows * (fmax(ks * step * w, epi * w) + handoff);
+      n[i] += rows;
     }
+    total += region;
+    if (n[i]) len[i] = region / n[i];
   }
-  if (ntiles == 0) return 0;
-  double t = fmax(total / workers, ceil(ntiles / workers) * (total / ntiles));
+  if (n[0] + n[1] == 0) return 0;
+  double t = fmax(total / workers, makespan(n[0], len[0], n[1], len[1], (long long)workers));
   if (splits > 1) t += 2.0 * splits * out_bytes / 6.4e12 / 0.2e-6;
   return t;
 }
@@ -871,30 +921,55 @@ bool tc_gemm_usable(const caat_ctx* ctx, int K_r) {
 // Any partition S: TMA wants 16-byte coordinates along a row's channels, so the private products start at S_lo; their
 // S - S_lo extra columns land in the scratch columns that no row kernel reads.  (Partitions off the 8-channel grid ran on
 // the CUDA-core GEMM before: a training step of a block at h = 2048, 2999 tokens, p = 0.7 took 17.5 ms, now 0.61 ms.)
+// A shared tile's contraction is t times a private one's, and with few tokens there are only a handful of them: the
+// GEMM then waits for its longest tiles (T = 300 at the 7B MLP shapes: 16 tiles of 176 k-steps where the even share of a
+// worker is 76).  Given `planes` ([max_groups][T][S_hi] fp32 scratch), the rank loop may be split into groups of ranks:
+// every group's partial sum is a tile of its own, and the row kernel adds the planes where it would read the sum (alone,
+// GEMM of that layer alone, 300 tokens: 67 -> 41 us; 80 tokens: 54 -> 21).  The cost model
+// decides.
+struct ForwardPlan { TileCfg tile; int groups, qper; };
+
+static ForwardPlan forward_plan(const RowparShapes& s, int max_groups) {
+  const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0, ksteps = (s.K_r + BK - 1) / BK;
+  ForwardPlan f{};
+  for (int per = s.t; per >= 1; per = per > 1 ? (per + 1) / 2 : 0) {
+    const int g = (s.t + per - 1) / per;
+    if (g > 1 && (n_sh == 0 || g > max_groups)) break;
+    const RegionShape rs[2] = {{s.T, n_sh, g, ksteps * per}, {s.T, n_pr, s.t, ksteps}};
+    TileCfg c = pick_tile(rs, 2, false, 1, 0.0);
+    if (g > 1) c.cost += (8.0 * g * s.T * s.S_hi / 10e12 + 1e-6) / 0.2e-6;   // the planes' round trip through L2
+    if (g == 1 || c.cost < f.tile.cost) f = ForwardPlan{c, g, per};
+  }
+  return f;
+}
+
+int tc_forward_groups(const RowparShapes& s, int max_groups) { return forward_plan(s, max_groups).groups; }
+
 cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* W, void* zs, void* zp,
-                              cudaStream_t st, const PushTarget* push) {
+                              cudaStream_t st, const PushTarget* push, void* planes, int max_groups, int* groups_out) {
   CUtensorMap maps[4], cmaps[2];
   PeerMaps pmaps{};
   Params p{};
   const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
   const int ksteps = (s.K_r + BK - 1) / BK;
-  {
-    const RegionShape rs[2] = {{s.T, n_sh, 1, ksteps * s.t}, {s.T, n_pr, s.t, ksteps}};
-    const TileCfg c = pick_tile(rs, 2, false, 1, 0.0);
-    p.BN = c.bn; p.cg = c.cg;
-  }
+  const ForwardPlan plan = forward_plan(s, planes ? max_groups : 1);
+  const int groups = plan.groups, qper = plan.qper;
+  p.BN = plan.tile.bn; p.cg = plan.tile.cg;
+  if (groups_out) *groups_out = groups;
   if (!make_map(&maps[0], Y, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, BK, BM)) return cudaErrorInvalidValue;
   if (!make_map(&maps[1], W, s.K_r, s.h, s.t, s.K_r, (long long)s.h * s.K_r, BK, p.BN / p.cg)) return cudaErrorInvalidValue;
   maps[2] = maps[0];
   maps[3] = maps[1];
-  p.a_mn = 0; p.b_mn = 0; p.out_f32 = 0; p.splits = 1;
+  p.a_mn = 0; p.b_mn = 0;  p.splits = 1;
   int g = 0;
   if (n_sh > 0) {
     Region& r = p.r[g++];
     r.nunits = 1;
     r.u[0] = Unit{0, 1, 0, 0, 0, 0, /*a_zb*/ 0, /*a_zq*/ 1, /*b_zb*/ 0, /*b_zq*/ 1, s.t, ksteps};
     r.M = s.T; r.N = n_sh; r.batch = 1; r.b_slowest = 0;
-    if (!make_cmap(&cmaps[g - 1], zs, n_sh, s.T, 1, s.S_hi, (long long)s.T * s.S_hi, false)) return cudaErrorInvalidValue;
+    if (groups > 1) { r.splits = groups; r.qper = qper; r.out_f32 = 1; }
+    if (!make_cmap(&cmaps[g - 1], groups > 1 ? planes : zs, n_sh, s.T, groups, s.S_hi, (long long)s.T * s.S_hi, groups > 1))
+      return cudaErrorInvalidValue;
   }
   if (n_pr > 0) {
     Region& r = p.r[g++];
@@ -905,7 +980,7 @@ cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* 
   }
   if (g == 1) cmaps[1] = cmaps[0];
   p.nregions = g;
-  if (push && n_sh > 0) {
+  if (push && n_sh > 0 && groups == 1) {
     // shared tiles go to the owners' receive slots: slot `rank` of GPU q is [slice, S] 16-bit elements; the map of
     // owner q covers only the tokens q really owns, so rows past the end of a ragged last slice are clipped
     if (push->world < 1 || push->world > CAAT_MAX_PEERS || push->slice % (BM * p.cg) != 0) return cudaErrorInvalidValue;
@@ -919,7 +994,18 @@ cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* 
     p.push_slice = push->slice;
   }
   finish_tiles(p);
-  return launch(maps, cmaps, p, CAAT_K_TC_FORWARD, st, push && n_sh > 0 ? &pmaps : nullptr);
+  const cudaError_t e = launch(maps, cmaps, p, CAAT_K_TC_FORWARD, st, push && n_sh > 0 && groups == 1 ? &pmaps : nullptr);
+  if (e != cudaSuccess || groups == 1 || groups_out) return e;
+  const long long n8 = (long long)s.T * s.S_hi / 8;
+  const int blocks = (int)((n8 + 255) / 256 < 8 * sm_count() ? (n8 + 255) / 256 : 8 * sm_count());
+  LaunchScope scope(CAAT_K_SPLITK_REDUCE, st);
+  SlotTarget slots{};
+  if (push) {
+    slots.slice = push->slice; slots.rank = push->rank;
+    for (int q = 0; q < push->world; ++q) slots.recv[q] = static_cast<uint4*>(push->recv[q]);
+  }
+  return launch_pdl(sum_groups_kernel, dim3(blocks), dim3(256), 0, st, static_cast<const float4*>(planes), static_cast<uint4*>(zs),
+                    s.T, s.S_hi / 8, groups, slots);
 }
 
 // ---- decode forward (few tokens): zt[m][i][l] = sum_k W[m][l][k] Y[m][i][k], fp32, for ALL channels.
@@ -947,7 +1033,7 @@ cudaError_t launch_tc_forward_decode(int t, int T, int h, const DecodeProblem* p
   p.BN = (T + 31) / 32 * 32;
   if (p.BN > 256) return cudaErrorInvalidValue;
   p.cg = 1;
-  p.a_mn = 0; p.b_mn = 0; p.out_f32 = 1; p.splits = 1;
+  p.a_mn = 0; p.b_mn = 0;  p.splits = 1;
   p.out_transposed = 1; p.out_t_ld = h;
   // longer contraction first: round-robin dealing then fills the tail with the short items
   int order[2] = {0, 1};
@@ -1005,7 +1091,7 @@ cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOpe
   if (!okA0 || !okA1) return cudaErrorInvalidValue;
   if (n_sh == 0) maps[0] = maps[2];
   if (n_pr == 0) maps[2] = maps[0];
-  p.a_mn = 0; p.b_mn = 1; p.out_f32 = 0; p.splits = 1;
+  p.a_mn = 0; p.b_mn = 1;  p.splits = 1;
   Region& r = p.r[0];
   int nu = 0;
   if (n_sh > 0) r.u[nu++] = Unit{0, 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, (n_sh + BK - 1) / BK};
@@ -1050,7 +1136,7 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
   if (n_sh == 0) maps[0] = maps[2];
   if (n_pr == 0) maps[2] = maps[0];
   maps[3] = maps[1];
-  p.a_mn = 1; p.b_mn = 1; p.out_f32 = 1; p.splits = splits;
+  p.a_mn = 1; p.b_mn = 1;  p.splits = splits;
   const int ksteps = (s.T + BK - 1) / BK;
   float* out = splits > 1 ? static_cast<float*>(splitk) : dW;
   int g = 0;
@@ -1058,6 +1144,7 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
     Region& r = p.r[g++];
     r.nunits = 1;
     r.u[0] = Unit{0, 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, ksteps};
+    r.out_f32 = 1;
     r.M = n_sh; r.N = s.K_r; r.batch = s.t; r.b_slowest = 0;   // the shared gradient panel serves all ranks at once
     r.scale = 1.0f;
     if (!make_cmap(&cmaps[g - 1], out, s.K_r, n_sh, (long long)s.t * splits, s.K_r, (long long)s.h * s.K_r, true))
@@ -1067,6 +1154,7 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
     Region& r = p.r[g++];
     r.nunits = 1;
     r.u[0] = Unit{2, 1, 0, pv.col0, 0, 0, 1, 0, 1, 0, 1, ksteps};
+    r.out_f32 = 1;
     r.M = n_pr; r.N = s.K_r; r.batch = s.t; r.b_slowest = 1;
     r.scale = pv.alpha;
     r.skip = s.S - s.S_lo;

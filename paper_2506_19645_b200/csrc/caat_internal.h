@@ -22,12 +22,16 @@ struct caat_ctx {
   int no_decode;   // CAAT_OPT_DECODE
   int bwd_reduce;  // CAAT_OPT_BACKWARD_REDUCE
   int groups;      // CAAT_OPT_TP_GROUPS: this context holds t of t * groups tensor-parallel ranks
+  int lean_scratch;   // set in the copy that the no-allocation entry point uses when the full scratch does not fit
   int block_overlap;  // CAAT_OPT_BLOCK_OVERLAP: the block forward runs the first layer's row kernel beside the second GEMM
 };
 
 namespace caat {
 
 constexpr int kLayoutVec = 8;        // column granularity of the scratch layout (elements)
+// Scratch for the rank groups of a split shared region: as many planes as fit here, at most t.  A split pays only while
+// the shared tiles are few, that is while a plane is small (2.4 MB at 300 tokens of S = 2048).
+constexpr size_t kGroupPlanesBytes = 32u << 20;
 constexpr int kMaxPartialRows = 1184;  // upper bound on rows of norm-gradient partials (8 x 148)
 
 inline int round_down(int x, int m) { return x / m * m; }
@@ -47,6 +51,8 @@ struct Scratch {
   size_t splitk_off, splitk_bytes;  // backward: split-K partials of the weight gradient
   size_t wt_off;           // backward: the private rows of W times alpha, [t, h, K_r] (tensor-core path, alpha != 1)
   size_t zt_off;           // forward, few tokens: fp32 per-rank partials [t, T, h]
+  size_t gp_off;           // forward: fp32 partial sums of the shared columns over groups of ranks, [gp_groups, T, S_hi]
+  int gp_groups;           // 0: no room reserved (too many tokens for a split to pay)
   size_t total;
 };
 
@@ -87,8 +93,13 @@ bool tc_gemm_usable(const caat_ctx* ctx, int K_r);
 // (exchange of the slab over peer memory): recv[q] is GPU q's receive buffer [world][slice][S] as this GPU
 // addresses it, the owner of token i is i / slice, slice a multiple of 256
 struct PushTarget { int world, rank, slice; void* const* recv; };
+// planes / max_groups: scratch for a split of the rank loop; with a split the shared part is left in the planes and
+// *groups says how many (1: it is in zs), or - groups == nullptr - it is summed into zs by one more launch
 cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* W, void* zs, void* zp,
-                              cudaStream_t st, const PushTarget* push = nullptr);
+                              cudaStream_t st, const PushTarget* push = nullptr, void* planes = nullptr, int max_groups = 1,
+                              int* groups = nullptr);
+// the split launch_tc_forward would choose (for a caller that launches the row kernel later)
+int tc_forward_groups(const RowparShapes& s, int max_groups);
 // The private part of dZt as the backward GEMMs read it: element (m, i, l) for l >= S_lo sits at
 // ptr[(m * T + i) * ld + col0 + (l - S_lo)], and the gradient is alpha times the stored value for l >= S.
 //   the residual gradient itself (per rank):  {dR, h, S_lo, alpha}   (no scaled copy is written at all)
@@ -123,6 +134,12 @@ struct RowFwdArgs {
   int compact;
   const void* Rs;
   void* Hns;
+  // zgroups > 1: the shared part comes as fp32 partial sums over groups of ranks, zplanes [zgroups][T][S_hi]; their sum in
+  // ascending order, rounded to the run's type, stands in for zs
+  const float* zplanes;
+  int zgroups;
+  // set by the launchers of the bulk-copy kernels, see unit_range()
+  int flat;
 };
 // direct: 0 = automatic (warp-per-token kernels for short rows, else the bulk-copy staged kernels
 // whenever a ring of at least two stages fits in shared memory), 1 = plain-load kernels,

@@ -28,7 +28,8 @@ using namespace rows;
 
 // ------------------------------------------------------------------ forward
 // CL: compact residual layout (shared part of R / Hn stored once, [T, S]; private parts [t, T, P])
-template <typename T_, int CPT, bool LN, bool CL>
+// FEW: the shared part may come as planes of a split GEMM
+template <typename T_, int CPT, bool LN, bool CL, bool FEW>
 __global__ void __launch_bounds__(512, CPT == 1 ? 2 : 1) rows_forward_kernel(const RowFwdArgs a) {
   using V_ = VT<T_>;
   using raw = typename V_::raw;
@@ -72,7 +73,10 @@ __global__ void __launch_bounds__(512, CPT == 1 ? 2 : 1) rows_forward_kernel(con
     if (act[j]) {
       V_::unpack(ldg<raw>(static_cast<const char*>(a.gamma) + (long long)col[j] * ES), gam[j]);
       if (LN && a.beta) V_::unpack(ldg<raw>(static_cast<const char*>(a.beta) + (long long)col[j] * ES), bet[j]);
-      if (cls[j] != 1) V_::unpack(ldg<raw>(static_cast<const char*>(a.zs) + (i * a.S_hi + col[j]) * ES), zs[j]);
+      if (cls[j] != 1) {
+        V_::unpack(FEW && a.zgroups > 1 ? sum_planes<T_>(a.zplanes + i * a.S_hi + col[j], (long long)a.T * a.S_hi, a.zgroups)
+                                 : ldg<raw>(static_cast<const char*>(a.zs) + (i * a.S_hi + col[j]) * ES), zs[j]);
+      }
     }
   }
 
@@ -761,10 +765,14 @@ cudaError_t launch_fwd_t(const RowFwdArgs& a, const RowGeom& g, cudaStream_t st)
   const dim3 block(g.TX, g.TY);
   const dim3 grid((a.T + g.TY - 1) / g.TY);
   LaunchScope scope(CAAT_K_ROWS_FORWARD, st);
+  const bool few = sizeof(T_) == 2 && a.zgroups > 1;
   switch (g.CPT) {
-    case 1: rows_forward_kernel<T_, 1, LN, CL><<<grid, block, g.smem_fwd, st>>>(a); break;
-    case 2: rows_forward_kernel<T_, 2, LN, CL><<<grid, block, g.smem_fwd, st>>>(a); break;
-    case 4: rows_forward_kernel<T_, 4, LN, CL><<<grid, block, g.smem_fwd, st>>>(a); break;
+    case 1: few ? rows_forward_kernel<T_, 1, LN, CL, true><<<grid, block, g.smem_fwd, st>>>(a)
+                : rows_forward_kernel<T_, 1, LN, CL, false><<<grid, block, g.smem_fwd, st>>>(a); break;
+    case 2: few ? rows_forward_kernel<T_, 2, LN, CL, true><<<grid, block, g.smem_fwd, st>>>(a)
+                : rows_forward_kernel<T_, 2, LN, CL, false><<<grid, block, g.smem_fwd, st>>>(a); break;
+    case 4: few ? rows_forward_kernel<T_, 4, LN, CL, true><<<grid, block, g.smem_fwd, st>>>(a)
+                : rows_forward_kernel<T_, 4, LN, CL, false><<<grid, block, g.smem_fwd, st>>>(a); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -143,6 +143,59 @@ __device__ __forceinline__ int chunk_class(int col, int V, int S) {
   return (col + V <= S) ? 0 : (col >= S ? 1 : 2);
 }
 
+// The (token group, rank) units of a persistent CTA of the forward: `total` units from (n0, m0) on, the next group nstep
+// further.  The ranks of a token are independent in the forward.  Strided: whole groups, the CTAs side by side in memory.
+// Flat: an even share of the units, starting and stopping inside a token.  Strided streams better (8192 tokens of 8 x 2048:
+// 174 us against 179; 16384 of 4 x 768: 66.5 against 69.7), flat evens out few groups (300 tokens of 8 x 4096 on 296 CTAs:
+// 9 units on the busiest instead of 16, 17.8 us against 14.9): flat when the busiest CTA's share drops by a tenth.
+struct UnitRange { int n0, m0, nstep; long long total; };
+__device__ __forceinline__ UnitRange unit_range(bool flat, int ngroups, int t) {
+  UnitRange u;
+  if (flat) {
+    const long long units = (long long)ngroups * t;
+    const long long u0 = units * blockIdx.x / gridDim.x;
+    u.n0 = (int)(u0 / t);
+    u.m0 = (int)(u0 - (long long)u.n0 * t);
+    u.nstep = 1;
+    u.total = units * (blockIdx.x + 1) / gridDim.x - u0;
+  } else {
+    u.n0 = blockIdx.x;
+    u.m0 = 0;
+    u.nstep = gridDim.x;
+    u.total = (int)blockIdx.x < ngroups ? (long long)((ngroups - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) * t : 0;
+  }
+  return u;
+}
+// Decides and trims the grid.  A compact stream updated in place (Rs == Hns) stays whole: rank 0's unit overwrites the
+// shared part that the token's other units read.
+inline int flat_units(const RowFwdArgs& a, int ngroups, int& grid) {
+  const long long units = (long long)ngroups * a.t;
+  const int g = (long long)grid < units ? grid : (int)units;
+  const long long strided = (long long)((ngroups + grid - 1) / grid) * a.t, flat = (units + g - 1) / g;
+  if (10 * strided > 11 * flat && !(a.compact && a.Rs == a.Hns)) { grid = g; return 1; }
+  if (grid > ngroups) grid = ngroups;
+  return 0;
+}
+
+// A chunk of the shared sum from the planes of a split GEMM: groups ascending, rounded once to the storage type.  Only
+// the few-token variants of the kernels (template flag FEW) contain it: its loads in flight cost registers that the main
+// loops of long launches need.
+template <typename T_>
+__device__ __forceinline__ typename VT<T_>::raw sum_planes(const float* src, long long plane, int groups) {
+  constexpr int V = VT<T_>::N;
+  float z[V];
+#pragma unroll
+  for (int e = 0; e < V; ++e) z[e] = 0.f;
+#pragma unroll 4
+  for (int g = 0; g < groups; ++g, src += plane) {
+#pragma unroll
+    for (int e = 0; e < V; e += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(src + e);
+      z[e] += v.x; z[e + 1] += v.y; z[e + 2] += v.z; z[e + 3] += v.w;
+    }
+  }
+  return VT<T_>::pack(z);
+}
 
 struct RowGeom {
   int TX, TY, CPT;

@@ -23,7 +23,8 @@ using namespace rows;
 // ------------------------------------------------------------------ forward
 // stage buffers: a = R rows [TY, h], b = zp rows [TY, P], c = zs rows [TY, S_hi] (rank 0 only)
 // compact layout (CL): a = private residual rows [TY, P], d = shared residual rows [TY, S] (rank 0 only)
-template <typename T_, int CPT, bool LN, int MAXT, bool CL>
+// FEW: few tokens - units dealt inside tokens, the shared part possibly as planes of a split GEMM
+template <typename T_, int CPT, bool LN, int MAXT, bool CL, bool FEW>
 __global__ void __launch_bounds__(MAXT, MinBlocks<CPT, MAXT>::value)
 rows_forward_staged(const RowFwdArgs a, const StageGeom sg, int ngroups, unsigned int* status) {
   using V_ = VT<T_>;
@@ -43,40 +44,42 @@ rows_forward_staged(const RowFwdArgs a, const StageGeom sg, int ngroups, unsigne
   const bool has_priv = a.P > 0 && a.S < a.h;
   const bool has_shared = a.S > 0;
 
-  // sequence k = n * t + m over this CTA's (token group n, rank m) pairs
-  const int my_groups = blockIdx.x < ngroups ? (ngroups - blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-  const long long total = (long long)my_groups * a.t;
+  const UnitRange ur = unit_range(FEW && a.flat, ngroups, a.t);
+  const long long total = ur.total;
 
   // Fetch the inputs of (token group nn, rank mm) into stage ss.  Every thread calls it (all keep the
   // counters); the copies of a stage are issued by lane 0 of DIFFERENT warps, so that no warp carries
   // more than one copy's issue latency into the next CTA barrier.  Warp 0 posts the expected bytes with
   // its arrival; a copy landing before that only drives the byte count negative for a moment, the phase
   // cannot complete before the arrival.
-  int nn = 0, mm = 0, ss = 0;
+  int nn = ur.n0, mm = ur.m0, ss = 0;
+  long long to_issue = total;
   const int issuer = __shfl_sync(0xffffffffu, (int)(threadIdx.y * TX + threadIdx.x) >> 5, 0);   // warp index, warp-uniform
   auto issue = [&]() {
-    if (nn >= my_groups) return;
+    if (to_issue == 0) return;
+    const bool first = mm == 0 || to_issue == total;     // the shared part comes with the token's first unit here
+    --to_issue;
     const int n = nn, m = mm, s = ss;
-    if (++mm == a.t) { mm = 0; ++nn; }
+    if (++mm == a.t) { mm = 0; nn += ur.nstep; }
     if (++ss == NS) ss = 0;
     if (issuer > 3) return;
-    const long long g = blockIdx.x + (long long)n * gridDim.x;
-    const long long i0 = g * TY;
+    const long long i0 = (long long)n * TY;
     const int rowsN = (int)((a.T - i0) < TY ? (a.T - i0) : TY);
     const uint32_t bar = bar0 + 8u * s;
     const uint32_t dst = smem_u32(ring + (size_t)s * sg.stage_bytes);
     const uint32_t bP = has_priv ? (uint32_t)rowsN * a.P * ES : 0u;
     const uint32_t bR = CL ? bP : (uint32_t)rowsN * a.h * ES;
-    const uint32_t bS = (m == 0 && has_shared) ? (uint32_t)rowsN * a.S_hi * ES : 0u;
+    const uint32_t bS = (first && has_shared) ? (uint32_t)rowsN * a.S_hi * ES : 0u;
+    const uint32_t bZ = FEW && a.zgroups > 1 ? 0u : bS;
     const long long row = (long long)m * a.T + i0;
     if (!elect_one()) return;
     if (issuer == 0) {
-      mbar_expect_tx(bar, bR + bP + (CL ? 2 * bS : bS) + sg.stall_bytes);
+      mbar_expect_tx(bar, bR + bP + bZ + (CL ? bS : 0u) + sg.stall_bytes);
       if (bR) bulk_g2s(dst + sg.off_a, static_cast<const char*>(a.R) + row * (CL ? a.P : a.h) * ES, bR, bar);
     } else if (issuer == 1) {
       if (bP) bulk_g2s(dst + sg.off_b, static_cast<const char*>(a.zp) + row * a.P * ES, bP, bar);
     } else if (issuer == 2) {
-      if (bS) bulk_g2s(dst + sg.off_c, static_cast<const char*>(a.zs) + i0 * a.S_hi * ES, bS, bar);
+      if (bZ) bulk_g2s(dst + sg.off_c, static_cast<const char*>(a.zs) + i0 * a.S_hi * ES, bZ, bar);
     } else {
       if (CL && bS) bulk_g2s(dst + sg.off_d, static_cast<const char*>(a.Rs) + i0 * a.S_hi * ES, bS, bar);
     }
@@ -132,9 +135,10 @@ rows_forward_staged(const RowFwdArgs a, const StageGeom sg, int ngroups, unsigne
   int cs = 0;
   uint32_t cph = 0;
   bool dead = false;
-  for (int n = 0; n < my_groups && !dead; ++n) {
-    const long long g = blockIdx.x + (long long)n * gridDim.x;
-    const long long i = g * TY + threadIdx.y;
+  int m_first = ur.m0;
+  for (int n = ur.n0; k < total && !dead; n += ur.nstep, m_first = 0) {
+    const long long i = (long long)n * TY + threadIdx.y;
+    const int m_end = total - k < a.t - m_first ? m_first + (int)(total - k) : a.t;
     const bool valid = i < a.T;
     bool act[CPT];
     float2 zs[CPT][H2];     // shared part of the layer output (compact: of the new stream), formed once per token
@@ -145,25 +149,27 @@ rows_forward_staged(const RowFwdArgs a, const StageGeom sg, int ngroups, unsigne
       act[j] = valid && colok[j];
       const long long off_h = (i * a.h + col[j]) * ES;
       if (CL) pHn[j] = cls[j] == 0 ? static_cast<char*>(a.Hns) + (i * a.S_hi + col[j]) * ES
-                                   : static_cast<char*>(a.Hn) + (i * a.P + (col[j] - a.S_lo)) * ES;
-      else pHn[j] = static_cast<char*>(a.Hn) + off_h;
-      pX[j] = static_cast<char*>(a.X) + off_h;
+                                   : static_cast<char*>(a.Hn) + (i * a.P + (col[j] - a.S_lo)) * ES + m_first * rank_hn;
+      else pHn[j] = static_cast<char*>(a.Hn) + off_h + m_first * rank_hn;
+      pX[j] = static_cast<char*>(a.X) + off_h + m_first * rank_h;
 #pragma unroll
       for (int q = 0; q < H2; ++q) zs[j][q] = f2(0.f);
     }
-    float* rstd_p = a.rstd + i;
-    float* mean_p = (LN && a.mean) ? a.mean + i : nullptr;
+    float* rstd_p = a.rstd + i + (long long)m_first * a.T;
+    float* mean_p = (LN && a.mean) ? a.mean + i + (long long)m_first * a.T : nullptr;
 
-    for (int m = 0; m < a.t; ++m, ++k) {
+    for (int m = m_first; m < m_end; ++m, ++k) {
       if (!mbar_wait(bar0 + 8u * cs, cph, sg.spin_cap)) *abort_flag = 1;
 
       float2 hn[CPT][H2];
       float2 acc = f2(0.f);
 #pragma unroll
       for (int j = 0; j < CPT; ++j) {
-        if (m == 0 && cls[j] != 1 && colok[j]) {
+        if (m == m_first && cls[j] != 1 && colok[j]) {
           const uint32_t os = ((uint32_t)threadIdx.y * a.S_hi + col[j]) * ES;
-          unpack2(lds32<raw>(sb + sg.off_c + os), zs[j]);
+          unpack2(FEW && a.zgroups > 1 ? (valid ? sum_planes<T_>(a.zplanes + i * a.S_hi + col[j], (long long)a.T * a.S_hi, a.zgroups)
+                                         : zero_raw<raw>())
+                                : lds32<raw>(sb + sg.off_c + os), zs[j]);
           if constexpr (CL) {       // the shared part of the new stream: zs + Rs
             float2 r0[H2];
             unpack2(lds32<raw>(sb + sg.off_d + os), r0);
@@ -609,8 +615,10 @@ cudaError_t launch_fwd_staged_t(const RowFwdArgs& a, const RowGeom& g, const Sta
   const int threads = g.TX * g.TY;
 #define CAAT_LAUNCH(CPT_, MAXT_)                                                                   \
   do {                                                                                             \
-    e = set_smem(rows_forward_staged<T_, CPT_, LN, MAXT_, CL>, sg.smem);                                        \
-    if (e == cudaSuccess) e = launch_pdl(rows_forward_staged<T_, CPT_, LN, MAXT_, CL>, dim3(grid), block, sg.smem, st, a, sg, ngroups, status);   \
+    auto k = a.flat || a.zgroups > 1 ? rows_forward_staged<T_, CPT_, LN, MAXT_, CL, true>           \
+                                     : rows_forward_staged<T_, CPT_, LN, MAXT_, CL, false>;         \
+    e = set_smem(k, sg.smem);                                                                       \
+    if (e == cudaSuccess) e = launch_pdl(k, dim3(grid), block, sg.smem, st, a, sg, ngroups, status); \
   } while (0)
   if (g.CPT == 1 && threads <= 256) CAAT_LAUNCH(1, 256);
   else if (g.CPT == 1) CAAT_LAUNCH(1, 512);
@@ -664,7 +672,8 @@ bool rows_staged_usable(int h, int t, int S_lo, int S_hi, caat_dtype dtype, bool
   return sg.nstages >= 2;
 }
 
-cudaError_t launch_rows_forward_staged(const RowFwdArgs& a, caat_dtype dtype, cudaStream_t st) {
+cudaError_t launch_rows_forward_staged(const RowFwdArgs& args, caat_dtype dtype, cudaStream_t st) {
+  RowFwdArgs a = args;
   const RowGeom g = row_geometry(a.h, dtype);
   const int ES = (int)elem_size(dtype);
   const LaunchLimits lim = effective_limits();
@@ -680,7 +689,7 @@ cudaError_t launch_rows_forward_staged(const RowFwdArgs& a, caat_dtype dtype, cu
   const int ngroups = (a.T + g.TY - 1) / g.TY;
   int grid = sm_count() * per_sm;
   if (lim.rows_ctas > 0 && grid > lim.rows_ctas) grid = lim.rows_ctas;
-  if (grid > ngroups) grid = ngroups;
+  a.flat = flat_units(a, ngroups, grid);
   unsigned int* status = device_status_word();
   if (!status) return cudaErrorUnknown;
   if (cl) {

@@ -84,7 +84,8 @@ struct WarpGeom {
 // ------------------------------------------------------------------ forward
 // stage: a = R rows [kW, h], b = zp rows [kW, P], c = zs rows [kW, S_hi] (rank 0 only)
 // compact layout (CL): a = private residual rows [kW, P], d = shared residual rows [kW, S] (rank 0 only)
-template <typename T_, int CPT, bool LN, bool CL>
+// FEW: few tokens - units dealt inside tokens, the shared part possibly as planes of a split GEMM
+template <typename T_, int CPT, bool LN, bool CL, bool FEW>
 __global__ void __launch_bounds__(kThreads, 3)
 rows_forward_warp(const RowFwdArgs a, const WarpGeom sg, int ngroups, unsigned int* status) {
   using V_ = VT<T_>;
@@ -98,7 +99,7 @@ rows_forward_warp(const RowFwdArgs a, const WarpGeom sg, int ngroups, unsigned i
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int NS = sg.nstages;
   const bool has_priv = a.P > 0 && a.S < a.h, has_shared = a.S > 0;
-  const int my_groups = blockIdx.x < ngroups ? (ngroups - blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+  const UnitRange ur = unit_range(FEW && a.flat, ngroups, a.t);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, kW); }
@@ -117,25 +118,27 @@ rows_forward_warp(const RowFwdArgs a, const WarpGeom sg, int ngroups, unsigned i
       int s = 0; uint32_t ph = 0;
       long long issued = 0;
       bool ok = true;
-      for (int n = 0; n < my_groups && ok; ++n) {
-        const long long i0 = (blockIdx.x + (long long)n * gridDim.x) * kW;
+      int n = ur.n0, m = ur.m0;
+      for (long long u = 0; u < ur.total; ++u) {
+        const long long i0 = (long long)n * kW;
         const int rowsN = (int)((a.T - i0) < kW ? (a.T - i0) : kW);
-        for (int m = 0; m < a.t; ++m) {
-          if (!mbar_wait(empty0 + 8u * s, ph ^ 1u, abort_flag, sg.spin_cap)) { ok = false; break; }
-          const uint32_t bar = full0 + 8u * s;
-          const uint32_t dst = smem_u32(ring + (size_t)s * sg.stage_bytes);
-          const uint32_t bP = has_priv ? (uint32_t)rowsN * a.P * ES : 0u;
-          const uint32_t bR = CL ? bP : (uint32_t)rowsN * a.h * ES;
-          const uint32_t bS = (m == 0 && has_shared) ? (uint32_t)rowsN * a.S_hi * ES : 0u;
-          mbar_expect_tx(bar, bR + bP + (CL ? 2 * bS : bS) + sg.stall_bytes);
-          const long long row = (long long)m * a.T + i0;
-          if (bR) bulk_g2s(dst + sg.off_a, static_cast<const char*>(a.R) + row * (CL ? a.P : a.h) * ES, bR, bar);
-          if (bP) bulk_g2s(dst + sg.off_b, static_cast<const char*>(a.zp) + row * a.P * ES, bP, bar);
-          if (bS) bulk_g2s(dst + sg.off_c, static_cast<const char*>(a.zs) + i0 * a.S_hi * ES, bS, bar);
-          if (CL && bS) bulk_g2s(dst + sg.off_d, static_cast<const char*>(a.Rs) + i0 * a.S_hi * ES, bS, bar);
-          ++issued;
-          if (++s == NS) { s = 0; ph ^= 1u; }
-        }
+        if (!mbar_wait(empty0 + 8u * s, ph ^ 1u, abort_flag, sg.spin_cap)) { ok = false; break; }
+        const uint32_t bar = full0 + 8u * s;
+        const uint32_t dst = smem_u32(ring + (size_t)s * sg.stage_bytes);
+        const bool first = m == 0 || u == 0;          // the shared part comes with the token's first unit here
+        const uint32_t bP = has_priv ? (uint32_t)rowsN * a.P * ES : 0u;
+        const uint32_t bR = CL ? bP : (uint32_t)rowsN * a.h * ES;
+        const uint32_t bS = (first && has_shared) ? (uint32_t)rowsN * a.S_hi * ES : 0u;
+        const uint32_t bZ = FEW && a.zgroups > 1 ? 0u : bS;
+        mbar_expect_tx(bar, bR + bP + bZ + (CL ? bS : 0u) + sg.stall_bytes);
+        const long long row = (long long)m * a.T + i0;
+        if (bR) bulk_g2s(dst + sg.off_a, static_cast<const char*>(a.R) + row * (CL ? a.P : a.h) * ES, bR, bar);
+        if (bP) bulk_g2s(dst + sg.off_b, static_cast<const char*>(a.zp) + row * a.P * ES, bP, bar);
+        if (bZ) bulk_g2s(dst + sg.off_c, static_cast<const char*>(a.zs) + i0 * a.S_hi * ES, bZ, bar);
+        if (CL && bS) bulk_g2s(dst + sg.off_d, static_cast<const char*>(a.Rs) + i0 * a.S_hi * ES, bS, bar);
+        ++issued;
+        if (++s == NS) { s = 0; ph ^= 1u; }
+        if (++m == a.t) { m = 0; n += ur.nstep; }
       }
       if (!ok) {
         *abort_flag = 1;
@@ -185,8 +188,12 @@ rows_forward_warp(const RowFwdArgs a, const WarpGeom sg, int ngroups, unsigned i
   int s = 0; uint32_t ph = 0;
   uint32_t sb = ring32;
   bool dead = false;
-  for (int n = 0; n < my_groups && !dead; ++n) {
-    const long long i = (blockIdx.x + (long long)n * gridDim.x) * kW + warp;
+  int m_first = ur.m0;
+  long long left = ur.total;
+  for (int n = ur.n0; left > 0 && !dead; n += ur.nstep, m_first = 0) {
+    const long long i = (long long)n * kW + warp;
+    const int m_end = left < a.t - m_first ? m_first + (int)left : a.t;
+    left -= m_end - m_first;
     const bool valid = i < a.T;
     float2 zs[CPT][H2];
 #pragma unroll
@@ -194,11 +201,11 @@ rows_forward_warp(const RowFwdArgs a, const WarpGeom sg, int ngroups, unsigned i
 #pragma unroll
       for (int q = 0; q < H2; ++q) zs[j][q] = f2(0.f);
     // compact: column l of the private rows sits at l - S
-    char* pHn = CL ? static_cast<char*>(a.Hn) + (i * a.P - a.S_lo) * ES : static_cast<char*>(a.Hn) + i * a.h * ES;
-    char* pX = static_cast<char*>(a.X) + i * a.h * ES;
-    float* rstd_p = a.rstd + i;
-    float* mean_p = (LN && a.mean) ? a.mean + i : nullptr;
-    for (int m = 0; m < a.t; ++m) {
+    char* pHn = (CL ? static_cast<char*>(a.Hn) + (i * a.P - a.S_lo) * ES : static_cast<char*>(a.Hn) + i * a.h * ES) + m_first * rank_hn;
+    char* pX = static_cast<char*>(a.X) + i * a.h * ES + m_first * rank_h;
+    float* rstd_p = a.rstd + i + (long long)m_first * a.T;
+    float* mean_p = (LN && a.mean) ? a.mean + i + (long long)m_first * a.T : nullptr;
+    for (int m = m_first; m < m_end; ++m) {
       if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8u * s, ph, abort_flag, sg.spin_cap))) {   // warp-uniform verdict
         consumer_gave_up(status, 8u, abort_flag, full0, s, ph, NS, lane);
         dead = true;
@@ -209,9 +216,11 @@ rows_forward_warp(const RowFwdArgs a, const WarpGeom sg, int ngroups, unsigned i
 #pragma unroll
       for (int j = 0; j < CPT; ++j) {
         const bool act = valid && colok[j];
-        if (m == 0 && cls[j] != 1 && colok[j]) {
+        if (m == m_first && cls[j] != 1 && colok[j]) {
           const uint32_t os = ((uint32_t)warp * a.S_hi + col[j]) * ES;
-          unpack2(lds32<raw>(sb + sg.off_c + os), zs[j]);
+          unpack2(FEW && a.zgroups > 1 ? (valid ? sum_planes<T_>(a.zplanes + i * a.S_hi + col[j], (long long)a.T * a.S_hi, a.zgroups)
+                                         : zero_raw<raw>())
+                                : lds32<raw>(sb + sg.off_c + os), zs[j]);
           if constexpr (CL) {       // the shared part of the new stream, formed once: zs + Rs
             float2 r0[H2];
             unpack2(lds32<raw>(sb + sg.off_d + os), r0);
@@ -620,8 +629,9 @@ cudaError_t launch_fwd_warp_t(const RowFwdArgs& a, int cpt, const WarpGeom& g, i
   LaunchScope scope(CAAT_K_ROWS_FORWARD, st);
 #define CAAT_LAUNCH(CPT_)                                                                      \
   do {                                                                                         \
-    e = set_smem(rows_forward_warp<T_, CPT_, LN, CL>, g.smem);                                 \
-    if (e == cudaSuccess) e = launch_pdl(rows_forward_warp<T_, CPT_, LN, CL>, dim3(grid), dim3(kThreads), g.smem, st, a, g, ngroups, status); \
+    auto k = a.flat || a.zgroups > 1 ? rows_forward_warp<T_, CPT_, LN, CL, true> : rows_forward_warp<T_, CPT_, LN, CL, false>; \
+    e = set_smem(k, g.smem);                                                                   \
+    if (e == cudaSuccess) e = launch_pdl(k, dim3(grid), dim3(kThreads), g.smem, st, a, g, ngroups, status); \
   } while (0)
   switch (cpt) {
     case 1: CAAT_LAUNCH(1); break;
@@ -665,7 +675,8 @@ int rows_warp_cpt(int h, int t, caat_dtype dtype) {
   return (cpt >= 1 && cpt <= 4 && t <= 32) ? cpt : 0;
 }
 
-cudaError_t launch_rows_forward_warp(const RowFwdArgs& a, caat_dtype dtype, cudaStream_t st) {
+cudaError_t launch_rows_forward_warp(const RowFwdArgs& args, caat_dtype dtype, cudaStream_t st) {
+  RowFwdArgs a = args;
   const int cpt = rows_warp_cpt(a.h, a.t, dtype);
   const int ES = (int)elem_size(dtype);
   const LaunchLimits lim = effective_limits();
@@ -676,7 +687,7 @@ cudaError_t launch_rows_forward_warp(const RowFwdArgs& a, caat_dtype dtype, cuda
   const int ngroups = (a.T + kW - 1) / kW;
   int grid = sm_count() * per_sm;
   if (lim.rows_ctas > 0 && grid > lim.rows_ctas) grid = lim.rows_ctas;
-  if (grid > ngroups) grid = ngroups;
+  a.flat = flat_units(a, ngroups, grid);
   unsigned int* status = device_status_word();
   if (!status) return cudaErrorUnknown;
   if (a.compact) {

@@ -46,9 +46,10 @@ extern "C" caat_status caat_rowpar_forward_noalloc(const caat_ctx* ctx, caat_lay
   if (!ctx) return CAAT_EINVAL;
   caat_ctx plain = *ctx;
   size_t need = caat_workspace_bytes(ctx, layer, tokens, 0);
-  if (need > (size_t)CAAT_NOALLOC_SCRATCH_BYTES) {
-    // a few tokens of a wide layer: the decode path's fp32 planes do not fit, the large-batch path's scratch may
-    plain.no_decode = 1;
+  // the optional fp32 planes (rank groups; the few-token path's) may not fit where the rest of the scratch does
+  for (int step = 0; step < 2 && need > (size_t)CAAT_NOALLOC_SCRATCH_BYTES; ++step) {
+    if (step == 0) plain.lean_scratch = 1;
+    else plain.no_decode = 1;
     ctx = &plain;
     need = caat_workspace_bytes(ctx, layer, tokens, 0);
   }

@@ -268,7 +268,8 @@ caat_status caat_tp_forward_local_push(const caat_ctx* ctx, caat_layer layer, in
   char* wsb = static_cast<char*>(workspace);
   const RowparShapes sh{ctx->t, tokens, ctx->h, K_r, ctx->S, L.S_lo, L.S_hi, L.P};
   const PushTarget pt{peers->world, peers->rank, slice, pr.recv};
-  cudaError_t e = launch_tc_forward(sh, Y, W, wsb + L.zs_off, wsb + L.zp_off, st, &pt);
+  cudaError_t e = launch_tc_forward(sh, Y, W, wsb + L.zs_off, wsb + L.zp_off, st, &pt, L.gp_groups ? wsb + L.gp_off : nullptr,
+                                    L.gp_groups);
   if (e != cudaSuccess) return cuda_fail(e);
   LaunchScope scope(CAAT_K_TP_EXCHANGE, st);
   e = launch_pdl(tp_signal_kernel, dim3(1), dim3(32), 0, st, pr, peers->world, peers->rank, epoch);
