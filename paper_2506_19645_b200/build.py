@@ -1,8 +1,9 @@
-"""Builds libcaat.so (the C-ABI library) in-tree with nvcc for sm_100a.
+"""Builds libcaat.so (the C-ABI library) and _caatpy.so (the binding's native argument marshalling) in-tree.
 
 Run as ``python -m paper_2506_19645_b200.build``; cross-compiles without a GPU.  Every
-translation unit is compiled to an object file of its own (in parallel, and only when it or a
-header changed), then the objects are linked into the shared library.
+translation unit is compiled to an object file of its own with nvcc for sm_100a (in parallel, and only when
+it or a header changed), then the objects are linked into the shared library.  _caatpy.so is host code: g++ against the
+headers of the installed Python and torch, linked to libcaat.so beside it.
 """
 from __future__ import annotations
 
@@ -10,6 +11,7 @@ import os
 import shlex
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -17,6 +19,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "build")
 LIB = os.path.join(PKG, "libcaat.so")
+PYEXT_SRC, PYEXT = os.path.join(CSRC, "caat_py.cpp"), os.path.join(PKG, "_caatpy.so")
 SOURCES = ["caat_api.cu", "caat_rows.cu", "caat_rows_staged.cu", "caat_rows_lean.cu", "caat_rows_warp.cu", "caat_gemm_simt.cu",
            "caat_gemm_tc.cu", "caat_static.cu", "caat_colpar.cu", "caat_tp_push.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
@@ -62,7 +65,26 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("nvcc failed linking libcaat.so")
+    header = os.path.join(ROOT, "include", "caat.h")
+    if force or not os.path.exists(PYEXT) or os.path.getmtime(PYEXT) < max(
+            os.path.getmtime(f) for f in (PYEXT_SRC, header, os.path.abspath(__file__))):
+        _build_pyext(nvcc)
     return LIB
+
+
+def _build_pyext(nvcc: str) -> None:
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(nvcc)))
+    inc = [os.path.join(ROOT, "include"), os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *[f"-I{i}" for i in inc], PYEXT_SRC, "-o", PYEXT,
+           f"-L{PKG}", "-lcaat", f"-L{os.path.join(t, 'lib')}", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+           "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on caat_py.cpp:\n{r.stdout}{r.stderr}")
 
 
 if __name__ == "__main__":

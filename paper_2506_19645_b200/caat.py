@@ -1,6 +1,7 @@
-"""Thin ctypes binding of libcaat.so (the C ABI declared in include/caat.h).
+"""Thin binding of libcaat.so (the C ABI declared in include/caat.h).
 
-Argument marshalling only: every step of the path runs in the library's CUDA
+Argument marshalling only - natively for the layer, block and column-parallel calls
+(csrc/caat_py.cpp), through ctypes for the rest: every step of the path runs in the library's CUDA
 kernels.  PyTorch is used for device memory (``torch.empty``), ``data_ptr()`` and the
 current CUDA stream.  There is no CPU fallback: without the built library the import
 fails, and without a CUDA device the compute calls raise.
@@ -37,6 +38,10 @@ if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2506_19645_b200.build` "
                       "(there is no fallback path)")
 lib = ctypes.CDLL(LIB_PATH)
+try:
+    from . import _caatpy
+except ImportError as _e:
+    raise ImportError("_caatpy.so is missing or does not load: build it with `python -m paper_2506_19645_b200.build`") from _e
 
 _P = c_void_p
 _sigs = {
@@ -126,6 +131,14 @@ def _ptr(x, dtype=None, shape=None, name="tensor"):
     return x.data_ptr()
 
 
+def _explain(x, code, shape, name):
+    """Raises what `_ptr` raises for an argument that the native marshalling rejected (code -1: uint8, any shape)."""
+    _ptr(x, {CAAT_F32: torch.float32, CAAT_BF16: torch.bfloat16, -1: torch.uint8}[code], shape, name)
+
+
+_caatpy.set_explain(_explain)
+
+
 def _stream():
     return torch.cuda.current_stream().cuda_stream
 
@@ -141,6 +154,10 @@ class Context:
         self.norm = RMSNORM
         self.groups = 1
         _check(lib.caat_create(h, ffn, t, float(p), self.dtype_code, byref(self._h)), "caat_create")
+        self._set_dims()
+
+    def _set_dims(self):
+        self._dims = _caatpy.dims(self._h.value, self.dtype_code, self.t, self.h, self.k_r(CAAT_ATTN_OUT), self.k_r(CAAT_MLP_DOWN))
 
     def __del__(self):
         # at interpreter shutdown the module globals may already be gone
@@ -155,6 +172,7 @@ class Context:
             self.norm = int(value)
         if opt == CAAT_OPT_TP_GROUPS:
             self.groups = int(value)
+            self._set_dims()
         return self
 
     @property
@@ -185,89 +203,33 @@ class Context:
 
     # ---- compute: raw entry points (caller passes every buffer)
     def rowpar_forward(self, layer, tokens, Y, W, R, gamma, beta, Hn, X, rstd, mean, workspace):
-        td, t, h, k = self.torch_dtype, self.t, self.h, self.k_r(layer)
-        st = lib.caat_rowpar_forward(
-            self._h, layer, tokens,
-            _ptr(Y, td, (t, tokens, k), "Y"), _ptr(W, td, (t, h, k), "W"), _ptr(R, td, (t, tokens, h), "R"),
-            _ptr(gamma, td, (h,), "gamma"), _ptr(beta, td, (h,), "beta"),
-            _ptr(Hn, td, (t, tokens, h), "Hn"), _ptr(X, td, (t, tokens, h), "X"),
-            _ptr(rstd, torch.float32, (t, tokens), "rstd"), _ptr(mean, torch.float32, (t, tokens), "mean"),
-            _ptr(workspace, torch.uint8, None, "workspace"), workspace.numel() if workspace is not None else 0,
-            _stream())
-        _check(st, "caat_rowpar_forward")
+        _check(_caatpy.rowpar_forward(
+            self._dims, layer, tokens, Y, W, R, gamma, beta, Hn, X, rstd, mean, workspace), "caat_rowpar_forward")
 
     def rowpar_forward_noalloc(self, layer, tokens, Y, W, R, gamma, beta, Hn, X, rstd, mean):
         """caat_rowpar_forward without a caller workspace: for callers that cannot allocate device
         memory when the layer runs.  Scratch is the library's built-in array (32 MiB); larger
         problems raise CaatError(CAAT_ELIMIT).  Calls on one device must not overlap on the GPU."""
-        td, t, h, k = self.torch_dtype, self.t, self.h, self.k_r(layer)
-        st = lib.caat_rowpar_forward_noalloc(
-            self._h, layer, tokens,
-            _ptr(Y, td, (t, tokens, k), "Y"), _ptr(W, td, (t, h, k), "W"), _ptr(R, td, (t, tokens, h), "R"),
-            _ptr(gamma, td, (h,), "gamma"), _ptr(beta, td, (h,), "beta"),
-            _ptr(Hn, td, (t, tokens, h), "Hn"), _ptr(X, td, (t, tokens, h), "X"),
-            _ptr(rstd, torch.float32, (t, tokens), "rstd"), _ptr(mean, torch.float32, (t, tokens), "mean"),
-            _stream())
-        _check(st, "caat_rowpar_forward_noalloc")
+        _check(_caatpy.rowpar_forward_noalloc(
+            self._dims, layer, tokens, Y, W, R, gamma, beta, Hn, X, rstd, mean), "caat_rowpar_forward_noalloc")
 
     def rowpar_backward(self, layer, tokens, dX, dHn, Y, W, Hn, rstd, mean, gamma, dY, dW, dR, dgamma, dbeta,
                         workspace):
-        td, t, h, k = self.torch_dtype, self.t, self.h, self.k_r(layer)
-        f32 = torch.float32
-        st = lib.caat_rowpar_backward(
-            self._h, layer, tokens,
-            _ptr(dX, td, (t, tokens, h), "dX"), _ptr(dHn, td, (t, tokens, h), "dHn"),
-            _ptr(Y, td, (t, tokens, k), "Y"), _ptr(W, td, (t, h, k), "W"), _ptr(Hn, td, (t, tokens, h), "Hn"),
-            _ptr(rstd, f32, (t, tokens), "rstd"), _ptr(mean, f32, (t, tokens), "mean"), _ptr(gamma, td, (h,), "gamma"),
-            _ptr(dY, td, (t, tokens, k), "dY"), _ptr(dW, f32, (t, h, k), "dW"), _ptr(dR, td, (t, tokens, h), "dR"),
-            _ptr(dgamma, f32, (h,), "dgamma"), _ptr(dbeta, f32, (h,), "dbeta"),
-            _ptr(workspace, torch.uint8, None, "workspace"), workspace.numel() if workspace is not None else 0,
-            _stream())
-        _check(st, "caat_rowpar_backward")
+        _check(_caatpy.rowpar_backward(
+            self._dims, layer, tokens, dX, dHn, Y, W, Hn, rstd, mean, gamma, dY, dW, dR, dgamma, dbeta, workspace), "caat_rowpar_backward")
 
     def block_forward(self, tokens, Y_attn, W_o, Y_mlp, W_down, R0, gamma1, beta1, gamma2, beta2,
                       Hn1, X1, rstd1, mean1, Hn2, X2, rstd2, mean2, workspace):
-        td, t, h = self.torch_dtype, self.t, self.h
-        ka, km = self.k_r(CAAT_ATTN_OUT), self.k_r(CAAT_MLP_DOWN)
-        f32 = torch.float32
-        act = (t, tokens, h)
-        st = lib.caat_block_forward(
-            self._h, tokens,
-            _ptr(Y_attn, td, (t, tokens, ka), "Y_attn"), _ptr(W_o, td, (t, h, ka), "W_o"),
-            _ptr(Y_mlp, td, (t, tokens, km), "Y_mlp"), _ptr(W_down, td, (t, h, km), "W_down"),
-            _ptr(R0, td, act, "R0"), _ptr(gamma1, td, (h,), "gamma1"), _ptr(beta1, td, (h,), "beta1"),
-            _ptr(gamma2, td, (h,), "gamma2"), _ptr(beta2, td, (h,), "beta2"),
-            _ptr(Hn1, td, act, "Hn1"), _ptr(X1, td, act, "X1"), _ptr(rstd1, f32, (t, tokens), "rstd1"),
-            _ptr(mean1, f32, (t, tokens), "mean1"),
-            _ptr(Hn2, td, act, "Hn2"), _ptr(X2, td, act, "X2"), _ptr(rstd2, f32, (t, tokens), "rstd2"),
-            _ptr(mean2, f32, (t, tokens), "mean2"),
-            _ptr(workspace, torch.uint8, None, "workspace"), workspace.numel() if workspace is not None else 0,
-            _stream())
-        _check(st, "caat_block_forward")
+        _check(_caatpy.block_forward(
+            self._dims, tokens, Y_attn, W_o, Y_mlp, W_down, R0, gamma1, beta1, gamma2, beta2, Hn1, X1, rstd1, mean1, Hn2,
+            X2, rstd2, mean2, workspace), "caat_block_forward")
 
     def block_backward(self, tokens, dX1, dX2, dHn2, Y_attn, W_o, Y_mlp, W_down, Hn1, rstd1, mean1, Hn2, rstd2,
                        mean2, gamma1, gamma2, dY_attn, dW_o, dY_mlp, dW_down, dR0, dHn1, dgamma1, dbeta1,
                        dgamma2, dbeta2, workspace):
-        td, t, h = self.torch_dtype, self.t, self.h
-        ka, km = self.k_r(CAAT_ATTN_OUT), self.k_r(CAAT_MLP_DOWN)
-        f32 = torch.float32
-        act = (t, tokens, h)
-        st = lib.caat_block_backward(
-            self._h, tokens,
-            _ptr(dX1, td, act, "dX1"), _ptr(dX2, td, act, "dX2"), _ptr(dHn2, td, act, "dHn2"),
-            _ptr(Y_attn, td, (t, tokens, ka), "Y_attn"), _ptr(W_o, td, (t, h, ka), "W_o"),
-            _ptr(Y_mlp, td, (t, tokens, km), "Y_mlp"), _ptr(W_down, td, (t, h, km), "W_down"),
-            _ptr(Hn1, td, act, "Hn1"), _ptr(rstd1, f32, (t, tokens), "rstd1"), _ptr(mean1, f32, (t, tokens), "mean1"),
-            _ptr(Hn2, td, act, "Hn2"), _ptr(rstd2, f32, (t, tokens), "rstd2"), _ptr(mean2, f32, (t, tokens), "mean2"),
-            _ptr(gamma1, td, (h,), "gamma1"), _ptr(gamma2, td, (h,), "gamma2"),
-            _ptr(dY_attn, td, (t, tokens, ka), "dY_attn"), _ptr(dW_o, f32, (t, h, ka), "dW_o"),
-            _ptr(dY_mlp, td, (t, tokens, km), "dY_mlp"), _ptr(dW_down, f32, (t, h, km), "dW_down"),
-            _ptr(dR0, td, act, "dR0"), _ptr(dHn1, td, act, "dHn1"),
-            _ptr(dgamma1, f32, (h,), "dgamma1"), _ptr(dbeta1, f32, (h,), "dbeta1"),
-            _ptr(dgamma2, f32, (h,), "dgamma2"), _ptr(dbeta2, f32, (h,), "dbeta2"),
-            _ptr(workspace, torch.uint8, None, "workspace"), workspace.numel() if workspace is not None else 0,
-            _stream())
-        _check(st, "caat_block_backward")
+        _check(_caatpy.block_backward(
+            self._dims, tokens, dX1, dX2, dHn2, Y_attn, W_o, Y_mlp, W_down, Hn1, rstd1, mean1, Hn2, rstd2, mean2, gamma1,
+            gamma2, dY_attn, dW_o, dY_mlp, dW_down, dR0, dHn1, dgamma1, dbeta1, dgamma2, dbeta2, workspace), "caat_block_backward")
 
     # ---- compact residual layout: shared part [T, S] once, private parts [t, T, h - S]
     def rowpar_forward_compact(self, layer, tokens, Y, W, Rs, Rp, gamma, beta, Hns, Hnp, X, rstd, mean, workspace):
@@ -302,71 +264,28 @@ class Context:
 
     def block_forward_compact(self, tokens, Y_attn, W_o, Y_mlp, W_down, R0s, R0p, gamma1, beta1, gamma2, beta2,
                               Hn1s, Hn1p, X1, rstd1, mean1, Hn2s, Hn2p, X2, rstd2, mean2, workspace):
-        td, t, h, S = self.torch_dtype, self.t, self.h, self.shared_channels
-        ka, km = self.k_r(CAAT_ATTN_OUT), self.k_r(CAAT_MLP_DOWN)
-        sh, pr, act, st2, f32 = (tokens, S), (t, tokens, h - S), (t, tokens, h), (t, tokens), torch.float32
-        st = lib.caat_block_forward_compact(
-            self._h, tokens,
-            _ptr(Y_attn, td, (t, tokens, ka), "Y_attn"), _ptr(W_o, td, (t, h, ka), "W_o"),
-            _ptr(Y_mlp, td, (t, tokens, km), "Y_mlp"), _ptr(W_down, td, (t, h, km), "W_down"),
-            _ptr(R0s, td, sh, "R0s"), _ptr(R0p, td, pr, "R0p"),
-            _ptr(gamma1, td, (h,), "gamma1"), _ptr(beta1, td, (h,), "beta1"),
-            _ptr(gamma2, td, (h,), "gamma2"), _ptr(beta2, td, (h,), "beta2"),
-            _ptr(Hn1s, td, sh, "Hn1s"), _ptr(Hn1p, td, pr, "Hn1p"), _ptr(X1, td, act, "X1"),
-            _ptr(rstd1, f32, st2, "rstd1"), _ptr(mean1, f32, st2, "mean1"),
-            _ptr(Hn2s, td, sh, "Hn2s"), _ptr(Hn2p, td, pr, "Hn2p"), _ptr(X2, td, act, "X2"),
-            _ptr(rstd2, f32, st2, "rstd2"), _ptr(mean2, f32, st2, "mean2"),
-            _ptr(workspace, torch.uint8, None, "workspace"), workspace.numel() if workspace is not None else 0,
-            _stream())
-        _check(st, "caat_block_forward_compact")
+        _check(_caatpy.block_forward_compact(
+            self._dims, tokens, Y_attn, W_o, Y_mlp, W_down, R0s, R0p, gamma1, beta1, gamma2, beta2, Hn1s, Hn1p, X1, rstd1,
+            mean1, Hn2s, Hn2p, X2, rstd2, mean2, workspace), "caat_block_forward_compact")
 
     def block_backward_compact(self, tokens, dX1, dX2, dHn2s, dHn2p, Y_attn, W_o, Y_mlp, W_down, Hn1s, Hn1p, rstd1,
                                mean1, Hn2s, Hn2p, rstd2, mean2, gamma1, gamma2, dY_attn, dW_o, dY_mlp, dW_down,
                                dR0s, dR0p, dHn1s, dHn1p, dgamma1, dbeta1, dgamma2, dbeta2, workspace):
-        td, t, h, S = self.torch_dtype, self.t, self.h, self.shared_channels
-        ka, km = self.k_r(CAAT_ATTN_OUT), self.k_r(CAAT_MLP_DOWN)
-        sh, pr, act, st2, f32 = (tokens, S), (t, tokens, h - S), (t, tokens, h), (t, tokens), torch.float32
-        st = lib.caat_block_backward_compact(
-            self._h, tokens,
-            _ptr(dX1, td, act, "dX1"), _ptr(dX2, td, act, "dX2"), _ptr(dHn2s, td, sh, "dHn2s"), _ptr(dHn2p, td, pr, "dHn2p"),
-            _ptr(Y_attn, td, (t, tokens, ka), "Y_attn"), _ptr(W_o, td, (t, h, ka), "W_o"),
-            _ptr(Y_mlp, td, (t, tokens, km), "Y_mlp"), _ptr(W_down, td, (t, h, km), "W_down"),
-            _ptr(Hn1s, td, sh, "Hn1s"), _ptr(Hn1p, td, pr, "Hn1p"), _ptr(rstd1, f32, st2, "rstd1"), _ptr(mean1, f32, st2, "mean1"),
-            _ptr(Hn2s, td, sh, "Hn2s"), _ptr(Hn2p, td, pr, "Hn2p"), _ptr(rstd2, f32, st2, "rstd2"), _ptr(mean2, f32, st2, "mean2"),
-            _ptr(gamma1, td, (h,), "gamma1"), _ptr(gamma2, td, (h,), "gamma2"),
-            _ptr(dY_attn, td, (t, tokens, ka), "dY_attn"), _ptr(dW_o, f32, (t, h, ka), "dW_o"),
-            _ptr(dY_mlp, td, (t, tokens, km), "dY_mlp"), _ptr(dW_down, f32, (t, h, km), "dW_down"),
-            _ptr(dR0s, td, sh, "dR0s"), _ptr(dR0p, td, pr, "dR0p"), _ptr(dHn1s, td, sh, "dHn1s"), _ptr(dHn1p, td, pr, "dHn1p"),
-            _ptr(dgamma1, f32, (h,), "dgamma1"), _ptr(dbeta1, f32, (h,), "dbeta1"),
-            _ptr(dgamma2, f32, (h,), "dgamma2"), _ptr(dbeta2, f32, (h,), "dbeta2"),
-            _ptr(workspace, torch.uint8, None, "workspace"), workspace.numel() if workspace is not None else 0,
-            _stream())
-        _check(st, "caat_block_backward_compact")
+        _check(_caatpy.block_backward_compact(
+            self._dims, tokens, dX1, dX2, dHn2s, dHn2p, Y_attn, W_o, Y_mlp, W_down, Hn1s, Hn1p, rstd1, mean1, Hn2s, Hn2p,
+            rstd2, mean2, gamma1, gamma2, dY_attn, dW_o, dY_mlp, dW_down, dR0s, dR0p, dHn1s, dHn1p, dgamma1,
+            dbeta1, dgamma2, dbeta2, workspace), "caat_block_backward_compact")
 
     # ---- column-parallel half: pre = X A^T per rank, Y = act(pre)
     def colpar_workspace_bytes(self, act: int, n_out: int, tokens: int) -> int:
         return int(lib.caat_colpar_workspace_bytes(self._h, act, n_out, tokens))
 
     def colpar_forward(self, act, n_out, tokens, X, A, pre, Y):
-        td, t, h = self.torch_dtype, self.t, self.h
-        wy = n_out // 2 if act == CAAT_ACT_SWIGLU else n_out
-        st = lib.caat_colpar_forward(
-            self._h, act, n_out, tokens,
-            _ptr(X, td, (t, tokens, h), "X"), _ptr(A, td, (t, n_out, h), "A"), _ptr(pre, td, (t, tokens, n_out), "pre"),
-            _ptr(Y, td, (t, tokens, wy), "Y"), _stream())
-        _check(st, "caat_colpar_forward")
+        _check(_caatpy.colpar_forward(self._dims, act, n_out, tokens, X, A, pre, Y), "caat_colpar_forward")
 
     def colpar_backward(self, act, n_out, tokens, dY, X, A, pre, dX, dA, workspace):
-        td, t, h = self.torch_dtype, self.t, self.h
-        wy = n_out // 2 if act == CAAT_ACT_SWIGLU else n_out
-        st = lib.caat_colpar_backward(
-            self._h, act, n_out, tokens,
-            _ptr(dY, td, (t, tokens, wy), "dY"), _ptr(X, td, (t, tokens, h), "X"), _ptr(A, td, (t, n_out, h), "A"),
-            _ptr(pre, td, (t, tokens, n_out), "pre"), _ptr(dX, td, (t, tokens, h), "dX"),
-            _ptr(dA, torch.float32, (t, n_out, h), "dA"),
-            _ptr(workspace, torch.uint8, None, "workspace"), workspace.numel() if workspace is not None else 0,
-            _stream())
-        _check(st, "caat_colpar_backward")
+        _check(_caatpy.colpar_backward(
+            self._dims, act, n_out, tokens, dY, X, A, pre, dX, dA, workspace), "caat_colpar_backward")
 
     # ---- real tensor parallelism: the halves of a layer call around the caller's all-reduce
     def tp_slab(self, layer, tokens, backward, workspace):
