@@ -104,10 +104,11 @@ typedef enum {
   CAAT_OPT_BLOCK_OVERLAP = 9    /* caat_block_forward: 1 = the attention-out layer's row kernel (HBM-bound) runs on a second
                                    stream beside the MLP-down layer's GEMM (tensor-bound), which does not depend on it,
                                    when the workspace holds both layers' scratch (caat_block_workspace_bytes); 0 = the
-                                   layers' kernels run one after the other on the caller's stream; 2 (default) = 1
-                                   unless that GEMM is much the longer of the two kernels (ffn / t large, e.g. the 7B
-                                   shapes, where the GPU is at its power limit and running both at once gains nothing).
-                                   Worth 2-4 % of a training step at the 130M / 1.1B shapes                             */
+                                   layers' kernels run one after the other on the caller's stream; 2 (default) = one
+                                   row kernel for both layers after both GEMMs where it applies (bf16 on the tensor-core
+                                   path, rows of up to 8192 channels, both layers' scratch in the workspace; not
+                                   LayerNorm on rows of more than 1024 channels), else 1 unless that GEMM is much the
+                                   longer of the two kernels (ffn / t large).  The compact block forward follows 0 and 2 */
 } caat_option;
 
 /* Creates a context for hidden size h, MLP width ffn, t ranks, synchronisation

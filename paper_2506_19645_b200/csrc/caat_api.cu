@@ -538,7 +538,8 @@ size_t caat_block_workspace_bytes(const caat_ctx* ctx, int tokens, int backward)
 // variant (registers only); the GEMM gives up one pipeline stage, which leaves the row kernel's loads some L1.
 // Measured: the pair alone gains 13-19 % (7B shapes: 1.74 ms one after the other, 1.41-1.51 ms side by side), a whole
 // training step 2-4 % at the 130M and 1.1B shapes and 1-2 % at the 7B shapes (the GPU runs into its power limit there:
-// with both kernels active the clock drops, which eats the gain).  Hence the automatic choice below: side by side
+// with both kernels active the clock drops, which eats the gain).  Hence the automatic choice below, for shapes that the
+// one-pass row kernel of both layers does not take (that one is the faster schedule wherever it applies): side by side
 // unless the GEMM is the much longer of the two.
 static bool overlap_pays(const caat_ctx* ctx) {
   if (ctx->block_overlap != 2) return ctx->block_overlap == 1;
@@ -584,6 +585,41 @@ static caat_status block_forward_overlapped(const caat_ctx* ctx, int tokens, con
                       nullptr, 2);
 }
 
+// The block forward with both layers' row work in one pass: GEMM 1 -> GEMM 2 -> rows of both layers.  compact: R0 / Hn1 /
+// Hn2 are the private parts and R0s / Hn1s / Hn2s the shared part of the stream.
+static bool fused_rows_apply(const caat_ctx* ctx, int tokens, int compact) {
+  if (!ctx || ctx->block_overlap != 2 || ctx->direct_rows || check_common(ctx, CAAT_MLP_DOWN, tokens) != CAAT_OK) return false;
+  if (!tc_gemm_usable(ctx, layer_kr(ctx, CAAT_ATTN_OUT)) || !tc_gemm_usable(ctx, layer_kr(ctx, CAAT_MLP_DOWN))) return false;
+  const int S_lo = round_down(ctx->S, kLayoutVec), S_hi = round_up(ctx->S, kLayoutVec);
+  return rows_block_usable(ctx->h, ctx->h - S_lo, S_hi, ctx->dtype, compact, ctx->norm);
+}
+static size_t two_layer_scratch(const caat_ctx* ctx, int tokens) {
+  return align_up(scratch_layout(ctx, layer_kr(ctx, CAAT_ATTN_OUT), tokens, 0).total, 256) +
+         scratch_layout(ctx, layer_kr(ctx, CAAT_MLP_DOWN), tokens, 0).total;
+}
+static caat_status block_forward_fused(const caat_ctx* ctx, int tokens, const void* Y_attn, const void* W_o, const void* Y_mlp,
+                                       const void* W_down, const RowBlockArgs& rows, void* workspace, cudaStream_t st) {
+  RowBlockArgs a = rows;
+  char* ws = static_cast<char*>(workspace);
+  for (int l = 0; l < 2; ++l) {
+    const int K_r = layer_kr(ctx, l == 0 ? CAAT_ATTN_OUT : CAAT_MLP_DOWN);
+    const Scratch L = scratch_layout(ctx, K_r, tokens, 0);
+    const RowparShapes sh{ctx->t, tokens, ctx->h, K_r, ctx->S, L.S_lo, L.S_hi, L.P};
+    a.zs[l] = ws + L.zs_off; a.zp[l] = ws + L.zp_off;
+    a.zplanes[l] = reinterpret_cast<const float*>(ws + L.gp_off);
+    a.zgroups[l] = 1;
+    const cudaError_t ce = launch_tc_forward(sh, l == 0 ? Y_attn : Y_mlp, l == 0 ? W_o : W_down, ws + L.zs_off, ws + L.zp_off, st,
+                                             nullptr, L.gp_groups ? ws + L.gp_off : nullptr, L.gp_groups, &a.zgroups[l]);
+    if (ce != cudaSuccess) return cuda_fail(ce);
+    a.S_lo = L.S_lo; a.S_hi = L.S_hi; a.P = L.P;
+    ws += align_up(L.total, 256);
+  }
+  a.t = ctx->t; a.T = tokens; a.h = ctx->h; a.S = ctx->S;
+  a.alpha = (float)ctx->alpha; a.eps = (float)ctx->eps; a.norm = ctx->norm;
+  const cudaError_t ce = launch_rows_forward_block(a, st);
+  return ce == cudaSuccess ? CAAT_OK : cuda_fail(ce);
+}
+
 caat_status caat_block_forward(const caat_ctx* ctx, int tokens, const void* Y_attn, const void* W_o,
                                const void* Y_mlp, const void* W_down, const void* R0, const void* gamma1,
                                const void* beta1, const void* gamma2, const void* beta2, void* Hn1, void* X1,
@@ -593,6 +629,21 @@ caat_status caat_block_forward(const caat_ctx* ctx, int tokens, const void* Y_at
   if (block_decode_applies(ctx, tokens))
     return block_decode(ctx, tokens, Y_attn, W_o, Y_mlp, W_down, R0, gamma1, beta1, gamma2, beta2, Hn1, X1, rstd1, mean1,
                         Hn2, X2, rstd2, mean2, workspace, workspace_bytes, cuda_stream, 0, nullptr, nullptr, nullptr);
+  if (fused_rows_apply(ctx, tokens, 0) && Y_attn && W_o && Y_mlp && W_down && R0 && gamma1 && gamma2 && Hn1 && X1 && rstd1 && Hn2 &&
+      X2 && rstd2 && (ctx->norm == 0 || (mean1 && mean2)) && workspace && workspace_bytes >= two_layer_scratch(ctx, tokens)) {
+    const void* ptrs[] = {Y_attn, W_o, Y_mlp, W_down, R0, gamma1, beta1, gamma2, beta2, Hn1, X1, rstd1, mean1,
+                          Hn2, X2, rstd2, mean2, workspace};
+    bool aligned = true;
+    for (const void* p : ptrs)
+      if (p && !aligned16(p)) aligned = false;
+    if (aligned) {
+      RowBlockArgs a{};
+      a.R = R0; a.gamma[0] = gamma1; a.gamma[1] = gamma2; a.beta[0] = beta1; a.beta[1] = beta2;
+      a.Hn[0] = Hn1; a.Hn[1] = Hn2; a.X[0] = X1; a.X[1] = X2;
+      a.rstd[0] = rstd1; a.rstd[1] = rstd2; a.mean[0] = mean1; a.mean[1] = mean2;
+      return block_forward_fused(ctx, tokens, Y_attn, W_o, Y_mlp, W_down, a, workspace, static_cast<cudaStream_t>(cuda_stream));
+    }
+  }
   if (ctx && overlap_pays(ctx) && !ctx->direct_rows && check_common(ctx, CAAT_MLP_DOWN, tokens) == CAAT_OK &&
       tc_gemm_usable(ctx, layer_kr(ctx, CAAT_ATTN_OUT)) && tc_gemm_usable(ctx, layer_kr(ctx, CAAT_MLP_DOWN)) &&
       Y_attn && W_o && Y_mlp && W_down && R0 && gamma1 && gamma2 && Hn1 && X1 && rstd1 && Hn2 && X2 && rstd2 &&
@@ -693,6 +744,23 @@ caat_status caat_block_forward_compact(const caat_ctx* ctx, int tokens, const vo
   if (block_decode_applies(ctx, tokens))
     return block_decode(ctx, tokens, Y_attn, W_o, Y_mlp, W_down, R0p, gamma1, beta1, gamma2, beta2, Hn1p, X1, rstd1, mean1,
                         Hn2p, X2, rstd2, mean2, workspace, workspace_bytes, cuda_stream, 1, R0s, Hn1s, Hn2s);
+  if (fused_rows_apply(ctx, tokens, 1) && ctx->S % kLayoutVec == 0 && Y_attn && W_o && Y_mlp && W_down && gamma1 && gamma2 && X1 &&
+      rstd1 && X2 && rstd2 && (ctx->norm == 0 || (mean1 && mean2)) && (ctx->S == 0 || (R0s && Hn1s && Hn2s)) &&
+      (ctx->S == ctx->h || (R0p && Hn1p && Hn2p)) && workspace && workspace_bytes >= two_layer_scratch(ctx, tokens)) {
+    const void* ptrs[] = {Y_attn, W_o, Y_mlp, W_down, R0s, R0p, gamma1, beta1, gamma2, beta2, Hn1s, Hn1p, X1, rstd1, mean1,
+                          Hn2s, Hn2p, X2, rstd2, mean2, workspace};
+    bool aligned = true;
+    for (const void* p : ptrs)
+      if (p && !aligned16(p)) aligned = false;
+    if (aligned) {
+      RowBlockArgs a{};
+      a.R = R0p; a.Rs = R0s; a.gamma[0] = gamma1; a.gamma[1] = gamma2; a.beta[0] = beta1; a.beta[1] = beta2;
+      a.Hn[0] = Hn1p; a.Hn[1] = Hn2p; a.Hns[0] = Hn1s; a.Hns[1] = Hn2s; a.X[0] = X1; a.X[1] = X2;
+      a.rstd[0] = rstd1; a.rstd[1] = rstd2; a.mean[0] = mean1; a.mean[1] = mean2;
+      a.compact = 1;
+      return block_forward_fused(ctx, tokens, Y_attn, W_o, Y_mlp, W_down, a, workspace, static_cast<cudaStream_t>(cuda_stream));
+    }
+  }
   caat_status s = caat_rowpar_forward_compact(ctx, CAAT_ATTN_OUT, tokens, Y_attn, W_o, R0s, R0p, gamma1, beta1, Hn1s,
                                               Hn1p, X1, rstd1, mean1, workspace, workspace_bytes, cuda_stream);
   if (s != CAAT_OK) return s;

@@ -141,6 +141,21 @@ struct RowFwdArgs {
   // set by the launchers of the bulk-copy kernels, see unit_range()
   int flat;
 };
+// both layers of a block in one pass (the second layer's residual is the first one's new stream as stored)
+struct RowBlockArgs {
+  const void *zs[2], *zp[2];
+  const float* zplanes[2];
+  int zgroups[2];
+  const void *R, *Rs;               // Rs, Hns: compact stream
+  const void *gamma[2], *beta[2];
+  void *Hn[2], *Hns[2], *X[2];
+  float *rstd[2], *mean[2];
+  int t, T, h, S, S_lo, S_hi, P;
+  float alpha, eps;
+  int norm, compact, flat;
+};
+bool rows_block_usable(int h, int P, int S_hi, caat_dtype dtype, int compact, int norm);
+cudaError_t launch_rows_forward_block(const RowBlockArgs& a, cudaStream_t st);
 // direct: 0 = automatic (warp-per-token kernels for short rows, else the bulk-copy staged kernels
 // whenever a ring of at least two stages fits in shared memory), 1 = plain-load kernels,
 // 2 = staged kernels even for short rows.

@@ -166,13 +166,13 @@ __device__ __forceinline__ UnitRange unit_range(bool flat, int ngroups, int t) {
   }
   return u;
 }
-// Decides and trims the grid.  A compact stream updated in place (Rs == Hns) stays whole: rank 0's unit overwrites the
-// shared part that the token's other units read.
-inline int flat_units(const RowFwdArgs& a, int ngroups, int& grid) {
-  const long long units = (long long)ngroups * a.t;
+// Decides and trims the grid.  whole: keep tokens whole - a compact stream updated in place, whose shared part rank 0's
+// unit overwrites while the token's other units read it.
+inline int flat_units(int t, bool whole, int ngroups, int& grid) {
+  const long long units = (long long)ngroups * t;
   const int g = (long long)grid < units ? grid : (int)units;
-  const long long strided = (long long)((ngroups + grid - 1) / grid) * a.t, flat = (units + g - 1) / g;
-  if (10 * strided > 11 * flat && !(a.compact && a.Rs == a.Hns)) { grid = g; return 1; }
+  const long long strided = (long long)((ngroups + grid - 1) / grid) * t, flat = (units + g - 1) / g;
+  if (10 * strided > 11 * flat && !whole) { grid = g; return 1; }
   if (grid > ngroups) grid = ngroups;
   return 0;
 }

@@ -687,7 +687,7 @@ cudaError_t launch_rows_forward_warp(const RowFwdArgs& args, caat_dtype dtype, c
   const int ngroups = (a.T + kW - 1) / kW;
   int grid = sm_count() * per_sm;
   if (lim.rows_ctas > 0 && grid > lim.rows_ctas) grid = lim.rows_ctas;
-  a.flat = flat_units(a, ngroups, grid);
+  a.flat = flat_units(a.t, a.compact && a.Rs == a.Hns, ngroups, grid);
   unsigned int* status = device_status_word();
   if (!status) return cudaErrorUnknown;
   if (a.compact) {
