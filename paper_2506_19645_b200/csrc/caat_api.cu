@@ -99,7 +99,8 @@ caat_status cuda_fail(cudaError_t e) {
 }
 
 static size_t decode_planes_bytes(const caat_ctx* ctx, int tokens) {
-  return align_up((size_t)kDecodeMaxSplits * ctx->t * tokens * ctx->h * sizeof(float), 256);
+  // at most kDecodeMaxSplits planes per rank of either part; their rows are padded to the 8-channel grid
+  return align_up((size_t)kDecodeMaxSplits * ctx->t * tokens * (ctx->h + 2 * kLayoutVec) * sizeof(float), 256);
 }
 
 Scratch scratch_layout(const caat_ctx* ctx, int K_r, int tokens, int backward) {
@@ -186,12 +187,11 @@ static caat_status forward_impl(const caat_ctx* ctx, int K_r, int T, const void*
     // few tokens (decode): the weights dominate the traffic; stream them with swapped operands and
     // let the row kernel form the rank sum from fp32 per-rank partials
     float* zt = reinterpret_cast<float*>(wsb + L.zt_off);
-    const int splits = tc_decode_splits(K_r, K_r, T);
-    const DecodeProblem pr{K_r, Y, W, zt, splits};
-    ce = launch_tc_forward_decode(t, T, h, &pr, 1, st);
+    DecodeProblem pr{K_r, Y, W, zt};
+    ce = launch_tc_forward_decode(t, T, h, S, &pr, 1, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
     RowPartArgs a{};
-    a.L[0] = PartialLayer{zt, splits, gamma, beta, Hn, X, rstd, mean, Hns};
+    a.L[0] = PartialLayer{pr.zs, pr.zp, pr.ns, pr.np, gamma, beta, Hn, X, rstd, mean, Hns};
     a.nlayers = 1; a.R = R; a.t = t; a.T = T; a.h = h; a.S = S; a.compact = compact; a.Rs = Rs;
     a.alpha = (float)ctx->alpha; a.eps = (float)ctx->eps; a.norm = ctx->norm;
     ce = launch_rows_forward_partials(a, ctx->dtype, st);
@@ -372,14 +372,12 @@ static caat_status block_decode(const caat_ctx* ctx, int tokens, const void* Y_a
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   float* zt1 = reinterpret_cast<float*>(static_cast<char*>(workspace) + L.zt_off);
   float* zt2 = reinterpret_cast<float*>(static_cast<char*>(workspace) + L.zt_off + decode_planes_bytes(ctx, tokens));
-  const int kmin = ka < km ? ka : km;
-  const int sp1 = tc_decode_splits(ka, kmin, tokens), sp2 = tc_decode_splits(km, kmin, tokens);
-  const DecodeProblem pr[2] = {{ka, Y_attn, W_o, zt1, sp1}, {km, Y_mlp, W_down, zt2, sp2}};
-  cudaError_t ce = launch_tc_forward_decode(ctx->t, tokens, ctx->h, pr, 2, st);
+  DecodeProblem pr[2] = {{ka, Y_attn, W_o, zt1}, {km, Y_mlp, W_down, zt2}};
+  cudaError_t ce = launch_tc_forward_decode(ctx->t, tokens, ctx->h, ctx->S, pr, 2, st);
   if (ce != cudaSuccess) return cuda_fail(ce);
   RowPartArgs a{};
-  a.L[0] = PartialLayer{zt1, sp1, gamma1, beta1, Hn1, X1, rstd1, mean1, Hn1s};
-  a.L[1] = PartialLayer{zt2, sp2, gamma2, beta2, Hn2, X2, rstd2, mean2, Hn2s};
+  a.L[0] = PartialLayer{pr[0].zs, pr[0].zp, pr[0].ns, pr[0].np, gamma1, beta1, Hn1, X1, rstd1, mean1, Hn1s};
+  a.L[1] = PartialLayer{pr[1].zs, pr[1].zp, pr[1].ns, pr[1].np, gamma2, beta2, Hn2, X2, rstd2, mean2, Hn2s};
   a.nlayers = 2; a.R = R0; a.t = ctx->t; a.T = tokens; a.h = ctx->h; a.S = ctx->S;
   a.alpha = (float)ctx->alpha; a.eps = (float)ctx->eps; a.norm = ctx->norm;
   a.compact = compact; a.Rs = R0s;

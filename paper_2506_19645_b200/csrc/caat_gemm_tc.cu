@@ -20,9 +20,12 @@
 // word, drains its own copies in flight, frees tensor memory and returns.
 #include <cuda.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <mutex>
+#include <utility>
 
 #include "caat_internal.h"
 
@@ -51,6 +54,8 @@ constexpr int kAidMask = ~0;
 constexpr int kAidMask = 1024;
 #endif
 
+constexpr int kMaxRegions = 4;
+
 struct Unit {            // one contraction segment of a tile
   int mapA, mapB;        // indices into the tensor-map array
   int ak0, am0;          // offsets added to A's K / M coordinate
@@ -67,7 +72,8 @@ struct Region {          // a family of output tiles with the same operand wirin
   int M, N, batch;       // valid output extents per batch
   int mtiles, ntiles;    // the output goes through the region's own tensor map (TMA store);
                          // its z coordinate is split * batch + b
-  float* out_t;          // transposed direct-store output (decode), else unused
+  float* out_t;          // transposed direct-store output (few tokens): [z][N][out_ld] fp32, else unused
+  long long out_ld;
   // Weight gradient with a partition off the 8-channel grid: the private rows start at S_lo (TMA reads channels in
   // 16-byte units), and the first `skip` = S - S_lo rows, which belong to the shared region, are not stored.  Only the
   // region's first row tile has such rows; it stores fp32 straight from registers to skip_out (plane z of skip_plane
@@ -85,17 +91,15 @@ struct Region {          // a family of output tiles with the same operand wirin
 
 struct Params {
   int nregions;
-  Region r[2];
+  Region r[kMaxRegions];
   int BN;                // tile width (UMMA N): multiple of 16 (of 64 when B is N-major)
   int nstages;
   int a_mn, b_mn;        // 1: operand is MN-major in global memory
-  int out_transposed;    // 1: D is [channels x tokens]; store fp32 straight to the region's out_t[z][token][channel]
-  long long out_t_ld;    // channels per token row of out_t
   int cg;                // CTAs per tile: 1, or 2 (tcgen05 cta_group::2, clusters of two)
   int splits;            // split-K factor (only with a single unit and Q == 1)
   int push_slice;        // > 0: tiles of region 0 (the shared columns) are stored into the peer GPUs' receive slots, the
                          // owner of a tile being its first row / push_slice (a multiple of the tile's rows)
-  int tiles_r0;          // tiles of region 0 (including splits)
+  int tile_end[kMaxRegions];   // tiles of regions 0..i (including splits)
   int tiles_total;
   unsigned int* status;
   uint32_t spin_cap;     // polls of one mbarrier wait before the role gives up (kSpinCap; CAAT_TC_SPINCAP for the timeout test)
@@ -222,14 +226,50 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
 // Output maps of the peers' receive slots (the exchange of the shared-channel slab over peer memory).
 struct PeerMaps { CUtensorMap m[CAAT_MAX_PEERS]; };
 
+// Operand maps (A and B of up to two layers or units) and output maps, one per region.
+struct Maps { CUtensorMap ab[4], c[kMaxRegions]; };
+
+// The swapped variant's tiles dealt to CTAs by their length (longest first, each to the least loaded CTA): CTA w works
+// item[first[w]] .. item[first[w + 1] - 1].  dealt == 0: round-robin by tile number.
+constexpr int kMaxDealWorkers = 160, kMaxDealItems = 1024;
+struct Deal {
+  int dealt;
+  uint16_t first[kMaxDealWorkers + 1];
+  uint16_t item[kMaxDealItems];
+};
+template <bool SWAP> struct ExtraArg { using type = PeerMaps; };
+template <> struct ExtraArg<true> { using type = Deal; };
+
+// the tiles of one worker, in order
+template <bool SWAP>
+struct TileIter {
+  const typename ExtraArg<SWAP>::type& x;
+  int pos, end, step;
+  __device__ __forceinline__ TileIter(const typename ExtraArg<SWAP>::type& x_, int worker, int nworkers, int total) : x(x_) {
+    pos = worker; end = total; step = nworkers;
+    if constexpr (SWAP) {
+      if (x.dealt) { pos = x.first[worker]; end = x.first[worker + 1]; step = 1; }
+    }
+  }
+  __device__ __forceinline__ bool valid() const { return pos < end; }
+  __device__ __forceinline__ int tile() const {
+    if constexpr (SWAP) return x.dealt ? x.item[pos] : pos;
+    return pos;
+  }
+  __device__ __forceinline__ void next() { pos += step; }
+};
+
 struct TileCoord {
   int region, b, mt, nt, split;
 };
 
 __device__ __forceinline__ TileCoord decode_tile(const Params& p, int tile) {
   TileCoord c;
-  c.region = (tile >= p.tiles_r0) ? 1 : 0;
-  int rem = tile - (c.region ? p.tiles_r0 : 0);
+  c.region = 0;
+#pragma unroll
+  for (int g = 0; g + 1 < kMaxRegions; ++g)
+    if (tile >= p.tile_end[g]) c.region = g + 1;       // unused regions end where the last used one does: never reached
+  int rem = tile - (c.region ? p.tile_end[c.region - 1] : 0);
   const Region& r = p.r[c.region];
   c.nt = rem % r.ntiles; rem /= r.ntiles;
   c.split = rem % r.splits; rem /= r.splits;
@@ -314,10 +354,8 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {   // arrives on
 // SWAP: the operands are swapped (few tokens: weights on the 128-row side), fp32 planes stored straight from registers.
 template <int CG, bool SWAP>
 __global__ void __launch_bounds__(kThreads, 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
-               const __grid_constant__ CUtensorMap map2, const __grid_constant__ CUtensorMap map3,
-               const __grid_constant__ CUtensorMap cmap0, const __grid_constant__ CUtensorMap cmap1,
-               const __grid_constant__ PeerMaps pm, const Params p) {
+tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename ExtraArg<SWAP>::type extra,
+               const __grid_constant__ Params p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr int BMT = BM * CG;                     // rows of a tile (of the pair's tile)
   const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
@@ -340,8 +378,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const CUtensorMap* maps[4] = {&map0, &map1, &map2, &map3};
-  const CUtensorMap* cmaps[2] = {&cmap0, &cmap1};
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.nstages; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, 1); }
@@ -388,8 +424,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       int stage = 0; uint32_t phase = 0;
       long long issued = 0;
       bool ok = true;
-      for (int tile = worker; tile < p.tiles_total && ok; tile += nworkers) {
-        const TileCoord c = decode_tile(p, tile);
+      for (TileIter<SWAP> it(extra, worker, nworkers, p.tiles_total); it.valid() && ok; it.next()) {
+        const TileCoord c = decode_tile(p, it.tile());
         const Region& r = p.r[c.region];
         const uint32_t cols_cta = (uint32_t)tile_cols(p, r, c.nt, CG) / CG;    // B columns this CTA stages
         const uint32_t b_tile_bytes = cols_cta * BK * 2;
@@ -399,7 +435,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         const int nb = multi ? (isA ? BM / 64 : (int)cols_cta / 64) : 1;         // boxes of this tile's stages
         for (int ui = 0; ui < r.nunits && ok; ++ui) {
           const Unit& u = r.u[ui];
-          const CUtensorMap* map = maps[isA ? u.mapA : u.mapB];
+          const CUtensorMap* map = &mp.ab[isA ? u.mapA : u.mapB];
           int q0, q1, kb, ke;
           split_range(r, u, c.split, q0, q1, kb, ke);
           for (int q = q0; q < q1 && ok; ++q) {
@@ -423,7 +459,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
                     if (CG == 2) tma_load_3d_pair(dst, map, x, y, z, fb); else tma_load_3d(dst, map, x, y, z, fb);
                   };
                   if (isA) {
-                    if (!p.a_mn) load(sa, u.ak0 + kk * BK, m0);
+                    if (!p.a_mn) load(sa, u.ak0 + kk * BK, u.am0 + m0);
                     else load(sa + box * (64 * BK * 2), u.am0 + m0 + box * 64, u.ak0 + kk * BK);
                   } else {
                     if (!p.b_mn) load(sb, u.bk0 + kk * BK, u.bn0 + n0);
@@ -471,8 +507,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       const uint32_t a_lo0 = (uint32_t)a_const + (tiles_sa >> 4), b_lo0 = (uint32_t)b_const + ((tiles_sa + a_bytes) >> 4);
       uint32_t a_lo = a_lo0, b_lo = b_lo0;
       uint32_t full_bar = full0, empty_bar = empty0;
-      for (int tile = worker; tile < p.tiles_total && ok; tile += nworkers) {
-        const TileCoord c = decode_tile(p, tile);
+      for (TileIter<SWAP> it(extra, worker, nworkers, p.tiles_total); it.valid() && ok; it.next()) {
+        const TileCoord c = decode_tile(p, it.tile());
         const Region& r = p.r[c.region];
         if (!mbar_wait_warp(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, p.spin_cap)) { ok = false; break; }
         tc_fence_after();
@@ -521,8 +557,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     int acc = 0; uint32_t acc_phase = 0;
     uint32_t slab = 0;
     bool ok = true;
-    for (int tile = worker; tile < p.tiles_total && ok; tile += nworkers) {
-      const TileCoord c = decode_tile(p, tile);
+    for (TileIter<SWAP> it(extra, worker, nworkers, p.tiles_total); it.valid() && ok; it.next()) {
+      const TileCoord c = decode_tile(p, it.tile());
       const Region& r = p.r[c.region];
       // a tile whose contraction range is empty leaves the accumulator undefined: its value is 0
       int total_k = 0;
@@ -543,12 +579,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       const int zc = c.split * r.batch + c.b;
       // where this tile's rows go: the region's own output, or - shared columns of a multi-GPU forward - the
       // receive slot of the GPU that owns these token rows, through its own map (row 0 = the owner's first token)
-      const CUtensorMap* omap = cmaps[c.region];
+      const CUtensorMap* omap = &mp.c[c.region];
       int om0 = m0;
-      if (p.push_slice > 0 && c.region == 0) {
-        const int owner = m0 / p.push_slice;
-        omap = &pm.m[owner];
-        om0 = m0 - owner * p.push_slice;
+      if constexpr (!SWAP) {
+        if (p.push_slice > 0 && c.region == 0) {
+          const int owner = m0 / p.push_slice;
+          omap = &extra.m[owner];
+          om0 = m0 - owner * p.push_slice;
+        }
       }
       const int rr = quarter * 32 + lane;                 // row of the tile this thread holds
       const uint32_t sw = (uint32_t)(lane & 7);           // 128-byte swizzle: 16-byte chunk ^= row % 8
@@ -569,12 +607,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + cc), v);
           tmem_ld_wait();
           if (chan < r.M) {
-            float* dst = r.out_t + ((long long)zc * r.N + n0 + cc) * p.out_t_ld + chan;
+            float* dst = r.out_t + ((long long)zc * r.N + n0 + cc) * r.out_ld + chan;
             const int ntok = r.N - (n0 + cc);           // tokens left from this column on (>= 1)
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
               if (e < ntok) *dst = total_k == 0 ? 0.f : __uint_as_float(v[e]);
-              dst += p.out_t_ld;
+              dst += r.out_ld;
             }
           }
         }
@@ -842,8 +880,8 @@ TileCfg pick_tile(const RegionShape* r, int nr, bool b_n_major, int max_splits, 
   return best;
 }
 
-cudaError_t launch(const CUtensorMap maps[4], const CUtensorMap cmaps[2], Params& p, int kind, cudaStream_t st,
-                   const PeerMaps* peer_maps = nullptr) {
+cudaError_t launch(const Maps& maps, Params& p, int kind, cudaStream_t st, const PeerMaps* peer_maps = nullptr,
+                   const Deal* deal = nullptr) {
   const LaunchLimits lim = effective_limits();
   const int stage_bytes = BM * BK * 2 + (p.BN / p.cg) * BK * 2;
   const int budget = lim.gemm_smem > 0 && lim.gemm_smem < 227 * 1024 ? lim.gemm_smem : 227 * 1024;
@@ -874,6 +912,7 @@ cudaError_t launch(const CUtensorMap maps[4], const CUtensorMap cmaps[2], Params
             p.splits, nst, p.tiles_total, p.r[0].M, p.r[0].N, p.r[0].batch);
   int workers_max = sm_count() / p.cg;
   if (lim.gemm_workers > 0 && lim.gemm_workers / p.cg < workers_max) workers_max = lim.gemm_workers / p.cg;
+  if (deal && workers_max > kMaxDealWorkers) workers_max = kMaxDealWorkers;
   const int workers = p.tiles_total < workers_max ? p.tiles_total : workers_max;
   if (workers < 1) return cudaSuccess;
   cudaLaunchConfig_t cfg{};
@@ -891,13 +930,11 @@ cudaError_t launch(const CUtensorMap maps[4], const CUtensorMap cmaps[2], Params
   cfg.attrs = attr;
   cfg.numAttrs = pdl_enabled() ? 2 : 1;
   LaunchScope scope(kind, st);
+  if (deal) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, true>, maps, *deal, (const Params&)p);
   static const PeerMaps no_peers{};
   const PeerMaps& pm = peer_maps ? *peer_maps : no_peers;
-  if (p.out_transposed)
-    return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, true>, maps[0], maps[1], maps[2], maps[3], cmaps[0], cmaps[1], pm, p);
-  if (p.cg == 2)
-    return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, false>, maps[0], maps[1], maps[2], maps[3], cmaps[0], cmaps[1], pm, p);
-  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, false>, maps[0], maps[1], maps[2], maps[3], cmaps[0], cmaps[1], pm, p);
+  if (p.cg == 2) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, false>, maps, pm, (const Params&)p);
+  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, false>, maps, pm, (const Params&)p);
 }
 
 void finish_tiles(Params& p) {
@@ -907,8 +944,11 @@ void finish_tiles(Params& p) {
     r.ntiles = (r.N + p.BN - 1) / p.BN;
     if (r.splits < 1) r.splits = p.splits < 1 ? 1 : p.splits;
   }
-  p.tiles_r0 = p.r[0].mtiles * p.r[0].ntiles * p.r[0].batch * p.r[0].splits;
-  p.tiles_total = p.tiles_r0 + (p.nregions > 1 ? p.r[1].mtiles * p.r[1].ntiles * p.r[1].batch * p.r[1].splits : 0);
+  p.tiles_total = 0;
+  for (int g = 0; g < kMaxRegions; ++g) {
+    if (g < p.nregions) p.tiles_total += p.r[g].mtiles * p.r[g].ntiles * p.r[g].batch * p.r[g].splits;
+    p.tile_end[g] = p.tiles_total;
+  }
 }
 
 }  // namespace
@@ -947,7 +987,8 @@ int tc_forward_groups(const RowparShapes& s, int max_groups) { return forward_pl
 
 cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* W, void* zs, void* zp,
                               cudaStream_t st, const PushTarget* push, void* planes, int max_groups, int* groups_out) {
-  CUtensorMap maps[4], cmaps[2];
+  Maps mp;
+  CUtensorMap *maps = mp.ab, *cmaps = mp.c;
   PeerMaps pmaps{};
   Params p{};
   const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
@@ -978,7 +1019,6 @@ cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* 
     r.M = s.T; r.N = n_pr; r.batch = s.t; r.b_slowest = 1;
     if (!make_cmap(&cmaps[g - 1], zp, n_pr, s.T, s.t, s.P, (long long)s.T * s.P, false)) return cudaErrorInvalidValue;
   }
-  if (g == 1) cmaps[1] = cmaps[0];
   p.nregions = g;
   if (push && n_sh > 0 && groups == 1) {
     // shared tiles go to the owners' receive slots: slot `rank` of GPU q is [slice, S] 16-bit elements; the map of
@@ -994,7 +1034,7 @@ cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* 
     p.push_slice = push->slice;
   }
   finish_tiles(p);
-  const cudaError_t e = launch(maps, cmaps, p, CAAT_K_TC_FORWARD, st, push && n_sh > 0 && groups == 1 ? &pmaps : nullptr);
+  const cudaError_t e = launch(mp, p, CAAT_K_TC_FORWARD, st, push && n_sh > 0 && groups == 1 ? &pmaps : nullptr);
   if (e != cudaSuccess || groups == 1 || groups_out) return e;
   const long long n8 = (long long)s.T * s.S_hi / 8;
   const int blocks = (int)((n8 + 255) / 256 < 8 * sm_count() ? (n8 + 255) / 256 : 8 * sm_count());
@@ -1008,52 +1048,200 @@ cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* 
                     s.T, s.S_hi / 8, groups, slots);
 }
 
-// ---- decode forward (few tokens): zt[m][i][l] = sum_k W[m][l][k] Y[m][i][k], fp32, for ALL channels.
-// The operands are swapped (weights on the 128-row side, tokens on the narrow side) so that a tile
-// streams 128 x K_r weights however few tokens there are; every (rank, 128-channel block) is a tile,
-// which spreads the weight stream over all SMs.  The rank sum of the shared channels is left to the
-// row kernel (the partials are tiny at these token counts).
-int tc_decode_splits(int K_r, int K_r_min, int T) {
-  // Work items are (rank, 128-channel block, split).  Splitting the longer layer's contraction until its
-  // items are about as long as the shorter layer's makes the round-robin deal even; the fp32 partial
-  // planes this adds (t * splits * T * h * 4 bytes) are kept near a tenth of the layer's weight bytes.
-  const int ks = (K_r + BK - 1) / BK, ks_min = (K_r_min + BK - 1) / BK;
-  int sp = (ks + ks_min / 2) / (ks_min > 0 ? ks_min : 1);
-  const int cap_traffic = K_r / (20 * T);
-  if (sp > cap_traffic) sp = cap_traffic;
-  if (sp > kDecodeMaxSplits) sp = kDecodeMaxSplits;
-  if (sp > ks / 2) sp = ks / 2;
-  return sp < 1 ? 1 : sp;
+// ---- few tokens: the operands are swapped (weights on the 128-row side, tokens on the narrow side), so that a tile streams
+// 128 weight rows however few tokens there are, and the sums leave as fp32 planes for the row kernel:
+//   zs[g][i][l]  l < S     sum over the g-th group of qper ranks (qper = 0: one plane per rank and k-split)
+//   zp[k][m][i][l - S_lo]  l >= S, the k-th part of the contraction
+// A tile is (plane, 128 channels).  Both layers of a block go in one launch.  Tiles differ in length (qper ranks of k-steps
+// against one), so they are dealt longest first to the least loaded CTA.  Fewer, longer tiles mean fewer planes for the
+// row kernel - with many tokens every rank's CTA reads every shared plane - but a coarser deal; few_token_plan weighs them.
+namespace {
+struct FewPlan { FewSplit l[2]; Deal deal; int workers; };
+
+constexpr double kItemOverhead = 1.5;     // of a tile, in k-steps: refill of the pipeline and the epilogue
+constexpr double kStepUs = 0.38;          // a k-step of 16 KB of weights on one of 148 SMs at 6.4 TB/s
+
+struct FewItem { float len; uint16_t tile; };
+
+// tiles in the kernel's numbering (decode_tile with one column tile): region, then split fastest, then mt, then b
+int few_items(int t, int h, int S, const int* K_r, int n, const FewSplit* sp, FewItem* out) {
+  const int S_lo = round_down(S, kLayoutVec);
+  int cnt = 0;
+  for (int g = 0; g < n; ++g) {
+    const int ks = (K_r[g] + BK - 1) / BK;
+    for (int part = 0; part < 2; ++part) {
+      const int M = part == 0 ? S : (S < h ? h - S_lo : 0);
+      if (M <= 0) continue;
+      const int mt = (M + BM - 1) / BM;
+      const bool grouped = part == 0 && sp[g].qper > 0;
+      const int splits = part == 0 ? (grouped ? (t + sp[g].qper - 1) / sp[g].qper : sp[g].ksplits) : sp[g].ksplits;
+      const int batch = grouped ? 1 : t, per = (ks + splits - 1) / splits;
+      for (int b = 0; b < batch * mt; ++b)
+        for (int k = 0; k < splits; ++k) {
+          int len;
+          if (grouped) len = ks * ((k + 1) * sp[g].qper <= t ? sp[g].qper : t - k * sp[g].qper);
+          else len = per * (k + 1) <= ks ? per : (ks > per * k ? ks - per * k : 0);
+          if (cnt == kMaxDealItems) return -1;
+          out[cnt] = FewItem{(float)(len + kItemOverhead), (uint16_t)cnt};
+          ++cnt;
+        }
+    }
+  }
+  return cnt;
 }
 
-cudaError_t launch_tc_forward_decode(int t, int T, int h, const DecodeProblem* pr, int n, cudaStream_t st) {
+// longest first, each to the least loaded worker; returns the busiest worker's load, fills `deal` when given
+double few_deal(FewItem* it, int n, int workers, Deal* deal) {
+  std::sort(it, it + n, [](const FewItem& a, const FewItem& b) { return a.len > b.len || (a.len == b.len && a.tile < b.tile); });
+  std::pair<float, int> load[kMaxDealWorkers];
+  for (int w = 0; w < workers; ++w) load[w] = {0.f, w};
+  auto more = [](const std::pair<float, int>& a, const std::pair<float, int>& b) { return a > b; };
+  static thread_local uint8_t owner[kMaxDealItems];
+  std::make_heap(load, load + workers, more);
+  float worst = 0.f;
+  for (int i = 0; i < n; ++i) {
+    std::pop_heap(load, load + workers, more);
+    auto& l = load[workers - 1];
+    l.first += it[i].len;
+    worst = l.first > worst ? l.first : worst;
+    owner[i] = (uint8_t)l.second;
+    std::push_heap(load, load + workers, more);
+  }
+  if (deal) {
+    int pos = 0;
+    for (int w = 0; w < workers; ++w) {
+      deal->first[w] = (uint16_t)pos;
+      for (int i = 0; i < n; ++i)
+        if (owner[i] == w) deal->item[pos++] = it[i].tile;
+    }
+    deal->first[workers] = (uint16_t)pos;
+    deal->dealt = 1;
+  }
+  return worst;
+}
+
+// Chooses the splits of one or two layers.  The row kernel's share: a plane of the shared part is written once and read
+// by every rank's CTA (once per token when the ranks share it through a cluster), a private plane is read once.
+void few_token_plan(int t, int T, int h, int S, const int* K_r, int n, int sms, FewPlan* best) {
+  const int workers = sms < kMaxDealWorkers ? sms : kMaxDealWorkers;
+  static thread_local FewItem items[kMaxDealItems];
+  double best_cost = -1;
+  const bool clustered = (long long)T * t <= (long long)sms * 3 / 4;
+  FewSplit cand[2][16];
+  int nc[2] = {0, 0};
+  for (int g = 0; g < n; ++g) {
+    const int ks = (K_r[g] + BK - 1) / BK;
+    for (int q = t; q >= 1; q = q > 1 ? (q + 1) / 2 : 0)
+      if (nc[g] < 12) cand[g][nc[g]++] = FewSplit{q, 1};
+    for (int k = 2; k <= kDecodeMaxSplits && 2 * k <= ks; ++k) cand[g][nc[g]++] = FewSplit{0, k};
+  }
+  if (n == 1) { cand[1][0] = FewSplit{t, 1}; nc[1] = 1; }
+  best->l[0] = best->l[1] = FewSplit{1, 1};
+  // a deal is computed only where its lower bound (even share, longest tile, planes) can still win
+  struct Cand { double bound, rest; FewSplit l[2]; };
+  Cand all[256];
+  int na = 0;
+  for (int i = 0; i < nc[0]; ++i)
+    for (int j = 0; j < nc[1]; ++j) {
+      Cand c{0, 0, {cand[0][i], cand[1][j]}};
+      double total = 0, longest = 0;
+      for (int g = 0; g < n; ++g) {
+        const int ks = (K_r[g] + BK - 1) / BK, ns = few_shared_planes(c.l[g], t);
+        const int ms = (S + BM - 1) / BM, mp = S < h ? (h - round_down(S, kLayoutVec) + BM - 1) / BM : 0;
+        total += (double)(ms + mp) * t * ks + kItemOverhead * ((double)ms * ns + (double)mp * t * c.l[g].ksplits);
+        const double len = c.l[g].qper > 0 ? (S > 0 ? c.l[g].qper : 1) * ks : (ks + c.l[g].ksplits - 1) / c.l[g].ksplits;
+        if (len > longest) longest = len;
+        const double bytes = 4.0 * T * ((double)ns * S * (clustered ? 2 : 1 + t) + 2.0 * c.l[g].ksplits * t * (h - S));
+        c.rest += bytes / 8e12 * 1e6;
+      }
+      c.bound = fmax(total / workers, longest + kItemOverhead) * kStepUs + c.rest;
+      all[na++] = c;
+    }
+  std::sort(all, all + na, [](const Cand& a, const Cand& b) { return a.bound < b.bound; });
+  for (int i = 0; i < na && (best_cost < 0 || all[i].bound < best_cost); ++i) {
+    const int cnt = few_items(t, h, S, K_r, n, all[i].l, items);
+    if (cnt <= 0) continue;
+    const double cost = few_deal(items, cnt, workers, nullptr) * kStepUs + all[i].rest;
+    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best->l[0] = all[i].l[0]; best->l[1] = all[i].l[1]; }
+  }
+  const int cnt = few_items(t, h, S, K_r, n, best->l, items);
+  best->deal.dealt = 0;
+  best->workers = workers;
+  if (cnt > 0) {
+    if (cnt < workers) best->workers = cnt;
+    few_deal(items, cnt, best->workers, &best->deal);
+  }
+}
+
+// The plan depends on the shapes alone; the most recent ones are kept (the oldest is replaced).
+struct FewKey { int t, T, h, S, K0, K1, sms; bool operator==(const FewKey& o) const { return !memcmp(this, &o, sizeof(o)); } };
+constexpr int kFewPlans = 64;
+
+void few_plan_cached(int t, int T, int h, int S, const int* K_r, int n, FewPlan* out) {
+  static FewKey keys[kFewPlans];
+  static FewPlan plans[kFewPlans];
+  static int used = 0, next = 0;
+  static std::mutex m;
+  const FewKey key{t, T, h, S, K_r[0], n > 1 ? K_r[1] : 0, sm_count()};
+  std::lock_guard<std::mutex> lock(m);
+  for (int i = 0; i < used; ++i)
+    if (keys[i] == key) { *out = plans[i]; return; }
+  const int slot = used < kFewPlans ? used++ : (next++ % kFewPlans);
+  few_token_plan(t, T, h, S, K_r, n, key.sms, &plans[slot]);
+  keys[slot] = key;
+  *out = plans[slot];
+}
+}  // namespace
+
+cudaError_t launch_tc_forward_decode(int t, int T, int h, int S, DecodeProblem* pr, int n, cudaStream_t st) {
   if (n < 1 || n > 2) return cudaErrorInvalidValue;
-  CUtensorMap maps[4], cmaps[2];
+  static thread_local FewPlan plan;
+  {
+    const int K[2] = {pr[0].K_r, n > 1 ? pr[1].K_r : 0};
+    few_plan_cached(t, T, h, S, K, n, &plan);
+  }
+  Maps mp;
   Params p{};
   p.BN = (T + 31) / 32 * 32;
   if (p.BN > 256) return cudaErrorInvalidValue;
   p.cg = 1;
-  p.a_mn = 0; p.b_mn = 0;  p.splits = 1;
-  p.out_transposed = 1; p.out_t_ld = h;
-  // longer contraction first: round-robin dealing then fills the tail with the short items
-  int order[2] = {0, 1};
-  if (n == 2 && pr[1].K_r > pr[0].K_r) { order[0] = 1; order[1] = 0; }
-  for (int g = 0; g < n; ++g) {
-    const DecodeProblem& q = pr[order[g]];
-    if (!make_map(&maps[2 * g], q.W, q.K_r, h, t, q.K_r, (long long)h * q.K_r, BK, BM)) return cudaErrorInvalidValue;
-    if (!make_map(&maps[2 * g + 1], q.Y, q.K_r, T, t, q.K_r, (long long)T * q.K_r, BK, p.BN)) return cudaErrorInvalidValue;
-    Region& r = p.r[g];
-    r.nunits = 1;
-    r.u[0] = Unit{2 * g, 2 * g + 1, 0, 0, 0, 0, 1, 0, 1, 0, 1, (q.K_r + BK - 1) / BK};
-    r.M = h; r.N = T; r.batch = t; r.b_slowest = 1;
-    r.out_t = q.zt;
-    r.splits = q.splits;
+  p.splits = 1;
+  const int S_lo = round_down(S, kLayoutVec), S_hi = round_up(S, kLayoutVec), P = h - S_lo;
+  int g = 0;
+  for (int l = 0; l < n; ++l) {
+    DecodeProblem& q = pr[l];
+    const FewSplit sp = plan.l[l];
+    const int ks = (q.K_r + BK - 1) / BK;
+    q.ns = S > 0 ? few_shared_planes(sp, t) : 0;
+    q.np = S < h ? sp.ksplits : 0;
+    q.zp = q.zs + (size_t)q.ns * T * S_hi;
+    if (!make_map(&mp.ab[2 * l], q.W, q.K_r, h, t, q.K_r, (long long)h * q.K_r, BK, BM)) return cudaErrorInvalidValue;
+    if (!make_map(&mp.ab[2 * l + 1], q.Y, q.K_r, T, t, q.K_r, (long long)T * q.K_r, BK, p.BN)) return cudaErrorInvalidValue;
+    if (S > 0) {
+      Region& r = p.r[g++];
+      const bool grouped = sp.qper > 0;
+      r.nunits = 1;
+      r.u[0] = Unit{2 * l, 2 * l + 1, 0, 0, 0, 0, !grouped, grouped, !grouped, grouped, grouped ? t : 1, ks};
+      r.M = S; r.N = T; r.batch = grouped ? 1 : t; r.b_slowest = 1;
+      r.splits = grouped ? q.ns : sp.ksplits;
+      r.qper = sp.qper;
+      r.out_t = q.zs; r.out_ld = S_hi;
+    }
+    if (S < h) {
+      Region& r = p.r[g++];
+      r.nunits = 1;
+      r.u[0] = Unit{2 * l, 2 * l + 1, 0, S_lo, 0, 0, 1, 0, 1, 0, 1, ks};
+      r.M = P; r.N = T; r.batch = t; r.b_slowest = 1;
+      r.splits = sp.ksplits;
+      r.out_t = q.zp; r.out_ld = P;
+    }
   }
-  if (n == 1) { maps[2] = maps[0]; maps[3] = maps[1]; }
-  cmaps[0] = maps[0]; cmaps[1] = maps[0];          // unused: the epilogue stores directly
-  p.nregions = n;
+  if (n == 1) { mp.ab[2] = mp.ab[0]; mp.ab[3] = mp.ab[1]; }
+  for (int c = 0; c < kMaxRegions; ++c) mp.c[c] = mp.ab[0];          // unused: the epilogue stores directly
+  p.nregions = g;
   finish_tiles(p);
-  return launch(maps, cmaps, p, CAAT_K_TC_FORWARD, st);
+  if (plan.deal.dealt && plan.deal.first[plan.workers] != p.tiles_total) return cudaErrorInvalidValue;
+  return launch(mp, p, CAAT_K_TC_FORWARD, st, nullptr, &plan.deal);
 }
 
 // ---- dgrad: dY[m] = gs W[m][:S] + (alpha gp[m]) W[m][S:]
@@ -1063,7 +1251,8 @@ cudaError_t launch_tc_forward_decode(int t, int T, int h, const DecodeProblem* p
 // coordinate -(S - S_lo), so the shared columns among them meet rows that TMA fills with zeros.
 cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* W, void* dY,
                             void* w_scaled, bool w_scaled_ready, cudaStream_t st) {
-  CUtensorMap maps[4], cmaps[2];
+  Maps mp;
+  CUtensorMap *maps = mp.ab, *cmaps = mp.c;
   Params p{};
   {
     const RegionShape rs[1] = {{s.T, s.K_r, s.t, (s.S + BK - 1) / BK + (s.h - s.S_lo + BK - 1) / BK}};
@@ -1099,10 +1288,9 @@ cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOpe
   r.nunits = nu;
   r.M = s.T; r.N = s.K_r; r.batch = s.t; r.b_slowest = 1; r.scale = 1.0f;
   if (!make_cmap(&cmaps[0], dY, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, false)) return cudaErrorInvalidValue;
-  cmaps[1] = cmaps[0];
   p.nregions = 1;
   finish_tiles(p);
-  return launch(maps, cmaps, p, CAAT_K_TC_DGRAD, st);
+  return launch(mp, p, CAAT_K_TC_DGRAD, st);
 }
 
 static TileCfg wgrad_cfg(const RowparShapes& s) {
@@ -1119,7 +1307,8 @@ size_t tc_wgrad_splitk_bytes(const RowparShapes& s) {
 // ---- wgrad: dW[m][:S] = gs^T Y[m] ; dW[m][S:] = alpha gp[m]^T Y[m]      (fp32 out; alpha in the epilogue)
 cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* Y, float* dW,
                             void* splitk, size_t splitk_bytes, cudaStream_t st) {
-  CUtensorMap maps[4], cmaps[2];
+  Maps mp;
+  CUtensorMap *maps = mp.ab, *cmaps = mp.c;
   Params p{};
   const TileCfg wc = wgrad_cfg(s);
   p.BN = wc.bn; p.cg = wc.cg;
@@ -1164,10 +1353,9 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
                    (long long)s.h * s.K_r, true))
       return cudaErrorInvalidValue;
   }
-  if (g == 1) cmaps[1] = cmaps[0];
   p.nregions = g;
   finish_tiles(p);
-  cudaError_t e = launch(maps, cmaps, p, CAAT_K_TC_WGRAD, st);
+  cudaError_t e = launch(mp, p, CAAT_K_TC_WGRAD, st);
   if (e != cudaSuccess) return e;
   if (splits > 1) {
     const long long n4 = dw_elems / 4;   // K_r is a multiple of 8

@@ -113,13 +113,15 @@ cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOpe
 cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* Y, float* dW,
                             void* splitk, size_t splitk_bytes, cudaStream_t st);
 size_t tc_wgrad_splitk_bytes(const RowparShapes& s);
-// decode (few tokens): per-rank fp32 partials for all channels, zt[t, T, h]
+// few tokens: the sums leave the GEMM as fp32 planes, zs [ns][T][S_hi] shared and zp [np][t][T][h - S_lo] private
 constexpr int kDecodeMaxTokens = 64;
-// zt[split * t + m][i][l] = partial of sum_k W[m][l][k] Y[m][i][k]; one or two layers in one launch
-struct DecodeProblem { int K_r; const void* Y; const void* W; float* zt; int splits; };
-int tc_decode_splits(int K_r, int K_r_min, int T);
 constexpr int kDecodeMaxSplits = 4;
-cudaError_t launch_tc_forward_decode(int t, int T, int h, const DecodeProblem* pr, int n, cudaStream_t st);
+// qper > 0: a shared plane sums qper ranks; qper == 0: a plane per rank and k-split.  ksplits: private planes.
+struct FewSplit { int qper, ksplits; };
+inline int few_shared_planes(const FewSplit& s, int t) { return s.qper > 0 ? (t + s.qper - 1) / s.qper : t * s.ksplits; }
+// one or two layers in one launch; zs is the scratch of the layer's planes, zp, ns and np are set by the call
+struct DecodeProblem { int K_r; const void* Y; const void* W; float* zs; float* zp; int ns, np; };
+cudaError_t launch_tc_forward_decode(int t, int T, int h, int S, DecodeProblem* pr, int n, cudaStream_t st);
 
 // ---- row kernels ------------------------------------------------------------
 struct RowFwdArgs {
@@ -164,7 +166,7 @@ cudaError_t launch_rows_forward_staged(const RowFwdArgs& a, caat_dtype dtype, cu
 // forward row work from fp32 partial planes (decode); with two layers the second layer's residual is
 // the first layer's new residual stream (as stored), both layers in one launch
 struct PartialLayer {
-  const float* zt; int splits; const void* gamma; const void* beta; void* Hn; void* X; float* rstd; float* mean;
+  const float* zs; const float* zp; int ns, np; const void* gamma; const void* beta; void* Hn; void* X; float* rstd; float* mean;
   void* Hns;   // compact layout: the shared part of this layer's new stream, [T, S]; Hn then holds the private parts
 };
 struct RowPartArgs {

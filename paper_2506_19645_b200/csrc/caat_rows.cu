@@ -379,11 +379,10 @@ __global__ void __launch_bounds__(512, CPT == 1 ? 2 : 1) rows_backward_kernel(co
 }
 
 // ------------------------------------------------------------------ forward from fp32 partial planes (decode)
-// One CTA per (token, rank).  zt holds fp32 partial outputs [splits * t, T, h] for ALL channels (plane
-// z = split * t + rank).  Shared channels: sum of every plane, z ascending; private channels: sum over
-// the splits of this rank's planes, times alpha.  Every rank's CTA forms the shared sum for itself (a few
-// kilobytes, L2 hits), so no CTA waits for another.  With two layers the second one's residual is the
-// first one's new residual stream as stored (rounded to the storage type).
+// One CTA per (token, rank).  The sums come as fp32 planes, zs [ns][T][S_hi] of the shared channels (a plane holds a group
+// of ranks or a part of one rank's contraction), zp [np][t][T][h - S_lo] of the private ones; planes are added in
+// ascending order.  Every rank's CTA forms the shared sum for itself (L2 hits), so no CTA waits for another.  With two
+// layers the second one's residual is the first one's new residual stream as stored (rounded to the storage type).
 template <typename T_, bool LN>
 __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPartArgs a) {
   using V_ = VT<T_>;
@@ -397,11 +396,10 @@ __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPar
   int par = 0;
   const int i = blockIdx.x, m = blockIdx.y;
   const long long row = (long long)m * a.T + i;
-  const long long plane = (long long)a.T * a.h;
+  const int S_lo = a.S / V * V, S_hi = (a.S + V - 1) / V * V, P = a.h - S_lo;
   const float inv_h = 1.0f / (float)a.h;
   for (int layer = 0; layer < a.nlayers; ++layer) {
     const PartialLayer& L = a.L[layer];
-    const int nplanes = L.splits * a.t;
     float st[1] = {0.f};
     for (int c = threadIdx.x * V; c < a.h; c += blockDim.x * V) {
       float r[V], z[V], hn[V];
@@ -416,13 +414,14 @@ __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPar
 #pragma unroll
         for (int e = 0; e < V; ++e) r[e] = V_::round(hrow[c + e]);
       }
-      const float* base = L.zt + (long long)i * a.h + c;
-      auto plane_sum = [&](float (&out)[V], int z0, int zstep, int nz) {
+      const float* zs = L.zs + (long long)i * S_hi + c;
+      const float* zp = L.zp + row * P + (c - S_lo);
+      const long long ps = (long long)a.T * S_hi, pp = (long long)a.t * a.T * P;
+      auto plane_sum = [&](float (&out)[V], const float* pz, long long stride, int nz) {
 #pragma unroll
         for (int e = 0; e < V; ++e) out[e] = 0.f;
 #pragma unroll 8
-        for (int q = 0; q < nz; ++q) {
-          const float* pz = base + (long long)(z0 + q * zstep) * plane;
+        for (int q = 0; q < nz; ++q, pz += stride) {
 #pragma unroll
           for (int e = 0; e < V; e += 4) {
             const float4 v = *reinterpret_cast<const float4*>(pz + e);
@@ -430,12 +429,12 @@ __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPar
           }
         }
       };
-      plane_sum(z, shared_chunk ? 0 : m, shared_chunk ? 1 : a.t, shared_chunk ? nplanes : L.splits);
+      plane_sum(z, shared_chunk ? zs : zp, shared_chunk ? ps : pp, shared_chunk ? L.ns : L.np);
       const float scale = shared_chunk ? 1.f : a.alpha;
 #pragma unroll
       for (int e = 0; e < V; ++e) hn[e] = fmaf(scale, z[e], r[e]);
       if (mixed) {
-        plane_sum(z, 0, 1, nplanes);
+        plane_sum(z, zs, ps, L.ns);
 #pragma unroll
         for (int e = 0; e < V; ++e) hn[e] = c + e < a.S ? z[e] + r[e] : hn[e];
       }
@@ -507,7 +506,7 @@ inline size_t cluster_partials_smem(const RowPartArgs& a) {
   const int S4 = (a.S + 7) / 8 * 2, P4 = (a.h - a.S / 8 * 8) / 4;
   const int ns_max = (S4 + a.t - 1) / a.t;
   size_t f4 = (size_t)a.nlayers * S4 + 16;            // rank sums of the shared channels, reduction scratch
-  for (int l = 0; l < a.nlayers; ++l) f4 += (size_t)a.L[l].splits * ((size_t)a.t * ns_max + P4);
+  for (int l = 0; l < a.nlayers; ++l) f4 += (size_t)a.L[l].ns * ns_max + (size_t)a.L[l].np * P4;
   return f4 * sizeof(float4);
 }
 
@@ -529,7 +528,7 @@ __global__ void __launch_bounds__(512, MINB) rows_forward_partials_cluster_kerne
   float* red = reinterpret_cast<float*>(sm4 + a.nlayers * S4);
   float4* stage = sm4 + a.nlayers * S4 + 16;
   const long long row = (long long)m * a.T + i;
-  const long long plane = (long long)a.T * a.h;
+  const int S_hi = S4 * 4, P = P4 * 4;
   int par = 0;
   // a peer's shared memory may be written only once that CTA runs: arrive now, wait before the first remote store
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
@@ -542,18 +541,19 @@ __global__ void __launch_bounds__(512, MINB) rows_forward_partials_cluster_kerne
 #pragma unroll
     for (int l = 0; l < 2; ++l) {
       if (l >= a.nlayers) break;
-      const int splits = a.L[l].splits, nplanes = splits * a.t;
-      const float* zt = a.L[l].zt + (long long)i * a.h;
+      const int nplanes = a.L[l].ns, splits = a.L[l].np;
+      const float* zs0 = a.L[l].zs + (long long)i * S_hi + 4 * cs0;
+      const float* zp0 = a.L[l].zp + row * P;
       sh_off[l] = off;
       for (int idx = tid; idx < nplanes * ns; idx += nthr) {
         const int z = idx / ns, c = idx - z * ns;
-        cp_async16(stage + off + idx, zt + z * plane + 4 * (cs0 + c));
+        cp_async16(stage + off + idx, zs0 + (long long)z * a.T * S_hi + 4 * c);
       }
       off += nplanes * ns;
       pr_off[l] = off;
       for (int idx = tid; idx < splits * P4; idx += nthr) {
         const int q = idx / P4, c = idx - q * P4;
-        cp_async16(stage + off + idx, zt + (long long)(m + q * a.t) * plane + S_lo + 4 * c);
+        cp_async16(stage + off + idx, zp0 + (long long)q * a.t * a.T * P + 4 * c);
       }
       off += splits * P4;
     }
@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(512, MINB) rows_forward_partials_cluster_kerne
 #pragma unroll
   for (int l = 0; l < 2; ++l) {
       if (l >= a.nlayers) break;
-    const int splits = a.L[l].splits, nplanes = splits * a.t;
+    const int splits = a.L[l].np, nplanes = a.L[l].ns;
     for (int q = tid; q < ns; q += nthr) {
       const float4* src = stage + sh_off[l] + q;
       float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
