@@ -86,7 +86,7 @@ struct Region {          // a family of output tiles with the same operand wirin
   int out_f32;
   int b_slowest;         // tile order: 1 = rank index slowest (a rank's weights / activations stay
                          // hot in L2 while its row tiles stream), 0 = row tile slowest
-  float scale;           // fp32 outputs are multiplied by it in the epilogue (0 means 1)
+  float scale;           // outputs are multiplied by it in the epilogue (0 means 1)
 };
 
 struct Params {
@@ -639,7 +639,7 @@ tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename
         const bool out_f32 = r.out_f32 != 0;
         const int sub = out_f32 ? 32 : 64;
         const int cols = (p.debug & kAidMask & 2) ? 0 : (r.N - n0 < p.BN ? r.N - n0 : p.BN);
-        const bool scaled = out_f32 && r.scale != 0.f && r.scale != 1.f;
+        const bool scaled = r.scale != 0.f && r.scale != 1.f;
         if (cols <= 0) release();
         for (int cc = 0; cc < cols; cc += sub) {
           uint32_t v[32], w[32];
@@ -667,6 +667,13 @@ tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename
             for (int q4 = 0; q4 < 8; ++q4)
               sts128(rowaddr + (((uint32_t)q4 ^ sw) << 4), v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
           } else {
+            if (scaled) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) {
+                v[e] = __float_as_uint(__uint_as_float(v[e]) * r.scale);
+                w[e] = __float_as_uint(__uint_as_float(w[e]) * r.scale);
+              }
+            }
             auto pack = [](uint32_t lo, uint32_t hi) {
               __nv_bfloat162 bb = __floats2bfloat162_rn(__uint_as_float(lo), __uint_as_float(hi));
               return *reinterpret_cast<uint32_t*>(&bb);
@@ -1265,7 +1272,7 @@ cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOpe
   maps[3] = maps[1];
   if (n_pr > 0) {
     const void* wp = W;
-    if (pv.alpha != 1.0f) {
+    if (pv.alpha != 1.0f && !pv.gs_over_alpha) {
       // sum_l (alpha g[l]) W[l][k] = sum_l g[l] (alpha W[l][k]): the private gradient is read as stored in dR,
       // the weights' private rows (the small operand) carry alpha; they were scaled by the launch before this one
       if (!w_scaled || !w_scaled_ready) return cudaErrorInvalidValue;
@@ -1286,7 +1293,7 @@ cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOpe
   if (n_sh > 0) r.u[nu++] = Unit{0, 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, (n_sh + BK - 1) / BK};
   if (n_pr > 0) r.u[nu++] = Unit{2, 3, pv.col0, 0, s.S_lo - s.S, 0, 1, 0, 1, 0, 1, (n_pr + BK - 1) / BK};
   r.nunits = nu;
-  r.M = s.T; r.N = s.K_r; r.batch = s.t; r.b_slowest = 1; r.scale = 1.0f;
+  r.M = s.T; r.N = s.K_r; r.batch = s.t; r.b_slowest = 1; r.scale = pv.gs_over_alpha ? pv.alpha : 1.0f;
   if (!make_cmap(&cmaps[0], dY, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, false)) return cudaErrorInvalidValue;
   p.nregions = 1;
   finish_tiles(p);
@@ -1335,7 +1342,7 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
     r.u[0] = Unit{0, 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, ksteps};
     r.out_f32 = 1;
     r.M = n_sh; r.N = s.K_r; r.batch = s.t; r.b_slowest = 0;   // the shared gradient panel serves all ranks at once
-    r.scale = 1.0f;
+    r.scale = pv.gs_over_alpha ? pv.alpha : 1.0f;
     if (!make_cmap(&cmaps[g - 1], out, s.K_r, n_sh, (long long)s.t * splits, s.K_r, (long long)s.h * s.K_r, true))
       return cudaErrorInvalidValue;
   }

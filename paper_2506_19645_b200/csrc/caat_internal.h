@@ -104,7 +104,10 @@ int tc_forward_groups(const RowparShapes& s, int max_groups);
 // ptr[(m * T + i) * ld + col0 + (l - S_lo)], and the gradient is alpha times the stored value for l >= S.
 //   the residual gradient itself (per rank):  {dR, h, S_lo, alpha}   (no scaled copy is written at all)
 //   compact stream:                           {dRp, P, 0, alpha}
-struct PrivOperand { const void* ptr; int ld; int col0; float alpha; };
+// gs_over_alpha: the shared gradient gs was stored divided by alpha, so both products are alpha times what the operands
+// give and alpha rides on the epilogue; otherwise the data gradient needs the private rows of the weights times alpha
+// (the shared gradient is then somebody's result: the compact stream's dRs, the slab of a multi-GPU exchange).
+struct PrivOperand { const void* ptr; int ld; int col0; float alpha; int gs_over_alpha; };
 // dY[m] = [gs | alpha gp[m]] W[m];  w_scaled: [t, h, K_r] scratch for the alpha-scaled private rows of W
 // w_scaled_ready: the scaled rows are already in w_scaled (written by the row kernels' reduction launch)
 cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* W, void* dY,
@@ -199,6 +202,7 @@ struct RowBwdArgs {
   int compact;
   const void *Hns, *dHns;
   int reduce_mode;   // CAAT_OPT_BACKWARD_REDUCE (plain-load kernels only)
+  float gs_scale;    // the reduced shared gradient is stored times this (1, or 1 / alpha: see PrivOperand::gs_over_alpha)
   // optional side job of the norm-gradient reduction launch: w_dst[m][l][:] = alpha * w_src[m][l][:] for the
   // private rows l >= S of the layer's weights [t, h, w_Kr] (bf16), which the data gradient reads next
   const void* w_src;

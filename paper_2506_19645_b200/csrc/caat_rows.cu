@@ -329,7 +329,11 @@ __global__ void __launch_bounds__(512, CPT == 1 ? 2 : 1) rows_backward_kernel(co
 #pragma unroll
     for (int j = 0; j < CPT; ++j)
       if (act[j] && cls[j] != 1)
+      {
+#pragma unroll
+        for (int e = 0; e < V; ++e) gsum[j][e] *= a.gs_scale;
         stg<raw>(gs_row(a, i, ES) + (long long)col[j] * ES, V_::pack(gsum[j]));
+      }
   }
 
   // Partial norm-parameter gradients of this CTA: one row of [h] per CTA.  With several
@@ -718,20 +722,22 @@ cudaError_t launch_partials_cluster(const RowPartArgs& a, int threads, size_t sm
   return cudaLaunchKernelEx(&cfg, rows_forward_partials_cluster_kernel<T_, LN, MINB>, a);
 }
 
-// out[l] = sum over `rows` partial rows, fixed order: 32 row lanes then a serial combine.
+// out[l] = sum over `rows` partial rows, fixed order: 128 row lanes, then 8 x 16, then 8.  Eight columns (a 32-byte sector)
+// per block: a chain of a few loads per thread on most SMs.
 // Blocks past the first `nreduce` run an unrelated small job that has to happen between the row kernel and the
 // data gradient anyway and would otherwise cost a launch of its own: scaling the private rows of the weights.
 struct ScaleJob { const uint4* src; uint4* dst; int t, h, K_r, S; float alpha; };
 
 __global__ void __launch_bounds__(1024) reduce_partials_kernel(const float* __restrict__ part, float* __restrict__ out,
-                                                               int rows, int h, int nreduce, ScaleJob job) {
-  __shared__ float sm[32][33];
+                                                               const float* __restrict__ part2, float* __restrict__ out2, int rows,
+                                                               int h, int nreduce, ScaleJob job) {
+  __shared__ float sm[128][9];
   pdl_wait();
   if ((int)blockIdx.x >= nreduce) {
     const int row_chunks = job.K_r / 8;
     const long long per_rank = (long long)(job.h - job.S) * row_chunks, total = per_rank * job.t;
     const long long nthreads = (long long)(gridDim.x - nreduce) * 1024;
-    for (long long q = (long long)(blockIdx.x - nreduce) * 1024 + threadIdx.y * 32 + threadIdx.x; q < total; q += nthreads) {
+    for (long long q = (long long)(blockIdx.x - nreduce) * 1024 + threadIdx.y * 8 + threadIdx.x; q < total; q += nthreads) {
       const long long m = q / per_rank, r = q - m * per_rank;
       const long long idx = (m * job.h + job.S) * row_chunks + r;
       const uint4 v = job.src[idx];
@@ -747,15 +753,25 @@ __global__ void __launch_bounds__(1024) reduce_partials_kernel(const float* __re
     }
     return;
   }
-  const int c = blockIdx.x * 32 + threadIdx.x;
+  int block = blockIdx.x;
+  if (part2 != nullptr && 2 * block >= nreduce) { block -= nreduce / 2; part = part2; out = out2; }     // the bias gradients
+  const int c = block * 8 + threadIdx.x;
   float s = 0.f;
   if (c < h)
-    for (int r = threadIdx.y; r < rows; r += 32) s += part[(size_t)r * h + c];
+    for (int r = threadIdx.y; r < rows; r += 128) s += part[(size_t)r * h + c];
   sm[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y < 8) {
+    float t = 0.f;
+#pragma unroll
+    for (int y = 0; y < 16; ++y) t += sm[threadIdx.y * 16 + y][threadIdx.x];
+    sm[threadIdx.y * 16][threadIdx.x] = t;
+  }
   __syncthreads();
   if (threadIdx.y == 0 && c < h) {
     float tot = 0.f;
-    for (int y = 0; y < 32; ++y) tot += sm[y][threadIdx.x];
+#pragma unroll
+    for (int y = 0; y < 8; ++y) tot += sm[16 * y][threadIdx.x];
     out[c] = tot;
   }
 }
@@ -901,8 +917,9 @@ cudaError_t launch_rows_backward(const RowBwdArgs& a, caat_dtype dtype, int dire
   else
     e = a.norm == 1 ? launch_bwd_t<float, true, false>(a, g, rows, st) : launch_bwd_t<float, false, false>(a, g, rows, st);
   if (e != cudaSuccess) return e;
-  const dim3 rb(32, 32);
-  const int nreduce = (a.h + 31) / 32;
+  const dim3 rb(8, 128);
+  const bool bias = a.norm == 1 && a.dbeta && a.dbpart;
+  const int nreduce = (a.h + 7) / 8 * (bias ? 2 : 1);
   ScaleJob job{};
   int nscale = 0;
   if (a.w_dst && a.w_src && a.S < a.h) {
@@ -914,14 +931,8 @@ cudaError_t launch_rows_backward(const RowBwdArgs& a, caat_dtype dtype, int dire
   }
   {
     LaunchScope scope(CAAT_K_NORMGRAD_REDUCE, st);
-    e = launch_pdl(reduce_partials_kernel, dim3(nreduce + nscale), rb, 0, st, (const float*)a.dgpart, a.dgamma, rows, a.h,
-                   nreduce, job);
-    if (e != cudaSuccess) return e;
-  }
-  if (a.norm == 1 && a.dbeta && a.dbpart) {
-    LaunchScope scope(CAAT_K_NORMGRAD_REDUCE, st);
-    e = launch_pdl(reduce_partials_kernel, dim3(nreduce), rb, 0, st, (const float*)a.dbpart, a.dbeta, rows, a.h, nreduce,
-                   ScaleJob{});
+    e = launch_pdl(reduce_partials_kernel, dim3(nreduce + nscale), rb, 0, st, (const float*)a.dgpart, a.dgamma,
+                   bias ? (const float*)a.dbpart : (const float*)nullptr, a.dbeta, rows, a.h, nreduce, job);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();

@@ -71,6 +71,13 @@ __device__ __forceinline__ uint4 pack2(const float2 (&f)[4]) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 __device__ __forceinline__ float4 pack2(const float2 (&f)[2]) { return make_float4(f[0].x, f[0].y, f[1].x, f[1].y); }
+template <int H2>
+__device__ __forceinline__ auto pack2_scaled(const float2 (&f)[H2], float s) {
+  float2 g[H2];
+#pragma unroll
+  for (int q = 0; q < H2; ++q) g[q] = mul2(f[q], f2(s));
+  return pack2(g);
+}
 
 // 16-byte shared-memory load through a 32-bit shared address (volatile: stays behind the barrier waits)
 template <typename raw>

@@ -292,7 +292,7 @@ rows_backward_lean(const RowBwdArgs a, const StageGeom sg, int ngroups, unsigned
       }
 #pragma unroll
       for (int j = 0; j < CPT; ++j)
-        if (act[j] && shared_chunk(j)) stg<raw>(gs_row(a, (long long)i, ES) + (long long)col[j] * ES, pack2(gsum[j]));
+        if (act[j] && shared_chunk(j)) stg<raw>(gs_row(a, (long long)i, ES) + (long long)col[j] * ES, pack2_scaled(gsum[j], a.gs_scale));
       asm volatile("cp.async.wait_all;" ::: "memory");   // this thread's copies of the next group's statistics have landed
       __syncthreads();
     }
