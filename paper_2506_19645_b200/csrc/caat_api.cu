@@ -589,8 +589,8 @@ static caat_status block_forward_overlapped(const caat_ctx* ctx, int tokens, con
                       nullptr, 2);
 }
 
-// The block forward with both layers' row work in one pass: GEMM 1 -> GEMM 2 -> rows of both layers.  compact: R0 / Hn1 /
-// Hn2 are the private parts and R0s / Hn1s / Hn2s the shared part of the stream.
+// The block forward with both layers' row work in one pass: GEMMs (one launch or two) -> rows of both layers.  compact: R0 /
+// Hn1 / Hn2 are the private parts and R0s / Hn1s / Hn2s the shared part of the stream.
 static bool fused_rows_apply(const caat_ctx* ctx, int tokens, int compact) {
   if (!ctx || ctx->block_overlap != 2 || ctx->direct_rows || check_common(ctx, CAAT_MLP_DOWN, tokens) != CAAT_OK) return false;
   if (!tc_gemm_usable(ctx, layer_kr(ctx, CAAT_ATTN_OUT)) || !tc_gemm_usable(ctx, layer_kr(ctx, CAAT_MLP_DOWN))) return false;
@@ -605,19 +605,24 @@ static caat_status block_forward_fused(const caat_ctx* ctx, int tokens, const vo
                                        const void* W_down, const RowBlockArgs& rows, void* workspace, cudaStream_t st) {
   RowBlockArgs a = rows;
   char* ws = static_cast<char*>(workspace);
+  RowparShapes sh[2];
+  const void *Y[2] = {Y_attn, Y_mlp}, *W[2] = {W_o, W_down};
+  void *zs[2], *zp[2], *planes[2];
+  int max_groups[2];
   for (int l = 0; l < 2; ++l) {
     const int K_r = layer_kr(ctx, l == 0 ? CAAT_ATTN_OUT : CAAT_MLP_DOWN);
     const Scratch L = scratch_layout(ctx, K_r, tokens, 0);
-    const RowparShapes sh{ctx->t, tokens, ctx->h, K_r, ctx->S, L.S_lo, L.S_hi, L.P};
-    a.zs[l] = ws + L.zs_off; a.zp[l] = ws + L.zp_off;
-    a.zplanes[l] = reinterpret_cast<const float*>(ws + L.gp_off);
-    a.zgroups[l] = 1;
-    const cudaError_t ce = launch_tc_forward(sh, l == 0 ? Y_attn : Y_mlp, l == 0 ? W_o : W_down, ws + L.zs_off, ws + L.zp_off, st,
-                                             nullptr, L.gp_groups ? ws + L.gp_off : nullptr, L.gp_groups, &a.zgroups[l]);
-    if (ce != cudaSuccess) return cuda_fail(ce);
+    sh[l] = RowparShapes{ctx->t, tokens, ctx->h, K_r, ctx->S, L.S_lo, L.S_hi, L.P};
+    a.zs[l] = zs[l] = ws + L.zs_off;
+    a.zp[l] = zp[l] = ws + L.zp_off;
+    planes[l] = L.gp_groups ? ws + L.gp_off : nullptr;
+    a.zplanes[l] = static_cast<const float*>(planes[l]);
+    max_groups[l] = L.gp_groups;
     a.S_lo = L.S_lo; a.S_hi = L.S_hi; a.P = L.P;
     ws += align_up(L.total, 256);
   }
+  const cudaError_t ge = launch_tc_forward_block(sh, Y, W, zs, zp, planes, max_groups, a.zgroups, st);
+  if (ge != cudaSuccess) return cuda_fail(ge);
   a.t = ctx->t; a.T = tokens; a.h = ctx->h; a.S = ctx->S;
   a.alpha = (float)ctx->alpha; a.eps = (float)ctx->eps; a.norm = ctx->norm;
   const cudaError_t ce = launch_rows_forward_block(a, st);

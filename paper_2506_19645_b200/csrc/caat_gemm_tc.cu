@@ -812,13 +812,22 @@ bool make_cmap(CUtensorMap* m, const void* base, long long d0, long long d1, lon
 struct RegionShape { int M, N, batch, ksteps; };
 struct TileCfg { int bn, cg, splits; double cost; };
 
-// The busiest worker's load when n1 tiles of length a and then n2 of length b are dealt round-robin to W workers.
-double makespan(long long n1, double a, long long n2, double b, long long W) {
-  const long long r1 = n1 % W, rt = (n1 + n2) % W, edge[3] = {0, r1, rt};
+// The busiest worker's load when the regions' tiles, n[i] of length len[i], are dealt round-robin one region after the other.
+double makespan(const long long* n, const double* len, int nr, long long W) {
   double worst = 0;
-  for (long long w : edge) {
-    const long long c1 = n1 / W + (w < r1), ct = (n1 + n2) / W + (w < rt);
-    worst = fmax(worst, c1 * a + (ct - c1) * b);
+  long long start = 0;
+  for (int q = 0; q <= nr; ++q) {            // loads change only where a region's last round ends
+    const long long w = start % W;
+    double load = 0;
+    long long e = 0, before = 0;
+    for (int i = 0; i < nr; ++i) {
+      e += n[i];
+      const long long upto = e / W + (w < e % W);
+      load += (double)(upto - before) * len[i];
+      before = upto;
+    }
+    worst = fmax(worst, load);
+    if (q < nr) start += n[q];
   }
   return worst;
 }
@@ -828,8 +837,8 @@ double estimate_cost(const RegionShape* r, int nr, int bn, int cg, int splits, d
   const double step = (bn / 256.0) * fmax(1.0, 0.92 * (128.0 + (double)bn / cg) / bn);
   const double epi = 10.0 * bn / 256.0;
   const double handoff = cg == 2 ? 3.5 : 2.0;
-  double total = 0, len[2] = {0, 0};
-  long long n[2] = {0, 0};
+  double total = 0, len[kMaxRegions] = {};
+  long long n[kMaxRegions] = {}, tiles = 0;
   for (int i = 0; i < nr; ++i) {
     if (r[i].M <= 0 || r[i].N <= 0) continue;
     const long long rows = (long long)((r[i].M + 128 * cg - 1) / (128 * cg)) * r[i].batch * splits;
@@ -843,10 +852,11 @@ double estimate_cost(const RegionShape* r, int nr, int bn, int cg, int splits, d
       n[i] += rows;
     }
     total += region;
+    tiles += n[i];
     if (n[i]) len[i] = region / n[i];
   }
-  if (n[0] + n[1] == 0) return 0;
-  double t = fmax(total / workers, makespan(n[0], len[0], n[1], len[1], (long long)workers));
+  if (tiles == 0) return 0;
+  double t = fmax(total / workers, makespan(n, len, nr, (long long)workers));
   if (splits > 1) t += 2.0 * splits * out_bytes / 6.4e12 / 0.2e-6;
   return t;
 }
@@ -976,6 +986,10 @@ bool tc_gemm_usable(const caat_ctx* ctx, int K_r) {
 // decides.
 struct ForwardPlan { TileCfg tile; int groups, qper; };
 
+static double plane_cost(const RowparShapes& s, int groups) {      // the planes' round trip through L2
+  return groups > 1 ? (8.0 * groups * s.T * s.S_hi / 10e12 + 1e-6) / 0.2e-6 : 0;
+}
+
 static ForwardPlan forward_plan(const RowparShapes& s, int max_groups) {
   const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0, ksteps = (s.K_r + BK - 1) / BK;
   ForwardPlan f{};
@@ -984,10 +998,83 @@ static ForwardPlan forward_plan(const RowparShapes& s, int max_groups) {
     if (g > 1 && (n_sh == 0 || g > max_groups)) break;
     const RegionShape rs[2] = {{s.T, n_sh, g, ksteps * per}, {s.T, n_pr, s.t, ksteps}};
     TileCfg c = pick_tile(rs, 2, false, 1, 0.0);
-    if (g > 1) c.cost += (8.0 * g * s.T * s.S_hi / 10e12 + 1e-6) / 0.2e-6;   // the planes' round trip through L2
-    if (g == 1 || c.cost < f.tile.cost) f = ForwardPlan{c, g, per};
+    c.cost += plane_cost(s, g);
+    if (g == 1 || c.cost < f.tile.cost) { f = ForwardPlan{c, g, per}; }
   }
   return f;
+}
+
+// operand maps of one layer's forward product: mp.ab[2 l] = Y, mp.ab[2 l + 1] = W
+static bool forward_maps(Maps& mp, int l, const RowparShapes& s, const void* Y, const void* W, const Params& p) {
+  return make_map(&mp.ab[2 * l], Y, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, BK, BM) &&
+         make_map(&mp.ab[2 * l + 1], W, s.K_r, s.h, s.t, s.K_r, (long long)s.h * s.K_r, BK, p.BN / p.cg);
+}
+// the next region of the launch: the shared columns, all ranks in the contraction (or groups of qper ranks)
+static bool forward_shared(Maps& mp, Params& p, int l, const RowparShapes& s, void* zs, void* planes, int groups, int qper) {
+  const int g = p.nregions++;
+  Region& r = p.r[g];
+  r.nunits = 1;
+  r.u[0] = Unit{2 * l, 2 * l + 1, 0, 0, 0, 0, /*a_zb*/ 0, /*a_zq*/ 1, /*b_zb*/ 0, /*b_zq*/ 1, s.t, (s.K_r + BK - 1) / BK};
+  r.M = s.T; r.N = s.S; r.batch = 1; r.b_slowest = 0;
+  if (groups > 1) { r.splits = groups; r.qper = qper; r.out_f32 = 1; }
+  return make_cmap(&mp.c[g], groups > 1 ? planes : zs, s.S, s.T, groups, s.S_hi, (long long)s.T * s.S_hi, groups > 1);
+}
+// the next region: the private columns, per rank
+static bool forward_private(Maps& mp, Params& p, int l, const RowparShapes& s, void* zp) {
+  const int g = p.nregions++;
+  Region& r = p.r[g];
+  r.nunits = 1;
+  r.u[0] = Unit{2 * l, 2 * l + 1, 0, 0, 0, s.S_lo, 1, 0, 1, 0, 1, (s.K_r + BK - 1) / BK};
+  r.M = s.T; r.N = s.h - s.S_lo; r.batch = s.t; r.b_slowest = 1;
+  return make_cmap(&mp.c[g], zp, s.h - s.S_lo, s.T, s.t, s.P, (long long)s.T * s.P, false);
+}
+
+// Both layers' forward products of a block (they do not depend on each other): one launch where the cost model sees a
+// gain - one ramp, one tail and a finer deal where a layer's tiles do not fill the GPU - else one after the other.  Each
+// layer keeps the rank groups that it would have alone, so its sums do not depend on the schedule.
+// The rule: a launch of its own costs 2.4 us; against that, one launch has to be cheaper than the two by 5 % of its own
+// time, which is what it loses to the model when both layers' operands go through L2 and only one tile width is left to
+// choose.  Block forward on either side of the line (apart / merged, us): taken - h 768, 300 tokens 21.9 / 14.9; h 2048,
+// 300 tokens 44.0 / 38.8, 2000 tokens 147 / 143; h 4096, 600 tokens 153 / 147, 3000 tokens 571 / 539; not taken - h 4096,
+// 1400 tokens 273 / 285; h 5120, 1000 tokens 306 / 312; h 4096, p = 0.75 on 2 ranks, 300 tokens 75 / 87.
+cudaError_t launch_tc_forward_block(const RowparShapes* s, const void* const* Y, const void* const* W, void* const* zs,
+                                    void* const* zp, void* const* planes, const int* max_groups, int* groups, cudaStream_t st) {
+  constexpr double kLaunchGap = 12, kMargin = 1.05;      // units of 0.2 us
+  const ForwardPlan one[2] = {forward_plan(s[0], planes[0] ? max_groups[0] : 1), forward_plan(s[1], planes[1] ? max_groups[1] : 1)};
+  const int ks[2] = {(s[0].K_r + BK - 1) / BK, (s[1].K_r + BK - 1) / BK};
+  const int lead = ks[1] * one[1].qper >= ks[0] * one[0].qper ? 1 : 0;        // the layer with the longer shared tiles
+  RegionShape rs[4];
+  for (int i = 0; i < 2; ++i) {
+    const int l = i == 0 ? lead : 1 - lead;
+    rs[i] = RegionShape{s[l].T, s[l].S, one[l].groups, ks[l] * one[l].qper};
+    rs[2 + i] = RegionShape{s[l].T, s[l].S < s[l].h ? s[l].h - s[l].S_lo : 0, s[l].t, ks[l]};
+  }
+  TileCfg both = pick_tile(rs, 4, false, 1, 0.0);
+  for (int l = 0; l < 2; ++l) both.cost += plane_cost(s[l], one[l].groups);
+  if (both.cost * kMargin >= one[0].tile.cost + one[1].tile.cost + kLaunchGap) {
+    for (int l = 0; l < 2; ++l) {
+      const cudaError_t e = launch_tc_forward(s[l], Y[l], W[l], zs[l], zp[l], st, nullptr, planes[l], max_groups[l], &groups[l]);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
+  Maps mp;
+  Params p{};
+  p.BN = both.bn; p.cg = both.cg; p.splits = 1;
+  for (int l = 0; l < 2; ++l) {
+    groups[l] = one[l].groups;
+    if (!forward_maps(mp, l, s[l], Y[l], W[l], p)) return cudaErrorInvalidValue;
+  }
+  for (int i = 0; i < 2; ++i) {
+    const int l = i == 0 ? lead : 1 - lead;
+    if (s[l].S > 0 && !forward_shared(mp, p, l, s[l], zs[l], planes[l], one[l].groups, one[l].qper)) return cudaErrorInvalidValue;
+  }
+  for (int i = 0; i < 2; ++i) {
+    const int l = i == 0 ? lead : 1 - lead;
+    if (s[l].S < s[l].h && !forward_private(mp, p, l, s[l], zp[l])) return cudaErrorInvalidValue;
+  }
+  finish_tiles(p);
+  return launch(mp, p, CAAT_K_TC_FORWARD, st);
 }
 
 int tc_forward_groups(const RowparShapes& s, int max_groups) { return forward_plan(s, max_groups).groups; }
@@ -999,34 +1086,16 @@ cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* 
   PeerMaps pmaps{};
   Params p{};
   const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
-  const int ksteps = (s.K_r + BK - 1) / BK;
   const ForwardPlan plan = forward_plan(s, planes ? max_groups : 1);
   const int groups = plan.groups, qper = plan.qper;
   p.BN = plan.tile.bn; p.cg = plan.tile.cg;
   if (groups_out) *groups_out = groups;
-  if (!make_map(&maps[0], Y, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, BK, BM)) return cudaErrorInvalidValue;
-  if (!make_map(&maps[1], W, s.K_r, s.h, s.t, s.K_r, (long long)s.h * s.K_r, BK, p.BN / p.cg)) return cudaErrorInvalidValue;
+  p.a_mn = 0; p.b_mn = 0; p.splits = 1;
+  if (!forward_maps(mp, 0, s, Y, W, p)) return cudaErrorInvalidValue;
   maps[2] = maps[0];
   maps[3] = maps[1];
-  p.a_mn = 0; p.b_mn = 0;  p.splits = 1;
-  int g = 0;
-  if (n_sh > 0) {
-    Region& r = p.r[g++];
-    r.nunits = 1;
-    r.u[0] = Unit{0, 1, 0, 0, 0, 0, /*a_zb*/ 0, /*a_zq*/ 1, /*b_zb*/ 0, /*b_zq*/ 1, s.t, ksteps};
-    r.M = s.T; r.N = n_sh; r.batch = 1; r.b_slowest = 0;
-    if (groups > 1) { r.splits = groups; r.qper = qper; r.out_f32 = 1; }
-    if (!make_cmap(&cmaps[g - 1], groups > 1 ? planes : zs, n_sh, s.T, groups, s.S_hi, (long long)s.T * s.S_hi, groups > 1))
-      return cudaErrorInvalidValue;
-  }
-  if (n_pr > 0) {
-    Region& r = p.r[g++];
-    r.nunits = 1;
-    r.u[0] = Unit{0, 1, 0, 0, 0, s.S_lo, 1, 0, 1, 0, 1, ksteps};
-    r.M = s.T; r.N = n_pr; r.batch = s.t; r.b_slowest = 1;
-    if (!make_cmap(&cmaps[g - 1], zp, n_pr, s.T, s.t, s.P, (long long)s.T * s.P, false)) return cudaErrorInvalidValue;
-  }
-  p.nregions = g;
+  if (n_sh > 0 && !forward_shared(mp, p, 0, s, zs, planes, groups, qper)) return cudaErrorInvalidValue;
+  if (n_pr > 0 && !forward_private(mp, p, 0, s, zp)) return cudaErrorInvalidValue;
   if (push && n_sh > 0 && groups == 1) {
     // shared tiles go to the owners' receive slots: slot `rank` of GPU q is [slice, S] 16-bit elements; the map of
     // owner q covers only the tokens q really owns, so rows past the end of a ragged last slice are clipped

@@ -98,6 +98,9 @@ struct PushTarget { int world, rank, slice; void* const* recv; };
 cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* W, void* zs, void* zp,
                               cudaStream_t st, const PushTarget* push = nullptr, void* planes = nullptr, int max_groups = 1,
                               int* groups = nullptr);
+// both layers of a block; groups[l] as above
+cudaError_t launch_tc_forward_block(const RowparShapes* s, const void* const* Y, const void* const* W, void* const* zs,
+                                    void* const* zp, void* const* planes, const int* max_groups, int* groups, cudaStream_t st);
 // the split launch_tc_forward would choose (for a caller that launches the row kernel later)
 int tc_forward_groups(const RowparShapes& s, int max_groups);
 // The private part of dZt as the backward GEMMs read it: element (m, i, l) for l >= S_lo sits at

@@ -20,6 +20,8 @@ CASES = [
     (4, 2001, 768, 3072, 380, 1),       # the same with LayerNorm, persistent CTAs, a straddling chunk
     (4, 333, 1536, 6144, 200, 0),       # fewer than eight warps
     (2, 130, 264, 528, 131, 1),         # chunks past the row end
+    (8, 300, 2048, 5632, 1024, 0),      # both layers' GEMMs in one launch, planes of both
+    (8, 129, 2048, 5632, 2048, 0),      # the same with nothing private
 ]
 
 
