@@ -108,7 +108,8 @@ typedef enum {
                                    row kernel for both layers after both GEMMs where it applies (bf16 on the tensor-core
                                    path, rows of up to 8192 channels, both layers' scratch in the workspace; not
                                    LayerNorm on rows of more than 1024 channels), else 1 unless that GEMM is much the
-                                   longer of the two kernels (ffn / t large).  The compact block forward follows 0 and 2 */
+                                   longer of the two kernels (ffn / t large).  The compact block forward follows 0 and 2;
+                                   the block backward too: 2 = one row kernel for both layers where that is faster */
 } caat_option;
 
 /* Creates a context for hidden size h, MLP width ffn, t ranks, synchronisation
@@ -125,9 +126,9 @@ int caat_shared_channels(const caat_ctx *ctx);
 double caat_private_scale(const caat_ctx *ctx);
 
 /* Bytes of device scratch for the block calls (caat_block_forward / _backward and the compact variants):
- * enough for the two layers' scratch side by side, which lets the block forward overlap the first layer's row
- * kernel with the second layer's GEMM.  A workspace of only the larger of the two layers' caat_workspace_bytes
- * is accepted as well; the block forward then runs its kernels one after the other. */
+ * enough for the two layers' scratch side by side, which lets the block calls do both layers' row work in one pass
+ * (or the forward overlap the first layer's row kernel with the second layer's GEMM).  A workspace of only the
+ * larger of the two layers' caat_workspace_bytes is accepted as well; the layers then run one after the other. */
 size_t caat_block_workspace_bytes(const caat_ctx *ctx, int tokens, int backward);
 
 /* Bytes of device scratch for `tokens` tokens of `layer`: backward = 0, what the forward
@@ -254,7 +255,9 @@ caat_status caat_block_forward(const caat_ctx *ctx, int tokens,
  * Backward of the block: the MLP-down layer first (upstream dX2 through its norm,
  * dHn2 on the outgoing residual stream), then the attention-out layer whose
  * residual-stream gradient is the dR of the second layer (written to dHn1, an
- * output of this call, [t,T,h] dtype).  dHn2 may be NULL.
+ * output of this call, [t,T,h] dtype).  dHn2 may be NULL.  With a workspace of
+ * caat_block_workspace_bytes and CAAT_OPT_BLOCK_OVERLAP = 2 both layers' row work runs in one pass where
+ * that is faster; a dR0 that overlaps dHn1, Y_mlp or W_down keeps a pass per layer.
  */
 caat_status caat_block_backward(const caat_ctx *ctx, int tokens,
                                 const void *dX1, const void *dX2, const void *dHn2,

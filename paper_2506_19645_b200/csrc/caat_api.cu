@@ -258,6 +258,24 @@ static SideStream* side_stream_locked() {
 }
 
 // ---- backward of one layer -----------------------------------------------------
+// alpha of the private gradient: on the epilogues when the shared gradient may be stored divided by it (one scaling of
+// the weights' private rows less: 9 + 7 us of a 193 us step at 600 tokens of 8 x 2048), else on the weights
+static bool alpha_on_epilogues(const caat_ctx* ctx, int compact) {
+  return !compact && ctx->S < ctx->h && ctx->alpha != 1.0 && std::fabs(ctx->alpha) >= 0x1p-10 && std::fabs(ctx->alpha) <= 0x1p10;
+}
+
+// the tensor-core gradient GEMMs of one layer, after its row work
+static caat_status backward_gemms(const caat_ctx* ctx, int K_r, int T, const void* gs, const void* dR, const void* Y,
+                                  const void* W, void* dY, float* dW, char* wsb, const Scratch& L, int compact, bool over_alpha,
+                                  bool prescale, cudaStream_t st) {
+  RowparShapes sh{ctx->t, T, ctx->h, K_r, ctx->S, L.S_lo, L.S_hi, L.P};
+  const PrivOperand pv = compact ? PrivOperand{dR, L.P, 0, (float)ctx->alpha, 0}
+                                 : PrivOperand{dR, ctx->h, L.S_lo, (float)ctx->alpha, over_alpha};
+  cudaError_t ce = launch_tc_dgrad(sh, gs, pv, W, dY, wsb + L.wt_off, prescale, st);
+  if (ce == cudaSuccess) ce = launch_tc_wgrad(sh, gs, pv, Y, dW, wsb + L.splitk_off, L.splitk_bytes, st);
+  return ce == cudaSuccess ? CAAT_OK : cuda_fail(ce);
+}
+
 static caat_status backward_impl(const caat_ctx* ctx, int K_r, int T, const void* dX, const void* dHn, const void* Y,
                                  const void* W, const void* Hn, const float* rstd, const float* mean,
                                  const void* gamma, void* dY, float* dW, void* dR, float* dgamma, float* dbeta,
@@ -290,10 +308,7 @@ static caat_status backward_impl(const caat_ctx* ctx, int K_r, int T, const void
     a.gs_slice = push->slice; a.gs_rank = push->rank;
     for (int q = 0; q < push->world && q < CAAT_MAX_PEERS; ++q) a.gs_recv[q] = push->recv[q];
   }
-  // alpha of the private gradient: on the epilogues when the shared gradient may be stored divided by it (one scaling of
-  // the weights' private rows less: 9 + 7 us of a 193 us step at 600 tokens of 8 x 2048), else on the weights
-  const bool over_alpha = tc && !compact && phase == 0 && S < h && ctx->alpha != 1.0 && std::fabs(ctx->alpha) >= 0x1p-10 &&
-                          std::fabs(ctx->alpha) <= 0x1p10;
+  const bool over_alpha = tc && phase == 0 && alpha_on_epilogues(ctx, compact);
   a.gs_scale = over_alpha ? (float)(1.0 / ctx->alpha) : 1.0f;
   const bool prescale = tc && ctx->alpha != 1.0 && S < h && !over_alpha;
   if (prescale) { a.w_src = W; a.w_dst = wsb + L.wt_off; a.w_Kr = K_r; }
@@ -303,16 +318,7 @@ static caat_status backward_impl(const caat_ctx* ctx, int K_r, int T, const void
   }
   if (phase == 1) return CAAT_OK;
 
-  if (tc) {
-    RowparShapes sh{t, T, h, K_r, S, L.S_lo, L.S_hi, L.P};
-    const PrivOperand pv = compact ? PrivOperand{dR, L.P, 0, (float)ctx->alpha, 0}
-                                   : PrivOperand{dR, h, L.S_lo, (float)ctx->alpha, over_alpha};
-    ce = launch_tc_dgrad(sh, gs, pv, W, dY, wsb + L.wt_off, prescale, st);
-    if (ce != cudaSuccess) return cuda_fail(ce);
-    ce = launch_tc_wgrad(sh, gs, pv, Y, dW, wsb + L.splitk_off, L.splitk_bytes, st);
-    if (ce != cudaSuccess) return cuda_fail(ce);
-    return CAAT_OK;
-  }
+  if (tc) return backward_gemms(ctx, K_r, T, gs, dR, Y, W, dY, dW, wsb, L, compact, over_alpha, prescale, st);
   const char* zp_priv = static_cast<const char*>(zp) + (size_t)(S - L.S_lo) * e;
   {  // dY[m] = gs W[m][:S] + zp[m] W[m][S:]
     GemmProblem g{};
@@ -528,11 +534,11 @@ size_t caat_block_workspace_bytes(const caat_ctx* ctx, int tokens, int backward)
   const size_t a = caat_workspace_bytes(ctx, CAAT_ATTN_OUT, tokens, backward);
   const size_t m = caat_workspace_bytes(ctx, CAAT_MLP_DOWN, tokens, backward);
   if (a == 0 || m == 0) return 0;
-  // the forward's two scratch regions side by side; a training step's backward runs layer by layer in one region
-  const size_t side_by_side = align_up(caat_workspace_bytes(ctx, CAAT_ATTN_OUT, tokens, 0), 256) +
-                              caat_workspace_bytes(ctx, CAAT_MLP_DOWN, tokens, 0);
-  const size_t one = a > m ? a : m;
-  return side_by_side > one ? side_by_side : one;
+  // both layers' scratch side by side, of the forward and - a training step - of the backward
+  const size_t fwd = align_up(caat_workspace_bytes(ctx, CAAT_ATTN_OUT, tokens, 0), 256) +
+                     caat_workspace_bytes(ctx, CAAT_MLP_DOWN, tokens, 0);
+  const size_t bwd = backward ? align_up(a, 256) + m : 0;
+  return fwd > bwd ? fwd : bwd;
 }
 
 // The block forward with the attention-out layer's row kernel beside the MLP-down layer's GEMM:
@@ -675,6 +681,51 @@ caat_status caat_block_forward(const caat_ctx* ctx, int tokens, const void* Y_at
                              workspace, workspace_bytes, cuda_stream);
 }
 
+// ---- backward of a block with both layers' row work in one pass: rows -> norm-gradient sums -> the four GEMMs
+static bool fused_backward_applies(const caat_ctx* ctx, int tokens, int compact) {
+  if (!ctx || ctx->block_overlap != 2 || ctx->direct_rows || ctx->bwd_reduce || check_common(ctx, CAAT_MLP_DOWN, tokens) != CAAT_OK)
+    return false;
+  if (compact && ctx->S % kLayoutVec != 0) return false;
+  if (!tc_gemm_usable(ctx, layer_kr(ctx, CAAT_ATTN_OUT)) || !tc_gemm_usable(ctx, layer_kr(ctx, CAAT_MLP_DOWN))) return false;
+  const int S_lo = round_down(ctx->S, kLayoutVec);
+  return rows_block_bwd_usable(ctx->h, tokens, ctx->h - S_lo, round_up(ctx->S, kLayoutVec), ctx->dtype, compact, ctx->norm);
+}
+
+static bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return a && b && x < y + nb && y < x + na;
+}
+
+static caat_status block_backward_fused(const caat_ctx* ctx, int tokens, const RowBlockBwdArgs& rows, const void* Y_attn,
+                                        const void* W_o, const void* Y_mlp, const void* W_down, void* dY_attn, float* dW_o,
+                                        void* dY_mlp, float* dW_down, void* workspace, cudaStream_t st) {
+  RowBlockBwdArgs a = rows;
+  const bool over_alpha = alpha_on_epilogues(ctx, a.compact);
+  const bool prescale = ctx->alpha != 1.0 && ctx->S < ctx->h && !over_alpha;
+  char* wsb[2];
+  Scratch L[2];
+  int K_r[2];
+  for (int l = 0; l < 2; ++l) {
+    K_r[l] = layer_kr(ctx, l == 0 ? CAAT_ATTN_OUT : CAAT_MLP_DOWN);
+    L[l] = scratch_layout(ctx, K_r[l], tokens, 1);
+    wsb[l] = l == 0 ? static_cast<char*>(workspace) : wsb[0] + align_up(L[0].total, 256);
+    if (!a.compact) a.gs[l] = wsb[l] + L[l].zs_off;
+    a.dgpart[l] = reinterpret_cast<float*>(wsb[l] + L[l].dgpart_off);
+    a.dbpart[l] = reinterpret_cast<float*>(wsb[l] + L[l].dbpart_off);
+    if (prescale) { a.w_src[l] = l == 0 ? W_o : W_down; a.w_dst[l] = wsb[l] + L[l].wt_off; a.w_Kr[l] = K_r[l]; }
+  }
+  a.t = ctx->t; a.T = tokens; a.h = ctx->h; a.S = ctx->S; a.S_lo = L[0].S_lo; a.S_hi = L[0].S_hi; a.P = L[0].P;
+  a.alpha = (float)ctx->alpha; a.norm = ctx->norm;
+  a.gs_scale = over_alpha ? (float)(1.0 / ctx->alpha) : 1.0f;
+  const cudaError_t ce = launch_rows_backward_block(a, st);
+  if (ce != cudaSuccess) return cuda_fail(ce);
+  const caat_status s = backward_gemms(ctx, K_r[1], tokens, a.gs[1], a.dR[1], Y_mlp, W_down, dY_mlp, dW_down, wsb[1], L[1], a.compact,
+                                       over_alpha, prescale, st);
+  if (s != CAAT_OK) return s;
+  return backward_gemms(ctx, K_r[0], tokens, a.gs[0], a.dR[0], Y_attn, W_o, dY_attn, dW_o, wsb[0], L[0], a.compact, over_alpha, prescale,
+                        st);
+}
+
 caat_status caat_block_backward(const caat_ctx* ctx, int tokens, const void* dX1, const void* dX2, const void* dHn2,
                                 const void* Y_attn, const void* W_o, const void* Y_mlp, const void* W_down,
                                 const void* Hn1, const float* rstd1, const float* mean1, const void* Hn2,
@@ -683,6 +734,27 @@ caat_status caat_block_backward(const caat_ctx* ctx, int tokens, const void* dX1
                                 float* dgamma1, float* dbeta1, float* dgamma2, float* dbeta2, void* workspace,
                                 size_t workspace_bytes, void* cuda_stream) {
   if (!dHn1) return CAAT_EINVAL;
+  if (fused_backward_applies(ctx, tokens, 0) && workspace && workspace_bytes >= caat_block_workspace_bytes(ctx, tokens, 1) &&
+      dX1 && dX2 && Y_attn && W_o && Y_mlp && W_down && Hn1 && rstd1 && Hn2 && rstd2 && gamma1 && gamma2 && dY_attn && dW_o &&
+      dY_mlp && dW_down && dR0 && dgamma1 && dgamma2 && (ctx->norm == 0 || (mean1 && mean2 && dbeta1 && dbeta2))) {
+    const void* ptrs[] = {dX1, dX2, dHn2, Y_attn, W_o, Y_mlp, W_down, Hn1, rstd1, mean1, Hn2, rstd2, mean2, gamma1, gamma2, dY_attn,
+                          dW_o, dY_mlp, dW_down, dR0, dHn1, dgamma1, dbeta1, dgamma2, dbeta2, workspace};
+    bool ok = true;
+    for (const void* p : ptrs) ok = ok && (!p || aligned16(p));
+    const size_t stream = (size_t)ctx->t * tokens * ctx->h * 2, km = (size_t)layer_kr(ctx, CAAT_MLP_DOWN);
+    // dR0 is written before the second layer's GEMMs run, and while its row work does: element by element in place is fine
+    ok = ok && !overlaps(dR0, stream, dHn1, stream) && !overlaps(dR0, stream, Y_mlp, ctx->t * km * tokens * 2) &&
+         !overlaps(dR0, stream, W_down, ctx->t * km * ctx->h * 2);
+    for (const void* p : {dX2, Hn2, dHn2}) ok = ok && (p == dR0 || !overlaps(dR0, stream, p, stream));
+    if (ok) {
+      RowBlockBwdArgs a{};
+      a.dX[0] = dX1; a.dX[1] = dX2; a.Hn[0] = Hn1; a.Hn[1] = Hn2; a.gamma[0] = gamma1; a.gamma[1] = gamma2; a.dHn = dHn2;
+      a.rstd[0] = rstd1; a.rstd[1] = rstd2; a.mean[0] = mean1; a.mean[1] = mean2; a.dR[0] = dR0; a.dR[1] = dHn1;
+      a.dgamma[0] = dgamma1; a.dgamma[1] = dgamma2; a.dbeta[0] = dbeta1; a.dbeta[1] = dbeta2;
+      return block_backward_fused(ctx, tokens, a, Y_attn, W_o, Y_mlp, W_down, dY_attn, dW_o, dY_mlp, dW_down, workspace,
+                                  static_cast<cudaStream_t>(cuda_stream));
+    }
+  }
   caat_status s = caat_rowpar_backward(ctx, CAAT_MLP_DOWN, tokens, dX2, dHn2, Y_mlp, W_down, Hn2, rstd2, mean2,
                                        gamma2, dY_mlp, dW_down, dHn1, dgamma2, dbeta2, workspace, workspace_bytes,
                                        cuda_stream);
@@ -786,6 +858,38 @@ caat_status caat_block_backward_compact(const caat_ctx* ctx, int tokens, const v
                                         void* dR0s, void* dR0p, void* dHn1s, void* dHn1p, float* dgamma1,
                                         float* dbeta1, float* dgamma2, float* dbeta2, void* workspace,
                                         size_t workspace_bytes, void* cuda_stream) {
+  const bool has_s = ctx && ctx->S > 0, has_p = ctx && ctx->S < ctx->h;
+  const bool any_dh = (has_s && dHn2s) || (has_p && dHn2p);
+  if (fused_backward_applies(ctx, tokens, 1) && workspace && workspace_bytes >= caat_block_workspace_bytes(ctx, tokens, 1) &&
+      dX1 && dX2 && Y_attn && W_o && Y_mlp && W_down && rstd1 && rstd2 && gamma1 && gamma2 && dY_attn && dW_o && dY_mlp && dW_down &&
+      dgamma1 && dgamma2 && (!has_s || (Hn1s && Hn2s && dR0s && dHn1s && (!any_dh || dHn2s))) &&
+      (!has_p || (Hn1p && Hn2p && dR0p && dHn1p && (!any_dh || dHn2p))) &&
+      (ctx->norm == 0 || (mean1 && mean2 && dbeta1 && dbeta2))) {
+    const void* ptrs[] = {dX1, dX2, dHn2s, dHn2p, Y_attn, W_o, Y_mlp, W_down, Hn1s, Hn1p, rstd1, mean1, Hn2s, Hn2p, rstd2, mean2,
+                          gamma1, gamma2, dY_attn, dW_o, dY_mlp, dW_down, dR0s, dR0p, dHn1s, dHn1p, dgamma1, dbeta1, dgamma2,
+                          dbeta2, workspace};
+    bool ok = true;
+    for (const void* p : ptrs) ok = ok && (!p || aligned16(p));
+    const size_t sh = (size_t)tokens * ctx->S * 2, pr = (size_t)ctx->t * tokens * (ctx->h - ctx->S) * 2;
+    const size_t km = (size_t)layer_kr(ctx, CAAT_MLP_DOWN), full = (size_t)ctx->t * tokens * ctx->h * 2;
+    auto clash = [&](const void* p, size_t n, bool in_place) {      // as in caat_block_backward, for either part
+      return (!(in_place && p == dR0s) && overlaps(dR0s, sh, p, n)) || (!(in_place && p == dR0p) && overlaps(dR0p, pr, p, n));
+    };
+    ok = ok && !clash(dHn1s, sh, false) && !clash(dHn1p, pr, false) && !clash(dX2, full, false) &&
+         !clash(Y_mlp, ctx->t * km * tokens * 2, false) && !clash(W_down, ctx->t * km * ctx->h * 2, false) && !clash(Hn2s, sh, true) &&
+         !clash(Hn2p, pr, true) && !clash(dHn2s, sh, true) && !clash(dHn2p, pr, true);
+    if (ok) {
+      RowBlockBwdArgs a{};
+      a.compact = 1;
+      a.dX[0] = dX1; a.dX[1] = dX2; a.Hn[0] = Hn1p; a.Hn[1] = Hn2p; a.Hns[0] = Hn1s; a.Hns[1] = Hn2s;
+      a.gamma[0] = gamma1; a.gamma[1] = gamma2; a.dHn = has_p ? dHn2p : nullptr; a.dHns = has_s ? dHn2s : nullptr;
+      a.rstd[0] = rstd1; a.rstd[1] = rstd2; a.mean[0] = mean1; a.mean[1] = mean2;
+      a.dR[0] = dR0p; a.dR[1] = dHn1p; a.gs[0] = dR0s; a.gs[1] = dHn1s;
+      a.dgamma[0] = dgamma1; a.dgamma[1] = dgamma2; a.dbeta[0] = dbeta1; a.dbeta[1] = dbeta2;
+      return block_backward_fused(ctx, tokens, a, Y_attn, W_o, Y_mlp, W_down, dY_attn, dW_o, dY_mlp, dW_down, workspace,
+                                  static_cast<cudaStream_t>(cuda_stream));
+    }
+  }
   caat_status s = caat_rowpar_backward_compact(ctx, CAAT_MLP_DOWN, tokens, dX2, dHn2s, dHn2p, Y_mlp, W_down, Hn2s, Hn2p,
                                                rstd2, mean2, gamma2, dY_mlp, dW_down, dHn1s, dHn1p, dgamma2, dbeta2,
                                                workspace, workspace_bytes, cuda_stream);

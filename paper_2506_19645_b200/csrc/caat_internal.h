@@ -227,6 +227,28 @@ __device__ __forceinline__ char* gs_row(const RowBwdArgs& a, long long i, int ES
 }
 #endif
 cudaError_t launch_rows_backward(const RowBwdArgs& a, caat_dtype dtype, int direct, cudaStream_t st);
+// sums of the norm-gradient partials [rows][h] of one or two layers, and beside them dst[m][l][:] = alpha * src[m][l][:]
+// for the private rows l >= S of weights [t][h][K_r] (bf16)
+struct ScaleJob { const void* src; void* dst; int t, h, K_r, S; float alpha; };
+struct NormGradReduce { const float* part[4]; float* out[4]; int n, rows, h; ScaleJob scale[2]; };
+cudaError_t launch_norm_grad_reduce(const NormGradReduce& r, cudaStream_t st);
+// Both layers of a block in one pass (index 1: the second layer, whose residual gradient dR[1] is the first one's stream
+// gradient).  compact: Hn, dHn, dR hold the private parts, Hns / dHns the shared rows, gs[l] is the shared part of dR[l].
+struct RowBlockBwdArgs {
+  const void *dX[2], *Hn[2], *Hns[2], *gamma[2];
+  const void *dHn, *dHns;
+  const float *rstd[2], *mean[2];
+  void *dR[2], *gs[2];
+  float *dgpart[2], *dbpart[2], *dgamma[2], *dbeta[2];
+  int t, T, h, S, S_lo, S_hi, P;
+  float alpha, gs_scale;
+  int norm, compact;
+  const void* w_src[2];      // as in RowBwdArgs
+  void* w_dst[2];
+  int w_Kr[2];
+};
+bool rows_block_bwd_usable(int h, int T, int P, int S_hi, caat_dtype dtype, int compact, int norm);
+cudaError_t launch_rows_backward_block(const RowBlockBwdArgs& a, cudaStream_t st);
 cudaError_t launch_rows_backward_staged(const RowBwdArgs& a, caat_dtype dtype, int max_rows, int* rows_used,
                                         cudaStream_t st);
 cudaError_t launch_rows_backward_warp(const RowBwdArgs& a, caat_dtype dtype, int max_rows, int* rows_used,

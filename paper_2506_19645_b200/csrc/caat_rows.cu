@@ -726,35 +726,39 @@ cudaError_t launch_partials_cluster(const RowPartArgs& a, int threads, size_t sm
 // per block: a chain of a few loads per thread on most SMs.
 // Blocks past the first `nreduce` run an unrelated small job that has to happen between the row kernel and the
 // data gradient anyway and would otherwise cost a launch of its own: scaling the private rows of the weights.
-struct ScaleJob { const uint4* src; uint4* dst; int t, h, K_r, S; float alpha; };
-
-__global__ void __launch_bounds__(1024) reduce_partials_kernel(const float* __restrict__ part, float* __restrict__ out,
-                                                               const float* __restrict__ part2, float* __restrict__ out2, int rows,
-                                                               int h, int nreduce, ScaleJob job) {
+__global__ void __launch_bounds__(1024) reduce_partials_kernel(const NormGradReduce a, int nreduce) {
   __shared__ float sm[128][9];
   pdl_wait();
+  const int per = (a.h + 7) / 8;       // blocks per array
   if ((int)blockIdx.x >= nreduce) {
-    const int row_chunks = job.K_r / 8;
-    const long long per_rank = (long long)(job.h - job.S) * row_chunks, total = per_rank * job.t;
-    const long long nthreads = (long long)(gridDim.x - nreduce) * 1024;
-    for (long long q = (long long)(blockIdx.x - nreduce) * 1024 + threadIdx.y * 8 + threadIdx.x; q < total; q += nthreads) {
-      const long long m = q / per_rank, r = q - m * per_rank;
-      const long long idx = (m * job.h + job.S) * row_chunks + r;
-      const uint4 v = job.src[idx];
-      const unsigned w[4] = {v.x, v.y, v.z, v.w};
-      unsigned o[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        __nv_bfloat162 bb = __floats2bfloat162_rn(job.alpha * __uint_as_float(w[i] << 16),
-                                                  job.alpha * __uint_as_float(w[i] & 0xffff0000u));
-        o[i] = *reinterpret_cast<unsigned*>(&bb);
+    for (int l = 0; l < 2; ++l) {
+      const ScaleJob& job = a.scale[l];
+      if (!job.dst) continue;
+      const int row_chunks = job.K_r / 8;
+      const long long per_rank = (long long)(job.h - job.S) * row_chunks, total = per_rank * job.t;
+      const long long nthreads = (long long)(gridDim.x - nreduce) * 1024;
+      for (long long q = (long long)(blockIdx.x - nreduce) * 1024 + threadIdx.y * 8 + threadIdx.x; q < total; q += nthreads) {
+        const long long m = q / per_rank, r = q - m * per_rank;
+        const long long idx = (m * job.h + job.S) * row_chunks + r;
+        const uint4 v = static_cast<const uint4*>(job.src)[idx];
+        const unsigned w[4] = {v.x, v.y, v.z, v.w};
+        unsigned o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          __nv_bfloat162 bb = __floats2bfloat162_rn(job.alpha * __uint_as_float(w[i] << 16),
+                                                    job.alpha * __uint_as_float(w[i] & 0xffff0000u));
+          o[i] = *reinterpret_cast<unsigned*>(&bb);
+        }
+        static_cast<uint4*>(job.dst)[idx] = make_uint4(o[0], o[1], o[2], o[3]);
       }
-      job.dst[idx] = make_uint4(o[0], o[1], o[2], o[3]);
     }
     return;
   }
-  int block = blockIdx.x;
-  if (part2 != nullptr && 2 * block >= nreduce) { block -= nreduce / 2; part = part2; out = out2; }     // the bias gradients
+  const int which = (int)blockIdx.x / per, block = (int)blockIdx.x - which * per;
+  const float* __restrict__ part = a.part[which];
+  float* __restrict__ out = a.out[which];
+  const int rows = a.rows, h = a.h;
   const int c = block * 8 + threadIdx.x;
   float s = 0.f;
   if (c < h)
@@ -917,25 +921,25 @@ cudaError_t launch_rows_backward(const RowBwdArgs& a, caat_dtype dtype, int dire
   else
     e = a.norm == 1 ? launch_bwd_t<float, true, false>(a, g, rows, st) : launch_bwd_t<float, false, false>(a, g, rows, st);
   if (e != cudaSuccess) return e;
-  const dim3 rb(8, 128);
-  const bool bias = a.norm == 1 && a.dbeta && a.dbpart;
-  const int nreduce = (a.h + 7) / 8 * (bias ? 2 : 1);
-  ScaleJob job{};
-  int nscale = 0;
-  if (a.w_dst && a.w_src && a.S < a.h) {
-    job = ScaleJob{static_cast<const uint4*>(a.w_src), static_cast<uint4*>(a.w_dst), a.t, a.h, a.w_Kr, a.S, a.alpha};
-    const long long total = (long long)a.t * (a.h - a.S) * (a.w_Kr / 8);
-    nscale = (int)((total + 4 * 1024 - 1) / (4 * 1024));          // four 16-byte chunks per thread
-    if (nscale > 148) nscale = 148;
-    if (nscale < 1) nscale = 1;
-  }
-  {
-    LaunchScope scope(CAAT_K_NORMGRAD_REDUCE, st);
-    e = launch_pdl(reduce_partials_kernel, dim3(nreduce + nscale), rb, 0, st, (const float*)a.dgpart, a.dgamma,
-                   bias ? (const float*)a.dbpart : (const float*)nullptr, a.dbeta, rows, a.h, nreduce, job);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaGetLastError();
+  NormGradReduce r{};
+  r.rows = rows;
+  r.h = a.h;
+  r.part[r.n] = a.dgpart; r.out[r.n++] = a.dgamma;
+  if (a.norm == 1 && a.dbeta && a.dbpart) { r.part[r.n] = a.dbpart; r.out[r.n++] = a.dbeta; }
+  if (a.w_dst && a.w_src && a.S < a.h) r.scale[0] = ScaleJob{a.w_src, a.w_dst, a.t, a.h, a.w_Kr, a.S, a.alpha};
+  return launch_norm_grad_reduce(r, st);
+}
+
+cudaError_t launch_norm_grad_reduce(const NormGradReduce& r, cudaStream_t st) {
+  long long chunks = 0;
+  for (const ScaleJob& job : r.scale)
+    if (job.dst) chunks += (long long)job.t * (job.h - job.S) * (job.K_r / 8);
+  long long nscale = (chunks + 4 * 1024 - 1) / (4 * 1024);          // four 16-byte chunks per thread
+  if (nscale > 148) nscale = 148;
+  const int nreduce = r.n * ((r.h + 7) / 8);
+  LaunchScope scope(CAAT_K_NORMGRAD_REDUCE, st);
+  const cudaError_t e = launch_pdl(reduce_partials_kernel, dim3(nreduce + (int)nscale), dim3(8, 128), 0, st, r, nreduce);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace caat
