@@ -264,13 +264,16 @@ static bool alpha_on_epilogues(const caat_ctx* ctx, int compact) {
   return !compact && ctx->S < ctx->h && ctx->alpha != 1.0 && std::fabs(ctx->alpha) >= 0x1p-10 && std::fabs(ctx->alpha) <= 0x1p10;
 }
 
+static PrivOperand priv_operand(const caat_ctx* ctx, const Scratch& L, const void* dR, int compact, bool over_alpha) {
+  return compact ? PrivOperand{dR, L.P, 0, (float)ctx->alpha, 0} : PrivOperand{dR, ctx->h, L.S_lo, (float)ctx->alpha, over_alpha};
+}
+
 // the tensor-core gradient GEMMs of one layer, after its row work
 static caat_status backward_gemms(const caat_ctx* ctx, int K_r, int T, const void* gs, const void* dR, const void* Y,
                                   const void* W, void* dY, float* dW, char* wsb, const Scratch& L, int compact, bool over_alpha,
                                   bool prescale, cudaStream_t st) {
   RowparShapes sh{ctx->t, T, ctx->h, K_r, ctx->S, L.S_lo, L.S_hi, L.P};
-  const PrivOperand pv = compact ? PrivOperand{dR, L.P, 0, (float)ctx->alpha, 0}
-                                 : PrivOperand{dR, ctx->h, L.S_lo, (float)ctx->alpha, over_alpha};
+  const PrivOperand pv = priv_operand(ctx, L, dR, compact, over_alpha);
   cudaError_t ce = launch_tc_dgrad(sh, gs, pv, W, dY, wsb + L.wt_off, prescale, st);
   if (ce == cudaSuccess) ce = launch_tc_wgrad(sh, gs, pv, Y, dW, wsb + L.splitk_off, L.splitk_bytes, st);
   return ce == cudaSuccess ? CAAT_OK : cuda_fail(ce);
@@ -681,14 +684,24 @@ caat_status caat_block_forward(const caat_ctx* ctx, int tokens, const void* Y_at
                              workspace, workspace_bytes, cuda_stream);
 }
 
-// ---- backward of a block with both layers' row work in one pass: rows -> norm-gradient sums -> the four GEMMs
-static bool fused_backward_applies(const caat_ctx* ctx, int tokens, int compact) {
+// ---- backward of a block on both layers' scratch: rows of both layers (one pass, or one after the other) -> the four GEMMs
+// (one launch or four).  Applies where at least one of the two is one launch; else the layers run one after the other.
+struct BwdBlock { bool applies, one_pass; BwdBlockPlan plan; RowparShapes sh[2]; Scratch L[2]; };
+static BwdBlock backward_block_plan(const caat_ctx* ctx, int tokens, int compact) {
+  BwdBlock b{};
   if (!ctx || ctx->block_overlap != 2 || ctx->direct_rows || ctx->bwd_reduce || check_common(ctx, CAAT_MLP_DOWN, tokens) != CAAT_OK)
-    return false;
-  if (compact && ctx->S % kLayoutVec != 0) return false;
-  if (!tc_gemm_usable(ctx, layer_kr(ctx, CAAT_ATTN_OUT)) || !tc_gemm_usable(ctx, layer_kr(ctx, CAAT_MLP_DOWN))) return false;
-  const int S_lo = round_down(ctx->S, kLayoutVec);
-  return rows_block_bwd_usable(ctx->h, tokens, ctx->h - S_lo, round_up(ctx->S, kLayoutVec), ctx->dtype, compact, ctx->norm);
+    return b;
+  if (compact && ctx->S % kLayoutVec != 0) return b;
+  for (int l = 0; l < 2; ++l) {
+    const int K_r = layer_kr(ctx, l == 0 ? CAAT_ATTN_OUT : CAAT_MLP_DOWN);
+    if (!tc_gemm_usable(ctx, K_r)) return b;
+    b.L[l] = scratch_layout(ctx, K_r, tokens, 1);
+    b.sh[l] = RowparShapes{ctx->t, tokens, ctx->h, K_r, ctx->S, b.L[l].S_lo, b.L[l].S_hi, b.L[l].P};
+  }
+  b.one_pass = rows_block_bwd_usable(ctx->h, tokens, b.L[0].P, b.L[0].S_hi, ctx->dtype, compact, ctx->norm);
+  b.plan = tc_backward_block_plan(b.sh);
+  b.applies = b.one_pass || b.plan.merged;
+  return b;
 }
 
 static bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
@@ -696,34 +709,53 @@ static bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
   return a && b && x < y + nb && y < x + na;
 }
 
-static caat_status block_backward_fused(const caat_ctx* ctx, int tokens, const RowBlockBwdArgs& rows, const void* Y_attn,
-                                        const void* W_o, const void* Y_mlp, const void* W_down, void* dY_attn, float* dW_o,
-                                        void* dY_mlp, float* dW_down, void* workspace, cudaStream_t st) {
+static caat_status block_backward_fused(const caat_ctx* ctx, int tokens, const BwdBlock& b, const RowBlockBwdArgs& rows,
+                                        const void* Y_attn, const void* W_o, const void* Y_mlp, const void* W_down, void* dY_attn,
+                                        float* dW_o, void* dY_mlp, float* dW_down, void* workspace, cudaStream_t st) {
   RowBlockBwdArgs a = rows;
   const bool over_alpha = alpha_on_epilogues(ctx, a.compact);
   const bool prescale = ctx->alpha != 1.0 && ctx->S < ctx->h && !over_alpha;
-  char* wsb[2];
-  Scratch L[2];
-  int K_r[2];
+  char* wsb[2] = {static_cast<char*>(workspace), static_cast<char*>(workspace) + align_up(b.L[0].total, 256)};
+  BwdGemm g[2];
   for (int l = 0; l < 2; ++l) {
-    K_r[l] = layer_kr(ctx, l == 0 ? CAAT_ATTN_OUT : CAAT_MLP_DOWN);
-    L[l] = scratch_layout(ctx, K_r[l], tokens, 1);
-    wsb[l] = l == 0 ? static_cast<char*>(workspace) : wsb[0] + align_up(L[0].total, 256);
-    if (!a.compact) a.gs[l] = wsb[l] + L[l].zs_off;
-    a.dgpart[l] = reinterpret_cast<float*>(wsb[l] + L[l].dgpart_off);
-    a.dbpart[l] = reinterpret_cast<float*>(wsb[l] + L[l].dbpart_off);
-    if (prescale) { a.w_src[l] = l == 0 ? W_o : W_down; a.w_dst[l] = wsb[l] + L[l].wt_off; a.w_Kr[l] = K_r[l]; }
+    const Scratch& L = b.L[l];
+    if (!a.compact) a.gs[l] = wsb[l] + L.zs_off;
+    a.dgpart[l] = reinterpret_cast<float*>(wsb[l] + L.dgpart_off);
+    a.dbpart[l] = reinterpret_cast<float*>(wsb[l] + L.dbpart_off);
+    g[l] = BwdGemm{b.sh[l], a.gs[l], priv_operand(ctx, L, a.dR[l], a.compact, over_alpha), l == 0 ? W_o : W_down,
+                   l == 0 ? Y_attn : Y_mlp, prescale ? wsb[l] + L.wt_off : nullptr, l == 0 ? dY_attn : dY_mlp, l == 0 ? dW_o : dW_down};
+    if (prescale) { a.w_src[l] = g[l].W; a.w_dst[l] = wsb[l] + L.wt_off; a.w_Kr[l] = b.sh[l].K_r; }
   }
-  a.t = ctx->t; a.T = tokens; a.h = ctx->h; a.S = ctx->S; a.S_lo = L[0].S_lo; a.S_hi = L[0].S_hi; a.P = L[0].P;
+  a.t = ctx->t; a.T = tokens; a.h = ctx->h; a.S = ctx->S; a.S_lo = b.L[0].S_lo; a.S_hi = b.L[0].S_hi; a.P = b.L[0].P;
   a.alpha = (float)ctx->alpha; a.norm = ctx->norm;
   a.gs_scale = over_alpha ? (float)(1.0 / ctx->alpha) : 1.0f;
-  const cudaError_t ce = launch_rows_backward_block(a, st);
+  cudaError_t ce = cudaSuccess;
+  if (b.one_pass) {
+    ce = launch_rows_backward_block(a, st);
+  } else {
+    for (int l = 1; l >= 0 && ce == cudaSuccess; --l) {
+      // the second layer's residual gradient is the first one's stream gradient; an absent part of a given one borrows the
+      // other part's pointer
+      const void* dh = l == 1 ? (a.dHn ? a.dHn : a.dHns) : (a.dR[1] ? a.dR[1] : a.gs[1]);
+      const void* dhs = l == 1 ? (a.dHns ? a.dHns : a.dHn) : (a.gs[1] ? a.gs[1] : a.dR[1]);
+      RowBwdArgs r{a.dX[l], dh, a.Hn[l], a.gamma[l], a.rstd[l], a.mean[l], a.dR[l], a.gs[l], nullptr, a.dgpart[l], a.dbpart[l],
+                   a.dgamma[l], a.dbeta[l], a.t, a.T, a.h, a.S, a.S_lo, a.S_hi, a.P, a.alpha, a.norm};
+      r.compact = a.compact; r.Hns = a.Hns[l]; r.dHns = a.compact ? dhs : nullptr;
+      r.gs_scale = a.gs_scale;
+      r.w_src = a.w_src[l]; r.w_dst = a.w_dst[l]; r.w_Kr = a.w_Kr[l];
+      ce = launch_rows_backward(r, ctx->dtype, ctx->direct_rows, st);
+    }
+  }
   if (ce != cudaSuccess) return cuda_fail(ce);
-  const caat_status s = backward_gemms(ctx, K_r[1], tokens, a.gs[1], a.dR[1], Y_mlp, W_down, dY_mlp, dW_down, wsb[1], L[1], a.compact,
-                                       over_alpha, prescale, st);
-  if (s != CAAT_OK) return s;
-  return backward_gemms(ctx, K_r[0], tokens, a.gs[0], a.dR[0], Y_attn, W_o, dY_attn, dW_o, wsb[0], L[0], a.compact, over_alpha, prescale,
-                        st);
+  if (b.plan.merged) {
+    ce = launch_tc_backward_block(b.plan, g, st);
+    return ce == cudaSuccess ? CAAT_OK : cuda_fail(ce);
+  }
+  caat_status s = CAAT_OK;
+  for (int l = 1; l >= 0 && s == CAAT_OK; --l)
+    s = backward_gemms(ctx, b.sh[l].K_r, tokens, a.gs[l], a.dR[l], g[l].Y, g[l].W, g[l].dY, g[l].dW, wsb[l], b.L[l], a.compact,
+                       over_alpha, prescale, st);
+  return s;
 }
 
 caat_status caat_block_backward(const caat_ctx* ctx, int tokens, const void* dX1, const void* dX2, const void* dHn2,
@@ -734,7 +766,8 @@ caat_status caat_block_backward(const caat_ctx* ctx, int tokens, const void* dX1
                                 float* dgamma1, float* dbeta1, float* dgamma2, float* dbeta2, void* workspace,
                                 size_t workspace_bytes, void* cuda_stream) {
   if (!dHn1) return CAAT_EINVAL;
-  if (fused_backward_applies(ctx, tokens, 0) && workspace && workspace_bytes >= caat_block_workspace_bytes(ctx, tokens, 1) &&
+  const BwdBlock b = backward_block_plan(ctx, tokens, 0);
+  if (b.applies && workspace && workspace_bytes >= align_up(b.L[0].total, 256) + b.L[1].total &&
       dX1 && dX2 && Y_attn && W_o && Y_mlp && W_down && Hn1 && rstd1 && Hn2 && rstd2 && gamma1 && gamma2 && dY_attn && dW_o &&
       dY_mlp && dW_down && dR0 && dgamma1 && dgamma2 && (ctx->norm == 0 || (mean1 && mean2 && dbeta1 && dbeta2))) {
     const void* ptrs[] = {dX1, dX2, dHn2, Y_attn, W_o, Y_mlp, W_down, Hn1, rstd1, mean1, Hn2, rstd2, mean2, gamma1, gamma2, dY_attn,
@@ -751,7 +784,7 @@ caat_status caat_block_backward(const caat_ctx* ctx, int tokens, const void* dX1
       a.dX[0] = dX1; a.dX[1] = dX2; a.Hn[0] = Hn1; a.Hn[1] = Hn2; a.gamma[0] = gamma1; a.gamma[1] = gamma2; a.dHn = dHn2;
       a.rstd[0] = rstd1; a.rstd[1] = rstd2; a.mean[0] = mean1; a.mean[1] = mean2; a.dR[0] = dR0; a.dR[1] = dHn1;
       a.dgamma[0] = dgamma1; a.dgamma[1] = dgamma2; a.dbeta[0] = dbeta1; a.dbeta[1] = dbeta2;
-      return block_backward_fused(ctx, tokens, a, Y_attn, W_o, Y_mlp, W_down, dY_attn, dW_o, dY_mlp, dW_down, workspace,
+      return block_backward_fused(ctx, tokens, b, a, Y_attn, W_o, Y_mlp, W_down, dY_attn, dW_o, dY_mlp, dW_down, workspace,
                                   static_cast<cudaStream_t>(cuda_stream));
     }
   }
@@ -860,7 +893,8 @@ caat_status caat_block_backward_compact(const caat_ctx* ctx, int tokens, const v
                                         size_t workspace_bytes, void* cuda_stream) {
   const bool has_s = ctx && ctx->S > 0, has_p = ctx && ctx->S < ctx->h;
   const bool any_dh = (has_s && dHn2s) || (has_p && dHn2p);
-  if (fused_backward_applies(ctx, tokens, 1) && workspace && workspace_bytes >= caat_block_workspace_bytes(ctx, tokens, 1) &&
+  const BwdBlock b = backward_block_plan(ctx, tokens, 1);
+  if (b.applies && workspace && workspace_bytes >= align_up(b.L[0].total, 256) + b.L[1].total &&
       dX1 && dX2 && Y_attn && W_o && Y_mlp && W_down && rstd1 && rstd2 && gamma1 && gamma2 && dY_attn && dW_o && dY_mlp && dW_down &&
       dgamma1 && dgamma2 && (!has_s || (Hn1s && Hn2s && dR0s && dHn1s && (!any_dh || dHn2s))) &&
       (!has_p || (Hn1p && Hn2p && dR0p && dHn1p && (!any_dh || dHn2p))) &&
@@ -886,7 +920,7 @@ caat_status caat_block_backward_compact(const caat_ctx* ctx, int tokens, const v
       a.rstd[0] = rstd1; a.rstd[1] = rstd2; a.mean[0] = mean1; a.mean[1] = mean2;
       a.dR[0] = dR0p; a.dR[1] = dHn1p; a.gs[0] = dR0s; a.gs[1] = dHn1s;
       a.dgamma[0] = dgamma1; a.dgamma[1] = dgamma2; a.dbeta[0] = dbeta1; a.dbeta[1] = dbeta2;
-      return block_backward_fused(ctx, tokens, a, Y_attn, W_o, Y_mlp, W_down, dY_attn, dW_o, dY_mlp, dW_down, workspace,
+      return block_backward_fused(ctx, tokens, b, a, Y_attn, W_o, Y_mlp, W_down, dY_attn, dW_o, dY_mlp, dW_down, workspace,
                                   static_cast<cudaStream_t>(cuda_stream));
     }
   }

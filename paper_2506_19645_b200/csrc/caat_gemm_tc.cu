@@ -54,7 +54,7 @@ constexpr int kAidMask = ~0;
 constexpr int kAidMask = 1024;
 #endif
 
-constexpr int kMaxRegions = 4;
+constexpr int kMaxRegions = 6;      // four, but for the launch of a block's four gradient products
 
 struct Unit {            // one contraction segment of a tile
   int mapA, mapB;        // indices into the tensor-map array
@@ -87,6 +87,7 @@ struct Region {          // a family of output tiles with the same operand wirin
   int b_slowest;         // tile order: 1 = rank index slowest (a rank's weights / activations stay
                          // hot in L2 while its row tiles stream), 0 = row tile slowest
   float scale;           // outputs are multiplied by it in the epilogue (0 means 1)
+  int a_mn;              // MIXED launches: as Params::a_mn, per region
 };
 
 struct Params {
@@ -227,7 +228,9 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
 struct PeerMaps { CUtensorMap m[CAAT_MAX_PEERS]; };
 
 // Operand maps (A and B of up to two layers or units) and output maps, one per region.
-struct Maps { CUtensorMap ab[4], c[kMaxRegions]; };
+template <bool MIXED> struct MapsT { CUtensorMap ab[4], c[4]; };
+template <> struct MapsT<true> { CUtensorMap ab[14], c[kMaxRegions]; };
+using Maps = MapsT<false>;
 
 // The swapped variant's tiles dealt to CTAs by their length (longest first, each to the least loaded CTA): CTA w works
 // item[first[w]] .. item[first[w + 1] - 1].  dealt == 0: round-robin by tile number.
@@ -352,9 +355,9 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {   // arrives on
 // leader (cluster rank 0) issues the MMAs for both and the tensor cores read B from both CTAs'
 // shared memory, so the operand bytes a CTA pulls from L2 per flop drop by a third.
 // SWAP: the operands are swapped (few tokens: weights on the 128-row side), fp32 planes stored straight from registers.
-template <int CG, bool SWAP>
+template <int CG, bool SWAP, bool MIXED>
 __global__ void __launch_bounds__(kThreads, 1)
-tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename ExtraArg<SWAP>::type extra,
+tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ typename ExtraArg<SWAP>::type extra,
                const __grid_constant__ Params p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr int BMT = BM * CG;                     // rows of a tile (of the pair's tile)
@@ -413,7 +416,7 @@ tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename
     // barrier that is already free, 250 for the announcement and one box, 85 of loop), more than the 384-512
     // cycles the tensor cores take for it.
     constexpr int kKI = 2;
-    const bool multi = (isA ? p.a_mn : p.b_mn) != 0;
+    const bool multi = MIXED || (isA ? p.a_mn : p.b_mn) != 0;       // MIXED: some regions' A, every region's B
     const int nbmax = multi ? (isA ? BM / 64 : (int)(p.BN / CG) / 64) : 1;      // boxes per stage, at most
     // measured: pays for multi-box operands (dgrad / wgrad -5...-8 %) and the weight stream of the decode
     // path (-5 %); a K-major operand of the large GEMMs gains nothing (its tiles wait for L2, not for the
@@ -432,7 +435,8 @@ tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename
         const int m0 = c.mt * BMT + (int)rank * BM, n0 = c.nt * p.BN + (int)(rank * cols_cta);
         const uint32_t tx = (uint32_t)CG * (((p.debug & kAidMask & 4) ? 0u : a_bytes) + ((p.debug & kAidMask & 8) ? 0u : b_tile_bytes));
         const bool skip = isA ? (p.debug & kAidMask & (4 | 1024)) != 0 : (p.debug & kAidMask & 8) != 0;
-        const int nb = multi ? (isA ? BM / 64 : (int)cols_cta / 64) : 1;         // boxes of this tile's stages
+        const int a_mn = MIXED ? r.a_mn : p.a_mn;
+        const int nb = isA ? (a_mn ? BM / 64 : 1) : (multi ? (int)cols_cta / 64 : 1);         // boxes of this tile's stages
         for (int ui = 0; ui < r.nunits && ok; ++ui) {
           const Unit& u = r.u[ui];
           const CUtensorMap* map = &mp.ab[isA ? u.mapA : u.mapB];
@@ -459,7 +463,7 @@ tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename
                     if (CG == 2) tma_load_3d_pair(dst, map, x, y, z, fb); else tma_load_3d(dst, map, x, y, z, fb);
                   };
                   if (isA) {
-                    if (!p.a_mn) load(sa, u.ak0 + kk * BK, u.am0 + m0);
+                    if (!a_mn) load(sa, u.ak0 + kk * BK, u.am0 + m0);
                     else load(sa + box * (64 * BK * 2), u.am0 + m0 + box * 64, u.ak0 + kk * BK);
                   } else {
                     if (!p.b_mn) load(sb, u.bk0 + kk * BK, u.bn0 + n0);
@@ -491,7 +495,7 @@ tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader CTA only when CG == 2)
     if (rank == 0) {                              // the whole warp walks the schedule, one elected lane issues
-      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)p.a_mn << 15) | ((uint32_t)p.b_mn << 16) |
+      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(MIXED ? 0 : p.a_mn) << 15) | ((uint32_t)p.b_mn << 16) |
                               ((uint32_t)(BMT >> 4) << 24);
       int stage = 0; uint32_t phase = 0;
       int acc = 0; uint32_t acc_phase = 0;
@@ -499,12 +503,15 @@ tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename
       // Descriptors differ from stage to stage and from MMA to MMA only in their 14-bit address field:
       // the constant part is built once and the loop adds 16-byte units to the low word.  The issuing
       // thread's instruction count per k-step is what bounds short contractions.
-      const uint64_t a_const = p.a_mn ? make_desc(0, 64 * BK * 2, 1024) : make_desc(0, 16, 1024);
+      const uint64_t a_const = p.a_mn && !MIXED ? make_desc(0, 64 * BK * 2, 1024) : make_desc(0, 16, 1024);
+      const uint32_t a_mn_lo = (uint32_t)make_desc(0, 64 * BK * 2, 1024) - (uint32_t)make_desc(0, 16, 1024);
       const uint64_t b_const = p.b_mn ? make_desc(0, 64 * BK * 2, 1024) : make_desc(0, 16, 1024);
       const uint32_t a_hi = (uint32_t)(a_const >> 32), b_hi = (uint32_t)(b_const >> 32);
-      const uint32_t a_k16 = (p.a_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4, b_k16 = (p.b_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      uint32_t a_k16 = (p.a_mn && !MIXED ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      const uint32_t b_k16 = (p.b_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
       const uint32_t stage16 = stage_bytes >> 4;
-      const uint32_t a_lo0 = (uint32_t)a_const + (tiles_sa >> 4), b_lo0 = (uint32_t)b_const + ((tiles_sa + a_bytes) >> 4);
+      uint32_t a_lo0 = (uint32_t)a_const + (tiles_sa >> 4);
+      const uint32_t b_lo0 = (uint32_t)b_const + ((tiles_sa + a_bytes) >> 4);
       uint32_t a_lo = a_lo0, b_lo = b_lo0;
       uint32_t full_bar = full0, empty_bar = empty0;
       for (TileIter<SWAP> it(extra, worker, nworkers, p.tiles_total); it.valid() && ok; it.next()) {
@@ -513,7 +520,13 @@ tc_gemm_kernel(const __grid_constant__ Maps mp, const __grid_constant__ typename
         if (!mbar_wait_warp(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, p.spin_cap)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kAccCols);
-        const uint32_t idesc = idesc0 | ((uint32_t)(tile_cols(p, r, c.nt, CG) >> 3) << 17);
+        uint32_t idesc = idesc0 | ((uint32_t)(tile_cols(p, r, c.nt, CG) >> 3) << 17);
+        if constexpr (MIXED) {
+          idesc |= (uint32_t)r.a_mn << 15;
+          a_k16 = (r.a_mn ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+          a_lo0 = (uint32_t)a_const + (tiles_sa >> 4) + (r.a_mn ? a_mn_lo : 0u);
+          a_lo = a_lo0 + (uint32_t)stage * stage16;
+        }
         uint32_t accumulate = 0;
         for (int ui = 0; ui < r.nunits && ok; ++ui) {
           const Unit& u = r.u[ui];
@@ -897,7 +910,8 @@ TileCfg pick_tile(const RegionShape* r, int nr, bool b_n_major, int max_splits, 
   return best;
 }
 
-cudaError_t launch(const Maps& maps, Params& p, int kind, cudaStream_t st, const PeerMaps* peer_maps = nullptr,
+template <bool MIXED = false>
+cudaError_t launch(const MapsT<MIXED>& maps, Params& p, int kind, cudaStream_t st, const PeerMaps* peer_maps = nullptr,
                    const Deal* deal = nullptr) {
   const LaunchLimits lim = effective_limits();
   const int stage_bytes = BM * BK * 2 + (p.BN / p.cg) * BK * 2;
@@ -911,9 +925,11 @@ cudaError_t launch(const Maps& maps, Params& p, int kind, cudaStream_t st, const
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (std::lock_guard<std::mutex> lock(host_cache_mutex()); !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_gemm_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_gemm_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    auto allow = [](auto k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); };
+    cudaError_t e = allow(tc_gemm_kernel<1, false, MIXED>);
+    if (e == cudaSuccess) e = allow(tc_gemm_kernel<2, false, MIXED>);
+    if constexpr (!MIXED)
+      if (e == cudaSuccess) e = allow(tc_gemm_kernel<1, true, false>);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
@@ -947,11 +963,12 @@ cudaError_t launch(const Maps& maps, Params& p, int kind, cudaStream_t st, const
   cfg.attrs = attr;
   cfg.numAttrs = pdl_enabled() ? 2 : 1;
   LaunchScope scope(kind, st);
-  if (deal) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, true>, maps, *deal, (const Params&)p);
+  if constexpr (!MIXED)
+    if (deal) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, true, false>, maps, *deal, (const Params&)p);
   static const PeerMaps no_peers{};
   const PeerMaps& pm = peer_maps ? *peer_maps : no_peers;
-  if (p.cg == 2) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, false>, maps, pm, (const Params&)p);
-  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, false>, maps, pm, (const Params&)p);
+  if (p.cg == 2) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, false, MIXED>, maps, pm, (const Params&)p);
+  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, false, MIXED>, maps, pm, (const Params&)p);
 }
 
 void finish_tiles(Params& p) {
@@ -1313,7 +1330,7 @@ cudaError_t launch_tc_forward_decode(int t, int T, int h, int S, DecodeProblem* 
     }
   }
   if (n == 1) { mp.ab[2] = mp.ab[0]; mp.ab[3] = mp.ab[1]; }
-  for (int c = 0; c < kMaxRegions; ++c) mp.c[c] = mp.ab[0];          // unused: the epilogue stores directly
+  for (CUtensorMap& c : mp.c) c = mp.ab[0];          // unused: the epilogue stores directly
   p.nregions = g;
   finish_tiles(p);
   if (plan.deal.dealt && plan.deal.first[plan.workers] != p.tiles_total) return cudaErrorInvalidValue;
@@ -1325,46 +1342,53 @@ cudaError_t launch_tc_forward_decode(int t, int T, int h, int S, DecodeProblem* 
 // pv.alpha != 1, w_scaled ([t, h, K_r], only rows >= S are used) must hold alpha times the private rows of W.
 // Any partition S: the private gradient is read from column S_lo on, and the weights' map starts at row S with the
 // coordinate -(S - S_lo), so the shared columns among them meet rows that TMA fills with zeros.
-cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* W, void* dY,
-                            void* w_scaled, bool w_scaled_ready, cudaStream_t st) {
-  Maps mp;
-  CUtensorMap *maps = mp.ab, *cmaps = mp.c;
-  Params p{};
-  {
-    const RegionShape rs[1] = {{s.T, s.K_r, s.t, (s.S + BK - 1) / BK + (s.h - s.S_lo + BK - 1) / BK}};
-    const TileCfg c = pick_tile(rs, 1, true, 1, 0.0);
-    p.BN = c.bn; p.cg = c.cg;
-  }
+static RegionShape dgrad_shape(const RowparShapes& s) {
+  return RegionShape{s.T, s.K_r, s.t, (s.S + BK - 1) / BK + (s.h - s.S_lo + BK - 1) / BK};
+}
+
+// the next region of the launch: one layer's data gradient, its operand maps ab[b] .. ab[b + 3]
+template <typename M>
+static bool dgrad_region(M& mp, Params& p, int b, const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* W,
+                         void* dY, const void* w_scaled) {
+  CUtensorMap* maps = mp.ab + b;
   const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
   // B = W[m] as [h rows (contraction)][K_r contiguous (N)]: N-major, boxes of 64 (N) x 64 (K)
-  if (!make_map(&maps[1], W, s.K_r, s.h, s.t, s.K_r, (long long)s.h * s.K_r, 64, BK)) return cudaErrorInvalidValue;
+  if (!make_map(&maps[1], W, s.K_r, s.h, s.t, s.K_r, (long long)s.h * s.K_r, 64, BK)) return false;
   maps[3] = maps[1];
   if (n_pr > 0) {
     const void* wp = W;
     if (pv.alpha != 1.0f && !pv.gs_over_alpha) {
       // sum_l (alpha g[l]) W[l][k] = sum_l g[l] (alpha W[l][k]): the private gradient is read as stored in dR,
       // the weights' private rows (the small operand) carry alpha; they were scaled by the launch before this one
-      if (!w_scaled || !w_scaled_ready) return cudaErrorInvalidValue;
+      if (!w_scaled) return false;
       wp = w_scaled;
     }
     if (!make_map(&maps[3], static_cast<const __nv_bfloat16*>(wp) + (long long)s.S * s.K_r, s.K_r, s.h - s.S, s.t, s.K_r,
                   (long long)s.h * s.K_r, 64, BK))
-      return cudaErrorInvalidValue;
+      return false;
   }
-  bool okA0 = n_sh > 0 ? make_map(&maps[0], gs, n_sh, s.T, 1, s.S_hi, (long long)s.T * s.S_hi, BK, BM) : true;
-  bool okA1 = n_pr > 0 ? make_map(&maps[2], pv.ptr, pv.ld, s.T, s.t, pv.ld, (long long)s.T * pv.ld, BK, BM) : true;
-  if (!okA0 || !okA1) return cudaErrorInvalidValue;
+  if (n_sh > 0 && !make_map(&maps[0], gs, n_sh, s.T, 1, s.S_hi, (long long)s.T * s.S_hi, BK, BM)) return false;
+  if (n_pr > 0 && !make_map(&maps[2], pv.ptr, pv.ld, s.T, s.t, pv.ld, (long long)s.T * pv.ld, BK, BM)) return false;
   if (n_sh == 0) maps[0] = maps[2];
   if (n_pr == 0) maps[2] = maps[0];
-  p.a_mn = 0; p.b_mn = 1;  p.splits = 1;
-  Region& r = p.r[0];
+  Region& r = p.r[p.nregions];
   int nu = 0;
-  if (n_sh > 0) r.u[nu++] = Unit{0, 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, (n_sh + BK - 1) / BK};
-  if (n_pr > 0) r.u[nu++] = Unit{2, 3, pv.col0, 0, s.S_lo - s.S, 0, 1, 0, 1, 0, 1, (n_pr + BK - 1) / BK};
+  if (n_sh > 0) r.u[nu++] = Unit{b, b + 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, (n_sh + BK - 1) / BK};
+  if (n_pr > 0) r.u[nu++] = Unit{b + 2, b + 3, pv.col0, 0, s.S_lo - s.S, 0, 1, 0, 1, 0, 1, (n_pr + BK - 1) / BK};
   r.nunits = nu;
   r.M = s.T; r.N = s.K_r; r.batch = s.t; r.b_slowest = 1; r.scale = pv.gs_over_alpha ? pv.alpha : 1.0f;
-  if (!make_cmap(&cmaps[0], dY, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, false)) return cudaErrorInvalidValue;
-  p.nregions = 1;
+  return make_cmap(&mp.c[p.nregions++], dY, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, false);
+}
+
+cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* W, void* dY,
+                            void* w_scaled, bool w_scaled_ready, cudaStream_t st) {
+  Maps mp;
+  Params p{};
+  const RegionShape rs = dgrad_shape(s);
+  const TileCfg c = pick_tile(&rs, 1, true, 1, 0.0);
+  p.BN = c.bn; p.cg = c.cg;
+  p.a_mn = 0; p.b_mn = 1;  p.splits = 1;
+  if (!dgrad_region(mp, p, 0, s, gs, pv, W, dY, w_scaled_ready ? w_scaled : nullptr)) return cudaErrorInvalidValue;
   finish_tiles(p);
   return launch(mp, p, CAAT_K_TC_DGRAD, st);
 }
@@ -1381,55 +1405,64 @@ size_t tc_wgrad_splitk_bytes(const RowparShapes& s) {
 }
 
 // ---- wgrad: dW[m][:S] = gs^T Y[m] ; dW[m][S:] = alpha gp[m]^T Y[m]      (fp32 out; alpha in the epilogue)
-cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* Y, float* dW,
-                            void* splitk, size_t splitk_bytes, cudaStream_t st) {
-  Maps mp;
-  CUtensorMap *maps = mp.ab, *cmaps = mp.c;
-  Params p{};
-  const TileCfg wc = wgrad_cfg(s);
-  p.BN = wc.bn; p.cg = wc.cg;
+// operand maps of one layer: ab[b] the shared gradient, ab[b + 1] the activations, ab[b + 2] the private gradient
+template <typename M>
+static bool wgrad_maps(M& mp, int b, const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* Y) {
+  CUtensorMap* maps = mp.ab + b;
   const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
-  const int splits = wc.splits;
-  const long long dw_elems = (long long)s.t * s.h * s.K_r;
-  if (splits > 1 && splitk_bytes < (size_t)splits * dw_elems * sizeof(float)) return cudaErrorInvalidValue;
   // A = dZt as [T rows (contraction)][channels contiguous (M)]: M-major, boxes of 64 (M) x 64 (K)
-  bool okA0 = n_sh > 0 ? make_map(&maps[0], gs, n_sh, s.T, 1, s.S_hi, (long long)s.T * s.S_hi, 64, BK) : true;
-  bool okA1 = n_pr > 0 ? make_map(&maps[2], pv.ptr, pv.ld, s.T, s.t, pv.ld, (long long)s.T * pv.ld, 64, BK) : true;
+  if (n_sh > 0 && !make_map(&maps[0], gs, n_sh, s.T, 1, s.S_hi, (long long)s.T * s.S_hi, 64, BK)) return false;
+  if (n_pr > 0 && !make_map(&maps[2], pv.ptr, pv.ld, s.T, s.t, pv.ld, (long long)s.T * pv.ld, 64, BK)) return false;
   // B = Y[m] as [T rows (contraction)][K_r contiguous (N)]: N-major
-  if (!okA0 || !okA1 || !make_map(&maps[1], Y, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, 64, BK))
-    return cudaErrorInvalidValue;
+  if (!make_map(&maps[1], Y, s.K_r, s.T, s.t, s.K_r, (long long)s.T * s.K_r, 64, BK)) return false;
   if (n_sh == 0) maps[0] = maps[2];
   if (n_pr == 0) maps[2] = maps[0];
-  maps[3] = maps[1];
-  p.a_mn = 1; p.b_mn = 1;  p.splits = splits;
-  const int ksteps = (s.T + BK - 1) / BK;
-  float* out = splits > 1 ? static_cast<float*>(splitk) : dW;
-  int g = 0;
+  return true;
+}
+// the next region or regions of the launch; out: dW, or the split-K planes
+template <typename M>
+static bool wgrad_regions(M& mp, Params& p, int b, const RowparShapes& s, const PrivOperand& pv, float* out, int splits) {
+  const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0, ksteps = (s.T + BK - 1) / BK;
   if (n_sh > 0) {
-    Region& r = p.r[g++];
+    Region& r = p.r[p.nregions];
     r.nunits = 1;
-    r.u[0] = Unit{0, 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, ksteps};
+    r.u[0] = Unit{b, b + 1, 0, 0, 0, 0, 0, 0, 1, 0, 1, ksteps};
     r.out_f32 = 1;
+    r.a_mn = 1;
     r.M = n_sh; r.N = s.K_r; r.batch = s.t; r.b_slowest = 0;   // the shared gradient panel serves all ranks at once
     r.scale = pv.gs_over_alpha ? pv.alpha : 1.0f;
-    if (!make_cmap(&cmaps[g - 1], out, s.K_r, n_sh, (long long)s.t * splits, s.K_r, (long long)s.h * s.K_r, true))
-      return cudaErrorInvalidValue;
+    if (!make_cmap(&mp.c[p.nregions++], out, s.K_r, n_sh, (long long)s.t * splits, s.K_r, (long long)s.h * s.K_r, true)) return false;
   }
   if (n_pr > 0) {
-    Region& r = p.r[g++];
+    Region& r = p.r[p.nregions];
     r.nunits = 1;
-    r.u[0] = Unit{2, 1, 0, pv.col0, 0, 0, 1, 0, 1, 0, 1, ksteps};
+    r.u[0] = Unit{b + 2, b + 1, 0, pv.col0, 0, 0, 1, 0, 1, 0, 1, ksteps};
     r.out_f32 = 1;
+    r.a_mn = 1;
     r.M = n_pr; r.N = s.K_r; r.batch = s.t; r.b_slowest = 1;
     r.scale = pv.alpha;
     r.skip = s.S - s.S_lo;
     r.skip_out = out + (long long)s.S_lo * s.K_r;
     r.skip_plane = (long long)s.h * s.K_r;
-    if (!make_cmap(&cmaps[g - 1], out + (long long)s.S_lo * s.K_r, s.K_r, n_pr, (long long)s.t * splits, s.K_r,
+    if (!make_cmap(&mp.c[p.nregions++], out + (long long)s.S_lo * s.K_r, s.K_r, n_pr, (long long)s.t * splits, s.K_r,
                    (long long)s.h * s.K_r, true))
-      return cudaErrorInvalidValue;
+      return false;
   }
-  p.nregions = g;
+  return true;
+}
+
+cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* Y, float* dW,
+                            void* splitk, size_t splitk_bytes, cudaStream_t st) {
+  Maps mp;
+  Params p{};
+  const TileCfg wc = wgrad_cfg(s);
+  p.BN = wc.bn; p.cg = wc.cg;
+  const int splits = wc.splits;
+  const long long dw_elems = (long long)s.t * s.h * s.K_r;
+  if (splits > 1 && splitk_bytes < (size_t)splits * dw_elems * sizeof(float)) return cudaErrorInvalidValue;
+  p.a_mn = 1; p.b_mn = 1;  p.splits = splits;
+  if (!wgrad_maps(mp, 0, s, gs, pv, Y) || !wgrad_regions(mp, p, 0, s, pv, splits > 1 ? static_cast<float*>(splitk) : dW, splits))
+    return cudaErrorInvalidValue;
   finish_tiles(p);
   cudaError_t e = launch(mp, p, CAAT_K_TC_WGRAD, st);
   if (e != cudaSuccess) return e;
@@ -1442,6 +1475,58 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
                    reinterpret_cast<float4*>(dW), n4, splits);
   }
   return e;
+}
+
+// ---- a block's four gradient products, independent of one another once both layers' row work is done: one launch,
+// longest contractions first, so that the short tiles of the data gradients fill the last rounds of the weight gradients
+// and three ramps and tails go away.  A launch of its own is worth 2.4 us and one launch has to win by 5 % of its time, as
+// in the forward; and it has to be short: the CTAs of a long launch drift apart and stop sharing operands in L2, which costs
+// more than the tails.  Training step of a block, four launches / one (us): taken - 4 x 768, 300 tokens 56.9 / 39.8, 3000
+// tokens 148 / 131, 16384 tokens 606 / 596; 8 x 2048, 600 tokens 166 / 150, 2999 tokens (p = 0.7) 549 / 537, 8192 tokens
+// 1360 / 1340; 8 x 4096, 300 tokens 289 / 281, 1000 tokens 572 / 554; not taken - 3000 tokens 1500 / 1503, 16384 tokens
+// 7730 / 8250.
+BwdBlockPlan tc_backward_block_plan(const RowparShapes* shapes) {
+  constexpr double kLaunchGap = 12, kMargin = 1.05, kLongest = 1200;       // units of 0.2 us
+  RegionShape rs[kMaxRegions] = {};
+  BwdBlockPlan b{};
+  int n = 0;
+  b.wgrad_first = (shapes[0].T + BK - 1) / BK >= dgrad_shape(shapes[0]).ksteps;
+  double apart = 3 * kLaunchGap;
+  for (int pass = 0; pass < 2; ++pass)
+    for (int l = 1; l >= 0; --l) {
+      const RowparShapes& s = shapes[l];
+      if ((pass == 0) == b.wgrad_first) {
+        const int ksteps = (s.T + BK - 1) / BK;
+        apart += wgrad_cfg(s).cost;
+        rs[n++] = RegionShape{s.S, s.K_r, s.t, ksteps};
+        rs[n++] = RegionShape{s.S < s.h ? s.h - s.S_lo : 0, s.K_r, s.t, ksteps};
+      } else {
+        rs[n] = dgrad_shape(s);
+        apart += pick_tile(rs + n, 1, true, 1, 0.0).cost;
+        ++n;
+      }
+    }
+  const TileCfg c = pick_tile(rs, n, true, 1, 0.0);
+  b.bn = c.bn; b.cg = c.cg;
+  b.merged = c.cost * kMargin < apart && c.cost < kLongest;
+  return b;
+}
+
+cudaError_t launch_tc_backward_block(const BwdBlockPlan& b, const BwdGemm* L, cudaStream_t st) {
+  MapsT<true> mp;
+  Params p{};
+  p.BN = b.bn; p.cg = b.cg; p.b_mn = 1; p.splits = 1;
+  for (int l = 0; l < 2; ++l)
+    if (!wgrad_maps(mp, 8 + 3 * l, L[l].s, L[l].gs, L[l].pv, L[l].Y)) return cudaErrorInvalidValue;
+  for (int pass = 0; pass < 2; ++pass)
+    for (int l = 1; l >= 0; --l) {
+      const BwdGemm& g = L[l];
+      const bool ok = (pass == 0) == b.wgrad_first ? wgrad_regions(mp, p, 8 + 3 * l, g.s, g.pv, g.dW, 1)
+                                                   : dgrad_region(mp, p, 4 * l, g.s, g.gs, g.pv, g.W, g.dY, g.w_scaled);
+      if (!ok) return cudaErrorInvalidValue;
+    }
+  finish_tiles(p);
+  return launch<true>(mp, p, CAAT_K_TC_WGRAD, st);
 }
 
 }  // namespace caat

@@ -119,6 +119,11 @@ cudaError_t launch_tc_dgrad(const RowparShapes& s, const void* gs, const PrivOpe
 cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOperand& pv, const void* Y, float* dW,
                             void* splitk, size_t splitk_bytes, cudaStream_t st);
 size_t tc_wgrad_splitk_bytes(const RowparShapes& s);
+// dY and dW of both layers of a block in one launch (plan.merged: cheaper than four)
+struct BwdBlockPlan { bool merged, wgrad_first; int bn, cg; };
+struct BwdGemm { RowparShapes s; const void* gs; PrivOperand pv; const void *W, *Y, *w_scaled; void* dY; float* dW; };
+BwdBlockPlan tc_backward_block_plan(const RowparShapes* shapes);
+cudaError_t launch_tc_backward_block(const BwdBlockPlan& plan, const BwdGemm* L, cudaStream_t st);
 // few tokens: the sums leave the GEMM as fp32 planes, zs [ns][T][S_hi] shared and zp [np][t][T][h - S_lo] private
 constexpr int kDecodeMaxTokens = 64;
 constexpr int kDecodeMaxSplits = 4;

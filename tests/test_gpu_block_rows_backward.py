@@ -1,4 +1,5 @@
-"""Both layers' backward row work in one pass (the default block backward) against a pass per layer and against the oracle."""
+"""The default block backward - both layers' row work in one pass, their four gradient products in one launch, or both -
+against the layers one after the other and against the oracle."""
 import pytest
 import torch
 
@@ -20,6 +21,11 @@ CASES = [
     (4, 130, 768, 3072, 380, 0, False),      # three warps per token
     (2, 2050, 512, 1024, 256, 0, True),      # two tokens per CTA, many rounds
     (2, 77, 272, 544, 128, 1, True),         # chunks past the row end
+    # rows of the layers one after the other, their four gradient products in one launch
+    (8, 300, 2048, 5632, 1024, 1, True),
+    (2, 257, 2048, 5632, 2048, 1, False),    # nothing private
+    (2, 129, 5120, 10240, 0, 0, True),       # nothing shared
+    (4, 200, 2048, 4096, 1003, 1, True),     # a partition off the 8-channel grid
 ]
 
 
@@ -80,7 +86,7 @@ def test_block_backward_rows_in_one_pass(t, T, h, ffn, S, norm, dh, compact):
     ctx.set_option(caat.CAAT_OPT_BLOCK_OVERLAP, 0)
     two = _run(ctx, d, sv, T, compact, S, norm, dh)
     if not (compact and h <= 768 and T > 2000):                   # those keep a pass per layer
-        assert caat.kernel_launches() - mid == mid - before + 2   # one row kernel and one norm-gradient sum less
+        assert caat.kernel_launches() - mid >= mid - before + 2   # one row kernel and one norm-gradient sum less
     z = lambda x: None if x is None else f64(x)
     args = [z(d["Y_attn"]), z(d["W_o"]), z(d["Y_mlp"]), z(d["W_down"])]
     if compact:
