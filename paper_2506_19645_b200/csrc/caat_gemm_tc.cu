@@ -1046,6 +1046,10 @@ static bool forward_private(Maps& mp, Params& p, int l, const RowparShapes& s, v
   return make_cmap(&mp.c[g], zp, s.h - s.S_lo, s.T, s.t, s.P, (long long)s.T * s.P, false);
 }
 
+// When the products of a block's two layers share a launch (units of 0.2 us): a launch of its own is worth kLaunchGap, the
+// shared one has to win by kMargin, and it has to be shorter than kLongest.
+constexpr double kLaunchGap = 12, kMargin = 1.05, kLongest = 1200;
+
 // Both layers' forward products of a block (they do not depend on each other): one launch where the cost model sees a
 // gain - one ramp, one tail and a finer deal where a layer's tiles do not fill the GPU - else one after the other.  Each
 // layer keeps the rank groups that it would have alone, so its sums do not depend on the schedule.
@@ -1053,10 +1057,10 @@ static bool forward_private(Maps& mp, Params& p, int l, const RowparShapes& s, v
 // time, which is what it loses to the model when both layers' operands go through L2 and only one tile width is left to
 // choose.  Block forward on either side of the line (apart / merged, us): taken - h 768, 300 tokens 21.9 / 14.9; h 2048,
 // 300 tokens 44.0 / 38.8, 2000 tokens 147 / 143; h 4096, 600 tokens 153 / 147, 3000 tokens 571 / 539; not taken - h 4096,
-// 1400 tokens 273 / 285; h 5120, 1000 tokens 306 / 312; h 4096, p = 0.75 on 2 ranks, 300 tokens 75 / 87.
+// 1400 tokens 273 / 285; h 5120, 1000 tokens 306 / 312; h 4096, p = 0.75 on 2 ranks, 300 tokens 75 / 87; long launches (see
+// the backward's) - h 4096, 8192 tokens 1389 / 1394, whole step 3810 / 3832, 65536 tokens of 4 x 768 2309 / 2337.
 cudaError_t launch_tc_forward_block(const RowparShapes* s, const void* const* Y, const void* const* W, void* const* zs,
                                     void* const* zp, void* const* planes, const int* max_groups, int* groups, cudaStream_t st) {
-  constexpr double kLaunchGap = 12, kMargin = 1.05;      // units of 0.2 us
   const ForwardPlan one[2] = {forward_plan(s[0], planes[0] ? max_groups[0] : 1), forward_plan(s[1], planes[1] ? max_groups[1] : 1)};
   const int ks[2] = {(s[0].K_r + BK - 1) / BK, (s[1].K_r + BK - 1) / BK};
   const int lead = ks[1] * one[1].qper >= ks[0] * one[0].qper ? 1 : 0;        // the layer with the longer shared tiles
@@ -1068,7 +1072,7 @@ cudaError_t launch_tc_forward_block(const RowparShapes* s, const void* const* Y,
   }
   TileCfg both = pick_tile(rs, 4, false, 1, 0.0);
   for (int l = 0; l < 2; ++l) both.cost += plane_cost(s[l], one[l].groups);
-  if (both.cost * kMargin >= one[0].tile.cost + one[1].tile.cost + kLaunchGap) {
+  if (both.cost * kMargin >= one[0].tile.cost + one[1].tile.cost + kLaunchGap || both.cost >= kLongest) {
     for (int l = 0; l < 2; ++l) {
       const cudaError_t e = launch_tc_forward(s[l], Y[l], W[l], zs[l], zp[l], st, nullptr, planes[l], max_groups[l], &groups[l]);
       if (e != cudaSuccess) return e;
@@ -1486,7 +1490,6 @@ cudaError_t launch_tc_wgrad(const RowparShapes& s, const void* gs, const PrivOpe
 // 1360 / 1340; 8 x 4096, 300 tokens 289 / 281, 1000 tokens 572 / 554; not taken - 3000 tokens 1500 / 1503, 16384 tokens
 // 7730 / 8250.
 BwdBlockPlan tc_backward_block_plan(const RowparShapes* shapes) {
-  constexpr double kLaunchGap = 12, kMargin = 1.05, kLongest = 1200;       // units of 0.2 us
   RegionShape rs[kMaxRegions] = {};
   BwdBlockPlan b{};
   int n = 0;
