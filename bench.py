@@ -549,6 +549,9 @@ def kernel_table(prof, work, steps, peaks):
     """Per kernel kind: device time per step from CUDA events around every launch, and the achieved rate on the
     kind's algorithmic work against the peak that bounds it (both bf16 denominators named)."""
     total = sum(v[0] for v in prof.values()) or 1.0
+    if "tc_gemm_wgrad" in prof and "tc_gemm_dgrad" not in prof and "tc_gemm_dgrad" in work:
+        # a block's four gradient products in one launch, counted as the weight gradient's kind
+        work = dict(work, tc_gemm_wgrad={k: v + work["tc_gemm_dgrad"][k] for k, v in work["tc_gemm_wgrad"].items()})
     kernels = {}
     for kind, (kms, n) in prof.items():
         per_step_ms = kms / steps
@@ -758,7 +761,7 @@ def config_of(w, S, world, compact, m):
             "S": S, "passes": passes(w), "private_scale": "sqrt(t)", "norm": "rmsnorm", "parallelism": f"replicas x{world}",
             "residual_layout": "compact (shared channels of the stream stored once)" if compact else "per rank [t,T,h]",
             "launch": "cuda graph replay" if m["graph"] else "eager", "l2": l2_note(m),
-            "block_forward_schedule": {None: "library's choice by shape (side by side unless the GEMM is much the longer kernel)",
+            "block_forward_schedule": {None: "library's choice by shape (both layers' rows in one pass where it applies)",
                                        True: "row kernel of layer 1 beside the GEMM of layer 2 (two streams)",
                                        False: "kernels one after the other"}[BlockRunner.overlap]}
 

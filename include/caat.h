@@ -525,7 +525,7 @@ typedef enum {
   CAAT_K_GEMM_CUDA_CORE = 3, /* CUDA-core GEMM (fp32 and unaligned shapes)          */
   CAAT_K_TC_FORWARD = 4,     /* tcgen05 GEMM, forward                               */
   CAAT_K_TC_DGRAD = 5,       /* tcgen05 GEMM, data gradient                         */
-  CAAT_K_TC_WGRAD = 6,       /* tcgen05 GEMM, weight gradient                       */
+  CAAT_K_TC_WGRAD = 6,       /* tcgen05 GEMM, weight gradient (or a block's four gradient products in one launch) */
   CAAT_K_SPLITK_REDUCE = 7,  /* split-K reduction of the weight gradient            */
   CAAT_K_ACTIVATION = 8,     /* activation of the column-parallel half / its derivative */
   CAAT_K_TP_EXCHANGE = 9,    /* slab exchange over peer memory: scatter, reduce + gather, waits */
