@@ -86,7 +86,7 @@ struct Region {          // a family of output tiles with the same operand wirin
   int out_f32;
   int b_slowest;         // tile order: 1 = rank index slowest (a rank's weights / activations stay
                          // hot in L2 while its row tiles stream), 0 = row tile slowest
-  float scale;           // outputs are multiplied by it in the epilogue (0 means 1)
+  float scale = 1.f;     // outputs are multiplied by it in the epilogue
   int a_mn;              // MIXED launches: as Params::a_mn, per region
 };
 
@@ -652,7 +652,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
         const bool out_f32 = r.out_f32 != 0;
         const int sub = out_f32 ? 32 : 64;
         const int cols = (p.debug & kAidMask & 2) ? 0 : (r.N - n0 < p.BN ? r.N - n0 : p.BN);
-        const bool scaled = r.scale != 0.f && r.scale != 1.f;
+        const bool scaled = r.scale != 1.f;
         if (cols <= 0) release();
         for (int cc = 0; cc < cols; cc += sub) {
           uint32_t v[32], w[32];

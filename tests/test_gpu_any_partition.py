@@ -27,6 +27,11 @@ pytestmark = pytest.mark.gpu
     (4, 5, 768, 3072, caat.CAAT_ATTN_OUT, 3, None, 1),
     (8, 64, 1024, 4096, caat.CAAT_MLP_DOWN, 1017, None, 0),     # many rows: CTA per row / two CTAs per SM
     (3, 33, 264, 792, caat.CAAT_ATTN_OUT, 259, 0.5, 1),         # fewer than 8 private channels
+    (8, 300, 2048, 5632, caat.CAAT_MLP_DOWN, 1433, 0.0, 0),     # private scale 0: no gradient reaches the private rows
+    (8, 300, 2048, 5632, caat.CAAT_MLP_DOWN, 1432, 0.0, 0),     # the same on the grid
+    (2, 3000, 256, 1024, caat.CAAT_ATTN_OUT, 131, 0.0, 1),      # the same through split-K partials
+    (4, 257, 768, 3072, caat.CAAT_ATTN_OUT, 381, -1.5, 0),      # a negative scale, on the epilogues
+    (4, 257, 768, 3072, caat.CAAT_ATTN_OUT, 384, -4096.0, 0),   # the same on the scaled weights
 ])
 def test_layer_with_a_partition_off_the_grid(t, T, h, ffn, layer, S, alpha, norm):
     ctx = G.make_ctx(t, h, ffn, "bf16", S=S, alpha=alpha, norm=norm)

@@ -62,6 +62,17 @@ def _run(ctx, d, sv, T, compact, S, norm, dh):
 @pytest.mark.parametrize("compact", [False, True])
 @pytest.mark.parametrize("t,T,h,ffn,S,norm,dh", CASES)
 def test_block_backward_rows_in_one_pass(t, T, h, ffn, S, norm, dh, compact):
+    _check(t, T, h, ffn, S, norm, dh, compact)
+
+
+@pytest.mark.parametrize("compact", [False, True])
+@pytest.mark.parametrize("S", [1024, 1003])
+@pytest.mark.parametrize("alpha", [0.0, -1.5])
+def test_block_backward_at_any_private_scale(alpha, S, compact):
+    _check(8, 300, 2048, 5632, S, 0, True, compact, alpha)      # the four gradient products in one launch
+
+
+def _check(t, T, h, ffn, S, norm, dh, compact, alpha=None):
     if compact:
         S = S // 8 * 8
     w = synthetic.Workload("blk", t, T, h, ffn, S / h, "bf16", "block", True, T + S)
@@ -79,7 +90,7 @@ def test_block_backward_rows_in_one_pass(t, T, h, ffn, S, norm, dh, compact):
         mean = x.mean(2) if norm else 0 * x.mean(2)
         sv["mean" + l] = torch.from_numpy(mean).float() if norm else None
         sv["rstd" + l] = torch.from_numpy(((x - mean[:, :, None]) ** 2).mean(2) ** -0.5).float()
-    ctx = G.make_ctx(t, h, ffn, "bf16", S=S, norm=norm)
+    ctx = G.make_ctx(t, h, ffn, "bf16", S=S, norm=norm, alpha=alpha)
     before = caat.kernel_launches()
     one = _run(ctx, d, sv, T, compact, S, norm, dh)
     mid = caat.kernel_launches()
