@@ -259,9 +259,11 @@ static SideStream* side_stream_locked() {
 
 // ---- backward of one layer -----------------------------------------------------
 // alpha of the private gradient: on the epilogues when the shared gradient may be stored divided by it (one scaling of
-// the weights' private rows less: 9 + 7 us of a 193 us step at 600 tokens of 8 x 2048), else on the weights
+// the weights' private rows less: 9 + 7 us of a 193 us step at 600 tokens of 8 x 2048), else on the weights.  The
+// numerics-study modes round the sum themselves: divided and rounded once more it would not be the sum they model.
 static bool alpha_on_epilogues(const caat_ctx* ctx, int compact) {
-  return !compact && ctx->S < ctx->h && ctx->alpha != 1.0 && std::fabs(ctx->alpha) >= 0x1p-10 && std::fabs(ctx->alpha) <= 0x1p10;
+  return !compact && ctx->bwd_reduce == 0 && ctx->S < ctx->h && ctx->alpha != 1.0 && std::fabs(ctx->alpha) >= 0x1p-10 &&
+         std::fabs(ctx->alpha) <= 0x1p10;
 }
 
 static PrivOperand priv_operand(const caat_ctx* ctx, const Scratch& L, const void* dR, int compact, bool over_alpha) {

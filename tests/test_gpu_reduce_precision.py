@@ -36,6 +36,46 @@ def test_reduce_modes_match_their_model(mode, t):
         assert_close(gb[k], ob[k], "bf16", k)
 
 
+@pytest.mark.parametrize("block", [False, True])
+@pytest.mark.parametrize("mode", [1, 2])
+@pytest.mark.parametrize("t,S", [(8, 256), (2, 131)])      # private scales that are no power of two
+def test_rounded_sums_reach_the_weight_gradient_unchanged(t, S, mode, block):
+    """Y holds a single 1 per rank, so dW's shared rows in that column ARE the sum of that token as the products see it:
+    the ranks' rounded terms (dR as stored) added in fp32 and rounded once, or rounded after every addition."""
+    (_, h, ffn), _, d = _case(t, T=96, seed=t)
+    ctx = G.make_ctx(t, h, ffn, "bf16", S=S, bwd_reduce=mode)
+    Hn, rstd, mean = G.saved_from_oracle(ctx, G.oracle_forward(ctx, d))
+    tok, col = 37, 5
+    d["Y"] = torch.zeros_like(d["Y"])
+    d["Y"][:, tok, col] = 1.0
+    if block:
+        dev = {k: v.cuda() for k, v in d.items() if isinstance(v, torch.Tensor)}
+        T, K = 96, h // t
+        km = ctx.k_r(caat.CAAT_MLP_DOWN)
+        mk = lambda *s, dt=torch.bfloat16: torch.zeros(*s, dtype=dt, device="cuda")
+        f32 = torch.float32
+        dW, dR, dHn1 = mk(t, h, K, dt=f32), mk(t, T, h), mk(t, T, h)
+        H, r = Hn.cuda(), rstd.cuda()
+        ws = ctx.alloc_workspace(ctx.block_workspace_bytes(T, True))
+        ctx.block_backward(T, dev["dX"], dev["dX"], dev["dHn"], dev["Y"], dev["W"], mk(t, T, km), mk(t, h, km), H, r, None, H, r,
+                           None, dev["gamma"], dev["gamma"], mk(t, T, K), dW, mk(t, T, km), mk(t, h, km, dt=f32), dR, dHn1,
+                           mk(h, dt=f32), None, mk(h, dt=f32), None, ws)
+        torch.cuda.synchronize()
+        assert ctx.last_device_status() == caat.CAAT_OK
+        gb = {"dW": dW.cpu(), "dR": dR.cpu()}
+    else:
+        gb = G.gpu_backward(ctx, caat.CAAT_ATTN_OUT, d, Hn, rstd, mean)
+    terms = gb["dR"][:, tok, :S].float()
+    acc = torch.zeros(S)
+    for m in range(t):
+        acc = acc + terms[m]
+        if mode == 2:
+            acc = acc.bfloat16().float()
+    want = acc.bfloat16().float()
+    for m in range(t):
+        assert torch.equal(gb["dW"][m, :S, col], want), m
+
+
 def test_fp32_accumulation_beats_16_bit_sums_and_the_gap_grows_with_ranks():
     rows = []
     for t in (2, 4, 8, 16, 32):
