@@ -387,6 +387,8 @@ __global__ void __launch_bounds__(512, CPT == 1 ? 2 : 1) rows_backward_kernel(co
 // of ranks or a part of one rank's contraction), zp [np][t][T][h - S_lo] of the private ones; planes are added in
 // ascending order.  Every rank's CTA forms the shared sum for itself (L2 hits), so no CTA waits for another.  With two
 // layers the second one's residual is the first one's new residual stream as stored (rounded to the storage type).
+// With one CTA per token (gridDim.y == 1) it works the ranks from the last to the first: a compact stream updated in place
+// is stored by rank 0's turn, after every other rank has read the chunk, by the same thread.
 template <typename T_, bool LN>
 __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPartArgs a) {
   using V_ = VT<T_>;
@@ -398,12 +400,13 @@ __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPar
   float* hrow = sm;                       // [h] the new residual stream of this row, fp32
   float* red = sm + a.h;                  // reduction scratch
   int par = 0;
-  const int i = blockIdx.x, m = blockIdx.y;
-  const long long row = (long long)m * a.T + i;
+  const int i = blockIdx.x;
   const int S_lo = a.S / V * V, S_hi = (a.S + V - 1) / V * V, P = a.h - S_lo;
   const float inv_h = 1.0f / (float)a.h;
+  for (int m = a.t - 1 - (int)blockIdx.y; m >= 0; m -= (int)gridDim.y)
   for (int layer = 0; layer < a.nlayers; ++layer) {
     const PartialLayer& L = a.L[layer];
+    const long long row = (long long)m * a.T + i;
     float st[1] = {0.f};
     for (int c = threadIdx.x * V; c < a.h; c += blockDim.x * V) {
       float r[V], z[V], hn[V];
@@ -820,7 +823,11 @@ cudaError_t launch_rows_forward_partials(const RowPartArgs& a, caat_dtype dtype,
   int threads = round_up(a.h / V, 32);               // one chunk per thread when the row allows
   if (threads > 512) threads = 512;
   if (threads < 32) threads = 32;
-  const dim3 grid(a.T, a.t);
+  // A compact stream updated in place: rank 0 stores the shared row that the other ranks read as their residual.  The
+  // CTAs of a cluster have all read it before their barrier; without clusters one CTA works all ranks of a token.
+  bool in_place = false;
+  for (int l = 0; l < a.nlayers; ++l) in_place = in_place || (a.compact && a.Rs && a.Rs == a.L[l].Hns);
+  const dim3 grid(a.T, in_place ? 1 : a.t);
   const size_t smem = (size_t)a.h * sizeof(float) + 2 * 16 * 2 * sizeof(float);
   LaunchScope scope(CAAT_K_ROWS_FORWARD, st);
   // few rows: the cluster kernel, as long as all its CTAs are resident at once (portable cluster size 8,
@@ -834,7 +841,8 @@ cudaError_t launch_rows_forward_partials(const RowPartArgs& a, caat_dtype dtype,
     const size_t csm = cluster_partials_smem(a);
     bool launched = false;
     cudaError_t e = cudaSuccess;
-    if (csm <= 200 * 1024 && (long long)a.T * a.t <= (long long)sm_count() * 3 / 4) {
+    const bool two_per_sm = a.norm != 1 && csm <= 100 * 1024;
+    if (csm <= 200 * 1024 && ((long long)a.T * a.t <= (long long)sm_count() * 3 / 4 || (in_place && !two_per_sm))) {
       e = a.norm == 1 ? launch_partials_cluster<__nv_bfloat16, true, 1>(a, threads, csm, st, &launched)
                       : launch_partials_cluster<__nv_bfloat16, false, 1>(a, threads, csm, st, &launched);
       if (launched || e != cudaSuccess) return e;
@@ -842,15 +850,14 @@ cudaError_t launch_rows_forward_partials(const RowPartArgs& a, caat_dtype dtype,
     // more rows than that: two CTAs per SM (64 registers, RMSNorm variant), a few waves.  Pays when most
     // channels are shared, where the kernel below reads every shared plane once per rank (measured at
     // 64 tokens of the 7B shapes: 3 % faster at p = 1, 5 % slower at p = 0.5).
-    if (a.norm != 1 && csm <= 100 * 1024 && (long long)a.S * 4 > (long long)a.h * 3 &&
-        (long long)a.T * a.t <= (long long)sm_count() * 4) {
+    if (two_per_sm && (in_place || ((long long)a.S * 4 > (long long)a.h * 3 && (long long)a.T * a.t <= (long long)sm_count() * 4))) {
       e = launch_partials_cluster<__nv_bfloat16, false, 2>(a, threads, csm, st, &launched);
       if (launched || e != cudaSuccess) return e;
     }
   }
   // more rows than two CTAs of 512 threads per SM can hold at once (64 registers per thread): two chunks per thread in
   // CTAs of 256, four of which fit an SM, keep every row's CTA resident in one wave (7B shapes, 64 tokens: -3.6 %)
-  if (threads > 256 && (long long)a.T * a.t > 2LL * sm_count()) threads = 256;
+  if (threads > 256 && (long long)grid.x * grid.y > 2LL * sm_count()) threads = 256;
   auto go = [&](auto kernel) -> cudaError_t {
     if (smem > 48 * 1024) {   // long rows: more dynamic shared memory than a kernel gets without asking
       const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

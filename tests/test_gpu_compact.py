@@ -208,3 +208,50 @@ def test_compact_block_few_tokens(no_decode, T, t, h, ffn, S):
         g.check(k)
         if fo[k].size:
             assert_close(g.view.cpu(), fo[k], "bf16", k)
+
+
+@pytest.mark.parametrize("t,T,h,ffn,S,norm", [
+    (8, 61, 1024, 4096, 512, 0),      # more rows than one wave of clusters
+    (8, 61, 1024, 4096, 512, 1),      # the same with LayerNorm
+    (8, 64, 4096, 11008, 4096, 0),    # everything shared: the widest staging area of a cluster
+    (2, 3, 1024, 4096, 512, 0),       # one wave of clusters
+    (16, 64, 512, 2048, 256, 0),      # more ranks than a cluster holds: a CTA per token
+    (16, 5, 512, 2048, 256, 1),
+    (4, 40, 8192, 8192, 4096, 0),     # rows too long for the cluster kernel
+    (1, 30, 512, 2048, 256, 0),       # one rank
+])
+def test_few_tokens_in_place_on_the_compact_stream(t, T, h, ffn, S, norm):
+    w = synthetic.Workload("in_place", t, T, h, ffn, S / h, "bf16", "block", False, T)
+    d = {k: v.cuda() for k, v in synthetic.block_inputs(w, S).items()}
+    ctx = G.make_ctx(t, h, ffn, "bf16", S=S, norm=norm)
+    ws = ctx.alloc_workspace(ctx.block_workspace_bytes(T, False))
+    mk = lambda *s, dt=torch.bfloat16: torch.zeros(*s, dtype=dt, device="cuda")
+    R0s, R0p = d["R0"][0, :, :S].contiguous(), d["R0"][:, :, S:].contiguous()
+    stat = lambda: mk(t, T, dt=torch.float32)
+
+    def layer(in_place):
+        rs, rp = R0s.clone(), R0p.clone()
+        hs, hp = (rs, rp) if in_place else (mk(T, S), mk(t, T, h - S))
+        X, r, m = mk(t, T, h), stat(), stat() if norm else None
+        ctx.rowpar_forward_compact(caat.CAAT_MLP_DOWN, T, d["Y_mlp"], d["W_down"], rs, rp, d["gamma1"], None, hs, hp, X, r, m, ws)
+        return {"Hns": hs, "Hnp": hp, "X": X, "rstd": r}
+
+    def block(first, second):      # which layers' new streams go over the residual
+        rs, rp = R0s.clone(), R0p.clone()
+        h1 = (rs, rp) if first else (mk(T, S), mk(t, T, h - S))
+        h2 = (rs, rp) if second else (mk(T, S), mk(t, T, h - S))
+        X1, X2, r1, r2 = mk(t, T, h), mk(t, T, h), stat(), stat()
+        m1, m2 = (stat(), stat()) if norm else (None, None)
+        ctx.block_forward_compact(T, d["Y_attn"], d["W_o"], d["Y_mlp"], d["W_down"], rs, rp, d["gamma1"], None, d["gamma2"], None,
+                                  *h1, X1, r1, m1, *h2, X2, r2, m2, ws)
+        out = {"Hn2s": h2[0], "Hn2p": h2[1], "X1": X1, "rstd1": r1, "X2": X2, "rstd2": r2}
+        return out if first and second else dict(out, Hn1s=h1[0], Hn1p=h1[1])
+
+    for want, got in [(layer(False), layer(True))] + [(block(False, False), block(a, b)) for a, b in ((1, 0), (0, 1), (1, 1))]:
+        torch.cuda.synchronize()
+        assert ctx.last_device_status() == caat.CAAT_OK
+        for k in got:
+            if k.startswith("Hn"):      # the same sums, rounded once, in the same order
+                assert torch.equal(got[k], want[k]), k
+            else:                       # the row statistics may be summed in another order
+                assert_close(got[k], f64(want[k]), "bf16", k, scale=0.5)
