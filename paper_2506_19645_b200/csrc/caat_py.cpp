@@ -6,9 +6,9 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
-#include <exception>
 #include <initializer_list>
 
 #include "caat.h"
@@ -26,7 +26,7 @@ PyObject* g_explain = nullptr;      // explain(tensor, dtype code, shape, name):
 void free_dims(PyObject* cap) { delete static_cast<Dims*>(PyCapsule_GetPointer(cap, kDimsName)); }
 
 // dims(ctx address, dtype code, t, h, K_r of attention-out, K_r of MLP-down) -> capsule
-PyObject* make_dims(PyObject*, PyObject* const* a, Py_ssize_t n) {
+PyObject* dims(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (n != 6) { PyErr_SetString(PyExc_TypeError, "dims: six arguments"); return nullptr; }
   const unsigned long long p = PyLong_AsUnsignedLongLong(a[0]);
   long long v[5];
@@ -118,13 +118,7 @@ template <typename F>
 PyObject* call(Args& g, F f) {
   if (!g.ok) return nullptr;
   caat_status s;
-  void* st;
-  try {
-    st = c10::cuda::getCurrentCUDAStream().stream();
-  } catch (const std::exception& e) {      // no device
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
-  }
+  void* st = c10::cuda::getCurrentCUDAStream().stream();
   Py_BEGIN_ALLOW_THREADS
   s = f(st);
   Py_END_ALLOW_THREADS
@@ -288,11 +282,21 @@ CAAT_FN(colpar_backward) {
   });
 }
 
-#define CAAT_DEF(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
+// The entry of every call: a tensor's methods throw for a tensor without storage (inside vmap), a sparse one, a machine
+// without a device.  C++ exceptions must not leave through Python's C frames; torch's own translation raises what the same
+// method raises in Python.
+using Fn = PyObject* (*)(PyObject*, PyObject* const*, Py_ssize_t);
+template <Fn F>
+PyObject* entry(PyObject* self, PyObject* const* args, Py_ssize_t nargs) {
+  HANDLE_TH_ERRORS
+  return F(self, args, nargs);
+  END_HANDLE_TH_ERRORS
+}
+
+#define CAAT_DEF(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(entry<name>)), METH_FASTCALL, nullptr}
 PyMethodDef kMethods[] = {
-    {"dims", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(make_dims)), METH_FASTCALL, nullptr},
     {"set_explain", set_explain, METH_O, nullptr},
-    CAAT_DEF(rowpar_forward), CAAT_DEF(rowpar_forward_noalloc), CAAT_DEF(rowpar_backward), CAAT_DEF(block_forward),
+    CAAT_DEF(dims), CAAT_DEF(rowpar_forward), CAAT_DEF(rowpar_forward_noalloc), CAAT_DEF(rowpar_backward), CAAT_DEF(block_forward),
     CAAT_DEF(block_backward), CAAT_DEF(block_forward_compact), CAAT_DEF(block_backward_compact), CAAT_DEF(colpar_forward),
     CAAT_DEF(colpar_backward), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_caatpy", "Argument marshalling of the hot calls", -1, kMethods, nullptr, nullptr,
