@@ -1158,70 +1158,110 @@ struct FewPlan { FewSplit l[2]; Deal deal; int workers; };
 constexpr double kItemOverhead = 1.5;     // of a tile, in k-steps: refill of the pipeline and the epilogue
 constexpr double kStepUs = 0.38;          // a k-step of 16 KB of weights on one of 148 SMs at 6.4 TB/s
 
-struct FewItem { float len; uint16_t tile; };
+// The tiles of a plan by their length: at most full, last and empty ones of the shared and of the private part of either layer.
+// first, step, run: the tiles first + i * step + j, j < run, in the kernel's numbering (decode_tile with one column tile:
+// region, then split fastest, then mt, then b).
+struct FewRun { float len; int first, step, run, n; };
+struct FewTiles { int nruns, tiles; FewRun r[12]; };
 
-// tiles in the kernel's numbering (decode_tile with one column tile): region, then split fastest, then mt, then b
-int few_items(int t, int h, int S, const int* K_r, int n, const FewSplit* sp, FewItem* out) {
+FewTiles few_tiles(int t, int h, int S, const int* K_r, int n, const FewSplit* sp) {
+  FewTiles f{};
   const int S_lo = round_down(S, kLayoutVec);
-  int cnt = 0;
   for (int g = 0; g < n; ++g) {
     const int ks = (K_r[g] + BK - 1) / BK;
     for (int part = 0; part < 2; ++part) {
       const int M = part == 0 ? S : (S < h ? h - S_lo : 0);
       if (M <= 0) continue;
-      const int mt = (M + BM - 1) / BM;
       const bool grouped = part == 0 && sp[g].qper > 0;
-      const int splits = part == 0 ? (grouped ? (t + sp[g].qper - 1) / sp[g].qper : sp[g].ksplits) : sp[g].ksplits;
-      const int batch = grouped ? 1 : t, per = (ks + splits - 1) / splits;
-      for (int b = 0; b < batch * mt; ++b)
-        for (int k = 0; k < splits; ++k) {
-          int len;
-          if (grouped) len = ks * ((k + 1) * sp[g].qper <= t ? sp[g].qper : t - k * sp[g].qper);
-          else len = per * (k + 1) <= ks ? per : (ks > per * k ? ks - per * k : 0);
-          if (cnt == kMaxDealItems) return -1;
-          out[cnt] = FewItem{(float)(len + kItemOverhead), (uint16_t)cnt};
-          ++cnt;
-        }
+      const int splits = grouped ? (t + sp[g].qper - 1) / sp[g].qper : sp[g].ksplits;
+      const int outer = (M + BM - 1) / BM * (grouped ? 1 : t);
+      // a split is `per` pieces of `unit` k-steps long; the last one may be shorter, and those of a k-split past it are empty
+      const int pieces = grouped ? t : ks, unit = grouped ? ks : 1, per = grouped ? sp[g].qper : (ks + splits - 1) / splits;
+      const int full = pieces / per, rest = pieces - full * per, used = full + (rest > 0);
+      auto add = [&](int split, int count, int length) {
+        if (count > 0) f.r[f.nruns++] = FewRun{(float)(length * unit + kItemOverhead), f.tiles + split, splits, count, outer};
+      };
+      add(0, full, per);
+      add(full, used - full, rest);
+      add(used, splits - used, 0);
+      f.tiles += outer * splits;
     }
   }
-  return cnt;
+  std::sort(f.r, f.r + f.nruns, [](const FewRun& x, const FewRun& y) { return x.len > y.len || (x.len == y.len && x.first < y.first); });
+  return f;
 }
 
-// longest first, each to the least loaded worker; returns the busiest worker's load, fills `deal` when given
-double few_deal(FewItem* it, int n, int workers, Deal* deal) {
-  std::sort(it, it + n, [](const FewItem& a, const FewItem& b) { return a.len > b.len || (a.len == b.len && a.tile < b.tile); });
-  std::pair<float, int> load[kMaxDealWorkers];
-  for (int w = 0; w < workers; ++w) load[w] = {0.f, w};
-  auto more = [](const std::pair<float, int>& a, const std::pair<float, int>& b) { return a > b; };
-  static thread_local uint8_t owner[kMaxDealItems];
-  std::make_heap(load, load + workers, more);
-  float worst = 0.f;
-  for (int i = 0; i < n; ++i) {
-    std::pop_heap(load, load + workers, more);
-    auto& l = load[workers - 1];
-    l.first += it[i].len;
-    worst = l.first > worst ? l.first : worst;
-    owner[i] = (uint8_t)l.second;
-    std::push_heap(load, load + workers, more);
-  }
-  if (deal) {
-    int pos = 0;
-    for (int w = 0; w < workers; ++w) {
-      deal->first[w] = (uint16_t)pos;
-      for (int i = 0; i < n; ++i)
-        if (owner[i] == w) deal->item[pos++] = it[i].tile;
+// Longest first, each to the least loaded worker: the busiest worker's load.  Workers of equal load are one group and take
+// their next tiles together, so a deal costs a few dozen steps however many tiles there are.
+double few_makespan(const FewTiles& f, int workers) {
+  struct Group { float load; int count; } g[kMaxDealWorkers];
+  int ng = 1;
+  g[0] = Group{0.f, workers};
+  for (int i = 0; i < f.nruns; ++i)
+    for (int left = f.r[i].n * f.r[i].run; left > 0;) {
+      const int take = left < g[0].count ? left : g[0].count;
+      const float load = g[0].load + f.r[i].len;
+      left -= take;
+      int at = 0;
+      if ((g[0].count -= take) == 0) {           // the group is gone: the others move down past its new place
+        for (; at + 1 < ng && g[at + 1].load < load; ++at) g[at] = g[at + 1];
+        if (at + 1 < ng && g[at + 1].load == load) {
+          g[at] = g[at + 1];
+          g[at].count += take;
+          for (int k = at + 1; k + 1 < ng; ++k) g[k] = g[k + 1];
+          --ng;
+        } else {
+          g[at] = Group{load, take};
+        }
+      } else {
+        for (at = 1; at < ng && g[at].load < load;) ++at;
+        if (at < ng && g[at].load == load) {
+          g[at].count += take;
+        } else {
+          for (int k = ng++; k > at; --k) g[k] = g[k - 1];
+          g[at] = Group{load, take};
+        }
+      }
     }
-    deal->first[workers] = (uint16_t)pos;
-    deal->dealt = 1;
+  return g[ng - 1].load;
+}
+
+// the same deal, tile by tile
+void few_deal(const FewTiles& f, int workers, Deal* deal) {
+  struct Worker { float load; int id; bool operator<(const Worker& o) const { return load < o.load || (load == o.load && id < o.id); } };
+  Worker w[kMaxDealWorkers], merged[kMaxDealWorkers];       // ascending
+  uint16_t tile[kMaxDealItems];          // longest first
+  uint8_t owner[kMaxDealItems];
+  int count[kMaxDealWorkers] = {};
+  for (int i = 0; i < workers; ++i) w[i] = Worker{0.f, i};
+  int n = 0;
+  for (int i = 0; i < f.nruns; ++i) {
+    const int begin = n;
+    for (int o = 0; o < f.r[i].n; ++o)
+      for (int k = 0; k < f.r[i].run; ++k) tile[n++] = (uint16_t)(f.r[i].first + o * f.r[i].step + k);
+    for (int j = begin; j < n;) {
+      int take = 1;
+      while (take < workers && take < n - j && w[take].load == w[0].load) ++take;
+      for (int k = 0; k < take; ++k) {
+        owner[j++] = (uint8_t)w[k].id;
+        ++count[w[k].id];
+        w[k].load += f.r[i].len;
+      }
+      std::merge(w, w + take, w + take, w + workers, merged);
+      std::copy(merged, merged + workers, w);
+    }
   }
-  return worst;
+  int at[kMaxDealWorkers], pos = 0;
+  for (int i = 0; i < workers; ++i) { deal->first[i] = (uint16_t)pos; at[i] = pos; pos += count[i]; }
+  deal->first[workers] = (uint16_t)pos;
+  for (int j = 0; j < n; ++j) deal->item[at[owner[j]]++] = tile[j];
+  deal->dealt = 1;
 }
 
 // Chooses the splits of one or two layers.  The row kernel's share: a plane of the shared part is written once and read
 // by every rank's CTA (once per token when the ranks share it through a cluster), a private plane is read once.
 void few_token_plan(int t, int T, int h, int S, const int* K_r, int n, int sms, FewPlan* best) {
   const int workers = sms < kMaxDealWorkers ? sms : kMaxDealWorkers;
-  static thread_local FewItem items[kMaxDealItems];
   double best_cost = -1;
   const bool clustered = (long long)T * t <= (long long)sms * 3 / 4;
   FewSplit cand[2][16];
@@ -1256,37 +1296,54 @@ void few_token_plan(int t, int T, int h, int S, const int* K_r, int n, int sms, 
     }
   std::sort(all, all + na, [](const Cand& a, const Cand& b) { return a.bound < b.bound; });
   for (int i = 0; i < na && (best_cost < 0 || all[i].bound < best_cost); ++i) {
-    const int cnt = few_items(t, h, S, K_r, n, all[i].l, items);
-    if (cnt <= 0) continue;
-    const double cost = few_deal(items, cnt, workers, nullptr) * kStepUs + all[i].rest;
+    const FewTiles f = few_tiles(t, h, S, K_r, n, all[i].l);
+    if (f.tiles > kMaxDealItems) continue;
+    const double cost = few_makespan(f, workers) * kStepUs + all[i].rest;
     if (best_cost < 0 || cost < best_cost) { best_cost = cost; best->l[0] = all[i].l[0]; best->l[1] = all[i].l[1]; }
   }
-  const int cnt = few_items(t, h, S, K_r, n, best->l, items);
+  const FewTiles f = few_tiles(t, h, S, K_r, n, best->l);
   best->deal.dealt = 0;
   best->workers = workers;
-  if (cnt > 0) {
-    if (cnt < workers) best->workers = cnt;
-    few_deal(items, cnt, best->workers, &best->deal);
+  if (f.tiles <= kMaxDealItems) {
+    if (f.tiles < workers) best->workers = f.tiles;
+    few_deal(f, best->workers, &best->deal);
   }
 }
 
-// The plan depends on the shapes alone; the most recent ones are kept (the oldest is replaced).
+// The plan depends on the shapes alone.  Making one takes 4 us (7B shapes, on the host of the measurements); the 64 used last
+// are kept.  Plans are made outside the lock, so that one thread's new shape holds up no other thread's call.
 struct FewKey { int t, T, h, S, K0, K1, sms; bool operator==(const FewKey& o) const { return !memcmp(this, &o, sizeof(o)); } };
 constexpr int kFewPlans = 64;
 
 void few_plan_cached(int t, int T, int h, int S, const int* K_r, int n, FewPlan* out) {
   static FewKey keys[kFewPlans];
+  static unsigned long long used[kFewPlans] = {}, clock = 0;      // used == 0: an empty slot
   static FewPlan plans[kFewPlans];
-  static int used = 0, next = 0;
   static std::mutex m;
   const FewKey key{t, T, h, S, K_r[0], n > 1 ? K_r[1] : 0, sm_count()};
+  auto find = [&] {
+    for (int i = 0; i < kFewPlans; ++i)
+      if (used[i] && keys[i] == key) return i;
+    return -1;
+  };
+  {
+    std::lock_guard<std::mutex> lock(m);
+    const int i = find();
+    if (i >= 0) {
+      used[i] = ++clock;
+      *out = plans[i];
+      return;
+    }
+  }
+  few_token_plan(t, T, h, S, K_r, n, key.sms, out);
   std::lock_guard<std::mutex> lock(m);
-  for (int i = 0; i < used; ++i)
-    if (keys[i] == key) { *out = plans[i]; return; }
-  const int slot = used < kFewPlans ? used++ : (next++ % kFewPlans);
-  few_token_plan(t, T, h, S, K_r, n, key.sms, &plans[slot]);
-  keys[slot] = key;
-  *out = plans[slot];
+  int i = find();                     // another thread may have made it meanwhile
+  if (i < 0) {
+    i = (int)(std::min_element(used, used + kFewPlans) - used);
+    keys[i] = key;
+    plans[i] = *out;
+  }
+  used[i] = ++clock;
 }
 }  // namespace
 
