@@ -3,10 +3,11 @@
 Run as ``python -m paper_2506_19645_b200.build``; cross-compiles without a GPU.  Every
 translation unit is compiled to an object file of its own with nvcc for sm_100a (in parallel, and only when
 it or a header changed), then the objects are linked into the shared library.  _caatpy.so is host code: g++ against the
-headers of the installed Python and torch, linked to libcaat.so beside it.
+headers of the installed Python and torch, linked to libcaat.so beside it, and built again when either changes version.
 """
 from __future__ import annotations
 
+import importlib.metadata
 import os
 import shlex
 import subprocess
@@ -20,6 +21,7 @@ CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "build")
 LIB = os.path.join(PKG, "libcaat.so")
 PYEXT_SRC, PYEXT = os.path.join(CSRC, "caat_py.cpp"), os.path.join(PKG, "_caatpy.so")
+PYEXT_FOR = os.path.join(OBJ, "caat_py.for")      # the Python and torch that _caatpy.so was built for
 SOURCES = ["caat_api.cu", "caat_rows.cu", "caat_rows_staged.cu", "caat_rows_lean.cu", "caat_rows_block.cu",
            "caat_rows_block_bwd.cu", "caat_rows_warp.cu", "caat_gemm_simt.cu",
            "caat_gemm_tc.cu", "caat_static.cu", "caat_colpar.cu", "caat_tp_push.cu"]
@@ -66,11 +68,25 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("nvcc failed linking libcaat.so")
-    header = os.path.join(ROOT, "include", "caat.h")
-    if force or not os.path.exists(PYEXT) or os.path.getmtime(PYEXT) < max(
-            os.path.getmtime(f) for f in (PYEXT_SRC, header, os.path.abspath(__file__))):
+    if force or not pyext_current():
         _build_pyext(nvcc)
     return LIB
+
+
+def _abi() -> str:
+    return f"python {sys.version} torch {importlib.metadata.version('torch')}"
+
+
+def pyext_current() -> bool:
+    """Whether _caatpy.so is newer than its sources and built for this Python and torch (it uses torch's C++ interface)."""
+    try:
+        with open(PYEXT_FOR) as f:
+            if f.read() != _abi():
+                return False
+        sources = (PYEXT_SRC, os.path.join(ROOT, "include", "caat.h"), os.path.abspath(__file__))
+        return os.path.getmtime(PYEXT) >= max(os.path.getmtime(f) for f in sources)
+    except OSError:
+        return False
 
 
 def _build_pyext(nvcc: str) -> None:
@@ -86,6 +102,8 @@ def _build_pyext(nvcc: str) -> None:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed on caat_py.cpp:\n{r.stdout}{r.stderr}")
+    with open(PYEXT_FOR, "w") as f:
+        f.write(_abi())
 
 
 if __name__ == "__main__":
