@@ -963,8 +963,14 @@ cudaError_t launch(const MapsT<MIXED>& maps, Params& p, int kind, cudaStream_t s
   cfg.attrs = attr;
   cfg.numAttrs = pdl_enabled() ? 2 : 1;
   LaunchScope scope(kind, st);
-  if constexpr (!MIXED)
-    if (deal) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, true, false>, maps, *deal, (const Params&)p);
+  if constexpr (!MIXED) {
+    if (deal) {
+      // a deal to more CTAs than this launch has would leave tiles out: those go round by number instead
+      static const Deal by_number{};
+      const Deal& d = deal->dealt && deal->first[workers] != p.tiles_total ? by_number : *deal;
+      return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, true, false>, maps, d, (const Params&)p);
+    }
+  }
   static const PeerMaps no_peers{};
   const PeerMaps& pm = peer_maps ? *peer_maps : no_peers;
   if (p.cg == 2) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, false, MIXED>, maps, pm, (const Params&)p);
