@@ -580,7 +580,8 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
         split_range(r, r.u[ui], c.split, q0, q1, kb, ke);
         total_k += (ke - kb) * (q1 - q0);
       }
-      if (!mbar_wait(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) { ok = false; break; }
+      // one verdict for the warp: the tensor-memory loads below are instructions of all its lanes
+      if (!mbar_wait_warp(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) { ok = false; break; }
       tc_fence_after();
       // Every warp drains its 32 rows by itself in slabs of 128 bytes: TMEM -> registers -> swizzled staging buffer ->
       // TMA store (whole 128-byte lines; rows and columns outside the region's extents are clipped by the tensor map).
