@@ -29,7 +29,8 @@ CASES = [
 ]
 
 
-def _run(ctx, d, sv, T, compact, S, norm, dh):
+def _run(ctx, d, sv, T, compact, S, norm, dh, in_place=()):
+    """in_place: "dHn1" puts the second layer's residual gradient over the stream gradient, "dR0" the first one's over that."""
     t, h = ctx.t, ctx.h
     dev = {k: v.cuda() for k, v in d.items()}
     f32 = torch.float32
@@ -44,12 +45,20 @@ def _run(ctx, d, sv, T, compact, S, norm, dh):
     if compact:
         o.update(dR0s=mk(T, S), dR0p=mk(t, T, h - S), dHn1s=mk(T, S), dHn1p=mk(t, T, h - S))
         dHs, dHp = part(d["dHn2"]) if dh else (None, None)
+        if "dHn1" in in_place:
+            o["dHn1s"], o["dHn1p"] = dHs, dHp
+        if "dR0" in in_place:
+            o["dR0s"], o["dR0p"] = o["dHn1s"], o["dHn1p"]
         ctx.block_backward_compact(T, dev["dX1"], dev["dX2"], dHs, dHp, dev["Y_attn"], dev["W_o"], dev["Y_mlp"], dev["W_down"],
                                    *part(sv["Hn1"]), r1, m1, *part(sv["Hn2"]), r2, m2, dev["gamma1"], dev["gamma2"], o["dY_attn"],
                                    o["dW_o"], o["dY_mlp"], o["dW_down"], o["dR0s"], o["dR0p"], o["dHn1s"], o["dHn1p"], o["dgamma1"],
                                    o["dbeta1"], o["dgamma2"], o["dbeta2"], ws)
     else:
         o.update(dR0=mk(t, T, h), dHn1=mk(t, T, h))
+        if "dHn1" in in_place:
+            o["dHn1"] = dev["dHn2"]
+        if "dR0" in in_place:
+            o["dR0"] = o["dHn1"]
         ctx.block_backward(T, dev["dX1"], dev["dX2"], dev["dHn2"] if dh else None, dev["Y_attn"], dev["W_o"], dev["Y_mlp"],
                            dev["W_down"], sv["Hn1"].cuda(), r1, m1, sv["Hn2"].cuda(), r2, m2, dev["gamma1"], dev["gamma2"],
                            o["dY_attn"], o["dW_o"], o["dY_mlp"], o["dW_down"], o["dR0"], o["dHn1"], o["dgamma1"], o["dbeta1"],
@@ -72,9 +81,7 @@ def test_block_backward_at_any_private_scale(alpha, S, compact):
     _check(8, 300, 2048, 5632, S, 0, True, compact, alpha)      # the four gradient products in one launch
 
 
-def _check(t, T, h, ffn, S, norm, dh, compact, alpha=None):
-    if compact:
-        S = S // 8 * 8
+def _inputs(t, T, h, ffn, S, norm, compact):
     w = synthetic.Workload("blk", t, T, h, ffn, S / h, "bf16", "block", True, T + S)
     d = synthetic.block_inputs(w, S)
     g = torch.Generator().manual_seed(5)
@@ -90,6 +97,32 @@ def _check(t, T, h, ffn, S, norm, dh, compact, alpha=None):
         mean = x.mean(2) if norm else 0 * x.mean(2)
         sv["mean" + l] = torch.from_numpy(mean).float() if norm else None
         sv["rstd" + l] = torch.from_numpy(((x - mean[:, :, None]) ** 2).mean(2) ** -0.5).float()
+    return d, sv
+
+
+@pytest.mark.parametrize("compact", [False, True])
+@pytest.mark.parametrize("t,T,h,ffn,S,norm", [(8, 300, 2048, 5632, 1024, 0), (2, 2050, 512, 1024, 256, 0), (2, 333, 1536, 3072, 1536, 1),
+                                              (4, 701, 1024, 4096, 0, 0)])
+def test_block_backward_in_place(t, T, h, ffn, S, norm, compact):
+    d, sv = _inputs(t, T, h, ffn, S, norm, compact)
+    ctx = G.make_ctx(t, h, ffn, "bf16", S=S, norm=norm)
+    run = lambda *where: _run(ctx, d, sv, T, compact, S, norm, True, where)
+    want, got = run(), run("dHn1")                # every element of the stream gradient is read before its place is written
+    for k in want:
+        assert torch.equal(want[k], got[k]), k
+    chained = run("dR0"), run("dHn1", "dR0")      # these take the layers one after the other
+    ctx.set_option(caat.CAAT_OPT_BLOCK_OVERLAP, 0)
+    want = run()
+    for got in chained:
+        for k in want:
+            if not k.startswith("dHn1"):          # overwritten by dR0
+                assert torch.equal(want[k], got[k]), k
+
+
+def _check(t, T, h, ffn, S, norm, dh, compact, alpha=None):
+    if compact:
+        S = S // 8 * 8
+    d, sv = _inputs(t, T, h, ffn, S, norm, compact)
     ctx = G.make_ctx(t, h, ffn, "bf16", S=S, norm=norm, alpha=alpha)
     before = caat.kernel_launches()
     one = _run(ctx, d, sv, T, compact, S, norm, dh)

@@ -86,3 +86,44 @@ def test_row_kernel_waits_run_out_and_report_timeout():
     # every launch of a bulk-copy row kernel (forward, backward; three configurations) timed out and said so once
     assert line[:-1] == [caat.CAAT_ETIMEOUT, caat.CAAT_OK] * 6
     assert line[-1] == 1024
+
+
+BLOCK_CHILD = r"""
+import torch
+from paper_2506_19645_b200 import caat, synthetic
+mk = lambda *s, dt=torch.bfloat16: torch.zeros(*s, dtype=dt, device="cuda")
+f32 = torch.float32
+out = []
+# the one-pass kernels of a block, forward and backward: one chunk of a row per thread, two, a warp per token; either stream
+for h, compact in ((512, False), (2048, False), (768, False), (2048, True), (768, True)):
+    t, T, ffn = 2, 200, 2 * h
+    S = h // 2
+    ctx = caat.Context(h, ffn, t, 0.5, "bf16")
+    ka, km = ctx.k_r(caat.CAAT_ATTN_OUT), ctx.k_r(caat.CAAT_MLP_DOWN)
+    Ya, Wo, Ym, Wd, g, r = mk(t, T, ka), mk(t, h, ka), mk(t, T, km), mk(t, h, km), mk(h), mk(t, T, dt=f32)
+    full = lambda: mk(t, T, h)
+    stream = (lambda: (mk(T, S), mk(t, T, h - S))) if compact else (lambda: (full(),))
+    ws = ctx.alloc_workspace(ctx.block_workspace_bytes(T, True))
+    fwd = ctx.block_forward_compact if compact else ctx.block_forward
+    bwd = ctx.block_backward_compact if compact else ctx.block_backward
+    fwd(T, Ya, Wo, Ym, Wd, *stream(), g, None, g, None, *stream(), full(), r, None, *stream(), full(), mk(t, T, dt=f32), None, ws)
+    torch.cuda.synchronize()
+    out += [ctx.last_device_status(), ctx.last_device_status()]
+    bwd(T, full(), full(), *stream(), Ya, Wo, Ym, Wd, *stream(), r, None, *stream(), r, None, g, g, mk(t, T, ka),
+        mk(t, h, ka, dt=f32), mk(t, T, km), mk(t, h, km, dt=f32), *stream(), *stream(), mk(h, dt=f32), None, mk(h, dt=f32), None, ws)
+    torch.cuda.synchronize()
+    out += [ctx.last_device_status(), ctx.last_device_status()]
+x = torch.ones(1024, device="cuda").sum().item()   # the context still works
+print("STATUS", *out, int(x))
+"""
+
+
+def test_one_pass_block_kernels_waits_run_out_and_report_timeout():
+    from paper_2506_19645_b200 import caat
+    env = dict(os.environ, CAAT_ROWS_STALL="1", CAAT_ROWS_SPINCAP="64")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", BLOCK_CHILD], env=env, cwd=root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    line = [int(v) for v in [l for l in out.stdout.splitlines() if l.startswith("STATUS")][-1].split()[1:]]
+    assert line[:-1] == [caat.CAAT_ETIMEOUT, caat.CAAT_OK] * 10
+    assert line[-1] == 1024
