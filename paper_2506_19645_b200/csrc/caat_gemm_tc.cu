@@ -517,9 +517,22 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
       for (TileIter<SWAP> it(extra, worker, nworkers, p.tiles_total); it.valid() && ok; it.next()) {
         const TileCoord c = decode_tile(p, it.tile());
         const Region& r = p.r[c.region];
-        if (!mbar_wait_warp(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, p.spin_cap)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kAccCols);
+        uint32_t d_tmem = 0, accumulate = 0;
+        auto begin = [&]() {                        // the next free accumulator
+          if (!mbar_wait_warp(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, p.spin_cap)) return false;
+          tc_fence_after();
+          d_tmem = tmem_base + (uint32_t)(acc * kAccCols);
+          accumulate = 0;
+          return true;
+        };
+        auto finish = [&]() {                       // accumulator complete (in both CTAs)
+          if (elect_one()) {
+            if (CG == 2) umma_commit_pair(tfull0 + 8u * acc); else umma_commit(tfull0 + 8u * acc);
+          }
+          acc ^= 1;
+          if (acc == 0) acc_phase ^= 1u;
+        };
+        if (!SWAP && !begin()) { ok = false; break; }
         uint32_t idesc = idesc0 | ((uint32_t)(tile_cols(p, r, c.nt, CG) >> 3) << 17);
         if constexpr (MIXED) {
           idesc |= (uint32_t)r.a_mn << 15;
@@ -527,12 +540,12 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
           a_lo0 = (uint32_t)a_const + (tiles_sa >> 4) + (r.a_mn ? a_mn_lo : 0u);
           a_lo = a_lo0 + (uint32_t)stage * stage16;
         }
-        uint32_t accumulate = 0;
         for (int ui = 0; ui < r.nunits && ok; ++ui) {
           const Unit& u = r.u[ui];
           int q0, q1, kb, ke;
           split_range(r, u, c.split, q0, q1, kb, ke);
           for (int q = q0; q < q1 && ok; ++q) {
+            if (SWAP && !begin()) { ok = false; break; }      // an accumulator per rank, see the epilogue
             for (int kk = kb; kk < ke; ++kk) {
               if (!mbar_wait_warp(full_bar, phase, abort_flag, p.spin_cap)) { ok = false; break; }
               tc_fence_after();
@@ -554,13 +567,10 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
                 a_lo = a_lo0; b_lo = b_lo0; full_bar = full0; empty_bar = empty0;
               }
             }
+            if (SWAP && ok) finish();
           }
         }
-        if (ok && elect_one()) {                    // accumulator complete (in both CTAs)
-          if (CG == 2) umma_commit_pair(tfull0 + 8u * acc); else umma_commit(tfull0 + 8u * acc);
-        }
-        acc ^= 1;
-        if (acc == 0) acc_phase ^= 1u;
+        if (!SWAP && ok) finish();
       }
       if (!ok && lane == 0) { *abort_flag = 1; atomicExch(p.status, 2u); }
     }
@@ -574,11 +584,64 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
       const TileCoord c = decode_tile(p, it.tile());
       const Region& r = p.r[c.region];
       // a tile whose contraction range is empty leaves the accumulator undefined: its value is 0
-      int total_k = 0;
+      int total_k = 0, nq = 0;
       for (int ui = 0; ui < r.nunits; ++ui) {
         int q0, q1, kb, ke;
         split_range(r, r.u[ui], c.split, q0, q1, kb, ke);
         total_k += (ke - kb) * (q1 - q0);
+        nq += q1 - q0;
+      }
+      const int n0 = c.nt * p.BN;
+      const int m0 = c.mt * BMT + (int)rank * BM;
+      const int zc = c.split * r.batch + c.b;
+      const int rr = quarter * 32 + lane;                 // row of the tile this thread holds
+      // this warp's part of the accumulator is drained: tell the MMA issuer
+      auto release = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if (CG == 2) mbar_arrive_cluster(mapa_rank(tempty0 + 8u * acc, 0)); else mbar_arrive(tempty0 + 8u * acc);
+        }
+      };
+      if constexpr (SWAP) {
+        // swap-AB (decode): TMEM lane = output channel, column = token.  Every rank of the tile's group comes in an
+        // accumulator of its own and the ranks are added here, as the row kernel adds the planes: one accumulator over all
+        // ranks rounds every k-step's partial sum in the tensor core, which cost the row statistics a factor of three in
+        // accuracy (7B shapes, 1 and 61 tokens: 2.5e-7 against 7.0e-7 from the exact ones).
+        float sum[kDecodeMaxTokens / 32][32];
+        for (int q = 0; q < nq; ++q) {
+          if (!mbar_wait_warp(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) { ok = false; break; }
+          tc_fence_after();
+#pragma unroll
+          for (int cc = 0; cc < kDecodeMaxTokens / 32; ++cc) {
+            if (cc * 32 >= r.N) break;
+            uint32_t v[32];
+            tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + 32 * cc), v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) sum[cc][e] = q == 0 ? __uint_as_float(v[e]) : sum[cc][e] + __uint_as_float(v[e]);
+          }
+          release();
+          acc ^= 1;
+          if (acc == 0) acc_phase ^= 1u;
+        }
+        if (!ok) break;
+        // for a fixed token the 32 lanes of a warp hold 32 consecutive channels: plain 128-byte coalesced stores
+        const long long chan = (long long)m0 + rr;
+        if (chan < r.M) {
+#pragma unroll
+          for (int cc = 0; cc < kDecodeMaxTokens / 32; ++cc) {
+            const int ntok = r.N - 32 * cc;             // tokens left from this column on
+            if (ntok <= 0) break;
+            float* dst = r.out_t + ((long long)zc * r.N + 32 * cc) * r.out_ld + chan;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+              if (e < ntok) *dst = total_k == 0 ? 0.f : sum[cc][e];
+              dst += r.out_ld;
+            }
+          }
+        }
+        continue;
       }
       // one verdict for the warp: the tensor-memory loads below are instructions of all its lanes
       if (!mbar_wait_warp(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) { ok = false; break; }
@@ -588,9 +651,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
       // Two buffers per warp, no barrier across warps.  Short contractions are bound by this drain: the forward GEMM at
       // t = 8, K_r = 256, h = 2048, 8192 tokens took 79.3 us with slabs of 64 bytes x 128 rows and a barrier per slab
       // (54.5 without any epilogue), 71.5 like this; at p = 0.25 89.7 -> 78.8.
-      const int n0 = c.nt * p.BN;
-      const int m0 = c.mt * BMT + (int)rank * BM;
-      const int zc = c.split * r.batch + c.b;
+      //
       // where this tile's rows go: the region's own output, or - shared columns of a multi-GPU forward - the
       // receive slot of the GPU that owns these token rows, through its own map (row 0 = the owner's first token)
       const CUtensorMap* omap = &mp.c[c.region];
@@ -602,36 +663,8 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
           om0 = m0 - owner * p.push_slice;
         }
       }
-      const int rr = quarter * 32 + lane;                 // row of the tile this thread holds
       const uint32_t sw = (uint32_t)(lane & 7);           // 128-byte swizzle: 16-byte chunk ^= row % 8
-      // this warp's part of the accumulator is drained: tell the MMA issuer
-      auto release = [&]() {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          if (CG == 2) mbar_arrive_cluster(mapa_rank(tempty0 + 8u * acc, 0)); else mbar_arrive(tempty0 + 8u * acc);
-        }
-      };
-      if constexpr (SWAP) {
-        // swap-AB (decode): TMEM lane = output channel, column = token.  For a fixed token the 32
-        // lanes of a warp hold 32 consecutive channels: plain 128-byte coalesced stores.
-        const long long chan = (long long)m0 + rr;
-        for (int cc = 0; cc < p.BN && n0 + cc < r.N; cc += 32) {
-          uint32_t v[32];
-          tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + cc), v);
-          tmem_ld_wait();
-          if (chan < r.M) {
-            float* dst = r.out_t + ((long long)zc * r.N + n0 + cc) * r.out_ld + chan;
-            const int ntok = r.N - (n0 + cc);           // tokens left from this column on (>= 1)
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              if (e < ntok) *dst = total_k == 0 ? 0.f : __uint_as_float(v[e]);
-              dst += r.out_ld;
-            }
-          }
-        }
-        release();
-      } else if (r.skip > 0 && c.mt == 0) {
+      if (r.skip > 0 && c.mt == 0) {
         const int row = m0 + rr;
         float* dst = r.skip_out + (long long)zc * r.skip_plane + (long long)row * r.N + n0;
         for (int cc = 0; cc < p.BN && n0 + cc < r.N; cc += 16) {
@@ -1364,7 +1397,7 @@ cudaError_t launch_tc_forward_decode(int t, int T, int h, int S, DecodeProblem* 
   Maps mp;
   Params p{};
   p.BN = (T + 31) / 32 * 32;
-  if (p.BN > 256) return cudaErrorInvalidValue;
+  if (p.BN > kDecodeMaxTokens) return cudaErrorInvalidValue;
   p.cg = 1;
   p.splits = 1;
   const int S_lo = round_down(S, kLayoutVec), S_hi = round_up(S, kLayoutVec), P = h - S_lo;

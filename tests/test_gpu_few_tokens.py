@@ -27,6 +27,17 @@ def test_few_token_layer(t, T, h, ffn, layer, S):
     _check_forward(ctx, layer, d, "bf16")
 
 
+@pytest.mark.parametrize("T", [1, 61])
+def test_row_statistics_keep_the_accuracy_of_a_sum_per_rank(T):
+    """rstd is stored in fp32.  A rank's contraction is one chain of tensor-core accumulations (512 to 1376 long here); ranks are
+    added in fp32 outside of it.  Such sums leave rstd 2.5e-7 from the exact one, a single chain over all ranks 7e-7."""
+    t, h, ffn, S, layer = 8, 4096, 11008, 2048, caat.CAAT_ATTN_OUT
+    ctx = G.make_ctx(t, h, ffn, "bf16", S=S)
+    d = _layer_case(t, T, h, ctx.k_r(layer), "bf16", S, seed=T)
+    got, want = G.gpu_forward(ctx, layer, d)["rstd"].double().numpy(), G.oracle_forward(ctx, d)["rstd"]
+    assert (((got - want) ** 2).sum() / (want ** 2).sum()) ** 0.5 < 4e-7
+
+
 def test_changing_batch_sizes_cost_little_host_time():
     # a serving loop whose token count and partition change from call to call: 192 shapes, more than the library keeps plans for
     t, h, ffn, layer = 8, 4096, 11008, caat.CAAT_MLP_DOWN
