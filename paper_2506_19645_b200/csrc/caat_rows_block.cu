@@ -332,8 +332,12 @@ cudaError_t launch_t(const RowBlockArgs& a, const RowGeom& g, const BlockGeom& s
   } while (0)
   if (g.CPT == 3) CAAT_LAUNCH(3, 128);
   else if (g.CPT == 1) CAAT_LAUNCH(1, 256);
-  else if (threads <= 256) CAAT_LAUNCH(2, 256);
-  else CAAT_LAUNCH(2, 512);
+  else if constexpr (!LN) {
+    if (threads <= 256) CAAT_LAUNCH(2, 256);
+    else CAAT_LAUNCH(2, 512);
+  } else {
+    return cudaErrorInvalidValue;       // rows_block_usable leaves these to a pass per layer
+  }
 #undef CAAT_LAUNCH
   return e != cudaSuccess ? e : cudaGetLastError();
 }
