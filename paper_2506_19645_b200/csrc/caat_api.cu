@@ -120,12 +120,12 @@ Scratch scratch_layout(const caat_ctx* ctx, int K_r, int tokens, int backward) {
   if (!backward && few && tc_gemm_usable(ctx, K_r))   // two layers' planes
     off = align_up(off + 2 * decode_planes_bytes(ctx, tokens), 256);
   s.gp_off = off;
-  if (!backward && !few && !ctx->lean_scratch && ctx->S > 0 && tc_gemm_usable(ctx, K_r)) {
-    const size_t plane = (size_t)tokens * s.S_hi * sizeof(float), fit = kGroupPlanesBytes / plane;
-    if (fit >= 2) {
-      s.gp_groups = fit < (size_t)ctx->t ? (int)fit : ctx->t;
-      off = align_up(off + s.gp_groups * plane, 256);
-    }
+  if (!backward && !few && !ctx->lean_scratch && ctx->S > 0 && ctx->t > 1 && tc_gemm_usable(ctx, K_r)) {
+    // reserved for any number of tokens, also where no two planes fit: a workspace made for more tokens serves fewer
+    const size_t plane = (size_t)tokens * s.S_hi * sizeof(float), all = ctx->t * plane;
+    const size_t room = all < kGroupPlanesBytes ? all : kGroupPlanesBytes;
+    if (room / plane >= 2) s.gp_groups = (int)(room / plane);
+    off = align_up(off + room, 256);
   }
   if (backward) {
     const size_t rows = (size_t)rows_backward_partial_rows(ctx->h, tokens, ctx->dtype);
@@ -146,6 +146,16 @@ Scratch scratch_layout(const caat_ctx* ctx, int K_r, int tokens, int backward) {
   }
   s.total = off;
   return s;
+}
+
+// The context to run a forward of few tokens with.  A partition off the 8-channel grid runs without the fp32 planes where the
+// workspace has no room for them (one made for more tokens, which need none); nullptr: it is too small for that as well.
+static const caat_ctx* forward_ctx(const caat_ctx* ctx, int K_r, int tokens, size_t bytes, caat_ctx* spare) {
+  if (bytes >= scratch_layout(ctx, K_r, tokens, 0).total) return ctx;
+  if (ctx->S % kLayoutVec == 0 || tokens > kDecodeMaxTokens || ctx->no_decode) return nullptr;
+  *spare = *ctx;
+  spare->no_decode = 1;
+  return bytes >= scratch_layout(spare, K_r, tokens, 0).total ? spare : nullptr;
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -358,9 +368,12 @@ static caat_status backward_impl(const caat_ctx* ctx, int K_r, int T, const void
 // The two layers' GEMMs do not depend on each other, so both weight streams run in ONE launch, and one
 // row kernel walks both layers of a (token, rank) row.  compact: R0 / Hn1 / Hn2 are the private parts
 // [t, T, h - S] and R0s / Hn1s / Hn2s the shared part [T, S] of the stream.
-static bool block_decode_applies(const caat_ctx* ctx, int tokens) {
-  return ctx && tokens >= 1 && tokens <= kDecodeMaxTokens && !ctx->no_decode &&
-         tc_gemm_usable(ctx, layer_kr(ctx, CAAT_ATTN_OUT)) && tc_gemm_usable(ctx, layer_kr(ctx, CAAT_MLP_DOWN));
+static bool block_decode_applies(const caat_ctx* ctx, int tokens, size_t workspace_bytes) {
+  if (!ctx || tokens < 1 || tokens > kDecodeMaxTokens || ctx->no_decode || !tc_gemm_usable(ctx, layer_kr(ctx, CAAT_ATTN_OUT)) ||
+      !tc_gemm_usable(ctx, layer_kr(ctx, CAAT_MLP_DOWN)))
+    return false;
+  caat_ctx spare;                     // short of room and able to do without the planes: layer by layer
+  return forward_ctx(ctx, layer_kr(ctx, CAAT_MLP_DOWN), tokens, workspace_bytes, &spare) != &spare;
 }
 
 static caat_status block_decode(const caat_ctx* ctx, int tokens, const void* Y_attn, const void* W_o, const void* Y_mlp,
@@ -513,8 +526,10 @@ caat_status caat_rowpar_forward(const caat_ctx* ctx, caat_layer layer, int token
   for (const void* p : ptrs)
     if (p && !aligned16(p)) return CAAT_EALIGN;
   const int K_r = layer_kr(ctx, layer);
-  if (!workspace || workspace_bytes < scratch_layout(ctx, K_r, tokens, 0).total) return CAAT_EWORKSPACE;
-  return forward_impl(ctx, K_r, tokens, Y, W, R, gamma, beta, Hn, X, rstd, mean, workspace,
+  caat_ctx spare;
+  const caat_ctx* run = workspace ? forward_ctx(ctx, K_r, tokens, workspace_bytes, &spare) : nullptr;
+  if (!run) return CAAT_EWORKSPACE;
+  return forward_impl(run, K_r, tokens, Y, W, R, gamma, beta, Hn, X, rstd, mean, workspace,
                       static_cast<cudaStream_t>(cuda_stream));
 }
 
@@ -646,7 +661,7 @@ caat_status caat_block_forward(const caat_ctx* ctx, int tokens, const void* Y_at
                                float* rstd1, float* mean1, void* Hn2, void* X2, float* rstd2, float* mean2,
                                void* workspace, size_t workspace_bytes, void* cuda_stream) {
   // Two reduces per block (Appendix C): attention-out, then MLP-down on the new residual stream.
-  if (block_decode_applies(ctx, tokens))
+  if (block_decode_applies(ctx, tokens, workspace_bytes))
     return block_decode(ctx, tokens, Y_attn, W_o, Y_mlp, W_down, R0, gamma1, beta1, gamma2, beta2, Hn1, X1, rstd1, mean1,
                         Hn2, X2, rstd2, mean2, workspace, workspace_bytes, cuda_stream, 0, nullptr, nullptr, nullptr);
   if (fused_rows_apply(ctx, tokens, 0) && Y_attn && W_o && Y_mlp && W_down && R0 && gamma1 && gamma2 && Hn1 && X1 && rstd1 && Hn2 &&
@@ -857,7 +872,7 @@ caat_status caat_block_forward_compact(const caat_ctx* ctx, int tokens, const vo
                                        void* Hn1s, void* Hn1p, void* X1, float* rstd1, float* mean1, void* Hn2s,
                                        void* Hn2p, void* X2, float* rstd2, float* mean2, void* workspace,
                                        size_t workspace_bytes, void* cuda_stream) {
-  if (block_decode_applies(ctx, tokens))
+  if (block_decode_applies(ctx, tokens, workspace_bytes))
     return block_decode(ctx, tokens, Y_attn, W_o, Y_mlp, W_down, R0p, gamma1, beta1, gamma2, beta2, Hn1p, X1, rstd1, mean1,
                         Hn2p, X2, rstd2, mean2, workspace, workspace_bytes, cuda_stream, 1, R0s, Hn1s, Hn2s);
   if (fused_rows_apply(ctx, tokens, 1) && ctx->S % kLayoutVec == 0 && Y_attn && W_o && Y_mlp && W_down && gamma1 && gamma2 && X1 &&

@@ -60,6 +60,16 @@ def test_options(caat):
     assert caat.lib.caat_strerror(caat.CAAT_EWORKSPACE).decode().startswith("workspace")
 
 
+@pytest.mark.parametrize("t,h,ffn,S", [(4, 768, 3072, 384), (8, 2048, 5632, 1433), (8, 4096, 11008, 2048), (2, 1024, 4096, 512)])
+def test_a_workspace_for_more_tokens_serves_fewer(caat, t, h, ffn, S):
+    # past the few-token path, whose fp32 planes are larger than what a few hundred tokens need
+    c = caat.Context(h, ffn, t, 0.5, "bf16").set_option(caat.CAAT_OPT_SHARED_CHANNELS, S)
+    for size in (lambda T: c.workspace_bytes(caat.CAAT_MLP_DOWN, T, False), lambda T: c.workspace_bytes(caat.CAAT_ATTN_OUT, T, True),
+                 lambda T: c.block_workspace_bytes(T, False)):
+        sizes = [size(T) for T in [*range(65, 2000, 41), *range(2000, 20000, 173)]]
+        assert sizes == sorted(sizes)
+
+
 def test_workspace_and_argument_errors_before_launch(caat):
     c = caat.Context(768, 3072, 4, 0.5, "bf16")
     T = 256        # above the few-token (decode) threshold, whose forward scratch holds fp32 planes

@@ -62,3 +62,29 @@ def test_two_layer_few_token_block_with_a_partition_off_the_grid(T, S):
                          f64(d["gamma1"]), f64(d["gamma2"]), S=S, alpha=ctx.private_scale)
     for name, g in (("Hn1", Hn1), ("X1", X1), ("Hn2", Hn2), ("X2", X2), ("rstd1", rstd1), ("rstd2", rstd2)):
         assert_close(g, fo[name], "bf16", name)
+
+
+@pytest.mark.parametrize("T", [1, 64])
+def test_few_tokens_on_a_workspace_made_for_more(T):
+    # 100 tokens need less scratch than the fp32 planes of a few; such a call goes without them
+    t, h, ffn, S = 8, 2048, 5632, 1433
+    ctx = G.make_ctx(t, h, ffn, "bf16", S=S)
+    w = synthetic.Workload("blk", t, T, h, ffn, S / h, "bf16", "block", False, T)
+    d = synthetic.block_inputs(w, S)
+    dev = {k: v.cuda() for k, v in d.items()}
+    mk = lambda *s, dt=torch.bfloat16: torch.empty(*s, dtype=dt, device="cuda")
+    Hn1, X1, Hn2, X2 = (mk(t, T, h) for _ in range(4))
+    rstd1, rstd2 = mk(t, T, dt=torch.float32), mk(t, T, dt=torch.float32)
+    small = ctx.alloc_workspace(ctx.workspace_bytes(caat.CAAT_MLP_DOWN, 100, False))
+    assert T == 1 or small.numel() < ctx.workspace_bytes(caat.CAAT_MLP_DOWN, T, False)
+    fo = O.block_forward(f64(d["Y_attn"]), f64(d["W_o"]), f64(d["Y_mlp"]), f64(d["W_down"]), f64(d["R0"]),
+                         f64(d["gamma1"]), f64(d["gamma2"]), S=S, alpha=ctx.private_scale)
+    ctx.block_forward(T, dev["Y_attn"], dev["W_o"], dev["Y_mlp"], dev["W_down"], dev["R0"], dev["gamma1"], None,
+                      dev["gamma2"], None, Hn1, X1, rstd1, None, Hn2, X2, rstd2, None, small)
+    torch.cuda.synchronize()
+    for name, g in (("Hn1", Hn1), ("X1", X1), ("Hn2", Hn2), ("X2", X2)):
+        assert_close(g, fo[name], "bf16", name)
+    ctx.rowpar_forward(caat.CAAT_ATTN_OUT, T, dev["Y_attn"], dev["W_o"], dev["R0"], dev["gamma1"], None, Hn2, X2, rstd2, None, small)
+    torch.cuda.synchronize()
+    assert_close(Hn2, fo["Hn1"], "bf16", "Hn1 of the layer call")
+    assert ctx.last_device_status() == caat.CAAT_OK
