@@ -266,11 +266,12 @@ struct TileCoord {
   int region, b, mt, nt, split;
 };
 
+template <int NREGIONS>
 __device__ __forceinline__ TileCoord decode_tile(const Params& p, int tile) {
   TileCoord c;
   c.region = 0;
 #pragma unroll
-  for (int g = 0; g + 1 < kMaxRegions; ++g)
+  for (int g = 0; g + 1 < NREGIONS; ++g)
     if (tile >= p.tile_end[g]) c.region = g + 1;       // unused regions end where the last used one does: never reached
   int rem = tile - (c.region ? p.tile_end[c.region - 1] : 0);
   const Region& r = p.r[c.region];
@@ -428,7 +429,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
       long long issued = 0;
       bool ok = true;
       for (TileIter<SWAP> it(extra, worker, nworkers, p.tiles_total); it.valid() && ok; it.next()) {
-        const TileCoord c = decode_tile(p, it.tile());
+        const TileCoord c = decode_tile<MIXED ? kMaxRegions : 4>(p, it.tile());
         const Region& r = p.r[c.region];
         const uint32_t cols_cta = (uint32_t)tile_cols(p, r, c.nt, CG) / CG;    // B columns this CTA stages
         const uint32_t b_tile_bytes = cols_cta * BK * 2;
@@ -515,7 +516,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
       uint32_t a_lo = a_lo0, b_lo = b_lo0;
       uint32_t full_bar = full0, empty_bar = empty0;
       for (TileIter<SWAP> it(extra, worker, nworkers, p.tiles_total); it.valid() && ok; it.next()) {
-        const TileCoord c = decode_tile(p, it.tile());
+        const TileCoord c = decode_tile<MIXED ? kMaxRegions : 4>(p, it.tile());
         const Region& r = p.r[c.region];
         uint32_t d_tmem = 0, accumulate = 0;
         auto begin = [&]() {                        // the next free accumulator
@@ -581,7 +582,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
     uint32_t slab = 0;
     bool ok = true;
     for (TileIter<SWAP> it(extra, worker, nworkers, p.tiles_total); it.valid() && ok; it.next()) {
-      const TileCoord c = decode_tile(p, it.tile());
+      const TileCoord c = decode_tile<MIXED ? kMaxRegions : 4>(p, it.tile());
       const Region& r = p.r[c.region];
       // a tile whose contraction range is empty leaves the accumulator undefined: its value is 0
       int total_k = 0, nq = 0;
@@ -608,39 +609,58 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
         // accumulator of its own and the ranks are added here, as the row kernel adds the planes: one accumulator over all
         // ranks rounds every k-step's partial sum in the tensor core, which cost the row statistics a factor of three in
         // accuracy (7B shapes, 1 and 61 tokens: 2.5e-7 against 7.0e-7 from the exact ones).
-        float sum[kDecodeMaxTokens / 32][32];
-        for (int q = 0; q < nq; ++q) {
-          if (!mbar_wait_warp(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) { ok = false; break; }
-          tc_fence_after();
+        const long long chan = (long long)m0 + rr;
+        // for a fixed token the 32 lanes of a warp hold 32 consecutive channels: plain 128-byte coalesced stores
+        auto store = [&](int cc, const auto& value) {
+          if (chan >= r.M) return;
+          float* dst = r.out_t + ((long long)zc * r.N + cc) * r.out_ld + chan;
+          const int ntok = r.N - cc;                      // tokens left from this column on (>= 1)
 #pragma unroll
-          for (int cc = 0; cc < kDecodeMaxTokens / 32; ++cc) {
-            if (cc * 32 >= r.N) break;
-            uint32_t v[32];
-            tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + 32 * cc), v);
-            tmem_ld_wait();
-#pragma unroll
-            for (int e = 0; e < 32; ++e) sum[cc][e] = q == 0 ? __uint_as_float(v[e]) : sum[cc][e] + __uint_as_float(v[e]);
+          for (int e = 0; e < 32; ++e) {
+            if (e < ntok) *dst = total_k == 0 ? 0.f : value(e);
+            dst += r.out_ld;
           }
+        };
+        auto next = [&]() {
+          if (!mbar_wait_warp(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) return false;
+          tc_fence_after();
+          return true;
+        };
+        auto done = [&]() {
           release();
           acc ^= 1;
           if (acc == 0) acc_phase ^= 1u;
+        };
+        const uint32_t tlane = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        if (nq == 1) {          // short code of its own: it runs once or twice a launch (0.4 us of 11 at 57 tokens of 4 x 768)
+          if (!next()) { ok = false; break; }
+          for (int cc = 0; cc < r.N; cc += 32) {
+            uint32_t v[32];
+            tmem_ld32(tlane + (uint32_t)(acc * kAccCols + cc), v);
+            tmem_ld_wait();
+            store(cc, [&](int e) { return __uint_as_float(v[e]); });
+          }
+          done();
+          continue;
+        }
+        float sum[kDecodeMaxTokens / 32][32] = {};
+        for (int q = 0; q < nq; ++q) {
+          if (!next()) { ok = false; break; }
+#pragma unroll
+          for (int j = 0; j < kDecodeMaxTokens / 32; ++j) {
+            if (32 * j >= r.N) break;
+            uint32_t v[32];
+            tmem_ld32(tlane + (uint32_t)(acc * kAccCols + 32 * j), v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) sum[j][e] += __uint_as_float(v[e]);
+          }
+          done();
         }
         if (!ok) break;
-        // for a fixed token the 32 lanes of a warp hold 32 consecutive channels: plain 128-byte coalesced stores
-        const long long chan = (long long)m0 + rr;
-        if (chan < r.M) {
 #pragma unroll
-          for (int cc = 0; cc < kDecodeMaxTokens / 32; ++cc) {
-            const int ntok = r.N - 32 * cc;             // tokens left from this column on
-            if (ntok <= 0) break;
-            float* dst = r.out_t + ((long long)zc * r.N + 32 * cc) * r.out_ld + chan;
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              if (e < ntok) *dst = total_k == 0 ? 0.f : sum[cc][e];
-              dst += r.out_ld;
-            }
-          }
-        }
+        for (int j = 0; j < kDecodeMaxTokens / 32; ++j)
+          if (32 * j < r.N) store(32 * j, [&](int e) { return sum[j][e]; });
         continue;
       }
       // one verdict for the warp: the tensor-memory loads below are instructions of all its lanes
@@ -1193,10 +1213,14 @@ cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* 
 // against one), so they are dealt longest first to the least loaded CTA.  Fewer, longer tiles mean fewer planes for the
 // row kernel - with many tokens every rank's CTA reads every shared plane - but a coarser deal; few_token_plan weighs them.
 namespace {
-struct FewPlan { FewSplit l[2]; Deal deal; int workers; };
+struct FewPlan { FewSplit l[2]; Deal deal; };
 
 constexpr double kItemOverhead = 1.5;     // of a tile, in k-steps: refill of the pipeline and the epilogue
 constexpr double kStepUs = 0.38;          // a k-step of 16 KB of weights on one of 148 SMs at 6.4 TB/s
+// Where the tiles leave SMs idle a k-step is bound by the CTA's own round trips (4 x 768: every k-step less on 48 tiles takes
+// 0.25 us off), and a split of the contraction costs more than its planes' bytes (0.3 us beside them).  A block of 4 x 768, split
+// in four by the bytes alone / as now: 64 tokens 12.7 / 10.0 us, 57 tokens of nothing shared 11.1 / 9.5, 16 tokens 9.7 / 8.7.
+constexpr double kLoneStepUs = 0.27, kSplitUs = 0.3;
 
 // The tiles of a plan by their length: at most full, last and empty ones of the shared and of the private part of either layer.
 // first, step, run: the tiles first + i * step + j, j < run, in the kernel's numbering (decode_tile with one column tile:
@@ -1329,25 +1353,22 @@ void few_token_plan(int t, int T, int h, int S, const int* K_r, int n, int sms, 
         const double len = c.l[g].qper > 0 ? (S > 0 ? c.l[g].qper : 1) * ks : (ks + c.l[g].ksplits - 1) / c.l[g].ksplits;
         if (len > longest) longest = len;
         const double bytes = 4.0 * T * ((double)ns * S * (clustered ? 2 : 1 + t) + 2.0 * c.l[g].ksplits * t * (h - S));
-        c.rest += bytes / 8e12 * 1e6;
+        c.rest += bytes / 8e12 * 1e6 + kSplitUs * (c.l[g].ksplits - 1);
       }
-      c.bound = fmax(total / workers, longest + kItemOverhead) * kStepUs + c.rest;
+      c.bound = fmax(total / workers * kStepUs, (longest + kItemOverhead) * kLoneStepUs) + c.rest;
       all[na++] = c;
     }
   std::sort(all, all + na, [](const Cand& a, const Cand& b) { return a.bound < b.bound; });
   for (int i = 0; i < na && (best_cost < 0 || all[i].bound < best_cost); ++i) {
     const FewTiles f = few_tiles(t, h, S, K_r, n, all[i].l);
     if (f.tiles > kMaxDealItems) continue;
-    const double cost = few_makespan(f, workers) * kStepUs + all[i].rest;
+    const double share = kStepUs * (f.tiles < workers ? f.tiles : workers) / workers;
+    const double cost = few_makespan(f, workers) * fmax(share, kLoneStepUs) + all[i].rest;
     if (best_cost < 0 || cost < best_cost) { best_cost = cost; best->l[0] = all[i].l[0]; best->l[1] = all[i].l[1]; }
   }
   const FewTiles f = few_tiles(t, h, S, K_r, n, best->l);
   best->deal.dealt = 0;
-  best->workers = workers;
-  if (f.tiles <= kMaxDealItems) {
-    if (f.tiles < workers) best->workers = f.tiles;
-    few_deal(f, best->workers, &best->deal);
-  }
+  if (f.tiles > workers && f.tiles <= kMaxDealItems) few_deal(f, workers, &best->deal);     // else a tile each, or by number
 }
 
 // The plan depends on the shapes alone.  Making one takes 4 us (7B shapes, on the host of the measurements); the 64 used last
@@ -1434,7 +1455,6 @@ cudaError_t launch_tc_forward_decode(int t, int T, int h, int S, DecodeProblem* 
   for (CUtensorMap& c : mp.c) c = mp.ab[0];          // unused: the epilogue stores directly
   p.nregions = g;
   finish_tiles(p);
-  if (plan.deal.dealt && plan.deal.first[plan.workers] != p.tiles_total) return cudaErrorInvalidValue;
   return launch(mp, p, CAAT_K_TC_FORWARD, st, nullptr, &plan.deal);
 }
 

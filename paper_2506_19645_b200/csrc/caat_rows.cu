@@ -387,7 +387,8 @@ __global__ void __launch_bounds__(512, CPT == 1 ? 2 : 1) rows_backward_kernel(co
 // of ranks or a part of one rank's contraction), zp [np][t][T][h - S_lo] of the private ones; planes are added in
 // ascending order.  Every rank's CTA forms the shared sum for itself (L2 hits), so no CTA waits for another.  With two
 // layers the second one's residual is the first one's new residual stream as stored (rounded to the storage type).
-template <typename T_, bool LN>
+// GRID: the partition is on the 8-channel grid.
+template <typename T_, bool LN, bool GRID>
 __device__ __forceinline__ void partials_row(const RowPartArgs& a, float* sm, int i, int m) {
   using V_ = VT<T_>;
   using raw = typename V_::raw;
@@ -397,7 +398,7 @@ __device__ __forceinline__ void partials_row(const RowPartArgs& a, float* sm, in
   float* red = sm + a.h;                  // reduction scratch
   int par = 0;
   const long long row = (long long)m * a.T + i;
-  const int S_lo = a.S / V * V, S_hi = (a.S + V - 1) / V * V, P = a.h - S_lo;
+  const int S_lo = GRID ? a.S : a.S / V * V, S_hi = GRID ? a.S : (a.S + V - 1) / V * V, P = a.h - S_lo;
   const float inv_h = 1.0f / (float)a.h;
   for (int layer = 0; layer < a.nlayers; ++layer) {
     const PartialLayer& L = a.L[layer];
@@ -405,7 +406,7 @@ __device__ __forceinline__ void partials_row(const RowPartArgs& a, float* sm, in
     for (int c = threadIdx.x * V; c < a.h; c += blockDim.x * V) {
       float r[V], z[V], hn[V];
       const bool shared_chunk = c + V <= a.S;
-      const bool mixed = !shared_chunk && c < a.S;     // the one chunk that straddles a partition off the 8-channel grid
+      const bool mixed = !GRID && !shared_chunk && c < a.S;     // the one chunk that straddles a partition off the 8-channel grid
       // compact layout (partition on the grid): where this chunk of the stream lives (shared part once, private part per rank)
       const long long coff = shared_chunk ? ((long long)i * a.S + c) * ES : (row * (a.h - a.S) + (c - a.S)) * ES;
       if (layer == 0) {
@@ -483,11 +484,11 @@ __device__ __forceinline__ void partials_row(const RowPartArgs& a, float* sm, in
   }
 }
 
-template <typename T_, bool LN>
+template <typename T_, bool LN, bool GRID>
 __global__ void __launch_bounds__(512) rows_forward_partials_kernel(const RowPartArgs a) {
   extern __shared__ float sm[];
   pdl_wait();
-  partials_row<T_, LN>(a, sm, blockIdx.x, blockIdx.y);
+  partials_row<T_, LN, GRID>(a, sm, blockIdx.x, blockIdx.y);
 }
 
 // One CTA per token, the ranks from the last to the first: a compact stream updated in place is stored in rank 0's turn, after
@@ -498,7 +499,7 @@ __global__ void __launch_bounds__(512) rows_forward_partials_token_kernel(const 
   extern __shared__ float sm[];
   pdl_wait();
   for (int m = a.t - 1; m >= 0; --m) {
-    partials_row<T_, LN>(a, sm, blockIdx.x, m);
+    partials_row<T_, LN, true>(a, sm, blockIdx.x, m);       // a compact stream
     __syncthreads();                      // the reduction scratch is used again
   }
 }
@@ -881,7 +882,8 @@ cudaError_t launch_rows_forward_partials(const RowPartArgs& a, caat_dtype dtype,
   using bf16 = __nv_bfloat16;          // the only type of the tensor-core GEMM that leaves the planes
   if (dtype != CAAT_BF16) return cudaErrorInvalidValue;
   if (in_place) return a.norm == 1 ? go(rows_forward_partials_token_kernel<bf16, true>) : go(rows_forward_partials_token_kernel<bf16, false>);
-  return a.norm == 1 ? go(rows_forward_partials_kernel<bf16, true>) : go(rows_forward_partials_kernel<bf16, false>);
+  if (a.S % V) return a.norm == 1 ? go(rows_forward_partials_kernel<bf16, true, false>) : go(rows_forward_partials_kernel<bf16, false, false>);
+  return a.norm == 1 ? go(rows_forward_partials_kernel<bf16, true, true>) : go(rows_forward_partials_kernel<bf16, false, true>);
 }
 
 RowsHooks rows_hooks() {
