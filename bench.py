@@ -9,7 +9,7 @@ ranks are simulated as a batch dimension on one GPU.
   python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME] [--impl reference]
   python -m torch.distributed.run ... bench.py --gpus N --mode tp      (real tensor parallelism, p sweep)
 
-Prints ONE JSON line (rank 0).  With N > 1 (launched by torch.distributed.run) every GPU
+Prints ONE JSON line (rank 0); the per-kernel tables and the other workloads go to ``--detail``.  With N > 1 (launched by torch.distributed.run) every GPU
 runs an independent replica of the workload (the path as benchmarked has no cross-GPU
 exchange step): weak scaling, no data-path collective; time is the max over ranks.
 ``--mode tp`` instead splits the tensor-parallel ranks over the GPUs and exchanges the
@@ -190,6 +190,15 @@ def step_work(w, S, compact=False):
             a = tot.setdefault(kind, {"flops": 0.0, "bytes": 0.0, "bytes_interface": 0.0})
             for k in a:
                 a[k] += v[k]
+    if w.kind == "block":
+        # the stream between the layers (and its gradient) is an output of the block: written, and read by no other tensor's
+        # formation once both layers' rows are worked in one pass
+        full = w.t * w.tokens * w.h * esize(w)
+        between = (w.tokens * S + w.t * w.tokens * (w.h - S)) * esize(w) if compact else full
+        for kind in ("rows_forward", "rows_backward"):
+            for k in ("bytes", "bytes_interface"):
+                if kind in tot:
+                    tot[kind][k] -= between
     if w.dtype == "f32":      # fp32 runs the CUDA-core GEMM (TF32 cannot meet the 1e-4 tolerance)
         tot["gemm_cuda_core"] = tot.pop("tc_gemm_forward")
     return tot
@@ -212,6 +221,8 @@ def paper_level_work(w, S, compact=False):
         if w.backward:
             fl += 4.0 * T * K * h
             by += e * (full + 3 * stream + 2 * T * K + K * h) + 4 * K * h
+    if w.kind == "block":      # the stream between the layers, and its gradient, are outputs: not read back
+        by -= e * stream * (2 if w.backward else 1)
     return fl, by
 
 
@@ -920,10 +931,25 @@ def run_cuda(args):
             result["cpu_baseline"] = cpu_baseline(w)
         else:
             result["cpu_baseline"] = None
-        print(json.dumps(result), flush=True)
+        print_result(result, args.detail)
     if dist_on:
         torch.distributed.barrier()
         torch.distributed.destroy_process_group()
+
+
+def print_result(result, detail):
+    """The whole record - per-kernel tables, the other workloads, projections: tens of kilobytes - goes to the file `detail`;
+    stdout gets one short line."""
+    try:
+        with open(detail, "w") as f:
+            json.dump(result, f, indent=1)
+    except OSError as ex:
+        sys.stderr.write(f"bench: {detail} not written ({ex})\n")
+    line = {k: result[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                                   "vs_baseline", "dtype", "data", "config", "clocks", "gpu_launches", "e2e", "roofline",
+                                   "cpu_baseline", "step_ms")}
+    line["path_roofline_frac"] = result["path_roofline"]["frac"]
+    print(json.dumps(line), flush=True)
 
 
 # --------------------------------------------------------------------------- the reference arm (oracle on host cores)
@@ -981,6 +1007,8 @@ def main():
                          "(CAAT_OPT_BLOCK_OVERLAP = 1); default: the library chooses by shape")
     ap.add_argument("--layout", default="per_rank", choices=["per_rank", "compact"],
                     help="residual-stream layout: per rank [t,T,h] (the benchmark's configuration) or compact")
+    ap.add_argument("--detail", default=os.path.join(ROOT, "bench_detail.json"),
+                    help="file for the whole record (per-kernel tables, the other workloads); stdout has one short line")
     ap.add_argument("--tokens", type=int, default=0, help="override the workload's token count (profiling on a small case)")
     args = ap.parse_args()
     if args.steps < 1:
