@@ -30,8 +30,9 @@
  *   Errors     a caat_status is returned; argument errors are found on the host
  *              before any launch and leave all outputs untouched.  There is no CPU
  *              fallback: without a usable CUDA device calls return CAAT_ECUDA.
- *   Determinism  same inputs, same device: bit-identical outputs (no floating-point
- *              atomics; rank sums run m = 0..t-1).
+ *   Determinism  same inputs, same device, same options and workspace size: bit-identical
+ *              outputs (no floating-point atomics).  Rank sums run in a fixed order: m = 0..t-1,
+ *              or groups of neighbouring ranks first and then the groups in order.
  *   Aliasing   Hn may alias R (in-place residual update); dR may alias dHn; nothing
  *              else may overlap.
  *   Threads    compute calls may be made from several host threads at once (each with its
@@ -43,8 +44,9 @@
  *              sets it; the call that reads it clears it) and the caat_profile_* benchmark
  *              aid (one recording at a time, not thread-safe).
  *   Limits     h must be a multiple of 8 and at most 16384 (bf16) or 8192 (fp32) channels,
- *              t * tokens at most 2e9 (CAAT_EUNSUPPORTED otherwise); t divides h and ffn.  The tensor-core GEMM is used for CAAT_BF16 when K_r and S
- *              are multiples of 8; other shapes run a slower CUDA-core GEMM.
+ *              t * tokens at most 2e9 (CAAT_EUNSUPPORTED otherwise); t divides h and ffn.  The
+ *              tensor-core GEMM is used for CAAT_BF16 when K_r is a multiple of 8, for any S;
+ *              other shapes run a slower CUDA-core GEMM.
  */
 #ifndef CAAT_H_
 #define CAAT_H_
@@ -134,7 +136,12 @@ size_t caat_block_workspace_bytes(const caat_ctx *ctx, int tokens, int backward)
 /* Bytes of device scratch for `tokens` tokens of `layer`: backward = 0, what the forward
  * call needs; backward = 1, enough for the forward AND the backward call (a training step
  * runs both on one buffer; neither keeps anything in it between calls).  The block calls
- * have their own figure, caat_block_workspace_bytes.
+ * have their own figure, caat_block_workspace_bytes.  With more than 64 tokens a buffer sized for
+ * a forward of more tokens serves fewer.  Included, whether a call comes to use it or not: up to
+ * 32 MB of partial sums per layer (forward), and a copy of the weights [t, h, K_r] in the run dtype
+ * when alpha != 1 and S < h (backward; written where alpha cannot ride on the products' results:
+ * the compact stream, the halves of a multi-GPU call, |alpha| outside [2^-10, 2^10],
+ * CAAT_OPT_BACKWARD_REDUCE 1 and 2).
  * 0 on bad arguments. */
 size_t caat_workspace_bytes(const caat_ctx *ctx, caat_layer layer, int tokens, int backward);
 
@@ -240,7 +247,9 @@ caat_status caat_rowpar_backward(const caat_ctx *ctx, caat_layer layer, int toke
  * kernel runs on a stream of the library's own, forked from and joined back into `cuda_stream` with events
  * inside this call (legal inside a stream capture; the library creates that stream on the first such call per
  * device, so make one call before capturing): everything the call enqueued is ordered before whatever the caller
- * enqueues on `cuda_stream` next.  Results do not depend on the schedule.
+ * enqueues on `cuda_stream` next.  The schedules form the same sums Hn1 and Hn2; X1, X2 and the row statistics may
+ * differ in their last bits between schedules (a row's statistics are summed in another order), and so may the
+ * gradients of the block backward.  The schedule follows the option and the workspace size.
  */
 caat_status caat_block_forward(const caat_ctx *ctx, int tokens,
                                const void *Y_attn, const void *W_o,
@@ -390,8 +399,9 @@ caat_status caat_colpar_backward(const caat_ctx *ctx, caat_activation act, int n
  * (caat_tp_slab; the forward and the backward slab may sit at different offsets).  Both halves of a
  * direction must get the same workspace, untouched in between except for the slab.  Tensor-core path
  * only (bf16, K_r and S multiples of 8): CAAT_EUNSUPPORTED otherwise.  Workspace size:
- * caat_workspace_bytes.  With G = 1 the two halves and no collective give caat_rowpar_forward /
- * _backward's results for more than 64 tokens (few-token calls take another route there).
+ * caat_workspace_bytes.  With G = 1 and more than 64 tokens (few-token calls take another route) the two halves and no
+ * collective give caat_rowpar_forward's results bit for bit, and caat_rowpar_backward's where alpha is a power of two;
+ * else dY and dW agree to their rounding (the single call divides the shared gradient by alpha before it is stored).
  */
 caat_status caat_tp_slab(const caat_ctx *ctx, caat_layer layer, int tokens, int backward,
                          size_t *offset_bytes, int *rows, int *cols);

@@ -1054,7 +1054,7 @@ bool tc_gemm_usable(const caat_ctx* ctx, int K_r) {
 // ---- forward: zs[T,S] = sum_m Y[m] W[m][:S]^T ; zp[m][T,h-S_lo] = Y[m] W[m][S_lo:]^T
 // Any partition S: TMA wants 16-byte coordinates along a row's channels, so the private products start at S_lo; their
 // S - S_lo extra columns land in the scratch columns that no row kernel reads.  (Partitions off the 8-channel grid ran on
-// the CUDA-core GEMM before: a training step of a block at h = 2048, 2999 tokens, p = 0.7 took 17.5 ms, now 0.61 ms.)
+// the CUDA-core GEMM before: a training step of a block at h = 2048, 2999 tokens, p = 0.7 took 17.5 ms, now 0.52 ms.)
 // A shared tile's contraction is t times a private one's, and with few tokens there are only a handful of them: the
 // GEMM then waits for its longest tiles (T = 300 at the 7B MLP shapes: 16 tiles of 176 k-steps where the even share of a
 // worker is 76).  Given `planes` ([max_groups][T][S_hi] fp32 scratch), the rank loop may be split into groups of ranks:

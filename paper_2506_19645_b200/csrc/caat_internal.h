@@ -30,7 +30,8 @@ namespace caat {
 
 constexpr int kLayoutVec = 8;        // column granularity of the scratch layout (elements)
 // Scratch for the rank groups of a split shared region: as many planes as fit here, at most t.  A split pays only while
-// the shared tiles are few, that is while a plane is small (2.4 MB at 300 tokens of S = 2048).
+// the shared tiles are few, that is while a plane is small (2.4 MB at 300 tokens of S = 2048).  The room is reserved for any
+// number of tokens.
 constexpr size_t kGroupPlanesBytes = 32u << 20;
 constexpr int kMaxPartialRows = 1184;  // upper bound on rows of norm-gradient partials (8 x 148)
 
@@ -52,7 +53,7 @@ struct Scratch {
   size_t wt_off;           // backward: the private rows of W times alpha, [t, h, K_r] (tensor-core path, alpha != 1)
   size_t zt_off;           // forward, few tokens: fp32 per-rank partials [t, T, h]
   size_t gp_off;           // forward: fp32 partial sums of the shared columns over groups of ranks, [gp_groups, T, S_hi]
-  int gp_groups;           // 0: no room reserved (too many tokens for a split to pay)
+  int gp_groups;           // 0: a single plane or none fits (too many tokens for a split to pay)
   size_t total;
 };
 
