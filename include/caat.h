@@ -83,7 +83,9 @@ typedef enum {
   CAAT_OPT_EPS = 1,             /* norm epsilon, default 1e-5                           */
   CAAT_OPT_PRIVATE_SCALE = 2,   /* alpha; default sqrt(t); 1 switches scaling off       */
   CAAT_OPT_SHARED_CHANNELS = 3, /* override S with an explicit integer in [0, h]        */
-  CAAT_OPT_GEMM = 4,            /* 0 = automatic (default), 1 = force the CUDA-core GEMM */
+  CAAT_OPT_GEMM = 4,            /* 0 = automatic (default; fp32 products of some size run on the tensor
+                                   cores, every operand split exactly into three bf16 parts),
+                                   1 = force the CUDA-core GEMM */
   CAAT_OPT_ROWS = 5,            /* row kernels: 0 = automatic (default: warp-per-token kernels for
                                    rows of at most 1024 bf16 channels, bulk-copy staged kernels
                                    otherwise), 1 = plain-load kernels, 2 = staged kernels always */
@@ -532,7 +534,7 @@ typedef enum {
   CAAT_K_ROWS_FORWARD = 0,   /* reduce hand-off + scale + residual + norm           */
   CAAT_K_ROWS_BACKWARD = 1,  /* norm backward + residual gradient + backward reduce */
   CAAT_K_NORMGRAD_REDUCE = 2,/* second stage of dgamma / dbeta                      */
-  CAAT_K_GEMM_CUDA_CORE = 3, /* CUDA-core GEMM (fp32 and unaligned shapes)          */
+  CAAT_K_GEMM_CUDA_CORE = 3, /* CUDA-core GEMM (small fp32 products, unaligned bf16)  */
   CAAT_K_TC_FORWARD = 4,     /* tcgen05 GEMM, forward                               */
   CAAT_K_TC_DGRAD = 5,       /* tcgen05 GEMM, data gradient                         */
   CAAT_K_TC_WGRAD = 6,       /* tcgen05 GEMM, weight gradient (or a block's four gradient products in one launch) */

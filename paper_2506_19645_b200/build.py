@@ -23,7 +23,7 @@ LIB = os.path.join(PKG, "libcaat.so")
 PYEXT_SRC, PYEXT = os.path.join(CSRC, "caat_py.cpp"), os.path.join(PKG, "_caatpy.so")
 PYEXT_FOR = os.path.join(OBJ, "caat_py.for")      # the Python and torch that _caatpy.so was built for
 SOURCES = ["caat_api.cu", "caat_rows.cu", "caat_rows_staged.cu", "caat_rows_lean.cu", "caat_rows_block.cu",
-           "caat_rows_block_bwd.cu", "caat_rows_warp.cu", "caat_gemm_simt.cu",
+           "caat_rows_block_bwd.cu", "caat_rows_warp.cu", "caat_gemm_simt.cu", "caat_gemm_f32.cu",
            "caat_gemm_tc.cu", "caat_static.cu", "caat_colpar.cu", "caat_tp_push.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 

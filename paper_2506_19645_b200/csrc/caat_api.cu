@@ -233,7 +233,7 @@ static caat_status forward_impl(const caat_ctx* ctx, int K_r, int T, const void*
       g.C = static_cast<char*>(zp) + (size_t)(S - L.S_lo) * e;
       g.sCb = (long long)T * L.P; g.sCi = L.P; g.M = T; g.N = h - S; g.batch = t; g.c_f32 = 0;
     }
-    ce = launch_gemm_simt(pr, 2, ctx->dtype, st);
+    ce = launch_gemm_simt(pr, 2, ctx->dtype, ctx->force_simt, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
   }
   if (phase == 1) return CAAT_OK;
@@ -342,7 +342,7 @@ static caat_status backward_impl(const caat_ctx* ctx, int K_r, int T, const void
     g.seg[1] = GemmSeg{zp_priv, static_cast<const char*>(W) + (size_t)S * K_r * e,
                        (long long)T * L.P, 0, L.P, 1, (long long)h * K_r, 0, K_r, 1, 1, h - S};
     g.C = dY; g.sCb = (long long)T * K_r; g.sCi = K_r; g.M = T; g.N = K_r; g.batch = t; g.c_f32 = 0;
-    ce = launch_gemm_simt(&g, 1, ctx->dtype, st);
+    ce = launch_gemm_simt(&g, 1, ctx->dtype, ctx->force_simt, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
   }
   GemmProblem pw[2] = {};
@@ -359,7 +359,7 @@ static caat_status backward_impl(const caat_ctx* ctx, int K_r, int T, const void
     g.C = dW + (size_t)S * K_r; g.sCb = (long long)h * K_r; g.sCi = K_r; g.M = h - S; g.N = K_r; g.batch = t;
     g.c_f32 = 1;
   }
-  ce = launch_gemm_simt(pw, 2, ctx->dtype, st);
+  ce = launch_gemm_simt(pw, 2, ctx->dtype, ctx->force_simt, st);
   if (ce != cudaSuccess) return cuda_fail(ce);
   return CAAT_OK;
 }
@@ -1012,7 +1012,7 @@ caat_status caat_colpar_forward(const caat_ctx* ctx, caat_activation act, int n_
     g.nseg = 1;
     g.seg[0] = GemmSeg{X, A, (long long)T * h, 0, h, 1, (long long)n_out * h, 0, 1, h, 1, h};
     g.C = pre; g.sCb = (long long)T * n_out; g.sCi = n_out; g.M = T; g.N = n_out; g.batch = t; g.c_f32 = 0;
-    ce = launch_gemm_simt(&g, 1, ctx->dtype, st);
+    ce = launch_gemm_simt(&g, 1, ctx->dtype, ctx->force_simt, st);
   }
   if (ce != cudaSuccess) return cuda_fail(ce);
   if (act != CAAT_ACT_NONE) {
@@ -1059,7 +1059,7 @@ caat_status caat_colpar_backward(const caat_ctx* ctx, caat_activation act, int n
     g.nseg = 1;
     g.seg[0] = GemmSeg{dpre, A, (long long)T * n_out, 0, n_out, 1, (long long)n_out * h, 0, h, 1, 1, n_out};
     g.C = dX; g.sCb = (long long)T * h; g.sCi = h; g.M = T; g.N = h; g.batch = t; g.c_f32 = 0;
-    ce = launch_gemm_simt(&g, 1, ctx->dtype, st);
+    ce = launch_gemm_simt(&g, 1, ctx->dtype, ctx->force_simt, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
   }
   {  // dA[m] = dpre[m]^T X[m]
@@ -1067,7 +1067,7 @@ caat_status caat_colpar_backward(const caat_ctx* ctx, caat_activation act, int n
     g.nseg = 1;
     g.seg[0] = GemmSeg{dpre, X, (long long)T * n_out, 0, 1, n_out, (long long)T * h, 0, h, 1, 1, T};
     g.C = dA; g.sCb = (long long)n_out * h; g.sCi = h; g.M = n_out; g.N = h; g.batch = t; g.c_f32 = 1;
-    ce = launch_gemm_simt(&g, 1, ctx->dtype, st);
+    ce = launch_gemm_simt(&g, 1, ctx->dtype, ctx->force_simt, st);
     if (ce != cudaSuccess) return cuda_fail(ce);
   }
   return CAAT_OK;

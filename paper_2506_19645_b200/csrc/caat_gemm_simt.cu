@@ -1,7 +1,7 @@
 // Generic strided batched GEMM on CUDA cores with fp32 accumulation.
 //
-// It serves the fp32 configuration (TF32 tensor cores cannot meet a 1e-4 relative tolerance) and bf16 shapes the
-// tensor-core kernels do not take (K_r not a multiple of 8).  Every operand is addressed through element strides, one
+// It serves small fp32 products (large ones run on the tensor cores in three bf16 parts per operand, caat_gemm_f32.cu, unless
+// the CUDA cores are asked for) and bf16 shapes the tensor-core kernels do not take (K_r not a multiple of 8).  Every operand is addressed through element strides, one
 // of which is 1, so the same kernels run the forward product, the data gradient and the weight gradient; the "two
 // segment" form covers the [shared | private] split of the contraction axis, and the products of a call that do not
 // depend on each other (shared and private columns) share one launch.
@@ -522,7 +522,7 @@ cudaError_t launch_typed(GemmList& L, bool ak, bool bk, cudaStream_t st) {
 
 }  // namespace
 
-cudaError_t launch_gemm_simt(const GemmProblem* problems, int n, caat_dtype dtype, cudaStream_t st) {
+cudaError_t launch_gemm_simt(const GemmProblem* problems, int n, caat_dtype dtype, int force_simt, cudaStream_t st) {
   GemmList L{};
   for (int i = 0; i < n; ++i) {
     if (problems[i].M <= 0 || problems[i].N <= 0 || problems[i].batch <= 0) continue;
@@ -560,6 +560,8 @@ cudaError_t launch_gemm_simt(const GemmProblem* problems, int n, caat_dtype dtyp
     }
   }
   if (dtype == CAAT_BF16) return launch_typed<__nv_bfloat16, false>(L, ak, bk, st);
+  cudaError_t err;
+  if (!force_simt && launch_gemm_f32(L.p, L.n, ak, bk, vec, st, &err)) return err;
   return vec ? launch_typed<float, true>(L, ak, bk, st) : launch_typed<float, false>(L, ak, bk, st);
 }
 

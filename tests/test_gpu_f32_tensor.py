@@ -1,0 +1,97 @@
+"""fp32 products on the bf16 tensor cores (operands split in three parts): tiles, pairs and clusters at their edges, both
+operand majors, 16-byte and element-wise loads, accuracy against 64 bits beside the CUDA-core path, values that are not finite."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2506_19645_b200 import caat
+from tests import gpu_harness as G
+from tests.test_gpu_parity import _check_backward, _check_forward, _layer_case
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("t,T,h,ffn,layer,S", [
+    (4, 64, 768, 3072, caat.CAAT_MLP_DOWN, 384),      # few tokens: the weights on the 128-row side, contractions over clusters
+    (4, 257, 768, 3072, caat.CAAT_MLP_DOWN, 384),     # one row past a pair's tile
+    (4, 999, 768, 3000, caat.CAAT_MLP_DOWN, 285),     # K_r = 750 and an odd partition: element-wise loads, remainders everywhere
+    (4, 640, 768, 3088, caat.CAAT_MLP_DOWN, 380),     # K_r = 772: 16-byte loads with remainders
+    (2, 777, 1032, 4104, caat.CAAT_MLP_DOWN, 1032),   # nothing private
+    (2, 777, 1032, 4104, caat.CAAT_MLP_DOWN, 0),      # nothing shared
+    (1, 1500, 1032, 2064, caat.CAAT_MLP_DOWN, 8),     # one rank, a shared tile of 8 columns
+    (8, 300, 2048, 5632, caat.CAAT_MLP_DOWN, 1024),   # more tiles than clusters: partial tiles and the next item's operands
+    (2, 3000, 1024, 4096, caat.CAAT_ATTN_OUT, 512),   # tiles for several rounds
+])
+def test_f32_layer(t, T, h, ffn, layer, S):
+    ctx = G.make_ctx(t, h, ffn, "f32", S=S)
+    d = _layer_case(t, T, h, ctx.k_r(layer), "f32", S, seed=T + S, backward=True)
+    _check_forward(ctx, layer, d, "f32")
+    _check_backward(ctx, layer, d, "f32")
+
+
+def _rel(a, b):
+    return float(((a.double().numpy() - b) ** 2).sum() ** 0.5 / (b ** 2).sum() ** 0.5)
+
+
+@pytest.mark.parametrize("t,T,h,ffn,p", [(4, 2000, 768, 3072, 0.5), (8, 64, 2048, 5632, 0.91), (2, 300, 1024, 4096, 0.0)])
+def test_no_further_from_64_bits_than_fma_chains(t, T, h, ffn, p):
+    """The three parts hold all 24 bits and a partial sum of 64 products is added in fp32 registers: 1.0e-7 to 1.4e-7 here, where
+    the CUDA-core kernels' chains of FMAs give 1.0e-7 to 5.7e-7."""
+    layer, out = caat.CAAT_MLP_DOWN, []
+    for force in (True, False):
+        ctx = G.make_ctx(t, h, ffn, "f32", p=p, force_simt=force)
+        d = _layer_case(t, T, h, ctx.k_r(layer), "f32", ctx.shared_channels, seed=5, backward=True)
+        fo = G.oracle_forward(ctx, d)
+        Hn, rstd, mean = G.saved_from_oracle(ctx, fo)
+        got, gb, ob = G.gpu_forward(ctx, layer, d), G.gpu_backward(ctx, layer, d, Hn, rstd, mean), G.oracle_backward(ctx, d, Hn, rstd, mean)
+        out.append([_rel(got["Hn"], fo["Hn"]), _rel(gb["dY"], ob["dY"]), _rel(gb["dW"], ob["dW"])])
+    for simt, tensor in zip(*out):
+        assert tensor < 2.5e-7 and tensor < 1.1 * simt
+
+
+def test_values_that_are_not_finite():
+    """An infinite or NaN operand gives what a chain of FMAs gives, also where the other operand's lower parts are zero."""
+    t, T, h, ffn, layer = 2, 300, 512, 4096, caat.CAAT_MLP_DOWN
+    ctx = G.make_ctx(t, h, ffn, "f32", S=256)
+    k = ctx.k_r(layer)
+    d = _layer_case(t, T, h, k, "f32", 256, seed=2)
+    d["W"] = d["W"].abs().bfloat16().float() + 0.0     # positive, lower parts zero
+    d["Y"][0, 7, 11] = float("inf")
+    d["Y"][1, 140, 500] = float("nan")
+    d["Y"][1, 299, k - 1] = 3.4e38                     # its first part would round to infinity
+    d["W"][0, 300, 5] = -float("inf")                  # a private column of rank 0
+    got = G.gpu_forward(ctx, layer, d)["Hn"].double().numpy()
+    with np.errstate(all="ignore"):
+        want = G.oracle_forward(ctx, d)["Hn"].astype(np.float32).astype(np.float64)
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
+    ok = np.isfinite(want)
+    assert np.isposinf(got[0, 7, 0]) and np.isnan(got[1, 140, 400]) and np.all(np.abs(got[ok] - want[ok]) <= 1e-4 * np.maximum(np.abs(want[ok]), 1))
+
+
+CHILD = r"""
+import torch
+from paper_2506_19645_b200 import caat, synthetic
+t, T, h, ffn, layer = 4, 700, 768, 3072, caat.CAAT_MLP_DOWN
+ctx = caat.Context(h, ffn, t, 0.5, "f32")
+d = synthetic.layer_inputs(t, T, h, ctx.k_r(layer), "f32", seed=1, S=ctx.shared_channels, device="cuda")
+mk = lambda *s: torch.empty(*s, dtype=torch.float32, device="cuda")
+Hn, X, rstd = mk(t, T, h), mk(t, T, h), mk(t, T)
+ws = ctx.alloc_workspace(ctx.workspace_bytes(layer, T, False))
+ctx.rowpar_forward(layer, T, d["Y"], d["W"], d["R"], d["gamma"], None, Hn, X, rstd, None, ws)
+torch.cuda.synchronize()
+print("STATUS", ctx.last_device_status(), ctx.last_device_status(), int(torch.ones(1024, device="cuda").sum().item()))
+"""
+
+
+def test_waits_run_out_and_report_timeout():
+    """Stages that are filled but never announced: every role gives up within its poll limit, partial tiles of a cluster included."""
+    env = dict(os.environ, CAAT_TC_DEBUG="1024", CAAT_TC_SPINCAP="2048")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", CHILD], env=env, cwd=root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    line = [l for l in out.stdout.splitlines() if l.startswith("STATUS")][-1].split()
+    assert [int(x) for x in line[1:]] == [caat.CAAT_ETIMEOUT, caat.CAAT_OK, 1024]
