@@ -10,7 +10,8 @@
 // output 2.1e-7 / 1.2e-7, data gradient 3.5e-7 / 1.1e-7, weight gradient 5.7e-7 / 1.4e-7; 8 x 5120, 60 tokens, the worst of
 // the three 6.4e-7 / 1.9e-7.
 //
-// The three products of a step at 4 x 768, 2000 tokens (28 GFLOP; an event around every launch): 783 -> 210 us.  What bounds a
+// A layer's training step at 4 x 768, 2000 tokens (28 GFLOP of products): 811 -> 269 us (three ring stages per pair instead of two,
+// which leave the first-level cache too little: products 211 -> 230 us).  What bounds a
 // stage (2.4 to 4 k cycles where its 24 products take 1.5 k) is the way round: loads, split, stores, barrier, products, barrier.
 //
 // A value below 2^-110 loses the bits of its last part that bf16 cannot hold.  A result that is not finite is computed
@@ -627,9 +628,9 @@ cudaError_t launch_layout(bool ak, bool bk, const XParams& p, int ctas, int kind
 }  // namespace
 
 // Products of fewer operations than this stay on the CUDA cores, whose 32 x 32 tiles are spread over more SMs.  Either side of
-// the lines (layer, CUDA cores / here, us): forward, 0.07 GFLOP 12.1 / 16.0, 0.3 GFLOP 24.6 / 22.7; forward and backward,
-// 0.3 GFLOP a product 119 / 61.
-constexpr double kMinForward = 2.0e8, kMinGradient = 1.2e8;
+// the lines (layer, CUDA cores / here, us): forward, 0.07 GFLOP 12.1 / 16.0, 0.21 GFLOP 27.2 / 20.4, 0.30 GFLOP 19.5 / 17.2;
+// backward, 0.13 GFLOP a product 25.8 / 28.5 (2 x 256) but 44.2 / 26.3 (2 x 512), 0.15 GFLOP 40.6 / 34.4.
+constexpr double kMinForward = 2.0e8, kMinGradient = 1.45e8;
 
 bool launch_gemm_f32(const GemmProblem* problems, int n, bool ak, bool bk, bool vec, cudaStream_t st, cudaError_t* err) {
   double work = 0;
