@@ -130,11 +130,11 @@ struct Deal {
   uint16_t first[kMaxDealWorkers + 1];
   uint16_t item[kMaxDealItems];
 };
-template <bool SWAP> struct ExtraArg { using type = PeerMaps; };
-template <> struct ExtraArg<true> { using type = Deal; };
+template <int SWAP> struct ExtraArg { using type = Deal; };
+template <> struct ExtraArg<0> { using type = PeerMaps; };
 
 // the tiles of one worker, in order
-template <bool SWAP>
+template <int SWAP>
 struct TileIter {
   const typename ExtraArg<SWAP>::type& x;
   int pos, end, step;
@@ -215,8 +215,9 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
 // (tcgen05 cta_group::2): each CTA stages its own 128 rows of A and HALF of the B tile, the
 // leader (cluster rank 0) issues the MMAs for both and the tensor cores read B from both CTAs'
 // shared memory, so the operand bytes a CTA pulls from L2 per flop drop by a third.
-// SWAP: the operands are swapped (few tokens: weights on the 128-row side), fp32 planes stored straight from registers.
-template <int CG, bool SWAP, bool MIXED>
+// SWAP: the operands are swapped (weights on the 128-row side) and the sums are stored straight from registers: 1 = few tokens,
+// fp32 planes, an accumulator per rank; 2 = some hundreds of tokens, one accumulator per tile, in the run's type or fp32 planes.
+template <int CG, int SWAP, bool MIXED>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ typename ExtraArg<SWAP>::type extra,
                const __grid_constant__ Params p) {
@@ -393,7 +394,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
           acc ^= 1;
           if (acc == 0) acc_phase ^= 1u;
         };
-        if (!SWAP && !begin()) { ok = false; break; }
+        if (SWAP != 1 && !begin()) { ok = false; break; }
         uint32_t idesc = idesc0 | ((uint32_t)(tile_cols(p, r, c.nt, CG) >> 3) << 17);
         if constexpr (MIXED) {
           idesc |= (uint32_t)r.a_mn << 15;
@@ -406,7 +407,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
           int q0, q1, kb, ke;
           split_range(r, u, c.split, q0, q1, kb, ke);
           for (int q = q0; q < q1 && ok; ++q) {
-            if (SWAP && !begin()) { ok = false; break; }      // an accumulator per rank, see the epilogue
+            if (SWAP == 1 && !begin()) { ok = false; break; }      // an accumulator per rank, see the epilogue
             for (int kk = kb; kk < ke; ++kk) {
               if (!mbar_wait_warp(full_bar, phase, abort_flag, p.spin_cap)) { ok = false; break; }
               tc_fence_after();
@@ -428,10 +429,10 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
                 a_lo = a_lo0; b_lo = b_lo0; full_bar = full0; empty_bar = empty0;
               }
             }
-            if (SWAP && ok) finish();
+            if (SWAP == 1 && ok) finish();
           }
         }
-        if (!SWAP && ok) finish();
+        if (SWAP != 1 && ok) finish();
       }
       if (!ok && lane == 0) { *abort_flag = 1; atomicExch(p.status, 2u); }
     }
@@ -464,7 +465,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
           if (CG == 2) mbar_arrive_remote(mapa_rank(tempty0 + 8u * acc, 0)); else mbar_arrive(tempty0 + 8u * acc);
         }
       };
-      if constexpr (SWAP) {
+      if constexpr (SWAP == 1) {
         // swap-AB (decode): TMEM lane = output channel, column = token.  Every rank of the tile's group comes in an
         // accumulator of its own and the ranks are added here, as the row kernel adds the planes: one accumulator over all
         // ranks rounds every k-step's partial sum in the tensor core, which cost the row statistics a factor of three in
@@ -521,6 +522,42 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
 #pragma unroll
         for (int j = 0; j < kDecodeMaxTokens / 32; ++j)
           if (32 * j < r.N) store(32 * j, [&](int e) { return sum[j][e]; });
+        continue;
+      }
+      if constexpr (SWAP == 2) {
+        // TMEM lane = output channel, column = token: for a token the 32 lanes of a warp hold 32 consecutive channels, stored
+        // as one run of 64 (128) bytes
+        if (!mbar_wait_warp(tfull0 + 8u * acc, acc_phase, abort_flag, p.spin_cap)) { ok = false; break; }
+        tc_fence_after();
+        const long long chan = (long long)m0 + rr;
+        const int ntok = r.N - n0 < p.BN ? r.N - n0 : p.BN;
+        const long long at = ((long long)zc * r.N + n0) * r.out_ld + chan;
+        float* f32 = r.out_t + at;
+        __nv_bfloat16* b16 = reinterpret_cast<__nv_bfloat16*>(r.out_t) + at;
+        const bool mine = chan < r.M;
+        for (int cc = 0; cc < ntok; cc += 32) {
+          uint32_t v[32];
+          __syncwarp();
+          tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccCols + cc), v);
+          tmem_ld_wait();
+          if (cc + 32 >= ntok) release();
+          if (total_k == 0) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] = 0u;
+          }
+          const int left = mine ? ntok - cc : 0;
+          if (r.out_f32) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e, f32 += r.out_ld)
+              if (e < left) *f32 = __uint_as_float(v[e]);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 32; ++e, b16 += r.out_ld)
+              if (e < left) *b16 = __float2bfloat16_rn(__uint_as_float(v[e]));
+          }
+        }
+        acc ^= 1;
+        if (acc == 0) acc_phase ^= 1u;
         continue;
       }
       // one verdict for the warp: the tensor-memory loads below are instructions of all its lanes
@@ -840,10 +877,12 @@ cudaError_t launch(const MapsT<MIXED>& maps, Params& p, int kind, cudaStream_t s
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (std::lock_guard<std::mutex> lock(host_cache_mutex()); !attr_set[dev]) {
     auto allow = [](auto k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); };
-    cudaError_t e = allow(tc_gemm_kernel<1, false, MIXED>);
-    if (e == cudaSuccess) e = allow(tc_gemm_kernel<2, false, MIXED>);
-    if constexpr (!MIXED)
-      if (e == cudaSuccess) e = allow(tc_gemm_kernel<1, true, false>);
+    cudaError_t e = allow(tc_gemm_kernel<1, 0, MIXED>);
+    if (e == cudaSuccess) e = allow(tc_gemm_kernel<2, 0, MIXED>);
+    if constexpr (!MIXED) {
+      if (e == cudaSuccess) e = allow(tc_gemm_kernel<1, 1, false>);
+      if (e == cudaSuccess) e = allow(tc_gemm_kernel<2, 2, false>);
+    }
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
@@ -882,13 +921,14 @@ cudaError_t launch(const MapsT<MIXED>& maps, Params& p, int kind, cudaStream_t s
       // a deal to more CTAs than this launch has would leave tiles out: those go round by number instead
       static const Deal by_number{};
       const Deal& d = deal->dealt && deal->first[workers] != p.tiles_total ? by_number : *deal;
-      return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, true, false>, maps, d, (const Params&)p);
+      if (p.cg == 2) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, 2, false>, maps, d, (const Params&)p);
+      return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, 1, false>, maps, d, (const Params&)p);
     }
   }
   static const PeerMaps no_peers{};
   const PeerMaps& pm = peer_maps ? *peer_maps : no_peers;
-  if (p.cg == 2) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, false, MIXED>, maps, pm, (const Params&)p);
-  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, false, MIXED>, maps, pm, (const Params&)p);
+  if (p.cg == 2) return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<2, 0, MIXED>, maps, pm, (const Params&)p);
+  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<1, 0, MIXED>, maps, pm, (const Params&)p);
 }
 
 void finish_tiles(Params& p) {
@@ -966,105 +1006,6 @@ static bool forward_private(Maps& mp, Params& p, int l, const RowparShapes& s, v
   return make_cmap(&mp.c[g], zp, s.h - s.S_lo, s.T, s.t, s.P, (long long)s.T * s.P, false);
 }
 
-// When the products of a block's two layers share a launch (units of 0.2 us): a launch of its own is worth kLaunchGap, the
-// shared one has to win by kMargin, and it has to be shorter than kLongest.
-constexpr double kLaunchGap = 12, kMargin = 1.05, kLongest = 1200;
-
-// Both layers' forward products of a block (they do not depend on each other): one launch where the cost model sees a
-// gain - one ramp, one tail and a finer deal where a layer's tiles do not fill the GPU - else one after the other.  Each
-// layer keeps the rank groups that it would have alone, so its sums do not depend on the schedule.
-// The rule: a launch of its own costs 2.4 us; against that, one launch has to be cheaper than the two by 5 % of its own
-// time, which is what it loses to the model when both layers' operands go through L2 and only one tile width is left to
-// choose.  Block forward on either side of the line (apart / merged, us): taken - h 768, 300 tokens 21.9 / 14.9; h 2048,
-// 300 tokens 44.0 / 38.8, 2000 tokens 147 / 143; h 4096, 600 tokens 153 / 147, 3000 tokens 571 / 539; not taken - h 4096,
-// 1400 tokens 273 / 285; h 5120, 1000 tokens 306 / 312; h 4096, p = 0.75 on 2 ranks, 300 tokens 75 / 87; long launches (see
-// the backward's) - h 4096, 8192 tokens 1389 / 1394, whole step 3810 / 3832, 65536 tokens of 4 x 768 2309 / 2337.
-cudaError_t launch_tc_forward_block(const RowparShapes* s, const void* const* Y, const void* const* W, void* const* zs,
-                                    void* const* zp, void* const* planes, const int* max_groups, int* groups, cudaStream_t st) {
-  const ForwardPlan one[2] = {forward_plan(s[0], planes[0] ? max_groups[0] : 1), forward_plan(s[1], planes[1] ? max_groups[1] : 1)};
-  const int ks[2] = {(s[0].K_r + BK - 1) / BK, (s[1].K_r + BK - 1) / BK};
-  const int lead = ks[1] * one[1].qper >= ks[0] * one[0].qper ? 1 : 0;        // the layer with the longer shared tiles
-  RegionShape rs[4];
-  for (int i = 0; i < 2; ++i) {
-    const int l = i == 0 ? lead : 1 - lead;
-    rs[i] = RegionShape{s[l].T, s[l].S, one[l].groups, ks[l] * one[l].qper};
-    rs[2 + i] = RegionShape{s[l].T, s[l].S < s[l].h ? s[l].h - s[l].S_lo : 0, s[l].t, ks[l]};
-  }
-  TileCfg both = pick_tile(rs, 4, false, 1, 0.0);
-  for (int l = 0; l < 2; ++l) both.cost += plane_cost(s[l], one[l].groups);
-  if (both.cost * kMargin >= one[0].tile.cost + one[1].tile.cost + kLaunchGap || both.cost >= kLongest) {
-    for (int l = 0; l < 2; ++l) {
-      const cudaError_t e = launch_tc_forward(s[l], Y[l], W[l], zs[l], zp[l], st, nullptr, planes[l], max_groups[l], &groups[l]);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-  }
-  Maps mp;
-  Params p{};
-  p.BN = both.bn; p.cg = both.cg; p.splits = 1;
-  for (int l = 0; l < 2; ++l) {
-    groups[l] = one[l].groups;
-    if (!forward_maps(mp, l, s[l], Y[l], W[l], p)) return cudaErrorInvalidValue;
-  }
-  for (int i = 0; i < 2; ++i) {
-    const int l = i == 0 ? lead : 1 - lead;
-    if (s[l].S > 0 && !forward_shared(mp, p, l, s[l], zs[l], planes[l], one[l].groups, one[l].qper)) return cudaErrorInvalidValue;
-  }
-  for (int i = 0; i < 2; ++i) {
-    const int l = i == 0 ? lead : 1 - lead;
-    if (s[l].S < s[l].h && !forward_private(mp, p, l, s[l], zp[l])) return cudaErrorInvalidValue;
-  }
-  finish_tiles(p);
-  return launch(mp, p, CAAT_K_TC_FORWARD, st);
-}
-
-int tc_forward_groups(const RowparShapes& s, int max_groups) { return forward_plan(s, max_groups).groups; }
-
-cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* W, void* zs, void* zp,
-                              cudaStream_t st, const PushTarget* push, void* planes, int max_groups, int* groups_out) {
-  Maps mp;
-  CUtensorMap *maps = mp.ab, *cmaps = mp.c;
-  PeerMaps pmaps{};
-  Params p{};
-  const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
-  const ForwardPlan plan = forward_plan(s, planes ? max_groups : 1);
-  const int groups = plan.groups, qper = plan.qper;
-  p.BN = plan.tile.bn; p.cg = plan.tile.cg;
-  if (groups_out) *groups_out = groups;
-  p.a_mn = 0; p.b_mn = 0; p.splits = 1;
-  if (!forward_maps(mp, 0, s, Y, W, p)) return cudaErrorInvalidValue;
-  maps[2] = maps[0];
-  maps[3] = maps[1];
-  if (n_sh > 0 && !forward_shared(mp, p, 0, s, zs, planes, groups, qper)) return cudaErrorInvalidValue;
-  if (n_pr > 0 && !forward_private(mp, p, 0, s, zp)) return cudaErrorInvalidValue;
-  if (push && n_sh > 0 && groups == 1) {
-    // shared tiles go to the owners' receive slots: slot `rank` of GPU q is [slice, S] 16-bit elements; the map of
-    // owner q covers only the tokens q really owns, so rows past the end of a ragged last slice are clipped
-    if (push->world < 1 || push->world > CAAT_MAX_PEERS || push->slice % (BM * p.cg) != 0) return cudaErrorInvalidValue;
-    for (int q = 0; q < push->world; ++q) {
-      long long rows = (long long)s.T - (long long)q * push->slice;
-      if (rows > push->slice) rows = push->slice;
-      if (rows < 1) { pmaps.m[q] = cmaps[0]; continue; }     // owns no token: never addressed
-      __nv_bfloat16* slot = static_cast<__nv_bfloat16*>(push->recv[q]) + (size_t)push->rank * push->slice * n_sh;
-      if (!make_cmap(&pmaps.m[q], slot, n_sh, rows, 1, n_sh, (long long)push->slice * n_sh, false)) return cudaErrorInvalidValue;
-    }
-    p.push_slice = push->slice;
-  }
-  finish_tiles(p);
-  const cudaError_t e = launch(mp, p, CAAT_K_TC_FORWARD, st, push && n_sh > 0 && groups == 1 ? &pmaps : nullptr);
-  if (e != cudaSuccess || groups == 1 || groups_out) return e;
-  const long long n8 = (long long)s.T * s.S_hi / 8;
-  const int blocks = (int)((n8 + 255) / 256 < 8 * sm_count() ? (n8 + 255) / 256 : 8 * sm_count());
-  LaunchScope scope(CAAT_K_SPLITK_REDUCE, st);
-  SlotTarget slots{};
-  if (push) {
-    slots.slice = push->slice; slots.rank = push->rank;
-    for (int q = 0; q < push->world; ++q) slots.recv[q] = static_cast<uint4*>(push->recv[q]);
-  }
-  return launch_pdl(sum_groups_kernel, dim3(blocks), dim3(256), 0, st, static_cast<const float4*>(planes), static_cast<uint4*>(zs),
-                    s.T, s.S_hi / 8, groups, slots);
-}
-
 // ---- few tokens: the operands are swapped (weights on the 128-row side, tokens on the narrow side), so that a tile streams
 // 128 weight rows however few tokens there are, and the sums leave as fp32 planes for the row kernel:
 //   zs[g][i][l]  l < S     sum over the g-th group of qper ranks (qper = 0: one plane per rank and k-split)
@@ -1088,7 +1029,7 @@ constexpr double kLoneStepUs = 0.27, kSplitUs = 0.3;
 struct FewRun { float len; int first, step, run, n; };
 struct FewTiles { int nruns, tiles; FewRun r[12]; };
 
-FewTiles few_tiles(int t, int h, int S, const int* K_r, int n, const FewSplit* sp) {
+FewTiles few_tiles(int t, int h, int S, const int* K_r, int n, const FewSplit* sp, int rows = BM, int ncols = 1, double overhead = kItemOverhead) {
   FewTiles f{};
   const int S_lo = round_down(S, kLayoutVec);
   for (int g = 0; g < n; ++g) {
@@ -1098,17 +1039,17 @@ FewTiles few_tiles(int t, int h, int S, const int* K_r, int n, const FewSplit* s
       if (M <= 0) continue;
       const bool grouped = part == 0 && sp[g].qper > 0;
       const int splits = grouped ? (t + sp[g].qper - 1) / sp[g].qper : sp[g].ksplits;
-      const int outer = (M + BM - 1) / BM * (grouped ? 1 : t);
+      const int outer = (M + rows - 1) / rows * (grouped ? 1 : t);
       // a split is `per` pieces of `unit` k-steps long; the last one may be shorter, and those of a k-split past it are empty
       const int pieces = grouped ? t : ks, unit = grouped ? ks : 1, per = grouped ? sp[g].qper : (ks + splits - 1) / splits;
       const int full = pieces / per, rest = pieces - full * per, used = full + (rest > 0);
       auto add = [&](int split, int count, int length) {
-        if (count > 0) f.r[f.nruns++] = FewRun{(float)(length * unit + kItemOverhead), f.tiles + split, splits, count, outer};
+        if (count > 0) f.r[f.nruns++] = FewRun{(float)(length * unit + overhead), f.tiles + split * ncols, splits * ncols, count * ncols, outer};
       };
       add(0, full, per);
       add(full, used - full, rest);
       add(used, splits - used, 0);
-      f.tiles += outer * splits;
+      f.tiles += outer * splits * ncols;
     }
   }
   std::sort(f.r, f.r + f.nruns, [](const FewRun& x, const FewRun& y) { return x.len > y.len || (x.len == y.len && x.first < y.first); });
@@ -1267,6 +1208,193 @@ void few_plan_cached(int t, int T, int h, int S, const int* K_r, int n, FewPlan*
   used[i] = ++clock;
 }
 }  // namespace
+
+// ---- a block's products with some hundreds of tokens: weights on the row side of a CTA pair's 256-row tiles, up to 256 tokens on
+// the column side, both layers in one launch, tiles dealt by length.  With tokens on the row side a tile is at least 128
+// tokens high and every one of them streams the weights again; what bounds these calls is the operand bytes from L2 (300
+// tokens of 8 x 4096: 550 MB, here 390 MB).  Outputs as in the normal forward: zs and zp, or fp32 planes of the shared part over
+// groups of ranks.  The groups are the normal forward's and every output's products are added in the same order, so the sums are
+// the same bits either way.
+// The rule: cheaper than the two layers' tiles by 5 % of the models' figures, and not so short that the launch alone decides.
+// Block forward on either side of the line, tokens on the rows / here, us: taken - 8 x 4096, 200 tokens 72.5 / 59.6, 300 tokens
+// 88.1 / 74.7, 400 tokens 93.6 / 88.0, nothing shared 78.3 / 69.9; 8 x 5120, 200 tokens 99.3 / 80.2, 300 tokens 118 / 106; 2 x 3072,
+// 300 tokens 50.6 / 37.6; 8 x 2048, 65 tokens 17.9 / 17.9, 300 tokens 37.6 / 34.2; 4 x 1536, 400 tokens 29.4 / 25.2; not taken -
+// 4 x 768, 65 tokens 15.5 / 16.8, 300 tokens 14.6 / 15.0 (short); 2 x 3072, 256 tokens 33.6 / 37.2 (a whole row tile pair);
+// 8 x 2048, 100 tokens 21.1 / 21.9; 8 x 4096, everything shared, 300 tokens 77.0 / 78.5.
+struct MidPlan { bool use; int bn, ncols; double us; };
+
+constexpr int kMidMaxTokens = 512;
+constexpr double kMidItem = 3.0;                    // of a tile beside its k-steps, in k-steps
+constexpr double kMidMargin = 1.05, kMidShortest = 6.0;
+static double mid_step_us(int bn) { return 0.09 + 0.10 * bn / 160.0; }
+
+static int mid_workers() { return sm_count() / 2 < kMaxDealWorkers ? sm_count() / 2 : kMaxDealWorkers; }
+
+static MidPlan mid_plan(const RowparShapes* s, const ForwardPlan* f) {
+  constexpr int n = 2;
+  MidPlan m{};
+  if (s[0].T <= kDecodeMaxTokens || s[0].T > kMidMaxTokens) return m;
+  m.ncols = (s[0].T + 255) / 256;
+  m.bn = round_up((s[0].T + m.ncols - 1) / m.ncols, 32);
+  FewSplit sp[2];
+  int K[2];
+  double us = 0;
+  for (int l = 0; l < n; ++l) {
+    sp[l] = FewSplit{f[l].qper, 1};
+    K[l] = s[l].K_r;
+    us += 0.2 * plane_cost(s[l], f[l].groups);
+  }
+  const FewTiles t = few_tiles(s[0].t, s[0].h, s[0].S, K, n, sp, 2 * BM, m.ncols, kMidItem);
+  m.us = us + few_makespan(t, mid_workers()) * mid_step_us(m.bn);
+  m.use = t.tiles <= kMaxDealItems && m.us >= kMidShortest && m.us * kMidMargin < 0.2 * (f[0].tile.cost + f[1].tile.cost);
+  return m;
+}
+
+static cudaError_t launch_mid(const RowparShapes* s, const MidPlan& m, const ForwardPlan* fp, const void* const* Y, const void* const* W,
+                              void* const* zs, void* const* zp, void* const* planes, cudaStream_t st) {
+  constexpr int n = 2;
+  Maps mp;
+  Params p{};
+  p.BN = m.bn; p.cg = 2; p.splits = 1;
+  FewSplit sp[2];
+  int K[2];
+  for (int l = 0; l < n; ++l) {
+    const int ks = (s[l].K_r + BK - 1) / BK;
+    K[l] = s[l].K_r;
+    sp[l] = FewSplit{fp[l].qper, 1};
+    if (!make_map(&mp.ab[2 * l], W[l], s[l].K_r, s[l].h, s[l].t, s[l].K_r, (long long)s[l].h * s[l].K_r, BK, BM) ||
+        !make_map(&mp.ab[2 * l + 1], Y[l], s[l].K_r, s[l].T, s[l].t, s[l].K_r, (long long)s[l].T * s[l].K_r, BK, p.BN / 2))
+      return cudaErrorInvalidValue;
+    if (s[l].S > 0) {
+      Region& r = p.r[p.nregions++];
+      r.nunits = 1;
+      r.u[0] = Unit{2 * l, 2 * l + 1, 0, 0, 0, 0, 0, 1, 0, 1, s[l].t, ks};
+      r.M = s[l].S; r.N = s[l].T; r.batch = 1; r.b_slowest = 1;
+      r.splits = fp[l].groups; r.qper = fp[l].groups > 1 ? fp[l].qper : 0;
+      r.out_f32 = fp[l].groups > 1;
+      r.out_t = static_cast<float*>(r.out_f32 ? planes[l] : zs[l]); r.out_ld = s[l].S_hi;
+    }
+    if (s[l].S < s[l].h) {
+      Region& r = p.r[p.nregions++];
+      r.nunits = 1;
+      r.u[0] = Unit{2 * l, 2 * l + 1, 0, s[l].S_lo, 0, 0, 1, 0, 1, 0, 1, ks};
+      r.M = s[l].P; r.N = s[l].T; r.batch = s[l].t; r.b_slowest = 1;
+      r.splits = 1;
+      r.out_t = static_cast<float*>(zp[l]); r.out_ld = s[l].P;
+    }
+  }
+  for (CUtensorMap& c : mp.c) c = mp.ab[0];          // unused: the epilogue stores directly
+  finish_tiles(p);
+  static thread_local Deal deal;
+  deal.dealt = 0;
+  const FewTiles f = few_tiles(s[0].t, s[0].h, s[0].S, K, n, sp, 2 * BM, m.ncols, kMidItem);
+  if (f.tiles > mid_workers() && f.tiles <= kMaxDealItems) few_deal(f, mid_workers(), &deal);
+  return launch(mp, p, CAAT_K_TC_FORWARD, st, nullptr, &deal);
+}
+
+// When the products of a block's two layers share a launch (units of 0.2 us): a launch of its own is worth kLaunchGap, the
+// shared one has to win by kMargin, and it has to be shorter than kLongest.
+constexpr double kLaunchGap = 12, kMargin = 1.05, kLongest = 1200;
+
+// Both layers' forward products of a block (they do not depend on each other): one launch where the cost model sees a
+// gain - one ramp, one tail and a finer deal where a layer's tiles do not fill the GPU - else one after the other.  Each
+// layer keeps the rank groups that it would have alone, so its sums do not depend on the schedule.
+// The rule: a launch of its own costs 2.4 us; against that, one launch has to be cheaper than the two by 5 % of its own
+// time, which is what it loses to the model when both layers' operands go through L2 and only one tile width is left to
+// choose.  Block forward on either side of the line (apart / merged, us): taken - h 768, 300 tokens 21.9 / 14.9; h 2048,
+// 300 tokens 44.0 / 38.8, 2000 tokens 147 / 143; h 4096, 600 tokens 153 / 147, 3000 tokens 571 / 539; not taken - h 4096,
+// 1400 tokens 273 / 285; h 5120, 1000 tokens 306 / 312; h 4096, p = 0.75 on 2 ranks, 300 tokens 75 / 87; long launches (see
+// the backward's) - h 4096, 8192 tokens 1389 / 1394, whole step 3810 / 3832, 65536 tokens of 4 x 768 2309 / 2337.
+cudaError_t launch_tc_forward_block(const RowparShapes* s, const void* const* Y, const void* const* W, void* const* zs,
+                                    void* const* zp, void* const* planes, const int* max_groups, int* groups, cudaStream_t st) {
+  const ForwardPlan one[2] = {forward_plan(s[0], planes[0] ? max_groups[0] : 1), forward_plan(s[1], planes[1] ? max_groups[1] : 1)};
+  const MidPlan mid = mid_plan(s, one);
+  if (mid.use) {
+    for (int l = 0; l < 2; ++l) groups[l] = one[l].groups;
+    return launch_mid(s, mid, one, Y, W, zs, zp, planes, st);
+  }
+  const int ks[2] = {(s[0].K_r + BK - 1) / BK, (s[1].K_r + BK - 1) / BK};
+  const int lead = ks[1] * one[1].qper >= ks[0] * one[0].qper ? 1 : 0;        // the layer with the longer shared tiles
+  RegionShape rs[4];
+  for (int i = 0; i < 2; ++i) {
+    const int l = i == 0 ? lead : 1 - lead;
+    rs[i] = RegionShape{s[l].T, s[l].S, one[l].groups, ks[l] * one[l].qper};
+    rs[2 + i] = RegionShape{s[l].T, s[l].S < s[l].h ? s[l].h - s[l].S_lo : 0, s[l].t, ks[l]};
+  }
+  TileCfg both = pick_tile(rs, 4, false, 1, 0.0);
+  for (int l = 0; l < 2; ++l) both.cost += plane_cost(s[l], one[l].groups);
+  if (both.cost * kMargin >= one[0].tile.cost + one[1].tile.cost + kLaunchGap || both.cost >= kLongest) {
+    for (int l = 0; l < 2; ++l) {
+      const cudaError_t e = launch_tc_forward(s[l], Y[l], W[l], zs[l], zp[l], st, nullptr, planes[l], max_groups[l], &groups[l]);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
+  Maps mp;
+  Params p{};
+  p.BN = both.bn; p.cg = both.cg; p.splits = 1;
+  for (int l = 0; l < 2; ++l) {
+    groups[l] = one[l].groups;
+    if (!forward_maps(mp, l, s[l], Y[l], W[l], p)) return cudaErrorInvalidValue;
+  }
+  for (int i = 0; i < 2; ++i) {
+    const int l = i == 0 ? lead : 1 - lead;
+    if (s[l].S > 0 && !forward_shared(mp, p, l, s[l], zs[l], planes[l], one[l].groups, one[l].qper)) return cudaErrorInvalidValue;
+  }
+  for (int i = 0; i < 2; ++i) {
+    const int l = i == 0 ? lead : 1 - lead;
+    if (s[l].S < s[l].h && !forward_private(mp, p, l, s[l], zp[l])) return cudaErrorInvalidValue;
+  }
+  finish_tiles(p);
+  return launch(mp, p, CAAT_K_TC_FORWARD, st);
+}
+
+int tc_forward_groups(const RowparShapes& s, int max_groups) { return forward_plan(s, max_groups).groups; }
+
+cudaError_t launch_tc_forward(const RowparShapes& s, const void* Y, const void* W, void* zs, void* zp,
+                              cudaStream_t st, const PushTarget* push, void* planes, int max_groups, int* groups_out) {
+  Maps mp;
+  CUtensorMap *maps = mp.ab, *cmaps = mp.c;
+  PeerMaps pmaps{};
+  Params p{};
+  const int n_sh = s.S, n_pr = s.S < s.h ? s.h - s.S_lo : 0;
+  const ForwardPlan plan = forward_plan(s, planes ? max_groups : 1);
+  const int groups = plan.groups, qper = plan.qper;
+  p.BN = plan.tile.bn; p.cg = plan.tile.cg;
+  if (groups_out) *groups_out = groups;
+  p.a_mn = 0; p.b_mn = 0; p.splits = 1;
+  if (!forward_maps(mp, 0, s, Y, W, p)) return cudaErrorInvalidValue;
+  maps[2] = maps[0];
+  maps[3] = maps[1];
+  if (n_sh > 0 && !forward_shared(mp, p, 0, s, zs, planes, groups, qper)) return cudaErrorInvalidValue;
+  if (n_pr > 0 && !forward_private(mp, p, 0, s, zp)) return cudaErrorInvalidValue;
+  if (push && n_sh > 0 && groups == 1) {
+    // shared tiles go to the owners' receive slots: slot `rank` of GPU q is [slice, S] 16-bit elements; the map of
+    // owner q covers only the tokens q really owns, so rows past the end of a ragged last slice are clipped
+    if (push->world < 1 || push->world > CAAT_MAX_PEERS || push->slice % (BM * p.cg) != 0) return cudaErrorInvalidValue;
+    for (int q = 0; q < push->world; ++q) {
+      long long rows = (long long)s.T - (long long)q * push->slice;
+      if (rows > push->slice) rows = push->slice;
+      if (rows < 1) { pmaps.m[q] = cmaps[0]; continue; }     // owns no token: never addressed
+      __nv_bfloat16* slot = static_cast<__nv_bfloat16*>(push->recv[q]) + (size_t)push->rank * push->slice * n_sh;
+      if (!make_cmap(&pmaps.m[q], slot, n_sh, rows, 1, n_sh, (long long)push->slice * n_sh, false)) return cudaErrorInvalidValue;
+    }
+    p.push_slice = push->slice;
+  }
+  finish_tiles(p);
+  const cudaError_t e = launch(mp, p, CAAT_K_TC_FORWARD, st, push && n_sh > 0 && groups == 1 ? &pmaps : nullptr);
+  if (e != cudaSuccess || groups == 1 || groups_out) return e;
+  const long long n8 = (long long)s.T * s.S_hi / 8;
+  const int blocks = (int)((n8 + 255) / 256 < 8 * sm_count() ? (n8 + 255) / 256 : 8 * sm_count());
+  LaunchScope scope(CAAT_K_SPLITK_REDUCE, st);
+  SlotTarget slots{};
+  if (push) {
+    slots.slice = push->slice; slots.rank = push->rank;
+    for (int q = 0; q < push->world; ++q) slots.recv[q] = static_cast<uint4*>(push->recv[q]);
+  }
+  return launch_pdl(sum_groups_kernel, dim3(blocks), dim3(256), 0, st, static_cast<const float4*>(planes), static_cast<uint4*>(zs),
+                    s.T, s.S_hi / 8, groups, slots);
+}
 
 cudaError_t launch_tc_forward_decode(int t, int T, int h, int S, DecodeProblem* pr, int n, cudaStream_t st) {
   if (n < 1 || n > 2) return cudaErrorInvalidValue;
