@@ -16,7 +16,8 @@
 //
 // A value below 2^-110 loses the bits of its last part that bf16 cannot hold.  A result that is not finite is computed
 // again from the operands with plain FMAs (an infinity times a part that is zero would turn into NaN), so infinities and
-// NaN come out as a chain of FMAs gives them.
+// NaN come out as chains of FMAs give them.  The epilogue only marks such a tile; a CTA goes over its marked tiles when its
+// products are complete and no role waits for another (redo_tile).
 //
 // Persistent CTAs, one per SM:
 //   warps 8..23  load fp32 operands (eight warps each; any of the two majors, 16-byte or element-wise), split them in
@@ -53,7 +54,10 @@ constexpr int kEpiWarps = 8, kProdWarp0 = 8, kProdWarps = 16, kMmaWarp = 24;
 // Seven warpgroups at 72 registers; B's producers and the last group (the issuing warp and three idle ones) give up what
 // the epilogue's two take: 2 x 96 + 2 x 72 + 2 x 64 + 40 = 7 x 72.
 constexpr int kThreads = 896;
-template <int CG> constexpr int kSmem = kStages<CG> * kStageBytes<CG> + 1024 + 256;
+// behind the ring: barriers, the tensor-memory address and the abort flag; then a bit per item (or group of items)
+constexpr int kBarBytes = 256, kMarkWords = 64;
+template <int CG> constexpr int kBars = 2 * kStages<CG> + 2 * kAccs + 3;
+template <int CG> constexpr int kSmem = kStages<CG> * kStageBytes<CG> + 1024 + kBarBytes + 4 * kMarkWords;
 constexpr uint32_t kSpinCap = 1u << 22;
 
 struct XSeg {                 // one segment of the contraction: A(b, q, row, k) and B(b, q, col, k)
@@ -169,23 +173,6 @@ __device__ __forceinline__ uint32_t piece_offset(int tid, int u) {
   return (uint32_t)((c >> 3) * (64 * XK * 2) + k * 128 + (((c & 7) ^ (k & 7)) << 4));
 }
 
-// one output from the operands, a chain of FMAs (results that are not finite)
-template <bool AK, bool BKM>
-__device__ __noinline__ float plain_dot(const XProblem& g, int b, int i, int j) {
-  float acc = 0.f;
-  for (int s = 0; s < g.nseg; ++s) {
-    const XSeg& e = g.seg[s];
-    for (int q = 0; q < e.Q; ++q) {
-      const float* A = e.A + b * e.sAb + q * e.sAq + (AK ? i * e.sAl : (long long)i);
-      const float* B = e.B + b * e.sBb + q * e.sBq + (BKM ? j * e.sBl : (long long)j);
-      for (int k = 0; k < e.Kd; ++k) {
-        acc = fmaf(A[AK ? (long long)k : k * e.sAl], B[BKM ? (long long)k : k * e.sBl], acc);
-        if (acc != acc) return acc;
-      }
-    }
-  }
-  return acc;
-}
 __device__ __forceinline__ bool not_finite(float x) { return !(fabsf(x) <= FLT_MAX); }
 
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t cap) {
@@ -205,6 +192,133 @@ __device__ __forceinline__ bool epi_all(bool ok) {       // barrier with a vote
   asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %1, 0;\n barrier.red.and.pred q, 1, %2, p;\n selp.s32 %0, 1, 0, q;\n}"
                : "=r"(r) : "r"((int)ok), "n"(kEpiWarps * 32) : "memory");
   return r != 0;
+}
+
+// ------------------------------------------------------------------ results that are not finite
+// the mark of a CTA's item: its number among the CTA's, several to a mark where there are more items than marks
+__device__ __forceinline__ int mark_of(int items, int n, int worker, int nworkers) {
+  int shift = 0;
+  while (items / nworkers >> shift >= 32 * kMarkWords) ++shift;
+  return (n - worker) / nworkers >> shift;
+}
+template <int BYTES>
+__device__ __forceinline__ void cp_async(uint32_t dst, const float* src, int bytes) {      // zeros behind the first `bytes`
+  if (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+// ROWS x 64 elements of an operand into [k][row] by 256 threads.  k contiguous: a warp copies 8 k of 4 rows at a time, whole sectors
+// into 32 banks (LD is 4 more than a multiple of 32).
+template <bool KM, bool VEC, int ROWS, int LD>
+__device__ __forceinline__ void redo_load(uint32_t dst, const float* p, long long ld, int rows, int k_left, int tid) {
+  constexpr int W = VEC && !KM ? 4 : 1, LANES = ROWS / W;               // elements of a copy, copies of a k
+  constexpr int STEP = KM ? 4 : 256 / LANES, N = KM ? ROWS / 4 : XK / STEP;
+  const int k = KM ? (tid >> 5) * 8 + (tid & 7) : tid / LANES, r = KM ? tid >> 3 & 3 : tid % LANES * W;
+  const int slow = KM ? r : k, slow_end = KM ? rows : k_left;
+  const int left = KM ? k_left - k : rows - r, bytes = 4 * (left <= 0 ? 0 : (left < W ? left : W));
+  const float* src = p + slow * ld + (KM ? k : r);
+  dst += (uint32_t)((k * LD + r) * 4);
+#pragma unroll 4
+  for (int u = 0; u < N; ++u, src += STEP * ld, dst += STEP * (KM ? 1 : LD) * 4) {
+    const int take = slow + u * STEP < slow_end ? bytes : 0;
+    cp_async<4 * W>(dst, take ? src : p, take);
+  }
+}
+// The results of 128 rows from i0 and the columns [j0, j1) that are not finite, from the operands by chains of FMAs.  The
+// epilogue's 256 threads, 64 columns at a time, 8 x 4 results per thread, both operands two chunks deep in `stage` (the ring).  A
+// warp whose 16 rows need nothing (finite, or NaN by now) only helps to load.  Two warps per scheduler bound it, and the few CTAs
+// that hold marked tiles.  A training step of one layer, CUDA cores (any data) / here with finite data / one infinite token / one
+// infinite value / all infinite, us: 4 x 768, 2000 tokens 827 / 263 / 484 / 733 / 832; 4 x 768, 8192 tokens 3197 / 917 / 1641 /
+// 1815 / 3029; 2 x 1024, 300 tokens 296 / 128 / 267 / 592 / 753; 8 x 5120, 100 tokens 1585 / 531 / 1486 / 2708 / 2972.
+constexpr int kRedoCols = 64, kRedoLdA = XM + 4, kRedoLdB = kRedoCols + 4, kRedoStage = XK * (kRedoLdA + kRedoLdB);
+static_assert(2 * kRedoStage * 4 <= kStages<2> * kStageBytes<2> && XM * kRedoCols == 32 * 256, "");
+
+template <bool AK, bool BKM, bool VEC>
+__device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int j0, int j1, float* stage, int tid) {
+  const int r8 = (tid >> 4) * 8, c4 = (tid & 15) * 4;
+  if (j1 > g.N) j1 = g.N;
+  for (int jc = j0; jc < j1; jc += kRedoCols) {
+    float* out = g.C + b * g.sCb + (i0 + r8) * g.sCi + (jc + c4) * g.sCj;
+    uint32_t todo = 0;                               // results of this thread that are not finite
+#pragma unroll 4
+    for (int e = 0; e < 32; ++e)
+      if (i0 + r8 + (e >> 2) < g.M && jc + c4 + (e & 3) < j1 && not_finite(out[(e >> 2) * g.sCi + (e & 3) * g.sCj])) todo |= 1u << e;
+    bool idle = __all_sync(0xffffffffu, todo == 0);
+    if (epi_all(idle)) continue;
+    auto load = [&](int n) {
+      const KPos pos = kpos_at(g, n);
+      const XSeg& s = g.seg[pos.seg];
+      const float* A = s.A + b * s.sAb + pos.q * s.sAq + (AK ? i0 * s.sAl + pos.k0 : pos.k0 * s.sAl + i0);
+      const float* B = s.B + b * s.sBb + pos.q * s.sBq + (BKM ? jc * s.sBl + pos.k0 : pos.k0 * s.sBl + jc);
+      const uint32_t dst = smem_u32(stage + (n & 1) * kRedoStage);
+      redo_load<AK, VEC, XM, kRedoLdA>(dst, A, s.sAl, g.M - i0, s.Kd - pos.k0, tid);
+      redo_load<BKM, VEC, kRedoCols, kRedoLdB>(dst + XK * kRedoLdA * 4, B, s.sBl, g.N - jc, s.Kd - pos.k0, tid);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc[32];
+#pragma unroll
+    for (int e = 0; e < 32; ++e) acc[e] = 0.f;
+    load(0);
+#pragma unroll 1
+    for (int n = 0; n < g.chunks; ++n) {
+      if (n + 1 < g.chunks) {
+        load(n + 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      epi_sync();
+      if (!idle) {
+        const float* A = stage + (n & 1) * kRedoStage + r8;
+        const float* B = stage + (n & 1) * kRedoStage + XK * kRedoLdA + c4;
+#pragma unroll 2
+        for (int k = 0; k < XK; ++k, A += kRedoLdA, B += kRedoLdB) {
+          const float4 a = *reinterpret_cast<const float4*>(A), c = *reinterpret_cast<const float4*>(A + 4);
+          const float4 v = *reinterpret_cast<const float4*>(B);
+          const float x[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w}, y[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int e = 0; e < 32; ++e) acc[e] = fmaf(x[e >> 2], y[e & 3], acc[e]);
+        }
+        uint32_t open = 0;                           // a sum that is NaN stays NaN
+#pragma unroll
+        for (int e = 0; e < 32; ++e) open |= acc[e] == acc[e] ? 1u << e : 0u;
+        idle = __all_sync(0xffffffffu, (todo & open) == 0);
+      }
+      if (epi_all(idle)) break;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    epi_sync();                                      // the next columns' copies go where these were read, or still land
+#pragma unroll
+    for (int e = 0; e < 32; ++e)
+      if (todo >> e & 1u) out[(e >> 2) * g.sCi + (e & 3) * g.sCj] = acc[e];
+  }
+}
+
+// The epilogue's last step, when every product of the CTA is complete: its ring is idle, and nobody waits for these warps but
+// barriers without a limit.  Reads its place anew, so that the loop before it keeps no registers for it.
+__device__ __forceinline__ uint8_t* ring_base() {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+}
+template <int CG, bool AK, bool BKM, bool VEC>
+__device__ __forceinline__ void redo_marked(const XParams& p) {
+  uint32_t tid, block, blocks;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+  asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
+  asm volatile("mov.u32 %0, %%nctaid.x;" : "=r"(blocks));
+  uint8_t* base = ring_base();
+  const unsigned int* marks = reinterpret_cast<const unsigned int*>(base + kStages<CG> * kStageBytes<CG> + kBarBytes);
+  const volatile int* aborted = reinterpret_cast<const volatile int*>(base + kStages<CG> * kStageBytes<CG> + 8 * kBars<CG> + 4);
+  epi_sync();                                        // the marks are complete; a wait that ran out has raised the flag
+  if (epi_all(tid >= kMarkWords || marks[tid % kMarkWords] == 0 || *aborted)) return;
+  const int ctas = p.csize * CG, cta = ctas > 1 ? (int)cluster_ctarank() : 0, crank = cta / CG;
+  const int worker = block / ctas, nworkers = blocks / ctas;
+  for (int n = worker; n < p.items; n += nworkers) {
+    const int m = mark_of(p.items, n, worker, nworkers);
+    const Item it = item_at<CG>(p, n, crank);
+    if (!(marks[m >> 5] >> (m & 31) & 1u) || !it.valid) continue;
+    const int cw = XN / p.csize, j0 = it.split ? it.j0 + crank * cw : it.j0;      // the columns that this CTA stored
+    redo_tile<AK, BKM, VEC>(p.p[it.prob], it.b, it.i0 + cta % CG * XM, j0, it.split ? j0 + cw : j0 + XN, reinterpret_cast<float*>(base), tid);
+  }
 }
 
 // ------------------------------------------------------------------ producers
@@ -300,19 +414,20 @@ __device__ __forceinline__ void produce(const XParams& p, int tid, int worker, i
 // AK / BKM: k is the contiguous axis of A / B (else its rows are)
 template <int CG, bool AK, bool BKM, bool VEC>
 __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_constant__ XParams p) {
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* base = ring_base();
   const uint32_t ring = smem_u32(base);
   // behind the ring: full, empty (a stage each), tfull[4], tempty[4], ready, data, done, tensor-memory address, abort flag
   const uint32_t full0 = ring + kStages<CG> * kStageBytes<CG>, empty0 = full0 + 8 * kStages<CG>, tfull0 = empty0 + 8 * kStages<CG>;
   const uint32_t tempty0 = tfull0 + 8 * kAccs, ready = tempty0 + 8 * kAccs, data = ready + 8, done = data + 8;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + kStages<CG> * kStageBytes<CG> + 8 * (2 * kStages<CG> + 2 * kAccs + 3));
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + kStages<CG> * kStageBytes<CG> + 8 * kBars<CG>);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  unsigned int* marks = reinterpret_cast<unsigned int*>(base + kStages<CG> * kStageBytes<CG> + kBarBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int csize = p.csize, ctas = csize * CG, cta = ctas > 1 ? (int)cluster_ctarank() : 0;      // of the cluster
   const int crank = cta / CG, pair_half = cta % CG, leader = cta - pair_half;
   const int worker = blockIdx.x / ctas, nworkers = gridDim.x / ctas;
 
+  if (threadIdx.x < kMarkWords) marks[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages<CG>; ++s) { mbar_init(full0 + 8 * s, kProdWarps * CG); mbar_init(empty0 + 8 * s, 1); }
     for (int a = 0; a < kAccs; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, kEpiWarps * CG); }
@@ -451,9 +566,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_cons
         if (j + 1 < g.N) { dst[g.sCj] = b; poison = fmaf(b, 0.f, poison); }
         if (j + 2 < g.N) { dst[2 * g.sCj] = c; poison = fmaf(c, 0.f, poison); }
       };
-      int jb = it.j0 + half * 64, je = jb + 64;          // the columns that this thread stores
       if (!it.split) {
         if (!ok) continue;
+        const int jb = it.j0 + half * 64;
         float* dst = crow + jb * g.sCj;
 #pragma unroll
         for (int e = 0; e < 64; e += 4, dst += 4 * g.sCj) store4(dst, jb + e, sum[e], sum[e + 1], sum[e + 2], sum[e + 3]);
@@ -480,7 +595,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_cons
         if (!epi_all(ok)) { ok = false; break; }
         const float* part = reinterpret_cast<const float*>(base) + row;
         const int c0 = half * (cw / 2);
-        jb = it.j0 + crank * cw + c0; je = jb + cw / 2;
         for (int c = c0; c < c0 + cw / 2; c += 4) {
           float s[4] = {0.f, 0.f, 0.f, 0.f};
           for (int src = 0; src < csize; ++src)
@@ -491,11 +605,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_cons
         epi_sync();
         if (threadIdx.x == 0) mbar_arrive(done);
       }
-      if (poison != poison && i < g.M)
-        for (int j = jb; j < je && j < g.N; ++j)
-          if (not_finite(crow[j * g.sCj])) crow[j * g.sCj] = plain_dot<AK, BKM>(g, it.b, i, j);
+      if (poison != poison) {
+        const int m = mark_of(p.items, n, worker, nworkers);
+        atomicOr(&marks[m >> 5], 1u << (m & 31));
+      }
     }
     if (!ok && lane == 0) { *abort_flag = 1; atomicExch(p.status, 3u); }
+    redo_marked<CG, AK, BKM, VEC>(p);
   }
 
   tc_fence_before();

@@ -72,6 +72,46 @@ def test_values_that_are_not_finite():
     assert np.isposinf(got[0, 7, 0]) and np.isnan(got[1, 140, 400]) and np.all(np.abs(got[ok] - want[ok]) <= 1e-4 * np.maximum(np.abs(want[ok]), 1))
 
 
+def _same_with_infinities(got, want, rel):
+    got, want = got.double().numpy(), want.astype(np.float32).astype(np.float64)
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isposinf(got), np.isposinf(want))
+    assert np.array_equal(np.isneginf(got), np.isneginf(want))
+    ok = np.isfinite(want)
+    assert ((got[ok] - want[ok]) ** 2).sum() ** 0.5 <= rel * (want[ok] ** 2).sum() ** 0.5
+
+
+@pytest.mark.parametrize("t,T,h,ffn,S", [
+    (4, 2000, 768, 3072, 384),      # forward: the shared part over clusters of CTAs; gradients: whole tiles of pairs
+    (2, 3000, 1024, 4096, 512),     # whole tiles of pairs, two to six a pair
+    (4, 999, 768, 3000, 285),       # element-wise loads; partial tiles of clusters of pairs in forward and weight gradient
+    (8, 300, 2048, 5632, 1024),     # more clusters' tiles than clusters
+    (2, 6000, 512, 2048, 0),        # weight gradient over clusters of pairs
+    (4, 64, 768, 3072, 384),        # data gradient over clusters of pairs; a contraction of one chunk
+])
+def test_an_infinite_token_and_channel(t, T, h, ffn, S):
+    """Whole gradients that are infinite: every tile is computed again, none of the waits around it runs out (the harness reads
+    the status), and a weight gradient keeps the sign that a chain gives."""
+    layer = caat.CAAT_MLP_DOWN
+    ctx = G.make_ctx(t, h, ffn, "f32", S=S)
+    d = _layer_case(t, T, h, ctx.k_r(layer), "f32", S, seed=T, backward=True)
+    fo = G.oracle_forward(ctx, d)
+    Hn, rstd, mean = G.saved_from_oracle(ctx, fo)
+    d["Y"][:, T // 2] = float("inf")                   # dW infinite wherever that token has a gradient
+    d["W"][0, h - 1] = float("inf")                    # a private channel of rank 0, all of dY[0]
+    with np.errstate(all="ignore"):
+        ob = G.oracle_backward(ctx, d, Hn, rstd, mean)
+    gb = G.gpu_backward(ctx, layer, d, Hn, rstd, mean)
+    assert np.isinf(ob["dW"]).all() and np.isinf(ob["dY"][0]).all()
+    for name in ("dY", "dW", "dR", "dgamma"):
+        _same_with_infinities(gb[name], ob[name], 1e-5)
+    d["Y"] = d["Y"].abs()                              # forward: a row of NaN or infinities per rank, a column of infinities
+    with np.errstate(all="ignore"):
+        fo = G.oracle_forward(ctx, d)
+    got = G.gpu_forward(ctx, layer, d)
+    assert not np.isfinite(fo["Hn"][0, :, h - 1]).any()
+    _same_with_infinities(got["Hn"], fo["Hn"], 1e-5)
+
+
 CHILD = r"""
 import torch
 from paper_2506_19645_b200 import caat, synthetic
