@@ -10,13 +10,15 @@
 // output 2.1e-7 / 1.2e-7, data gradient 3.5e-7 / 1.1e-7, weight gradient 5.7e-7 / 1.4e-7; 8 x 5120, 60 tokens, the worst of
 // the three 6.4e-7 / 1.9e-7.
 //
-// A layer's training step at 4 x 768, 2000 tokens (28 GFLOP of products): 811 -> 269 us (three ring stages per pair instead of two,
+// A layer's training step at 4 x 768, 2000 tokens (28 GFLOP of products): 811 -> 275 us (three ring stages per pair instead of two,
 // which leave the first-level cache too little: products 211 -> 230 us).  What bounds a
 // stage (2.4 to 4 k cycles where its 24 products take 1.5 k) is the way round: loads, split, stores, barrier, products, barrier.
 //
-// A value below 2^-110 loses the bits of its last part that bf16 cannot hold.  A result that is not finite is computed
-// again from the operands with plain FMAs (an infinity times a part that is zero would turn into NaN), so infinities and
-// NaN come out as chains of FMAs give them.  The epilogue only marks such a tile; a CTA goes over its marked tiles when its
+// Operands are multiplied by 2^16 on their way into parts and the accumulators' sums by 2^-32 where they are added up, both
+// exact: an operand below 2^-110 would lose the last part's bits under bf16's smallest number (2^-133); so every fp32 number
+// keeps all of them.  A result that is not finite is computed again from the operands with FMAs: sums of 2^96 and more,
+// which overflow in the accumulator, and infinities and NaN, which come out as chains of FMAs give them (an infinity times a
+// part that is zero would turn into NaN).  The epilogue only marks such a tile; a CTA goes over its marked tiles when its
 // products are complete and no role waits for another (redo_tile).
 //
 // Persistent CTAs, one per SM:
@@ -142,6 +144,7 @@ __device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
   const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&b);
 }
+constexpr float kScale = 65536.f;
 // the three parts of eight elements, stored at the same place of the three part tiles
 __device__ __forceinline__ float2 less(float2 x, uint32_t part) {      // x minus a pair of parts: exact
   return __ffma2_rn(make_float2(__uint_as_float(part << 16), __uint_as_float(part & 0xffff0000u)), make_float2(-1.f, -1.f), x);
@@ -152,8 +155,8 @@ __device__ __forceinline__ void split_store(const float (&v)[8], uint32_t dst) {
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     float2 x = make_float2(v[2 * q], v[2 * q + 1]);
-    h[q] = bf16x2(x.x, x.y);
-    x = less(x, h[q]);
+    h[q] = bf16x2(x.x * kScale, x.y * kScale);
+    x = make_float2(fmaf(x.x, kScale, -__uint_as_float(h[q] << 16)), fmaf(x.y, kScale, -__uint_as_float(h[q] & 0xffff0000u)));
     m[q] = bf16x2(x.x, x.y);
     x = less(x, m[q]);
     l[q] = bf16x2(x.x, x.y);
@@ -223,25 +226,25 @@ __device__ __forceinline__ void redo_load(uint32_t dst, const float* p, long lon
     cp_async<4 * W>(dst, take ? src : p, take);
   }
 }
-// The results of 128 rows from i0 and the columns [j0, j1) that are not finite, from the operands by chains of FMAs.  The
-// epilogue's 256 threads, 64 columns at a time, 8 x 4 results per thread, both operands two chunks deep in `stage` (the ring).  A
-// warp whose 16 rows need nothing (finite, or NaN by now) only helps to load.  Two warps per scheduler bound it, and the few CTAs
-// that hold marked tiles.  A training step of one layer, CUDA cores (any data) / here with finite data / one infinite token / one
-// infinite value / all infinite, us: 4 x 768, 2000 tokens 827 / 263 / 484 / 733 / 832; 4 x 768, 8192 tokens 3197 / 917 / 1641 /
-// 1815 / 3029; 2 x 1024, 300 tokens 296 / 128 / 267 / 592 / 753; 8 x 5120, 100 tokens 1585 / 531 / 1486 / 2708 / 2972.
-constexpr int kRedoCols = 64, kRedoLdA = XM + 4, kRedoLdB = kRedoCols + 4, kRedoStage = XK * (kRedoLdA + kRedoLdB);
-static_assert(2 * kRedoStage * 4 <= kStages<2> * kStageBytes<2> && XM * kRedoCols == 32 * 256, "");
+// The results of 128 rows from i0 and the columns [j0, j1) that are not finite, from the operands by chains of 64 FMAs, added up in
+// fp32.  The epilogue's 256 threads, 32 columns at a time, 4 x 4 results per thread, both operands two chunks deep in `stage`
+// (the ring).  A warp whose 16 rows need nothing (finite, or NaN by now) only helps to load.  Two warps per scheduler bound it,
+// and the few CTAs that hold marked tiles.  A training step of one layer, CUDA cores (any data) / here with one infinite token / one
+// infinite value / all infinite, us: 4 x 768, 2000 tokens 827 / 519 / 694 / 979; 4 x 768, 8192 tokens 3197 / 1808 / 2072 / 3769;
+// 2 x 1024, 300 tokens 296 / 272 / 506 / 607; 8 x 5120, 100 tokens 1585 / 1624 / 2520 / 2952.
+constexpr int kRedoCols = 32, kRedoLdA = XM + 4, kRedoLdB = kRedoCols + 4, kRedoStage = XK * (kRedoLdA + kRedoLdB);
+static_assert(2 * kRedoStage * 4 <= kStages<2> * kStageBytes<2> && XM * kRedoCols == 16 * 256, "");
 
 template <bool AK, bool BKM, bool VEC>
 __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int j0, int j1, float* stage, int tid) {
-  const int r8 = (tid >> 4) * 8, c4 = (tid & 15) * 4;
+  const int r4 = (tid >> 3) * 4, c4 = (tid & 7) * 4;
   if (j1 > g.N) j1 = g.N;
   for (int jc = j0; jc < j1; jc += kRedoCols) {
-    float* out = g.C + b * g.sCb + (i0 + r8) * g.sCi + (jc + c4) * g.sCj;
+    float* out = g.C + b * g.sCb + (i0 + r4) * g.sCi + (jc + c4) * g.sCj;
     uint32_t todo = 0;                               // results of this thread that are not finite
 #pragma unroll 4
-    for (int e = 0; e < 32; ++e)
-      if (i0 + r8 + (e >> 2) < g.M && jc + c4 + (e & 3) < j1 && not_finite(out[(e >> 2) * g.sCi + (e & 3) * g.sCj])) todo |= 1u << e;
+    for (int e = 0; e < 16; ++e)
+      if (i0 + r4 + (e >> 2) < g.M && jc + c4 + (e & 3) < j1 && not_finite(out[(e >> 2) * g.sCi + (e & 3) * g.sCj])) todo |= 1u << e;
     bool idle = __all_sync(0xffffffffu, todo == 0);
     if (epi_all(idle)) continue;
     auto load = [&](int n) {
@@ -254,9 +257,9 @@ __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int 
       redo_load<BKM, VEC, kRedoCols, kRedoLdB>(dst + XK * kRedoLdA * 4, B, s.sBl, g.N - jc, s.Kd - pos.k0, tid);
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float acc[32];
+    float sum[16];
 #pragma unroll
-    for (int e = 0; e < 32; ++e) acc[e] = 0.f;
+    for (int e = 0; e < 16; ++e) sum[e] = 0.f;
     load(0);
 #pragma unroll 1
     for (int n = 0; n < g.chunks; ++n) {
@@ -268,19 +271,24 @@ __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int 
       }
       epi_sync();
       if (!idle) {
-        const float* A = stage + (n & 1) * kRedoStage + r8;
+        const float* A = stage + (n & 1) * kRedoStage + r4;
         const float* B = stage + (n & 1) * kRedoStage + XK * kRedoLdA + c4;
+        float acc[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e] = 0.f;
 #pragma unroll 2
         for (int k = 0; k < XK; ++k, A += kRedoLdA, B += kRedoLdB) {
-          const float4 a = *reinterpret_cast<const float4*>(A), c = *reinterpret_cast<const float4*>(A + 4);
-          const float4 v = *reinterpret_cast<const float4*>(B);
-          const float x[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w}, y[4] = {v.x, v.y, v.z, v.w};
+          const float4 a = *reinterpret_cast<const float4*>(A), v = *reinterpret_cast<const float4*>(B);
+          const float x[4] = {a.x, a.y, a.z, a.w}, y[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int e = 0; e < 32; ++e) acc[e] = fmaf(x[e >> 2], y[e & 3], acc[e]);
+          for (int e = 0; e < 16; ++e) acc[e] = fmaf(x[e >> 2], y[e & 3], acc[e]);
         }
         uint32_t open = 0;                           // a sum that is NaN stays NaN
 #pragma unroll
-        for (int e = 0; e < 32; ++e) open |= acc[e] == acc[e] ? 1u << e : 0u;
+        for (int e = 0; e < 16; ++e) {
+          sum[e] += acc[e];
+          open |= sum[e] == sum[e] ? 1u << e : 0u;
+        }
         idle = __all_sync(0xffffffffu, (todo & open) == 0);
       }
       if (epi_all(idle)) break;
@@ -288,8 +296,8 @@ __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int 
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     epi_sync();                                      // the next columns' copies go where these were read, or still land
 #pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (todo >> e & 1u) out[(e >> 2) * g.sCi + (e & 3) * g.sCj] = acc[e];
+    for (int e = 0; e < 16; ++e)
+      if (todo >> e & 1u) out[(e >> 2) * g.sCi + (e & 3) * g.sCj] = sum[e];
   }
 }
 
@@ -534,7 +542,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_cons
           tmem_ld16(ta + e, v);
           tmem_ld_wait();
 #pragma unroll
-          for (int k = 0; k < 16; ++k) sum[e + k] += __uint_as_float(v[k]);
+          for (int k = 0; k < 16; ++k) sum[e + k] = fmaf(__uint_as_float(v[k]), 1 / (kScale * kScale), sum[e + k]);
         }
         tc_fence_before();
         __syncwarp();

@@ -53,6 +53,24 @@ def test_no_further_from_64_bits_than_fma_chains(t, T, h, ffn, p):
         assert tensor < 2.5e-7 and tensor < 1.1 * simt
 
 
+@pytest.mark.parametrize("ey,ew", [(-120, 100), (100, -120), (-126, 0), (0, -126), (-100, -30), (-70, -70), (60, 45)])
+def test_small_and_large_operands(ey, ew):
+    """Operands near the smallest normal numbers keep all their bits, products that are not normal and sums that are large
+    come out as the CUDA cores' chains give them."""
+    t, T, h, ffn, layer, out = 4, 300, 768, 3072, caat.CAAT_MLP_DOWN, []
+    for force in (True, False):
+        ctx = G.make_ctx(t, h, ffn, "f32", p=0.5, force_simt=force)
+        d = _layer_case(t, T, h, ctx.k_r(layer), "f32", ctx.shared_channels, seed=5, backward=True)
+        Hn, rstd, mean = G.saved_from_oracle(ctx, G.oracle_forward(ctx, d))
+        d["Y"], d["W"] = torch.ldexp(d["Y"], torch.tensor(ey)), torch.ldexp(d["W"], torch.tensor(ew))
+        d["R"].zero_()
+        want = G.oracle_forward(ctx, d)["Hn"]
+        got, gb, ob = G.gpu_forward(ctx, layer, d), G.gpu_backward(ctx, layer, d, Hn, rstd, mean), G.oracle_backward(ctx, d, Hn, rstd, mean)
+        out.append([_rel(got["Hn"], want), _rel(gb["dY"], ob["dY"]), _rel(gb["dW"], ob["dW"])])
+    for simt, tensor in zip(*out):
+        assert tensor < 1.1 * simt
+
+
 def test_values_that_are_not_finite():
     """An infinite or NaN operand gives what a chain of FMAs gives, also where the other operand's lower parts are zero."""
     t, T, h, ffn, layer = 2, 300, 512, 4096, caat.CAAT_MLP_DOWN
