@@ -411,7 +411,7 @@ __device__ __forceinline__ void produce(const XParams& p, int tid, int worker, i
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
     if ((tid & 31) == 0 && !p.stall) {
-      if (CG == 2) mbar_arrive_remote(full0 + 8 * stage); else mbar_arrive(full0 + 8 * stage);
+      if (CG == 2) mbar_arrive_shared(full0 + 8 * stage); else mbar_arrive(full0 + 8 * stage);
     }
     if (++stage == kStages<CG>) { stage = 0; phase ^= 1u; }
   }

@@ -133,12 +133,21 @@ __device__ __forceinline__ uint32_t mapa_rank(uint32_t saddr, uint32_t rank) {  
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// Arrival on a barrier of another CTA of the cluster.  The first form orders what the arriving thread did for the tensor core
-// (tcgen05 accesses behind their own fence, shared memory behind a proxy fence) and costs tens of cycles; the second one
-// also makes the thread's plain writes visible to the other CTA and waits for everything the thread has in flight, global
-// loads included: 1300 to 1600 cycles.
+// Arrival on a barrier of another CTA of the cluster, by what it hands over:
+//   remote   nothing in memory.  For accumulators that were read: the loads are complete (tcgen05.wait::ld) and behind
+//            tcgen05.fence::before_thread_sync, and what the other CTA's thread issues after its wait and its
+//            tcgen05.fence::after_thread_sync comes later.  No plain access is ordered: the default scope is the CTA.
+//   shared   what was written to shared memory, by the thread or by threads that it has synchronised with: a release at the
+//            cluster's scope that is restricted to shared memory, so that it does not wait for global loads in flight.
+//   release  everything: waits for all that the thread has in flight, 1300 to 1600 cycles where that is global loads.
+// In a loop that fills operand stages from global memory (fp32 products of a step at 4 x 768, 2000 tokens) the first one, which
+// does not order the stages' stores, gave 220 us, the second 225, the third 250.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_shared(uint32_t cluster_addr) {
+  asm volatile("fence.release.sync_restrict::shared::cta.cluster;\n mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];"
+               ::"r"(cluster_addr) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_release(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
