@@ -1175,40 +1175,50 @@ void few_token_plan(int t, int T, int h, int S, const int* K_r, int n, int sms, 
   if (f.tiles > workers && f.tiles <= kMaxDealItems) few_deal(f, workers, &best->deal);     // else a tile each, or by number
 }
 
-// The plan depends on the shapes alone.  Making one takes 4 us (7B shapes, on the host of the measurements); the 64 used last
-// are kept.  Plans are made outside the lock, so that one thread's new shape holds up no other thread's call.
-struct FewKey { int t, T, h, S, K0, K1, sms; bool operator==(const FewKey& o) const { return !memcmp(this, &o, sizeof(o)); } };
-constexpr int kFewPlans = 64;
+// Plans depend on the shapes (and the device's SMs) alone.  Making one takes 4 us (7B shapes, on the host of the measurements); the
+// 64 used last are kept.  They are made outside the lock, so that one thread's new shape holds up no other thread's call.
+template <typename Plan, int N>
+struct PlanCache {
+  struct Key { int v[N]; bool operator==(const Key& o) const { return !memcmp(v, o.v, sizeof(v)); } };
+  static constexpr int kPlans = 64;
+  Key keys[kPlans];
+  unsigned long long used[kPlans] = {}, clock = 0;      // used == 0: an empty slot
+  Plan plans[kPlans];
+  std::mutex m;
 
-void few_plan_cached(int t, int T, int h, int S, const int* K_r, int n, FewPlan* out) {
-  static FewKey keys[kFewPlans];
-  static unsigned long long used[kFewPlans] = {}, clock = 0;      // used == 0: an empty slot
-  static FewPlan plans[kFewPlans];
-  static std::mutex m;
-  const FewKey key{t, T, h, S, K_r[0], n > 1 ? K_r[1] : 0, sm_count()};
-  auto find = [&] {
-    for (int i = 0; i < kFewPlans; ++i)
+  int find(const Key& key) const {
+    for (int i = 0; i < kPlans; ++i)
       if (used[i] && keys[i] == key) return i;
     return -1;
-  };
-  {
-    std::lock_guard<std::mutex> lock(m);
-    const int i = find();
-    if (i >= 0) {
-      used[i] = ++clock;
-      *out = plans[i];
-      return;
+  }
+  template <typename Make>
+  void get(const Key& key, Plan* out, Make make) {
+    {
+      std::lock_guard<std::mutex> lock(m);
+      const int i = find(key);
+      if (i >= 0) {
+        used[i] = ++clock;
+        *out = plans[i];
+        return;
+      }
     }
+    make(out);
+    std::lock_guard<std::mutex> lock(m);
+    int i = find(key);                  // another thread may have made it meanwhile
+    if (i < 0) {
+      i = (int)(std::min_element(used, used + kPlans) - used);
+      keys[i] = key;
+      plans[i] = *out;
+    }
+    used[i] = ++clock;
   }
-  few_token_plan(t, T, h, S, K_r, n, key.sms, out);
-  std::lock_guard<std::mutex> lock(m);
-  int i = find();                     // another thread may have made it meanwhile
-  if (i < 0) {
-    i = (int)(std::min_element(used, used + kFewPlans) - used);
-    keys[i] = key;
-    plans[i] = *out;
-  }
-  used[i] = ++clock;
+};
+
+void few_plan_cached(int t, int T, int h, int S, const int* K_r, int n, FewPlan* out) {
+  static PlanCache<FewPlan, 7> cache;
+  const int sms = sm_count();
+  cache.get({{t, T, h, S, K_r[0], n > 1 ? K_r[1] : 0, sms}}, out,
+            [&](FewPlan* p) { few_token_plan(t, T, h, S, K_r, n, sms, p); });
 }
 }  // namespace
 
@@ -1224,7 +1234,7 @@ void few_plan_cached(int t, int T, int h, int S, const int* K_r, int n, FewPlan*
 // 300 tokens 50.6 / 37.6; 8 x 2048, 65 tokens 17.9 / 17.9, 300 tokens 37.6 / 34.2; 4 x 1536, 400 tokens 29.4 / 25.2; not taken -
 // 4 x 768, 65 tokens 15.5 / 16.8, 300 tokens 14.6 / 15.0 (short); 2 x 3072, 256 tokens 33.6 / 37.2 (a whole row tile pair);
 // 8 x 2048, 100 tokens 21.1 / 21.9; 8 x 4096, everything shared, 300 tokens 77.0 / 78.5.
-struct MidPlan { bool use; int bn, ncols; double us; };
+struct MidPlan { ForwardPlan one[2]; bool use; int bn, ncols; double us; Deal deal; };      // one: the layers' own plans
 
 constexpr int kMidMaxTokens = 512;
 constexpr double kMidItem = 3.0;                    // of a tile beside its k-steps, in k-steps
@@ -1233,10 +1243,15 @@ static double mid_step_us(int bn) { return 0.09 + 0.10 * bn / 160.0; }
 
 static int mid_workers() { return sm_count() / 2 < kMaxDealWorkers ? sm_count() / 2 : kMaxDealWorkers; }
 
-static MidPlan mid_plan(const RowparShapes* s, const ForwardPlan* f) {
+// max_groups: 1 where the layer has no planes
+static void mid_plan(const RowparShapes* s, const int* max_groups, MidPlan* out) {
   constexpr int n = 2;
-  MidPlan m{};
-  if (s[0].T <= kDecodeMaxTokens || s[0].T > kMidMaxTokens) return m;
+  MidPlan& m = *out;
+  const ForwardPlan* f = m.one;
+  for (int l = 0; l < n; ++l) m.one[l] = forward_plan(s[l], max_groups[l]);
+  m.use = false;
+  m.deal.dealt = 0;
+  if (s[0].T <= kDecodeMaxTokens || s[0].T > kMidMaxTokens) return;
   m.ncols = (s[0].T + 255) / 256;
   m.bn = round_up((s[0].T + m.ncols - 1) / m.ncols, 32);
   FewSplit sp[2];
@@ -1250,21 +1265,25 @@ static MidPlan mid_plan(const RowparShapes* s, const ForwardPlan* f) {
   const FewTiles t = few_tiles(s[0].t, s[0].h, s[0].S, K, n, sp, 2 * BM, m.ncols, kMidItem);
   m.us = us + few_makespan(t, mid_workers()) * mid_step_us(m.bn);
   m.use = t.tiles <= kMaxDealItems && m.us >= kMidShortest && m.us * kMidMargin < 0.2 * (f[0].tile.cost + f[1].tile.cost);
-  return m;
+  if (m.use && t.tiles > mid_workers()) few_deal(t, mid_workers(), &m.deal);
 }
 
-static cudaError_t launch_mid(const RowparShapes* s, const MidPlan& m, const ForwardPlan* fp, const void* const* Y, const void* const* W,
+// the plans of up to kMidMaxTokens tokens are kept; for more there is only forward_plan, once a call as ever
+static void mid_plan_cached(const RowparShapes* s, const int* max_groups, MidPlan* out) {
+  static PlanCache<MidPlan, 9> cache;
+  if (s[0].T > kMidMaxTokens) return mid_plan(s, max_groups, out);
+  cache.get({{s[0].t, s[0].T, s[0].h, s[0].S, s[0].K_r, s[1].K_r, max_groups[0], max_groups[1], sm_count()}}, out,
+            [&](MidPlan* p) { mid_plan(s, max_groups, p); });
+}
+
+static cudaError_t launch_mid(const RowparShapes* s, const MidPlan& m, const void* const* Y, const void* const* W,
                               void* const* zs, void* const* zp, void* const* planes, cudaStream_t st) {
-  constexpr int n = 2;
+  const ForwardPlan* fp = m.one;
   Maps mp;
   Params p{};
   p.BN = m.bn; p.cg = 2; p.splits = 1;
-  FewSplit sp[2];
-  int K[2];
-  for (int l = 0; l < n; ++l) {
+  for (int l = 0; l < 2; ++l) {
     const int ks = (s[l].K_r + BK - 1) / BK;
-    K[l] = s[l].K_r;
-    sp[l] = FewSplit{fp[l].qper, 1};
     if (!make_map(&mp.ab[2 * l], W[l], s[l].K_r, s[l].h, s[l].t, s[l].K_r, (long long)s[l].h * s[l].K_r, BK, BM) ||
         !make_map(&mp.ab[2 * l + 1], Y[l], s[l].K_r, s[l].T, s[l].t, s[l].K_r, (long long)s[l].T * s[l].K_r, BK, p.BN / 2))
       return cudaErrorInvalidValue;
@@ -1288,11 +1307,7 @@ static cudaError_t launch_mid(const RowparShapes* s, const MidPlan& m, const For
   }
   for (CUtensorMap& c : mp.c) c = mp.ab[0];          // unused: the epilogue stores directly
   finish_tiles(p);
-  static thread_local Deal deal;
-  deal.dealt = 0;
-  const FewTiles f = few_tiles(s[0].t, s[0].h, s[0].S, K, n, sp, 2 * BM, m.ncols, kMidItem);
-  if (f.tiles > mid_workers() && f.tiles <= kMaxDealItems) few_deal(f, mid_workers(), &deal);
-  return launch(mp, p, CAAT_K_TC_FORWARD, st, nullptr, &deal);
+  return launch(mp, p, CAAT_K_TC_FORWARD, st, nullptr, &m.deal);
 }
 
 // When the products of a block's two layers share a launch (units of 0.2 us): a launch of its own is worth kLaunchGap, the
@@ -1310,11 +1325,13 @@ constexpr double kLaunchGap = 12, kMargin = 1.05, kLongest = 1200;
 // the backward's) - h 4096, 8192 tokens 1389 / 1394, whole step 3810 / 3832, 65536 tokens of 4 x 768 2309 / 2337.
 cudaError_t launch_tc_forward_block(const RowparShapes* s, const void* const* Y, const void* const* W, void* const* zs,
                                     void* const* zp, void* const* planes, const int* max_groups, int* groups, cudaStream_t st) {
-  const ForwardPlan one[2] = {forward_plan(s[0], planes[0] ? max_groups[0] : 1), forward_plan(s[1], planes[1] ? max_groups[1] : 1)};
-  const MidPlan mid = mid_plan(s, one);
+  static thread_local MidPlan mid;
+  const int room[2] = {planes[0] ? max_groups[0] : 1, planes[1] ? max_groups[1] : 1};
+  mid_plan_cached(s, room, &mid);
+  const ForwardPlan* one = mid.one;
   if (mid.use) {
     for (int l = 0; l < 2; ++l) groups[l] = one[l].groups;
-    return launch_mid(s, mid, one, Y, W, zs, zp, planes, st);
+    return launch_mid(s, mid, Y, W, zs, zp, planes, st);
   }
   const int ks[2] = {(s[0].K_r + BK - 1) / BK, (s[1].K_r + BK - 1) / BK};
   const int lead = ks[1] * one[1].qper >= ks[0] * one[0].qper ? 1 : 0;        // the layer with the longer shared tiles

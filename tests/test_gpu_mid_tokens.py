@@ -19,6 +19,19 @@ pytestmark = pytest.mark.gpu
     (8, 511, 2048, 5632, 520),
 ])
 def test_block_forward_has_the_layers_bits(t, T, h, ffn, S):
+    _same_bits(t, T, h, ffn, S)
+
+
+def test_plans_kept_by_shape_serve_their_own_shape():
+    """More shapes than plans are kept, each of them twice, the second time in the other order; another partition and another
+    set of layers with the same token counts in between."""
+    shapes = [(2, T, 1024, 4096, 512) for T in range(65, 129)] + [(2, T, 1024, 4096, 1024) for T in (65, 100, 128)]
+    shapes += [(4, T, 1024, 3072, 512) for T in (65, 100, 128)]
+    for shape in shapes + shapes[::-1]:
+        _same_bits(*shape)
+
+
+def _same_bits(t, T, h, ffn, S):
     ctx = G.make_ctx(t, h, ffn, "bf16", S=S)
     w = synthetic.Workload("", t, T, h, ffn, S / h, "bf16", "block", False, T + S)
     i = synthetic.block_inputs(w, S, device="cuda")
