@@ -84,7 +84,8 @@ typedef enum {
   CAAT_OPT_PRIVATE_SCALE = 2,   /* alpha; default sqrt(t); 1 switches scaling off       */
   CAAT_OPT_SHARED_CHANNELS = 3, /* override S with an explicit integer in [0, h]        */
   CAAT_OPT_GEMM = 4,            /* 0 = automatic (default; fp32 products of some size run on the tensor
-                                   cores, every operand split exactly into three bf16 parts),
+                                   cores: every operand split exactly into three bf16 parts, what is
+                                   left out of their product is at most 2^-24 of it),
                                    1 = force the CUDA-core GEMM */
   CAAT_OPT_ROWS = 5,            /* row kernels: 0 = automatic (default: warp-per-token kernels for
                                    rows of at most 1024 bf16 channels, bulk-copy staged kernels

@@ -1,14 +1,17 @@
-// fp32 GEMMs on the bf16 tensor cores, with fp32 results at least as accurate as a chain of fp32 FMAs.
+// fp32 GEMMs on the bf16 tensor cores, with errors that on ordinary data are below those of chains of fp32 FMAs.
 //
 // Every fp32 operand is split exactly into three bf16 parts, x = h + m + l (8 + 8 + 8 bits of significand, each rounded
 // to nearest; Henry, Tang, Heinecke, "Leveraging the bfloat16 Artificial Intelligence Datatype For Higher-Precision
 // Computations", 2019), and a product is six products of parts: h h, h m, m h, m m, h l, l h.  What is left out (m l, l m,
-// l l) is below 2^-26 of the product.  The tensor core truncates when it adds to its fp32 accumulator (measured: 16
-// products 2.5e-8 of the result, 64 products 6.5e-8, 1024 products 4.7e-7, a bias towards zero), so an accumulator takes
-// 64 elements of the contraction, smallest parts first, and the epilogue adds those partial sums in fp32 registers, rounded
-// to nearest.  Relative error (2-norm) against 64 bits, chains of FMAs on the CUDA cores / here: 4 x 768, 2000 tokens, layer
-// output 2.1e-7 / 1.2e-7, data gradient 3.5e-7 / 1.1e-7, weight gradient 5.7e-7 / 1.4e-7; 8 x 5120, 60 tokens, the worst of
-// the three 6.4e-7 / 1.9e-7.
+// l l) is at most 2^-24 of the product (x = 1.0038986 = 1 + 2^-8 - 2^-17 squared), as much as one fp32 rounding, and above 2^-26 for
+// 2.8 % of random pairs.  The tensor core truncates when it adds to its fp32 accumulator (measured: 16 products 2.5e-8 of the
+// result, 64 products 6.5e-8, 1024 products 4.7e-7, a bias towards zero), so an accumulator takes 64 elements of the
+// contraction, smallest parts first, and the epilogue adds those partial sums in fp32 registers, rounded to nearest: results are
+// 4e-8 to 6e-8 too small on average, where chains of FMAs have no bias.  Relative error (2-norm) against 64 bits, chains of FMAs
+// on the CUDA cores / here: 4 x 768, 2000 tokens, layer output 2.1e-7 / 1.2e-7, data gradient 3.5e-7 / 1.1e-7, weight gradient
+// 5.7e-7 / 1.4e-7; 8 x 5120, 60 tokens, the worst of the three 6.4e-7 / 1.9e-7; a weight gradient over 16, 64, 256 and 4096
+// tokens 6.0e-8 / 4.8e-8, 1.1e-7 / 7.8e-8, 2.1e-7 / 8.8e-8, 2.9e-7 / 1.2e-7.  Operands made of that x and powers of two, where an FMA
+// chain hardly rounds: 7.7e-8 / 1.3e-7 over 4096.
 //
 // A layer's training step at 4 x 768, 2000 tokens (28 GFLOP of products): 811 -> 275 us (three ring stages per pair instead of two,
 // which leave the first-level cache too little: products 211 -> 230 us).  What bounds a

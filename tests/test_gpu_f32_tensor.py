@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2506_19645_b200 import caat
+from paper_2506_19645_b200 import caat, synthetic
 from tests import gpu_harness as G
 from tests.test_gpu_parity import _check_backward, _check_forward, _layer_case
 
@@ -51,6 +51,21 @@ def test_no_further_from_64_bits_than_fma_chains(t, T, h, ffn, p):
         out.append([_rel(got["Hn"], fo["Hn"]), _rel(gb["dY"], ob["dY"]), _rel(gb["dW"], ob["dW"])])
     for simt, tensor in zip(*out):
         assert tensor < 2.5e-7 and tensor < 1.1 * simt
+
+
+@pytest.mark.parametrize("spread", [0, 2])
+def test_operands_that_lose_the_most(spread):
+    """The square of 1.0038986 (parts 1, 2^-8, -2^-17) loses 2^-24 in the products that are left out, the most any product can.  A
+    sum of such products of one sign loses as much, and the accumulator's truncation and the fp32 additions of the partial
+    sums come on top: each stays below 2^-24 here (6e-8 and less, measured)."""
+    t, T, h, ffn, layer = 1, 2000, 1024, 4096, caat.CAAT_MLP_DOWN
+    ctx = G.make_ctx(t, h, ffn, "f32", S=0, alpha=1.0)
+    d = _layer_case(t, T, h, ctx.k_r(layer), "f32", 0, seed=1)
+    g = torch.Generator().manual_seed(1)
+    for n in ("Y", "W"):
+        d[n] = torch.ldexp(torch.full_like(d[n], 1.0038986206), torch.randint(-spread, spread + 1, d[n].shape, generator=g))
+    d["R"].zero_()
+    assert _rel(G.gpu_forward(ctx, layer, d)["Hn"], G.oracle_forward(ctx, d)["Hn"]) < 3 * 2.0 ** -24
 
 
 @pytest.mark.parametrize("ey,ew", [(-120, 100), (100, -120), (-126, 0), (0, -126), (-100, -30), (-70, -70), (60, 45)])
