@@ -53,7 +53,8 @@ def _colpar_gpu(ctx, act, n_out, d, pre_saved=None):
     (4, 300, 768, 1536, "bf16", False),     # 130M MLP: gate|up of ffn/t = 768
     (8, 257, 2048, 1408, "bf16", False),    # 1.1B MLP: 2 x 704
     (8, 130, 4096, 1536, "bf16", False),    # 7B QKV width 3 h / t
-    (2, 70, 256, 1024, "f32", False),       # fp32 runs on the CUDA-core GEMM
+    (2, 70, 256, 1024, "f32", False),       # a small fp32 product: the CUDA-core GEMM
+    (2, 300, 520, 2064, "f32", False),      # a larger one: three bf16 parts on the tensor cores
     (3, 45, 264, 176, "bf16", True),        # forced CUDA-core GEMM in bf16
     (8, 5000, 1024, 512, "bf16", False),    # many tokens, persistent CTAs walk many tiles
 ])

@@ -68,6 +68,50 @@ def test_operands_that_lose_the_most(spread):
     assert _rel(G.gpu_forward(ctx, layer, d)["Hn"], G.oracle_forward(ctx, d)["Hn"]) < 3 * 2.0 ** -24
 
 
+def _block_and_column_calls(ctx, T, compact, seed):
+    """A block's forward and backward on the layers' scratch, and a column-parallel layer's: every output by name."""
+    t, h, S, f32 = ctx.t, ctx.h, ctx.shared_channels, torch.float32
+    ka, km = ctx.k_r(caat.CAAT_ATTN_OUT), ctx.k_r(caat.CAAT_MLP_DOWN)
+    i = synthetic.block_inputs(synthetic.Workload("", t, T, h, km * t, S / h, "f32", "block", True, seed), S, device="cuda")
+    mk = lambda *s: torch.empty(*s, dtype=f32, device="cuda")  # noqa: E731
+    part = (lambda x: [x[0, :, :S].contiguous(), x[:, :, S:].contiguous()]) if compact else (lambda x: [x])
+    new = (lambda: [mk(T, S), mk(t, T, h - S)]) if compact else (lambda: [mk(t, T, h)])
+    ws = ctx.alloc_workspace(ctx.block_workspace_bytes(T, True))
+    Hn1, X1, r1, Hn2, X2, r2 = new(), mk(t, T, h), mk(t, T), new(), mk(t, T, h), mk(t, T)
+    (ctx.block_forward_compact if compact else ctx.block_forward)(
+        T, i["Y_attn"], i["W_o"], i["Y_mlp"], i["W_down"], *part(i["R0"]), i["gamma1"], None, i["gamma2"], None, *Hn1, X1, r1, None,
+        *Hn2, X2, r2, None, ws)
+    dYa, dWo, dYm, dWd, dR0, dHn1, dg1, dg2 = mk(t, T, ka), mk(t, h, ka), mk(t, T, km), mk(t, h, km), new(), new(), mk(h), mk(h)
+    (ctx.block_backward_compact if compact else ctx.block_backward)(
+        T, i["dX1"], i["dX2"], *part(i["dHn2"]), i["Y_attn"], i["W_o"], i["Y_mlp"], i["W_down"], *Hn1, r1, None, *Hn2, r2, None,
+        i["gamma1"], i["gamma2"], dYa, dWo, dYm, dWd, *dR0, *dHn1, dg1, None, dg2, None, ws)
+    n_out, act = 2 * km, caat.CAAT_ACT_SWIGLU
+    A, pre, Y, dX, dA = torch.cat([i["W_down"], -i["W_down"]], 2).transpose(1, 2).contiguous(), mk(t, T, n_out), mk(t, T, km), mk(t, T, h), mk(t, n_out, h)
+    ctx.colpar_forward(act, n_out, T, i["R0"], A, pre, Y)
+    ctx.colpar_backward(act, n_out, T, i["Y_mlp"], i["R0"], A, pre, dX, dA, ctx.alloc_workspace(ctx.colpar_workspace_bytes(act, n_out, T)))
+    torch.cuda.synchronize()
+    assert ctx.last_device_status() == caat.CAAT_OK
+    return dict(Hn1=Hn1[-1], X1=X1, Hn2=Hn2[-1], X2=X2, Hn1s=Hn1[0], Hn2s=Hn2[0], dYa=dYa, dWo=dWo, dYm=dYm, dWd=dWd, dR0=dR0[-1],
+                dR0s=dR0[0], dg1=dg1, dg2=dg2, pre=pre, Y=Y, dX=dX, dA=dA)
+
+
+@pytest.mark.parametrize("t,T,h,ffn,p,compact", [(4, 700, 768, 3072, 0.5, False), (4, 700, 768, 3072, 0.5, True), (2, 333, 1032, 4128, 0.3, False)])
+def test_blocks_and_column_parallel_layers(t, T, h, ffn, p, compact):
+    """The other entry points' products go the same way, none to the CUDA cores, and give what those give to both sides' rounding."""
+    out = []
+    for force in (True, False):
+        ctx = G.make_ctx(t, h, ffn, "f32", p=p, force_simt=force)
+        caat.profile_begin(64)
+        out.append(_block_and_column_calls(ctx, T, compact, seed=T))
+        kinds = set(caat.profile_end())
+        gemms = {k for k in kinds if "gemm" in k}
+        assert gemms == ({"gemm_cuda_core"} if force else {"tc_gemm_forward", "tc_gemm_dgrad", "tc_gemm_wgrad"})
+    for name, want in out[0].items():
+        got = out[1][name]
+        # chains of up to 4128 products: 6e-7 each side at most, twice through the block's second layer
+        assert float((got - want).double().norm() / want.double().norm()) < 3e-6, name
+
+
 @pytest.mark.parametrize("ey,ew", [(-120, 100), (100, -120), (-126, 0), (0, -126), (-100, -30), (-70, -70), (60, 45)])
 def test_small_and_large_operands(ey, ew):
     """Operands near the smallest normal numbers keep all their bits, products that are not normal and sums that are large

@@ -127,3 +127,25 @@ def test_one_pass_block_kernels_waits_run_out_and_report_timeout():
     line = [int(v) for v in [l for l in out.stdout.splitlines() if l.startswith("STATUS")][-1].split()[1:]]
     assert line[:-1] == [caat.CAAT_ETIMEOUT, caat.CAAT_OK] * 10
     assert line[-1] == 1024
+
+
+MID_CHILD = r"""
+import torch
+from tests.test_gpu_mid_tokens import Block
+b = Block(8, 300, 2048, 5632, 1024)
+b.block(b.R0())
+torch.cuda.synchronize()
+x = torch.ones(1024, device="cuda").sum().item()   # the context still works
+print("STATUS", b.ctx.last_device_status(), b.ctx.last_device_status(), int(x))
+"""
+
+
+def test_block_products_with_weights_on_the_rows_report_timeout():
+    from paper_2506_19645_b200 import caat
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, CAAT_TC_DEBUG="1024", CAAT_TC_SPINCAP="2048", CAAT_TC_VERBOSE="1", PYTHONPATH=root)
+    out = subprocess.run([sys.executable, "-c", MID_CHILD], env=env, cwd=root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    assert "cg=2" in out.stderr and "r0 M=1024 N=300" in out.stderr      # the form that is meant
+    line = [l for l in out.stdout.splitlines() if l.startswith("STATUS")][-1].split()
+    assert [int(v) for v in line[1:]] == [caat.CAAT_ETIMEOUT, caat.CAAT_OK, 1024]
