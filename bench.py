@@ -199,7 +199,7 @@ def step_work(w, S, compact=False):
             for k in ("bytes", "bytes_interface"):
                 if kind in tot:
                     tot[kind][k] -= between
-    if w.dtype == "f32":      # fp32 runs the CUDA-core GEMM (TF32 cannot meet the 1e-4 tolerance)
+    if w.dtype == "f32":      # the fp32 workload's products are small and run the CUDA-core GEMM
         tot["gemm_cuda_core"] = tot.pop("tc_gemm_forward")
     return tot
 

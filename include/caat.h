@@ -45,8 +45,8 @@
  *              aid (one recording at a time, not thread-safe).
  *   Limits     h must be a multiple of 8 and at most 16384 (bf16) or 8192 (fp32) channels,
  *              t * tokens at most 2e9 (CAAT_EUNSUPPORTED otherwise); t divides h and ffn.  The
- *              tensor-core GEMM is used for CAAT_BF16 when K_r is a multiple of 8, for any S;
- *              other shapes run a slower CUDA-core GEMM.
+ *              tensor-core GEMM is used for CAAT_BF16 when K_r is a multiple of 8, for any S, and for
+ *              CAAT_F32 products of some size (see CAAT_OPT_GEMM); the rest runs a slower CUDA-core GEMM.
  */
 #ifndef CAAT_H_
 #define CAAT_H_

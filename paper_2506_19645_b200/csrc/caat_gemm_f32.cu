@@ -53,7 +53,7 @@ constexpr int kPartA = 128 * XK * 2;              // one part of one operand of 
 template <int CG> constexpr int kPartB = kPartA / CG;
 constexpr int kOperandA = 3 * kPartA;
 template <int CG> constexpr int kStageBytes = kOperandA + 3 * kPartB<CG>;
-template <int CG> constexpr int kStages = 2;
+constexpr int kStages = 2;
 constexpr int kAccs = 4;                          // accumulators of 128 columns: all of tensor memory
 constexpr int kEpiWarps = 8, kProdWarp0 = 8, kProdWarps = 16, kMmaWarp = 24;
 // Seven warpgroups at 72 registers; B's producers and the last group (the issuing warp and three idle ones) give up what
@@ -61,8 +61,8 @@ constexpr int kEpiWarps = 8, kProdWarp0 = 8, kProdWarps = 16, kMmaWarp = 24;
 constexpr int kThreads = 896;
 // behind the ring: barriers, the tensor-memory address and the abort flag; then a bit per item (or group of items)
 constexpr int kBarBytes = 256, kMarkWords = 64;
-template <int CG> constexpr int kBars = 2 * kStages<CG> + 2 * kAccs + 3;
-template <int CG> constexpr int kSmem = kStages<CG> * kStageBytes<CG> + 1024 + kBarBytes + 4 * kMarkWords;
+constexpr int kBars = 2 * kStages + 2 * kAccs + 3;
+template <int CG> constexpr int kSmem = kStages * kStageBytes<CG> + 1024 + kBarBytes + 4 * kMarkWords;
 constexpr uint32_t kSpinCap = 1u << 22;
 
 struct XSeg {                 // one segment of the contraction: A(b, q, row, k) and B(b, q, col, k)
@@ -236,7 +236,7 @@ __device__ __forceinline__ void redo_load(uint32_t dst, const float* p, long lon
 // infinite value / all infinite, us: 4 x 768, 2000 tokens 827 / 519 / 694 / 979; 4 x 768, 8192 tokens 3197 / 1808 / 2072 / 3769;
 // 2 x 1024, 300 tokens 296 / 272 / 506 / 607; 8 x 5120, 100 tokens 1585 / 1624 / 2520 / 2952.
 constexpr int kRedoCols = 32, kRedoLdA = XM + 4, kRedoLdB = kRedoCols + 4, kRedoStage = XK * (kRedoLdA + kRedoLdB);
-static_assert(2 * kRedoStage * 4 <= kStages<2> * kStageBytes<2> && XM * kRedoCols == 16 * 256, "");
+static_assert(2 * kRedoStage * 4 <= kStages * kStageBytes<2> && XM * kRedoCols == 16 * 256, "");
 
 template <bool AK, bool BKM, bool VEC>
 __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int j0, int j1, float* stage, int tid) {
@@ -317,8 +317,8 @@ __device__ __forceinline__ void redo_marked(const XParams& p) {
   asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
   asm volatile("mov.u32 %0, %%nctaid.x;" : "=r"(blocks));
   uint8_t* base = ring_base();
-  const unsigned int* marks = reinterpret_cast<const unsigned int*>(base + kStages<CG> * kStageBytes<CG> + kBarBytes);
-  const volatile int* aborted = reinterpret_cast<const volatile int*>(base + kStages<CG> * kStageBytes<CG> + 8 * kBars<CG> + 4);
+  const unsigned int* marks = reinterpret_cast<const unsigned int*>(base + kStages * kStageBytes<CG> + kBarBytes);
+  const volatile int* aborted = reinterpret_cast<const volatile int*>(base + kStages * kStageBytes<CG> + 8 * kBars + 4);
   epi_sync();                                        // the marks are complete; a wait that ran out has raised the flag
   if (epi_all(tid >= kMarkWords || marks[tid % kMarkWords] == 0 || *aborted)) return;
   const int ctas = p.csize * CG, cta = ctas > 1 ? (int)cluster_ctarank() : 0, crank = cta / CG;
@@ -416,7 +416,7 @@ __device__ __forceinline__ void produce(const XParams& p, int tid, int worker, i
     if ((tid & 31) == 0 && !p.stall) {
       if (CG == 2) mbar_arrive_shared(full0 + 8 * stage); else mbar_arrive(full0 + 8 * stage);
     }
-    if (++stage == kStages<CG>) { stage = 0; phase ^= 1u; }
+    if (++stage == kStages) { stage = 0; phase ^= 1u; }
   }
   if (!ok && (tid & 31) == 0) { *abort_flag = 1; atomicExch(p.status, 1u); }
 }
@@ -428,11 +428,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_cons
   uint8_t* base = ring_base();
   const uint32_t ring = smem_u32(base);
   // behind the ring: full, empty (a stage each), tfull[4], tempty[4], ready, data, done, tensor-memory address, abort flag
-  const uint32_t full0 = ring + kStages<CG> * kStageBytes<CG>, empty0 = full0 + 8 * kStages<CG>, tfull0 = empty0 + 8 * kStages<CG>;
+  const uint32_t full0 = ring + kStages * kStageBytes<CG>, empty0 = full0 + 8 * kStages, tfull0 = empty0 + 8 * kStages;
   const uint32_t tempty0 = tfull0 + 8 * kAccs, ready = tempty0 + 8 * kAccs, data = ready + 8, done = data + 8;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + kStages<CG> * kStageBytes<CG> + 8 * kBars<CG>);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + kStages * kStageBytes<CG> + 8 * kBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  unsigned int* marks = reinterpret_cast<unsigned int*>(base + kStages<CG> * kStageBytes<CG> + kBarBytes);
+  unsigned int* marks = reinterpret_cast<unsigned int*>(base + kStages * kStageBytes<CG> + kBarBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int csize = p.csize, ctas = csize * CG, cta = ctas > 1 ? (int)cluster_ctarank() : 0;      // of the cluster
   const int crank = cta / CG, pair_half = cta % CG, leader = cta - pair_half;
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_cons
 
   if (threadIdx.x < kMarkWords) marks[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages<CG>; ++s) { mbar_init(full0 + 8 * s, kProdWarps * CG); mbar_init(empty0 + 8 * s, 1); }
+    for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, kProdWarps * CG); mbar_init(empty0 + 8 * s, 1); }
     for (int a = 0; a < kAccs; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, kEpiWarps * CG); }
     mbar_init(ready, csize); mbar_init(data, csize); mbar_init(done, 1);
     *abort_flag = 0;
@@ -476,50 +476,51 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_cons
     // ------------------------------------------------------------ MMA issuer
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     if (warp == kMmaWarp && pair_half == 0) {
-    const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)!AK << 15) | ((uint32_t)!BKM << 16) | ((uint32_t)((XM * CG) >> 4) << 24);
-    const uint64_t ac = AK ? make_desc(0, 16, 1024) : make_desc(0, 64 * XK * 2, 1024);
-    const uint64_t bc = BKM ? make_desc(0, 16, 1024) : make_desc(0, 64 * XK * 2, 1024);
-    constexpr uint32_t ak16 = (AK ? 32 : 2048) >> 4, bk16 = (BKM ? 32 : 2048) >> 4, pa16 = kPartA >> 4, pb16 = kPartB<CG> >> 4;
-    int stage = 0, acc = 0; uint32_t phase = 0, acc_phase = 0;
-    bool ok = true;
-    for (int n = worker; n < p.items && ok; n += nworkers) {
-      const Item it = item_at<CG>(p, n, crank);
-      if (!it.valid) continue;
-      const uint32_t idesc = idesc0 | ((uint32_t)(it.cols >> 3) << 17);
-      for (int c = it.c0; c < it.c1; ++c) {
-        const bool landed = CG == 2 ? __all_sync(0xffffffffu, mbar_wait_cluster(full0 + 8 * stage, phase, abort_flag, p.spin_cap))
-                                    : mbar_wait_warp(full0 + 8 * stage, phase, abort_flag, p.spin_cap);
-        if (!landed || !mbar_wait_warp(tempty0 + 8 * acc, acc_phase ^ 1u, abort_flag, p.spin_cap)) { ok = false; break; }
-        tc_fence_after();
-        if (elect_one()) {
-          const uint32_t sa = (ring & 0x3FFFFu) + (uint32_t)stage * kStageBytes<CG>;      // without the rank bits of a cluster's address
-          const uint32_t a0 = (uint32_t)ac + (sa >> 4), b0 = (uint32_t)bc + ((sa + kOperandA) >> 4);
-          const uint32_t d = tmem + (uint32_t)(acc * XN);
-          // parts of A, of B (two bits each, first product lowest): h l, l h, m m, h m, m h, h h
-          uint32_t parts_a = 0x118u, parts_b = 0x052u;
+      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)!AK << 15) | ((uint32_t)!BKM << 16) |
+                              ((uint32_t)((XM * CG) >> 4) << 24);
+      const uint64_t ac = AK ? make_desc(0, 16, 1024) : make_desc(0, 64 * XK * 2, 1024);
+      const uint64_t bc = BKM ? make_desc(0, 16, 1024) : make_desc(0, 64 * XK * 2, 1024);
+      constexpr uint32_t ak16 = (AK ? 32 : 2048) >> 4, bk16 = (BKM ? 32 : 2048) >> 4, pa16 = kPartA >> 4, pb16 = kPartB<CG> >> 4;
+      int stage = 0, acc = 0; uint32_t phase = 0, acc_phase = 0;
+      bool ok = true;
+      for (int n = worker; n < p.items && ok; n += nworkers) {
+        const Item it = item_at<CG>(p, n, crank);
+        if (!it.valid) continue;
+        const uint32_t idesc = idesc0 | ((uint32_t)(it.cols >> 3) << 17);
+        for (int c = it.c0; c < it.c1; ++c) {
+          const bool landed = CG == 2 ? __all_sync(0xffffffffu, mbar_wait_cluster(full0 + 8 * stage, phase, abort_flag, p.spin_cap))
+                                      : mbar_wait_warp(full0 + 8 * stage, phase, abort_flag, p.spin_cap);
+          if (!landed || !mbar_wait_warp(tempty0 + 8 * acc, acc_phase ^ 1u, abort_flag, p.spin_cap)) { ok = false; break; }
+          tc_fence_after();
+          if (elect_one()) {
+            const uint32_t sa = (ring & 0x3FFFFu) + (uint32_t)stage * kStageBytes<CG>;      // without the rank bits of a cluster's address
+            const uint32_t a0 = (uint32_t)ac + (sa >> 4), b0 = (uint32_t)bc + ((sa + kOperandA) >> 4);
+            const uint32_t d = tmem + (uint32_t)(acc * XN);
+            // parts of A, of B (two bits each, first product lowest): h l, l h, m m, h m, m h, h h
+            uint32_t parts_a = 0x118u, parts_b = 0x052u;
 #pragma unroll 1
-          for (int q = 0; q < 6; ++q, parts_a >>= 2, parts_b >>= 2) {
-            uint32_t al = a0 + (parts_a & 3u) * pa16, bl = b0 + (parts_b & 3u) * pb16;
+            for (int q = 0; q < 6; ++q, parts_a >>= 2, parts_b >>= 2) {
+              uint32_t al = a0 + (parts_a & 3u) * pa16, bl = b0 + (parts_b & 3u) * pb16;
 #pragma unroll
-            for (int k = 0; k < XK / 16; ++k) {
-              const uint64_t ad = (ac & 0xffffffff00000000ull) | (al + k * ak16), bd = (bc & 0xffffffff00000000ull) | (bl + k * bk16);
-              if (CG == 2) umma_bf16_pair(d, ad, bd, idesc, q + k > 0 ? 1u : 0u); else umma_bf16(d, ad, bd, idesc, q + k > 0 ? 1u : 0u);
+              for (int k = 0; k < XK / 16; ++k) {
+                const uint64_t ad = (ac & 0xffffffff00000000ull) | (al + k * ak16), bd = (bc & 0xffffffff00000000ull) | (bl + k * bk16);
+                if (CG == 2) umma_bf16_pair(d, ad, bd, idesc, q + k > 0 ? 1u : 0u); else umma_bf16(d, ad, bd, idesc, q + k > 0 ? 1u : 0u);
+              }
+            }
+            if (CG == 2) {
+              umma_commit_ctas(empty0 + 8 * stage, 3u << leader);
+              umma_commit_ctas(tfull0 + 8 * acc, 3u << leader);
+            } else {
+              umma_commit(empty0 + 8 * stage);
+              umma_commit(tfull0 + 8 * acc);
             }
           }
-          if (CG == 2) {
-            umma_commit_ctas(empty0 + 8 * stage, 3u << leader);
-            umma_commit_ctas(tfull0 + 8 * acc, 3u << leader);
-          } else {
-            umma_commit(empty0 + 8 * stage);
-            umma_commit(tfull0 + 8 * acc);
-          }
+          __syncwarp();
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          if (++acc == kAccs) { acc = 0; acc_phase ^= 1u; }
         }
-        __syncwarp();
-        if (++stage == kStages<CG>) { stage = 0; phase ^= 1u; }
-        if (++acc == kAccs) { acc = 0; acc_phase ^= 1u; }
       }
-    }
-    if (!ok && lane == 0) { *abort_flag = 1; atomicExch(p.status, 2u); }
+      if (!ok && lane == 0) { *abort_flag = 1; atomicExch(p.status, 2u); }
     }
   } else {
     // ------------------------------------------------------------ epilogue: 32 rows x 64 columns per warp
@@ -659,7 +660,8 @@ XProblem convert(const GemmProblem& g, bool ak, bool bk, bool swap, int cg) {
   return x;
 }
 
-// microseconds, fitted to the sizes above: a chunk of 64 of the contraction of a CTA's (a pair's) tile, what a tile costs beside its chunks, and a tile summed over a cluster on top
+// microseconds, fitted to the sizes above: a chunk of 64 of the contraction of a CTA's (a pair's) tile, what a tile costs beside
+// its chunks, and a tile summed over a cluster on top
 constexpr double kChunkUs[2] = {2.2, 1.7}, kTileUs = 1.0, kReduceUs = 4.0;
 
 double chunk_us(const XProblem& g, int cg) {      // narrow tiles: the A parts cost what they cost

@@ -1229,9 +1229,13 @@ void few_plan_cached(int t, int T, int h, int S, const int* K_r, int n, FewPlan*
 // groups of ranks.  The groups are the normal forward's and every output's products are added in the same order, so the sums are
 // the same bits either way.
 // The rule: cheaper than the two layers' tiles by 5 % of the models' figures, and not so short that the launch alone decides.
+// Of 280 sizes (seven models from 2 x 1024 to 8 x 5120, p = 0, 0.25, 0.5, 0.75, 1, eight token counts from 65 to 512; replayed from
+// graphs) 113 are taken, at 0.72 to 1.01 of the time with tokens on the rows.  The models underrate the gain elsewhere, and
+// sizes are refused that would be faster here: 8 x 4096, 65 / 100 / 128 tokens 48.8 / 41.3, 54.0 / 46.8, 57.6 / 50.0; 2 x 3072,
+// 400 / 512 tokens 53.7 / 43.0, 57.2 / 47.3; 8 x 5120, 256 / 512 tokens 95.8 / 89.1, 171.7 / 145.7; 4 x 1536, 512 tokens 29.1 / 26.9.
 // Block forward on either side of the line, tokens on the rows / here, us: taken - 8 x 4096, 200 tokens 72.5 / 59.6, 300 tokens
 // 88.1 / 74.7, 400 tokens 93.6 / 88.0, nothing shared 78.3 / 69.9; 8 x 5120, 200 tokens 99.3 / 80.2, 300 tokens 118 / 106; 2 x 3072,
-// 300 tokens 50.6 / 37.6; 8 x 2048, 65 tokens 17.9 / 17.9, 300 tokens 37.6 / 34.2; 4 x 1536, 400 tokens 29.4 / 25.2; not taken -
+// 300 tokens 50.6 / 37.6; 8 x 2048, 65 tokens 17.9 / 17.9, 300 tokens 37.6 / 34.2; 4 x 1536, 400 tokens 29.4 / 25.2; not taken and rightly so -
 // 4 x 768, 65 tokens 15.5 / 16.8, 300 tokens 14.6 / 15.0 (short); 2 x 3072, 256 tokens 33.6 / 37.2 (a whole row tile pair);
 // 8 x 2048, 100 tokens 21.1 / 21.9; 8 x 4096, everything shared, 300 tokens 77.0 / 78.5.
 struct MidPlan { ForwardPlan one[2]; bool use; int bn, ncols; double us; Deal deal; };      // one: the layers' own plans

@@ -86,7 +86,8 @@ def _block_and_column_calls(ctx, T, compact, seed):
         T, i["dX1"], i["dX2"], *part(i["dHn2"]), i["Y_attn"], i["W_o"], i["Y_mlp"], i["W_down"], *Hn1, r1, None, *Hn2, r2, None,
         i["gamma1"], i["gamma2"], dYa, dWo, dYm, dWd, *dR0, *dHn1, dg1, None, dg2, None, ws)
     n_out, act = 2 * km, caat.CAAT_ACT_SWIGLU
-    A, pre, Y, dX, dA = torch.cat([i["W_down"], -i["W_down"]], 2).transpose(1, 2).contiguous(), mk(t, T, n_out), mk(t, T, km), mk(t, T, h), mk(t, n_out, h)
+    A = torch.cat([i["W_down"], -i["W_down"]], 2).transpose(1, 2).contiguous()
+    pre, Y, dX, dA = mk(t, T, n_out), mk(t, T, km), mk(t, T, h), mk(t, n_out, h)
     ctx.colpar_forward(act, n_out, T, i["R0"], A, pre, Y)
     ctx.colpar_backward(act, n_out, T, i["Y_mlp"], i["R0"], A, pre, dX, dA, ctx.alloc_workspace(ctx.colpar_workspace_bytes(act, n_out, T)))
     torch.cuda.synchronize()
