@@ -462,10 +462,7 @@ tc_gemm_kernel(const __grid_constant__ MapsT<MIXED> mp, const __grid_constant__ 
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          // SWAP == 2 stores from registers, and a release would wait for those stores (8 x 4096, 300 tokens: 84.0 us, not 82.1)
-          if (CG == 2 && SWAP == 2) mbar_arrive_remote(mapa_rank(tempty0 + 8u * acc, 0));
-          else if (CG == 2) mbar_arrive_release(mapa_rank(tempty0 + 8u * acc, 0));
-          else mbar_arrive(tempty0 + 8u * acc);
+          if (CG == 2) mbar_arrive_remote(mapa_rank(tempty0 + 8u * acc, 0)); else mbar_arrive(tempty0 + 8u * acc);
         }
       };
       if constexpr (SWAP == 1) {
