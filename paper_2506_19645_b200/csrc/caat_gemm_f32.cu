@@ -759,6 +759,11 @@ cudaError_t launch_layout(bool ak, bool bk, const XParams& p, int ctas, int kind
 // Products of fewer operations than this stay on the CUDA cores, whose 32 x 32 tiles are spread over more SMs.  Either side of
 // the lines (layer, CUDA cores / here, us): forward, 0.07 GFLOP 12.1 / 16.0, 0.21 GFLOP 27.2 / 20.4, 0.30 GFLOP 19.5 / 17.2;
 // backward, 0.13 GFLOP a product 25.8 / 28.5 (2 x 256) but 44.2 / 26.3 (2 x 512), 0.15 GFLOP 40.6 / 34.4.
+// Above them forward products of few tiles and a long contraction stay there, which the plan below puts behind the CUDA cores'
+// (simt_forward_us): layer forward, 64 tokens of h 128, K 16384 23.5 / 60.7; 256 tokens 39.8 / 75.9; 100 tokens of 256,
+// 8192 23.7 / 42.5; 512 tokens of 64, 4096 15.5 / 23.7 - but 1024 tokens of 128, 16384 138 / 77; 64 tokens of 8 x 2048, 5632 at
+// p = 0.9 153 / 67.  (720 shapes of 0.02 to 5 GFLOP, timed from graphs: 85 were slower here than on the CUDA cores, up to 2.6 times;
+// now 22, by 22 % and less, most by 1 to 2 us.)
 constexpr double kMinForward = 2.0e8, kMinGradient = 1.45e8;
 
 bool launch_gemm_f32(const GemmProblem* problems, int n, bool ak, bool bk, bool vec, cudaStream_t st, cudaError_t* err) {
@@ -802,6 +807,7 @@ bool launch_gemm_f32(const GemmProblem* problems, int n, bool ak, bool bk, bool 
       }
     }
   }
+  if (ak && bk && best >= simt_forward_us(problems, n)) return false;
   p.status = device_status_word();
   if (!p.status) { *err = cudaErrorUnknown; return true; }
   static const uint32_t cap_env = [] { const char* e = getenv("CAAT_TC_SPINCAP"); return e ? (uint32_t)atoi(e) : 0u; }();

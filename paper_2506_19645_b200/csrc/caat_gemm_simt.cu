@@ -451,6 +451,19 @@ void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int
   cfg.numAttrs = pdl_enabled() ? 2 : 1;
 }
 
+// cluster size of the warp-tile kernel (tiles set): a power of two up to the portable size, while every warp has a k-tile
+int small_cluster(const GemmList& L, int* ktiles_out) {
+  const int slots = 2 * sm_count(), tiles = L.tile_end[L.n - 1];
+  int ktiles = 1, csize = 1;            // of the longest contraction
+  for (int i = 0; i < L.n; ++i) {
+    const int k = ktiles_of<SB>(L.p[i]);
+    if (k > ktiles) ktiles = k;
+  }
+  while (csize < 8 && 2 * csize * kSmallWarps <= ktiles && 2 * tiles * csize <= slots) csize *= 2;
+  *ktiles_out = ktiles;
+  return csize;
+}
+
 // Gradients of at least this much work per SM, in k-tiles of the CTA-tile kernel (0.26 MFLOP), run on it.  Measured
 // (whole backward of a layer, warp tiles / CTA tiles): 5.4 per SM 39 / 46 us, 13.8 67 / 57 us, 31 132 / 97 us.  Forward
 // products stay on the warp tiles at any size: 61 per SM 86 us against 119 on CTA tiles with the operands transposed on
@@ -490,13 +503,8 @@ cudaError_t launch_layout(GemmList& L, cudaStream_t st) {
   }
   set_tiles(L, SB, SB);
   const int tiles = L.tile_end[L.n - 1];
-  int ktiles = 1;                       // of the longest contraction
-  for (int i = 0; i < L.n; ++i) {
-    const int k = ktiles_of<SB>(L.p[i]);
-    if (k > ktiles) ktiles = k;
-  }
-  int csize = 1;                        // a power of two up to the portable cluster size, while every warp has a k-tile
-  while (csize < 8 && 2 * csize * kSmallWarps <= ktiles && 2 * tiles * csize <= slots) csize *= 2;
+  int ktiles;
+  const int csize = small_cluster(L, &ktiles);
   const int nbuf = ktiles > csize * kSmallWarps && tiles * csize <= sm_count() ? 2 : 1;
   const size_t smem = ((size_t)kSmallWarps * nbuf * kWarpTile + SB * SB) * sizeof(float);
   auto kernel = gemm_simt_small<T_, AK, BKF, VEC>;
@@ -521,6 +529,25 @@ cudaError_t launch_typed(GemmList& L, bool ak, bool bk, cudaStream_t st) {
 }
 
 }  // namespace
+
+// A forward product's time on the warp-tile kernel on the scale of the tensor-core kernel's plan (caat_gemm_f32.cu), in us: the
+// serial k-tiles of a warp and the k-tiles per SM.  Where no product is wider than a tile on its narrow side the
+// tensor-core kernel's tiles are at their emptiest, which its plan does not see.
+double simt_forward_us(const GemmProblem* problems, int n) {
+  GemmList L{};
+  bool narrow = true;
+  for (int i = 0; i < n; ++i) {
+    L.p[L.n++] = problems[i];
+    narrow &= problems[i].M <= SB || problems[i].N <= SB;
+  }
+  set_tiles(L, SB, SB);
+  int ktiles;
+  const int csize = small_cluster(L, &ktiles);
+  double work = 0;
+  for (int i = 0; i < L.n; ++i) work += (double)(L.tile_end[i] - (i ? L.tile_end[i - 1] : 0)) * ktiles_of<SB>(L.p[i]);
+  const int serial = (ktiles + csize * kSmallWarps - 1) / (csize * kSmallWarps);
+  return (2.25 * serial + 0.20 * work / sm_count()) * (narrow ? 0.8 : 1.0);
+}
 
 cudaError_t launch_gemm_simt(const GemmProblem* problems, int n, caat_dtype dtype, int force_simt, cudaStream_t st) {
   GemmList L{};

@@ -84,6 +84,7 @@ struct GemmProblem {
 // n <= 2 products that do not depend on each other, of one operand layout (forward, data or weight gradient), in one launch
 // fp32 products large enough for it run on the tensor cores (launch_gemm_f32) unless force_simt is set
 cudaError_t launch_gemm_simt(const GemmProblem* problems, int n, caat_dtype dtype, int force_simt, cudaStream_t st);
+double simt_forward_us(const GemmProblem* problems, int n);     // at most two products, none empty
 // ak / bk: k is the unit stride of A / B (else the row / column is); vec: every address along the unit strides is on a
 // 16-byte boundary.  false: the products are left to the CUDA cores; else *err is the launch's result.
 bool launch_gemm_f32(const GemmProblem* problems, int n, bool ak, bool bk, bool vec, cudaStream_t st, cudaError_t* err);

@@ -29,8 +29,40 @@ pytestmark = pytest.mark.gpu
 def test_f32_layer(t, T, h, ffn, layer, S):
     ctx = G.make_ctx(t, h, ffn, "f32", S=S)
     d = _layer_case(t, T, h, ctx.k_r(layer), "f32", S, seed=T + S, backward=True)
+    caat.profile_begin(64)
     _check_forward(ctx, layer, d, "f32")
     _check_backward(ctx, layer, d, "f32")
+    assert "gemm_cuda_core" not in caat.profile_end()
+
+
+@pytest.mark.parametrize("t,T,h,ffn,S,stays", [
+    (1, 64, 128, 16384, 64, "forward"),         # two row tiles and a contraction of 256 chunks
+    (1, 100, 256, 8192, 256, "forward"),
+    (1, 1024, 128, 16384, 64, ""),              # the same contraction, tiles for all SMs
+])
+def test_products_that_stay_on_the_cuda_cores(t, T, h, ffn, S, stays):
+    """Of the layer's three products the named one and no other; every output against the CUDA cores alone."""
+    layer, out, kinds = caat.CAAT_MLP_DOWN, [], None
+    for force in (True, False):
+        ctx = G.make_ctx(t, h, ffn, "f32", S=S, force_simt=force)
+        d = synthetic.layer_inputs(t, T, h, ctx.k_r(layer), "f32", seed=T, S=S, backward=True, device="cuda")
+        o = ctx.alloc_forward_outputs(T)
+        o.update(ctx.alloc_backward_outputs(layer, T))
+        ws = ctx.alloc_workspace(ctx.workspace_bytes(layer, T, True))
+        caat.profile_begin(64)
+        ctx.rowpar_forward(layer, T, d["Y"], d["W"], d["R"], d["gamma"], None, o["Hn"], o["X"], o["rstd"], None, ws)
+        ctx.rowpar_backward(layer, T, d["dX"], d["dHn"], d["Y"], d["W"], o["Hn"], o["rstd"], None, d["gamma"], o["dY"], o["dW"],
+                            o["dR"], o["dgamma"], None, ws)
+        torch.cuda.synchronize()
+        assert ctx.last_device_status() == caat.CAAT_OK
+        kinds = {k for k in caat.profile_end() if "gemm" in k}
+        out.append(o)
+    here = {"tc_gemm_forward", "tc_gemm_dgrad", "tc_gemm_wgrad"} - {"tc_gemm_" + stays}
+    assert kinds == here | ({"gemm_cuda_core"} if stays else set())
+    for name in ("Hn", "dY", "dW", "dR"):
+        a, b = out[0][name].double(), out[1][name].double()
+        # chains of up to 16384 products on the CUDA cores: 2^-24 sqrt(16384) / 2 = 3.8e-6 at most, through the norm into the gradients
+        assert float((a - b).norm() / a.norm()) < 8e-6, name
 
 
 def _rel(a, b):
