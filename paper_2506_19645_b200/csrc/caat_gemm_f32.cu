@@ -662,7 +662,10 @@ XProblem convert(const GemmProblem& g, bool ak, bool bk, bool swap, int cg) {
 
 // microseconds, fitted to the sizes above: a chunk of 64 of the contraction of a CTA's (a pair's) tile, what a tile costs beside
 // its chunks, and a tile summed over a cluster on top
-constexpr double kChunkUs[2] = {2.2, 1.7}, kTileUs = 1.0, kReduceUs = 4.0;
+// a tile that is stored element by element with the results' contiguous axis along a thread's columns, not along the lanes (backward at
+// p = 0.9, CUDA cores / without regard to it / here: 8 x 2048, 5632, 16 tokens 169 / 148 / 83, 64 tokens 218 / 166 / 93; 8 x 4096,
+// 11008, 16 tokens 597 / 472 / 240; long contractions choose as before: 4 x 1536, 333 tokens 163 / 163)
+constexpr double kChunkUs[2] = {2.2, 1.7}, kTileUs = 1.0, kReduceUs = 4.0, kScatterUs = 3.0;
 
 double chunk_us(const XProblem& g, int cg) {      // narrow tiles: the A parts cost what they cost
   const int last = g.N % XN, w = last ? (last + 15) / 16 * 16 : XN;
@@ -671,12 +674,12 @@ double chunk_us(const XProblem& g, int cg) {      // narrow tiles: the A parts c
 }
 
 // time of the busiest cluster, items dealt round-robin, problem after problem
-double plan_cost(const XProblem* g, int n, int cg, int csize, const int* split, int workers) {
+double plan_cost(const XProblem* g, int n, int cg, int csize, const int* split, int workers, bool vec) {
   double load_all = 0, worst = 0, len[2];
   long long items[2] = {0, 0};
   for (int i = 0; i < n; ++i) {
     const double c = split[i] ? (double)((g[i].chunks + csize - 1) / csize) : (double)g[i].chunks;
-    len[i] = c * chunk_us(g[i], cg) + kTileUs + (split[i] ? kReduceUs : 0.0);
+    len[i] = c * chunk_us(g[i], cg) + kTileUs + (split[i] ? kReduceUs : 0.0) + (!vec && g[i].sCj == 1 ? kScatterUs / (split[i] ? csize : 1) : 0.0);
     items[i] = split[i] ? g[i].tiles : (g[i].tiles + csize - 1) / csize;
     load_all += items[i] * len[i];
   }
@@ -792,7 +795,7 @@ bool launch_gemm_f32(const GemmProblem* problems, int n, bool ak, bool bk, bool 
         bool can = true;
         for (int i = 0; i < n; ++i) can &= !split[i] || g[i].chunks >= c;
         if (!can) continue;
-        const double cost = plan_cost(g, n, pair, c, split, workers);
+        const double cost = plan_cost(g, n, pair, c, split, workers, vec);
         if (best >= 0 && cost >= best) continue;
         best = cost; best_swap = swap != 0; cg = pair;
         p.nprob = n; p.csize = c;

@@ -39,6 +39,7 @@ def test_f32_layer(t, T, h, ffn, layer, S):
     (1, 64, 128, 16384, 64, "forward"),         # two row tiles and a contraction of 256 chunks
     (1, 100, 256, 8192, 256, "forward"),
     (1, 1024, 128, 16384, 64, ""),              # the same contraction, tiles for all SMs
+    (8, 64, 1024, 2816, 921, ""),               # short contractions, element by element: the results' contiguous axis on the lanes
 ])
 def test_products_that_stay_on_the_cuda_cores(t, T, h, ffn, S, stays):
     """Of the layer's three products the named one and no other; every output against the CUDA cores alone."""
