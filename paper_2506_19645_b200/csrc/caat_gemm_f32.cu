@@ -152,13 +152,17 @@ constexpr float kScale = 65536.f;
 __device__ __forceinline__ float2 less(float2 x, uint32_t part) {      // x minus a pair of parts: exact
   return __ffma2_rn(make_float2(__uint_as_float(part << 16), __uint_as_float(part & 0xffff0000u)), make_float2(-1.f, -1.f), x);
 }
+__device__ __forceinline__ uint32_t scaled(uint32_t h) {
+  const __nv_bfloat162 b = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&h), __float2bfloat162_rn(kScale));
+  return *reinterpret_cast<const uint32_t*>(&b);
+}
 template <int PART>
 __device__ __forceinline__ void split_store(const float (&v)[8], uint32_t dst) {
   uint32_t h[4], m[4], l[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     float2 x = make_float2(v[2 * q], v[2 * q + 1]);
-    h[q] = bf16x2(x.x * kScale, x.y * kScale);
+    h[q] = scaled(bf16x2(x.x, x.y));
     x = make_float2(fmaf(x.x, kScale, -__uint_as_float(h[q] << 16)), fmaf(x.y, kScale, -__uint_as_float(h[q] & 0xffff0000u)));
     m[q] = bf16x2(x.x, x.y);
     x = less(x, m[q]);
