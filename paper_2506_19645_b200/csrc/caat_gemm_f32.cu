@@ -152,7 +152,7 @@ constexpr float kScale = 65536.f;
 __device__ __forceinline__ float2 less(float2 x, uint32_t part) {      // x minus a pair of parts: exact
   return __ffma2_rn(make_float2(__uint_as_float(part << 16), __uint_as_float(part & 0xffff0000u)), make_float2(-1.f, -1.f), x);
 }
-__device__ __forceinline__ uint32_t scaled(uint32_t h) {
+__device__ __forceinline__ uint32_t scaled(uint32_t h) {      // a pair of first parts: exact, and one instruction for both
   const __nv_bfloat162 b = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&h), __float2bfloat162_rn(kScale));
   return *reinterpret_cast<const uint32_t*>(&b);
 }
@@ -211,38 +211,35 @@ __device__ __forceinline__ int mark_of(int items, int n, int worker, int nworker
   while (items / nworkers >> shift >= 32 * kMarkWords) ++shift;
   return (n - worker) / nworkers >> shift;
 }
-template <int BYTES>
-__device__ __forceinline__ void cp_async(uint32_t dst, const float* src, int bytes) {      // zeros behind the first `bytes`
-  if (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-// ROWS x 64 elements of an operand into [k][row] by 256 threads.  k contiguous: a warp copies 8 k of 4 rows at a time, whole sectors
-// into 32 banks (LD is 4 more than a multiple of 32).
-template <bool KM, bool VEC, int ROWS, int LD>
-__device__ __forceinline__ void redo_load(uint32_t dst, const float* p, long long ld, int rows, int k_left, int tid) {
-  constexpr int W = VEC && !KM ? 4 : 1, LANES = ROWS / W;               // elements of a copy, copies of a k
-  constexpr int STEP = KM ? 4 : 256 / LANES, N = KM ? ROWS / 4 : XK / STEP;
-  const int k = KM ? (tid >> 5) * 8 + (tid & 7) : tid / LANES, r = KM ? tid >> 3 & 3 : tid % LANES * W;
-  const int slow = KM ? r : k, slow_end = KM ? rows : k_left;
-  const int left = KM ? k_left - k : rows - r, bytes = 4 * (left <= 0 ? 0 : (left < W ? left : W));
+// ROWS x 64 elements of an operand into [k][row] by 256 threads.  k contiguous: a warp takes 8 k of 4 rows at a time, whole sectors
+// into 32 banks (LD is 4 more than a multiple of 32).  Through registers: with one cp.async anywhere in the kernel, executed or not,
+// the producers' fences above wait longer (three products of a step at 4 x 768, 2000 tokens: 218 -> 226 us).
+template <bool KM, int ROWS, int LD>
+__device__ __forceinline__ void redo_load(float* dst, const float* p, long long ld, int rows, int k_left, int tid) {
+  constexpr int STEP = KM ? 4 : 256 / ROWS, N = KM ? ROWS / 4 : XK / STEP, B = 8;       // B loads in flight
+  const int k = KM ? (tid >> 5) * 8 + (tid & 7) : tid / ROWS, r = KM ? tid >> 3 & 3 : tid % ROWS;
+  const int slow = KM ? r : k, slow_end = (KM ? k < k_left : r < rows) ? (KM ? rows : k_left) : 0;
   const float* src = p + slow * ld + (KM ? k : r);
-  dst += (uint32_t)((k * LD + r) * 4);
-#pragma unroll 4
-  for (int u = 0; u < N; ++u, src += STEP * ld, dst += STEP * (KM ? 1 : LD) * 4) {
-    const int take = slow + u * STEP < slow_end ? bytes : 0;
-    cp_async<4 * W>(dst, take ? src : p, take);
+  dst += k * LD + r;
+#pragma unroll 1
+  for (int u = 0; u < N; u += B, src += B * STEP * ld, dst += B * STEP * (KM ? 1 : LD)) {
+    float v[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) v[b] = slow + (u + b) * STEP < slow_end ? src[b * STEP * ld] : 0.f;
+#pragma unroll
+    for (int b = 0; b < B; ++b) dst[b * STEP * (KM ? 1 : LD)] = v[b];
   }
 }
 // The results of 128 rows from i0 and the columns [j0, j1) that are not finite, from the operands by chains of 64 FMAs, added up in
 // fp32.  The epilogue's 256 threads, 32 columns at a time, 4 x 4 results per thread, both operands two chunks deep in `stage`
 // (the ring).  A warp whose 16 rows need nothing (finite, or NaN by now) only helps to load.  Two warps per scheduler bound it,
 // and the few CTAs that hold marked tiles.  A training step of one layer, CUDA cores (any data) / here with one infinite token / one
-// infinite value / all infinite, us: 4 x 768, 2000 tokens 827 / 519 / 694 / 979; 4 x 768, 8192 tokens 3197 / 1808 / 2072 / 3769;
-// 2 x 1024, 300 tokens 296 / 272 / 506 / 607; 8 x 5120, 100 tokens 1585 / 1624 / 2520 / 2952.
+// infinite value / all infinite, us: 4 x 768, 2000 tokens 827 / 610 / 824 / 1134; 2 x 1024, 300 tokens 296 / 316 / 603 / 709;
+// 8 x 5120, 100 tokens 1585 / 2021 / 3412 / 3999.
 constexpr int kRedoCols = 32, kRedoLdA = XM + 4, kRedoLdB = kRedoCols + 4, kRedoStage = XK * (kRedoLdA + kRedoLdB);
 static_assert(2 * kRedoStage * 4 <= kStages * kStageBytes<2> && XM * kRedoCols == 16 * 256, "");
 
-template <bool AK, bool BKM, bool VEC>
+template <bool AK, bool BKM>
 __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int j0, int j1, float* stage, int tid) {
   const int r4 = (tid >> 3) * 4, c4 = (tid & 7) * 4;
   if (j1 > g.N) j1 = g.N;
@@ -259,10 +256,9 @@ __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int 
       const XSeg& s = g.seg[pos.seg];
       const float* A = s.A + b * s.sAb + pos.q * s.sAq + (AK ? i0 * s.sAl + pos.k0 : pos.k0 * s.sAl + i0);
       const float* B = s.B + b * s.sBb + pos.q * s.sBq + (BKM ? jc * s.sBl + pos.k0 : pos.k0 * s.sBl + jc);
-      const uint32_t dst = smem_u32(stage + (n & 1) * kRedoStage);
-      redo_load<AK, VEC, XM, kRedoLdA>(dst, A, s.sAl, g.M - i0, s.Kd - pos.k0, tid);
-      redo_load<BKM, VEC, kRedoCols, kRedoLdB>(dst + XK * kRedoLdA * 4, B, s.sBl, g.N - jc, s.Kd - pos.k0, tid);
-      asm volatile("cp.async.commit_group;" ::: "memory");
+      float* dst = stage + (n & 1) * kRedoStage;
+      redo_load<AK, XM, kRedoLdA>(dst, A, s.sAl, g.M - i0, s.Kd - pos.k0, tid);
+      redo_load<BKM, kRedoCols, kRedoLdB>(dst + XK * kRedoLdA, B, s.sBl, g.N - jc, s.Kd - pos.k0, tid);
     };
     float sum[16];
 #pragma unroll
@@ -270,12 +266,7 @@ __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int 
     load(0);
 #pragma unroll 1
     for (int n = 0; n < g.chunks; ++n) {
-      if (n + 1 < g.chunks) {
-        load(n + 1);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-      } else {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-      }
+      if (n + 1 < g.chunks) load(n + 1);
       epi_sync();
       if (!idle) {
         const float* A = stage + (n & 1) * kRedoStage + r4;
@@ -300,8 +291,6 @@ __device__ __forceinline__ void redo_tile(const XProblem& g, int b, int i0, int 
       }
       if (epi_all(idle)) break;
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    epi_sync();                                      // the next columns' copies go where these were read, or still land
 #pragma unroll
     for (int e = 0; e < 16; ++e)
       if (todo >> e & 1u) out[(e >> 2) * g.sCi + (e & 3) * g.sCj] = sum[e];
@@ -314,7 +303,7 @@ __device__ __forceinline__ uint8_t* ring_base() {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
 }
-template <int CG, bool AK, bool BKM, bool VEC>
+template <int CG, bool AK, bool BKM>
 __device__ __forceinline__ void redo_marked(const XParams& p) {
   uint32_t tid, block, blocks;
   asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
@@ -332,7 +321,7 @@ __device__ __forceinline__ void redo_marked(const XParams& p) {
     const Item it = item_at<CG>(p, n, crank);
     if (!(marks[m >> 5] >> (m & 31) & 1u) || !it.valid) continue;
     const int cw = XN / p.csize, j0 = it.split ? it.j0 + crank * cw : it.j0;      // the columns that this CTA stored
-    redo_tile<AK, BKM, VEC>(p.p[it.prob], it.b, it.i0 + cta % CG * XM, j0, it.split ? j0 + cw : j0 + XN, reinterpret_cast<float*>(base), tid);
+    redo_tile<AK, BKM>(p.p[it.prob], it.b, it.i0 + cta % CG * XM, j0, it.split ? j0 + cw : j0 + XN, reinterpret_cast<float*>(base), tid);
   }
 }
 
@@ -627,7 +616,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_f32_kernel(const __grid_cons
       }
     }
     if (!ok && lane == 0) { *abort_flag = 1; atomicExch(p.status, 3u); }
-    redo_marked<CG, AK, BKM, VEC>(p);
+    redo_marked<CG, AK, BKM>(p);
   }
 
   tc_fence_before();
