@@ -13,7 +13,7 @@
 // tokens 6.0e-8 / 4.8e-8, 1.1e-7 / 7.8e-8, 2.1e-7 / 8.8e-8, 2.9e-7 / 1.2e-7.  Operands made of that x and powers of two, where an FMA
 // chain hardly rounds: 7.7e-8 / 1.3e-7 over 4096.
 //
-// A layer's training step at 4 x 768, 2000 tokens (28 GFLOP of products): 811 -> 275 us (three ring stages per pair instead of two,
+// A layer's training step at 4 x 768, 2000 tokens (28 GFLOP of products): 811 -> 270 us (three ring stages per pair instead of two,
 // which leave the first-level cache too little: products 211 -> 230 us).  What bounds a
 // stage (2.4 to 4 k cycles where its 24 products take 1.5 k) is the way round: loads, split, stores, barrier, products, barrier.
 //
@@ -213,7 +213,7 @@ __device__ __forceinline__ int mark_of(int items, int n, int worker, int nworker
 }
 // ROWS x 64 elements of an operand into [k][row] by 256 threads.  k contiguous: a warp takes 8 k of 4 rows at a time, whole sectors
 // into 32 banks (LD is 4 more than a multiple of 32).  Through registers: with one cp.async anywhere in the kernel, executed or not,
-// the producers' fences above wait longer (three products of a step at 4 x 768, 2000 tokens: 218 -> 226 us).
+// the producers' fences above wait longer (three products of a step at 4 x 768, 2000 tokens: 217 -> 225 us).
 template <bool KM, int ROWS, int LD>
 __device__ __forceinline__ void redo_load(float* dst, const float* p, long long ld, int rows, int k_left, int tid) {
   constexpr int STEP = KM ? 4 : 256 / ROWS, N = KM ? ROWS / 4 : XK / STEP, B = 8;       // B loads in flight

@@ -144,7 +144,7 @@ __device__ __forceinline__ void cluster_sync() {
 // 256 tokens 27.3 / 27.3 / 28.8; 4 x 1536, 512 tokens 26.7 / 26.7 / 28.2; 8 x 4096, 300 tokens, whose epilogue stores from
 // registers, 82.1 / - / 84.0 with inputs rotated.
 // In a loop that fills operand stages from global memory (fp32 products of a step at 4 x 768, 2000 tokens) the first one, which
-// does not order the stages' stores, gave 220 us, the second 225, the third 250.
+// does not order the stages' stores, and the second one give 214 us, the third 244.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
